@@ -318,8 +318,8 @@ typedef enum {
  * is set in kernel_mask is bracketed by two CUDA events recorded on its
  * launch stream, for at most max_launches groups per id.  A group is the
  * kernels one step launches back to back under that id: one for
- * EXTREMES, OCTAGON, SORT_HIST, SORT_PASS (one per pass), FINISH; two for
- * EMIT (offsets, copy); two for FILTER with the two-pass schedule (count,
+ * EXTREMES, OCTAGON, SORT_HIST, SORT_PASS (one per pass), EMIT (the chain
+ * ranges' output offsets), FINISH (their copy); two for FILTER with the two-pass schedule (count,
  * scatter; in ch_hull each is its own group, KGON runs between them), one
  * with the single pass; two for CHAIN (chains, tree merge); for KGON three
  * (fan vertices, estimate, refine of the keep decisions; the count pass

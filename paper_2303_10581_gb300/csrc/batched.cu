@@ -156,27 +156,6 @@ __global__ void __launch_bounds__(kSetupThreads) bx_hullsize_kernel(void *ws, Ba
     if (threadIdx.x == 0) hull_offsets[B] = (int64_t)total;
 }
 
-// Output position p of the concatenated hulls -> its set (binary search over
-// hull_offsets) -> the lower chain, or the upper chain read backwards.
-__global__ void __launch_bounds__(256) bx_assemble_kernel(void *ws, Layout L, BatchLayout BL,
-                                                          const int64_t *__restrict__ hull_offsets, uint32_t *hull_idx)
-{
-    const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    if (bc->abort) return;
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const uint32_t *off0 = at<uint32_t>(ws, BL.sc_off[0]), *off1 = at<uint32_t>(ws, BL.sc_off[1]);
-    const uint32_t *lower = at<uint32_t>(ws, BL.lower), *upper = at<uint32_t>(ws, L.utmp);
-    const int64_t B = BL.num_sets;
-    const int64_t H = hull_offsets[B];
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < H; p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = last_le(B, (uint64_t)p, [&](int64_t i) { return (uint64_t)hull_offsets[i]; });
-        uint32_t l0, hl, u0, hu;
-        set_chain_sizes(sets[b], off0, off1, l0, hl, u0, hu);
-        const int64_t k = p - hull_offsets[b];
-        hull_idx[p] = k < hl ? lower[l0 + k] : upper[u0 + hu - 2 - (k - hl)];
-    }
-}
-
 }  // namespace
 
 cudaError_t launch_bx_setup(const int64_t *offsets, void *ws, const Layout &L, const BatchLayout &BL, int64_t n_cap,
@@ -194,8 +173,8 @@ cudaError_t launch_bx_finish(void *ws, const Layout &L, const BatchLayout &BL, u
 {
     probe_before(CH_K_FINISH, st);
     bx_hullsize_kernel<<<1, kSetupThreads, 0, st>>>(ws, BL, hull_offsets);
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.n, 256), sm_count() * 4));
-    bx_assemble_kernel<<<(unsigned)blocks, 256, 0, st>>>(ws, L, BL, hull_offsets, hull_idx);
+    const cudaError_t e = launch_bx_assemble(ws, L, BL, hull_offsets, hull_idx, st);
+    if (e != cudaSuccess) return e;
     note_kernels(CH_K_FINISH, 2);
     probe_after(CH_K_FINISH, st);
     return cudaGetLastError();

@@ -43,11 +43,13 @@
 //     chain; chunks whose range empties are unlinked from a list of live
 //     chunks.  Upper chains are handled the same way with the predicate
 //     mirrored.
-//  3. emit: one pass compacts the live ranges (decoupled look-back over
-//     super-chunk counts) into the lower chain and the upper chain, and the
-//     final kernel appends the upper chain, reversed and without its end
-//     points, behind the lower one: counter-clockwise from the
-//     lexicographically smallest point.
+//  3. emit: one pass finds the live ranges' output offsets (decoupled
+//     look-back over super-chunk counts), and the final kernel copies them
+//     to the hull: the lower chain, then the upper chain reversed and
+//     without its end points: counter-clockwise from the lexicographically
+//     smallest point.
+#include <algorithm>
+
 #include "common.cuh"
 #include "launch.h"
 
@@ -811,24 +813,17 @@ __global__ void __launch_bounds__(32) bx_merge_kernel(void *ws, Layout L, BatchL
     climb(P, j - sets[b].sc_base, sets[b].nsc, sets[b].sc_base, sets[b].node_base);
 }
 
-// Compacts the live chain ranges of super-chunks [0, nc): thread =
-// super-chunk, look-back over tiles of super-chunks, then the whole block
-// copies the tile's ranges (the original indices: low half of the payload),
-// each thread finding the super-chunk of an output position by binary
-// search over the tile's offsets.  Side 0 goes to out0, side 1 to out1.
-// With sc_off, each super-chunk's output offset per side is recorded too
-// (sc_off[side][nc] = side total).
-// copy = false: only the offsets (sc_off required); emit_copy_kernel then
-// writes the ranges with the whole grid.
+// Output offsets of the live chain ranges of super-chunks [0, nc), per side:
+// thread = super-chunk, look-back over tiles of kEmitThreads super-chunks.
+// sc_off[side][c] receives the entries of the ranges before c,
+// sc_off[side][nc] and h_total the side's total.
 struct EmitArgs {
-    uint32_t *out[2];
     uint32_t *sc_off[2];
     uint32_t *ticket;
     uint32_t *h_total[2];
-    bool copy;
 };
 
-__device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t nc, uint64_t s, const EmitArgs &E)
+__device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t nc, const EmitArgs &E)
 {
     const int64_t ntiles = ceil_div(nc, kEmitThreads);
     unsigned long long *status[2] = {at<unsigned long long>(ws, L.emit_status[0]),
@@ -837,9 +832,6 @@ __device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t
     __shared__ uint32_t s_tile;
     __shared__ uint32_t s_wsum[2][NW];
     __shared__ unsigned long long s_excl[2];
-    __shared__ uint32_t s_rel[2][kEmitThreads];   // offset of each super-chunk's range in the tile's output
-    __shared__ int32_t s_lo[2][kEmitThreads];     // and its first chain slot
-    __shared__ uint32_t s_tot[2];
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     for (;;) {
         if (tid == 0) s_tile = atomicAdd(E.ticket, 1u);
@@ -847,13 +839,12 @@ __device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t
         const int64_t tile = s_tile;
         if (tile >= ntiles) break;
         const int64_t c = tile * kEmitThreads + tid;
-        int32_t lo[2] = {0, 0}, cnt[2] = {0, 0};
+        int32_t cnt[2] = {0, 0};
         if (c < nc) {
 #pragma unroll
             for (int side = 0; side < 2; ++side) {
-                lo[side] = __ldcg(P.lo[side] + c);
-                const int32_t hi = __ldcg(P.hi[side] + c);
-                cnt[side] = hi >= lo[side] ? hi - lo[side] + 1 : 0;
+                const int32_t lo = __ldcg(P.lo[side] + c), hi = __ldcg(P.hi[side] + c);
+                cnt[side] = hi >= lo ? hi - lo + 1 : 0;
             }
         }
         uint32_t pre[2];
@@ -890,112 +881,92 @@ __device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t
             }
             if (lane == 0) {
                 s_excl[side] = excl;
-                s_tot[side] = total;
                 if (tile == ntiles - 1) {
                     *E.h_total[side] = (uint32_t)(excl + total);
-                    if (E.sc_off[side]) E.sc_off[side][nc] = (uint32_t)(excl + total);
+                    E.sc_off[side][nc] = (uint32_t)(excl + total);
                 }
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int side = 0; side < 2; ++side) {
-            const uint32_t rel = s_wsum[side][warp] + pre[side];
-            s_rel[side][tid] = rel;
-            s_lo[side][tid] = lo[side];
-            if (E.sc_off[side] && c < nc) E.sc_off[side][c] = (uint32_t)(s_excl[side] + rel);
-        }
-        __syncthreads();
-        if (!E.copy) continue;   // (the loop's first barrier orders the next tile's shared writes)
-        constexpr int B4 = 4;   // output positions per thread in flight
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-            const uint32_t T = s_tot[side];
-            const uint64_t excl = s_excl[side];
-            uint32_t *out = E.out[side];
-            const uint32_t *chain = P.pos[side];
-            for (uint32_t k0 = 0; k0 < T; k0 += B4 * kEmitThreads) {
-                uint32_t sp[B4];
-#pragma unroll
-                for (int u = 0; u < B4; ++u) {
-                    const uint32_t k = k0 + u * kEmitThreads + tid;
-                    sp[u] = 0u;
-                    if (k < T) {
-                        // the last super-chunk whose range starts at or before k
-                        // (empty ranges share their start with the next one)
-                        int lo_j = 0, hi_j = kEmitThreads - 1;
-                        while (lo_j < hi_j) {
-                            const int mid = (lo_j + hi_j + 1) >> 1;
-                            if (s_rel[side][mid] <= k) lo_j = mid;
-                            else hi_j = mid - 1;
-                        }
-                        const int64_t ci = tile * kEmitThreads + lo_j;
-                        sp[u] = __ldcg(chain + ci * CS + s_lo[side][lo_j] + (k - s_rel[side][lo_j]));
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < B4; ++u) {
-                    const uint32_t k = k0 + u * kEmitThreads + tid;
-                    if (k < T && excl + k < (uint64_t)s) out[excl + k] = (uint32_t)__ldg(P.pay + sp[u]);
-                }
-            }
-        }
-        __syncthreads();
+        for (int side = 0; side < 2; ++side)
+            if (c < nc) E.sc_off[side][c] = (uint32_t)(s_excl[side] + s_wsum[side][warp] + pre[side]);
+        // (the loop's first barrier orders the next tile's shared writes)
     }
 }
 
-__global__ void __launch_bounds__(kEmitThreads) emit_kernel(void *ws, Layout L, uint32_t *hull_idx)
+// One warp copies a part of super-chunk c's live range of one side to its
+// place in the hull: chain entry g of the side (off0: its entries before
+// this super-chunk) goes to position g on the lower side; the upper chain
+// (hu entries) follows the hl lower ones reversed and without its two ends.
+// The warp knows where its range goes, so no position is searched for and
+// the chains are copied once.  limit: positions the hull may fill (only a
+// look-back that gave up could pass it).
+constexpr int kCopyParts = 4;                  // a range is shared by so many warps
+constexpr int kCopyLen = CS / kCopyParts;      // entries per part
+static_assert(CS % kCopyParts == 0, "parts cover a super-chunk's slots");
+
+__device__ __forceinline__ void copy_chain_part(const ChainPtrs &P, int side, int64_t c, int part, uint32_t off0,
+                                                uint32_t hl, uint32_t hu, uint32_t *out, int64_t limit)
+{
+    const int32_t lo = __ldcg(P.lo[side] + c), cnt = __ldcg(P.hi[side] + c) - lo + 1;
+    const int32_t k1 = min(cnt, (part + 1) * kCopyLen);
+    const uint32_t *chain = P.pos[side] + c * CS + lo;
+    constexpr int U = 4;   // entries per lane in flight
+    for (int32_t k0 = part * kCopyLen + (int32_t)lane_id(); k0 < k1; k0 += 32 * U) {
+        uint32_t sp[U], ix[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) sp[u] = k0 + 32 * u < k1 ? __ldcg(chain + k0 + 32 * u) : 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) ix[u] = k0 + 32 * u < k1 ? (uint32_t)__ldg(P.pay + sp[u]) : 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k0 + 32 * u >= k1) continue;
+            const uint32_t g = off0 + (uint32_t)(k0 + 32 * u);
+            if (side == 1 && (g == 0u || g + 1u >= hu)) continue;   // the ends are the lower chain's
+            const int64_t p = side == 0 ? (int64_t)g : (int64_t)hl + (hu - 2u - g);
+            if (p < limit) out[p] = ix[u];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kEmitThreads) emit_kernel(void *ws, Layout L)
 {
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
     if (s == 0) return;
     const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
-    EmitArgs E{{hull_idx, at<uint32_t>(ws, L.utmp)},
-               {at<uint32_t>(ws, L.emit_off[0]), at<uint32_t>(ws, L.emit_off[1])},
+    EmitArgs E{{at<uint32_t>(ws, L.emit_off[0]), at<uint32_t>(ws, L.emit_off[1])},
                &ctrl->emit_ticket[0],
-               {&ctrl->h_lower, &ctrl->h_upper},
-               false};
-    emit_body(ws, L, P, ceil_div((int64_t)s, SC), s, E);
+               {&ctrl->h_lower, &ctrl->h_upper}};
+    emit_body(ws, L, P, ceil_div((int64_t)s, SC), E);
 }
 
-// The chains' surviving ranges into the outputs (lower chain to hull_idx,
-// upper chain to utmp: original indices, the low half of the payload),
-// every thread of the grid on its own output positions: the super-chunk
-// of position k is the last one whose offset (emit_off) is at most k
-// (binary search; an empty range shares its offset with the next one).
-// A hull with many vertices on few super-chunks (the unit circle after
-// the fan: about 2000 per super-chunk) is no longer copied by one block.
-__global__ void __launch_bounds__(kEmitThreads) emit_copy_kernel(void *ws, Layout L, uint32_t *hull_idx)
+// The hull and its vertex count: the chains' surviving ranges (original
+// indices, the low half of the payload) straight to their positions, a warp
+// per part of a super-chunk's range.
+__global__ void __launch_bounds__(kEmitThreads) hull_copy_kernel(void *ws, Layout L, uint32_t *hull_idx,
+                                                                 uint32_t *hull_count)
 {
     const Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
-    const Octagon *oct = at<Octagon>(ws, L.oct);
-    const uint32_t s = hull_stage_count(ctrl, oct);
+    if (ctrl->small_done) return;
+    const uint32_t hl = ctrl->h_lower, hu = ctrl->h_upper;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *hull_count = hl == 0 ? 0u : hl + (hu >= 2 ? hu - 2 : 0u);
+    const uint32_t s = hull_stage_count(ctrl, at<Octagon>(ws, L.oct));
     if (s == 0) return;
     const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
-    const int32_t nc = (int32_t)ceil_div((int64_t)s, SC);
-    const uint32_t gtid = blockIdx.x * kEmitThreads + threadIdx.x, gthreads = gridDim.x * kEmitThreads;
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-        const uint32_t T = side ? ctrl->h_upper : ctrl->h_lower;
-        const uint32_t *off = at<uint32_t>(ws, L.emit_off[side]);
-        uint32_t *out = side ? at<uint32_t>(ws, L.utmp) : hull_idx;
-        for (uint32_t k = gtid; k < T && k < s; k += gthreads) {
-            int lo_j = 0, hi_j = nc - 1;
-            while (lo_j < hi_j) {
-                const int mid = (lo_j + hi_j + 1) >> 1;
-                if (__ldg(off + mid) <= k) lo_j = mid;
-                else hi_j = mid - 1;
-            }
-            const uint32_t sp =
-                __ldcg(P.pos[side] + (int64_t)lo_j * CS + __ldcg(P.lo[side] + lo_j) + (k - __ldg(off + lo_j)));
-            out[k] = (uint32_t)__ldg(P.pay + sp);
-        }
+    const int64_t items = ceil_div((int64_t)s, SC) * 2 * kCopyParts;
+    const int64_t warps = (int64_t)gridDim.x * (kEmitThreads / 32);
+    for (int64_t it = ((int64_t)blockIdx.x * kEmitThreads + threadIdx.x) >> 5; it < items; it += warps) {
+        const int64_t c = it / (2 * kCopyParts);
+        const int side = (int)(it / kCopyParts) & 1;
+        copy_chain_part(P, side, c, (int)(it % kCopyParts), __ldg(at<uint32_t>(ws, L.emit_off[side]) + c), hl, hu,
+                        hull_idx, L.n);
     }
 }
 
-// all sets at once: lower chains to the batch's lower array, upper chains
-// to utmp, each set's part delimited by the per-super-chunk offsets
+// all sets at once: the offsets of every super-chunk's ranges
 __global__ void __launch_bounds__(kEmitThreads) bx_emit_kernel(void *ws, Layout L, BatchLayout BL)
 {
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -1003,26 +974,37 @@ __global__ void __launch_bounds__(kEmitThreads) bx_emit_kernel(void *ws, Layout 
     const int64_t nc = bc->nsc;
     if (nc == 0) return;
     const ChainPtrs P = chain_ptrs(ws, L, 0);
-    EmitArgs E{{at<uint32_t>(ws, BL.lower), at<uint32_t>(ws, L.utmp)},
-               {at<uint32_t>(ws, BL.sc_off[0]), at<uint32_t>(ws, BL.sc_off[1])},
+    EmitArgs E{{at<uint32_t>(ws, BL.sc_off[0]), at<uint32_t>(ws, BL.sc_off[1])},
                &bc->emit_ticket,
-               {&bc->h_lower, &bc->h_upper},
-               true};
-    emit_body(ws, L, P, nc, (uint64_t)L.n, E);
+               {&bc->h_lower, &bc->h_upper}};
+    emit_body(ws, L, P, nc, E);
 }
 
-// hull = lower chain, then the upper chain reversed without its two ends
-__global__ void finish_kernel(void *ws, Layout L, uint32_t *hull_idx, uint32_t *hull_count)
+// The sets' hulls: as hull_copy_kernel, every set's part of the output at
+// its hull_offsets entry (a set's hull has at most as many vertices as the
+// set has points).
+__global__ void __launch_bounds__(kEmitThreads) bx_assemble_kernel(void *ws, Layout L, BatchLayout BL,
+                                                                   const int64_t *__restrict__ hull_offsets,
+                                                                   uint32_t *hull_idx)
 {
-    Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
-    if (ctrl->small_done) return;
-    const uint32_t hl = ctrl->h_lower, hu = ctrl->h_upper;
-    const uint32_t mid = hu >= 2 ? hu - 2 : 0;
-    const uint32_t *utmp = at<uint32_t>(ws, L.utmp);
-    const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < mid; m += gthreads)
-        if (hl + m < L.n) hull_idx[hl + m] = utmp[hu - 2 - m];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *hull_count = hl == 0 ? 0u : hl + mid;
+    const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
+    if (bc->abort) return;
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const uint32_t *sc_set = at<uint32_t>(ws, BL.sc_set);
+    const uint32_t *off[2] = {at<uint32_t>(ws, BL.sc_off[0]), at<uint32_t>(ws, BL.sc_off[1])};
+    const ChainPtrs P = chain_ptrs(ws, L, 0);
+    const int64_t items = (int64_t)bc->nsc * 2 * kCopyParts;
+    const int64_t warps = (int64_t)gridDim.x * (kEmitThreads / 32);
+    for (int64_t it = ((int64_t)blockIdx.x * kEmitThreads + threadIdx.x) >> 5; it < items; it += warps) {
+        const int64_t j = it / (2 * kCopyParts);
+        const int side = (int)(it / kCopyParts) & 1;
+        const SetInfo &S = sets[sc_set[j]];
+        const int64_t ho = hull_offsets[sc_set[j]];
+        const uint32_t l0 = off[0][S.sc_base], u0 = off[1][S.sc_base];
+        copy_chain_part(P, side, j, (int)(it % kCopyParts), off[side][j] - (side ? u0 : l0),
+                        off[0][S.sc_base + S.nsc] - l0, off[1][S.sc_base + S.nsc] - u0, hull_idx + ho,
+                        S.pt_begin + S.n - ho);
+    }
 }
 
 // Few survivors (at most kSmallHull): one block sorts them by (x, y, index)
@@ -1148,17 +1130,14 @@ cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t
     if (eb > (int64_t)sms * 4) eb = (int64_t)sms * 4;
     if (eb < 1) eb = 1;
     probe_before(CH_K_EMIT, st);
-    emit_kernel<<<(unsigned)eb, kEmitThreads, 0, st>>>(ws, L, hull_idx);
-    emit_copy_kernel<<<(unsigned)sms * 4, kEmitThreads, 0, st>>>(ws, L, hull_idx);
-    note_kernels(CH_K_EMIT, 2);
+    emit_kernel<<<(unsigned)eb, kEmitThreads, 0, st>>>(ws, L);
+    note_kernels(CH_K_EMIT, 1);
     probe_after(CH_K_EMIT, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    int64_t fb = ceil_div(L.n, 256 * 8);
-    if (fb > (int64_t)sms * 4) fb = (int64_t)sms * 4;
-    if (fb < 1) fb = 1;
+    const int64_t fb = std::min<int64_t>(ceil_div(L.n_chunks * 2 * kCopyParts, kEmitThreads / 32), (int64_t)sms * 4);
     probe_before(CH_K_FINISH, st);
-    finish_kernel<<<(unsigned)fb, 256, 0, st>>>(ws, L, hull_idx, hull_count);
+    hull_copy_kernel<<<(unsigned)fb, kEmitThreads, 0, st>>>(ws, L, hull_idx, hull_count);
     note_kernels(CH_K_FINISH, 1);
     probe_after(CH_K_FINISH, st);
     return cudaGetLastError();
@@ -1191,6 +1170,15 @@ cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cu
     bx_emit_kernel<<<(unsigned)eb, kEmitThreads, 0, st>>>(ws, L, BL);
     note_kernels(CH_K_EMIT, 1);
     probe_after(CH_K_EMIT, st);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bx_assemble(void *ws, const Layout &L, const BatchLayout &BL, const int64_t *hull_offsets,
+                               uint32_t *hull_idx, cudaStream_t st)
+{
+    const int64_t blocks =
+        std::min<int64_t>(ceil_div(BL.tiles_max * 2 * kCopyParts, kEmitThreads / 32), (int64_t)sm_count() * 8);
+    bx_assemble_kernel<<<(unsigned)blocks, kEmitThreads, 0, st>>>(ws, L, BL, hull_offsets, hull_idx);
     return cudaGetLastError();
 }
 

@@ -293,7 +293,7 @@ struct BatchLayout {
     size_t tile_set;      // u32[tiles_max]: set of each point tile
     size_t sc_set;        // u32[tiles_max]: set of each super-chunk
     size_t sc_off[2];     // u32[tiles_max + 1]: lower / upper chain offset of each super-chunk
-    size_t lower;         // u32[n]: lower chains of all sets (set-local indices); aliases keys[1]
+    size_t lower;         // keys[1] again: free for the stages after the sort, which ends in buffer 0
     // the fan of the hull step, per set with many octagon survivors (kgon.cu)
     size_t soct;          // u32[B]: octagon survivors per set (in the zeroed range)
     size_t fan_id;        // i32[B]: the set's fan number, -1: none
@@ -396,7 +396,7 @@ __host__ __device__ inline BatchLayout make_batch_layout(const Layout &L, int64_
     B.sc_set = take((size_t)B.tiles_max * 4);
     B.sc_off[0] = take((size_t)(B.tiles_max + 1) * 4);
     B.sc_off[1] = take((size_t)(B.tiles_max + 1) * 4);
-    B.lower = L.keys[1];   // the second sort buffer is free once the sort ends in buffer 0
+    B.lower = L.keys[1];
     // a set with a fan has at least 2^16 points
     B.max_fan = sets < L.n / 65536 + 1 ? sets : L.n / 65536 + 1;
     B.max_items = B.tiles_max / kBxFanChunkMin + B.max_fan + 1;

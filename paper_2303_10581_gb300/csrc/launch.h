@@ -114,6 +114,9 @@ cudaError_t launch_bx_filter(const float *pts, void *ws, const Layout &L, const 
 cudaError_t launch_bx_fan(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
 cudaError_t launch_bx_sort(void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
 cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
+// copies every set's chains to its part of hull_idx (after hull_offsets)
+cudaError_t launch_bx_assemble(void *ws, const Layout &L, const BatchLayout &BL, const int64_t *hull_offsets,
+                               uint32_t *hull_idx, cudaStream_t st);
 cudaError_t launch_bx_finish(void *ws, const Layout &L, const BatchLayout &BL, uint32_t *hull_idx,
                              int64_t *hull_offsets, cudaStream_t st);
 
