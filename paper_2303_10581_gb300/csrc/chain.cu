@@ -1008,92 +1008,109 @@ __global__ void __launch_bounds__(kEmitThreads) bx_assemble_kernel(void *ws, Lay
 }
 
 // Few survivors (at most kSmallHull): one block sorts them by (x, y, index)
-// in shared memory (bitonic network over the packed keys and indices),
-// then one thread runs Andrew's monotone chain over them -- equal points
-// collapse to the first, a turn that is not strictly counter-clockwise
-// (exact sign) pops the middle point -- and writes the hull, counter-
-// clockwise from the first point; the sort and chain kernels launched
-// after it then stop at once.  More survivors: it does nothing.
+// -- a bitonic network with one point per thread, exchanged by shuffles
+// within a warp -- drops repeated points (the first, of the lowest index,
+// stays), and two warps run the strict-turn elimination passes of the chain
+// kernel, one per side, until nothing changes: a sequence with only strict
+// turns is its own monotone chain.  The later sort and chain kernels then
+// stop at once.  More survivors: it does nothing.
+// Bound by latency.  One thread's sequential chain took 60 of this kernel's
+// 67 us on the 69 survivors of 10^8 normal points (three dependent shared
+// loads and an orientation per step); the passes look at every point at
+// once and there are few of them.
 constexpr int kSmallHull = 512;
-constexpr int kSmallThreads = 256;
 
-__global__ void __launch_bounds__(kSmallThreads) small_hull_kernel(void *ws, Layout L, uint32_t *hull_idx,
-                                                                   uint32_t *hull_count)
+struct SmallSmem {
+    unsigned long long sk[kSmallHull];   // ord(x) << 32 | ord(y)
+    uint32_t si[kSmallHull];             // point index
+    float2 pt[kSmallHull];
+    uint16_t list[2][2][kSmallHull];     // per side: the sequence and the pass's output
+    uint32_t wsum[kSmallHull / 32];
+    int len[2], cur[2];
+};
+
+__global__ void __launch_bounds__(kSmallHull) small_hull_kernel(void *ws, Layout L, uint32_t *hull_idx,
+                                                                uint32_t *hull_count)
 {
+    __shared__ SmallSmem sm;
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
     if (s == 0 || s > (uint32_t)kSmallHull) return;
-    __shared__ unsigned long long sk[kSmallHull];   // ord(x) << 32 | ord(y)
-    __shared__ uint32_t si[kSmallHull];             // point index
-    __shared__ uint16_t st[2 * kSmallHull + 2];     // chain stack: sorted positions
-    const uint32_t *keys = at<uint32_t>(ws, L.keys[ctrl->sort_in]);
-    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[ctrl->sort_in]);
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5, lt = (1u << lane) - 1u;
+    unsigned long long k = ~0ull;   // after every point
+    uint32_t ix = ~0u;
+    if (t < s) {
+        const unsigned long long pv = at<unsigned long long>(ws, L.pay[ctrl->sort_in])[t];
+        k = ((unsigned long long)at<uint32_t>(ws, L.keys[ctrl->sort_in])[t] << 32) | (pv >> 32);
+        ix = (uint32_t)pv;
+    }
     uint32_t m = 32;
     while (m < s) m <<= 1;
-    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
-        if (i < s) {
-            const unsigned long long pv = pay[i];
-            sk[i] = ((unsigned long long)keys[i] << 32) | (pv >> 32);
-            si[i] = (uint32_t)pv;
-        } else {
-            sk[i] = ~0ull;   // after every point
-            si[i] = ~0u;
+    for (uint32_t g = 2; g <= m; g <<= 1) {
+        for (uint32_t j = g >> 1; j > 0; j >>= 1) {
+            unsigned long long ok;
+            uint32_t oi;
+            if (j >= 32) {
+                sm.sk[t] = k;
+                sm.si[t] = ix;
+                __syncthreads();
+                ok = sm.sk[t ^ j];
+                oi = sm.si[t ^ j];
+                __syncthreads();
+            } else {
+                ok = __shfl_xor_sync(0xffffffffu, k, j);
+                oi = __shfl_xor_sync(0xffffffffu, ix, j);
+            }
+            const bool less = k < ok || (k == ok && ix < oi);   // (padding entries are equal: either order)
+            if (less != (((t & g) == 0) == ((t & j) == 0))) {
+                k = ok;
+                ix = oi;
+            }
+        }
+    }
+    sm.sk[t] = k;
+    __syncthreads();
+    // equal points: the first stays
+    const bool first = t < s && (t == 0 || sm.sk[t - 1] != k);
+    const uint32_t bal = __ballot_sync(0xffffffffu, first);
+    if (lane == 0) sm.wsum[warp] = __popc(bal);
+    __syncthreads();
+    uint32_t before = 0, u = 0;
+#pragma unroll
+    for (int w = 0; w < kSmallHull / 32; ++w) {
+        if (w < (int)warp) before += sm.wsum[w];
+        u += sm.wsum[w];
+    }
+    if (first) {
+        const uint32_t p = before + __popc(bal & lt);
+        sm.pt[p] = key_point(k);
+        sm.si[p] = ix;
+        sm.list[0][0][p] = sm.list[1][0][p] = (uint16_t)p;
+    }
+    __syncthreads();
+    if (warp < 2) {
+        int len = (int)u, cur = 0;
+        while (len > 2) {   // each pass but the last drops a point
+            const int kept = warp_elim_pass(sm.pt, sm.list[warp][cur], sm.list[warp][cur ^ 1], len, (int)warp,
+                                            (int)lane, lt);
+            cur ^= 1;
+            if (kept == len) break;
+            len = kept;
+        }
+        if (lane == 0) {
+            sm.len[warp] = len;
+            sm.cur[warp] = cur;
         }
     }
     __syncthreads();
-    for (uint32_t k = 2; k <= m; k <<= 1) {
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
-                const uint32_t l = i ^ j;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const bool gt = sk[i] > sk[l] || (sk[i] == sk[l] && si[i] > si[l]);
-                    if (gt == up) {
-                        const unsigned long long tk = sk[i];
-                        sk[i] = sk[l];
-                        sk[l] = tk;
-                        const uint32_t ti = si[i];
-                        si[i] = si[l];
-                        si[l] = ti;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+    const uint32_t hl = (uint32_t)sm.len[0], hu = (uint32_t)sm.len[1], mid = hu >= 2 ? hu - 2 : 0;
+    if (t < hl) hull_idx[t] = sm.si[sm.list[0][sm.cur[0]][t]];
+    if (t < mid) hull_idx[hl + t] = sm.si[sm.list[1][sm.cur[1]][hu - 2 - t]];
+    if (t == 0) {
+        *hull_count = hl + mid;
+        ctrl->small_done = 1u;
     }
-    if (threadIdx.x != 0) return;
-    // equal points: the first (lowest index) stays
-    uint32_t u = 0;
-    for (uint32_t i = 0; i < s; ++i) {
-        if (u > 0 && sk[i] == sk[u - 1]) continue;
-        sk[u] = sk[i];
-        si[u] = si[i];
-        ++u;
-    }
-    auto px = [&](uint32_t k) { return key_float((uint32_t)(sk[k] >> 32)); };
-    auto py = [&](uint32_t k) { return key_float((uint32_t)sk[k]); };
-    uint32_t h = 0;
-    if (u == 1) {
-        hull_idx[0] = si[0];
-        h = 1;
-    } else {
-        for (uint32_t k = 0; k < u; ++k) {   // lower chain, left to right
-            while (h >= 2 && orient(px(st[h - 2]), py(st[h - 2]), px(st[h - 1]), py(st[h - 1]), px(k), py(k)) <= 0)
-                --h;
-            st[h++] = (uint16_t)k;
-        }
-        const uint32_t base = h + 1;
-        for (int k = (int)u - 2; k >= 0; --k) {   // upper chain, right to left
-            while (h >= base && orient(px(st[h - 2]), py(st[h - 2]), px(st[h - 1]), py(st[h - 1]), px(k), py(k)) <= 0)
-                --h;
-            st[h++] = (uint16_t)k;
-        }
-        --h;   // the last point is the first again
-        for (uint32_t k = 0; k < h; ++k) hull_idx[k] = si[st[k]];
-    }
-    *hull_count = h;
-    ctrl->small_done = 1u;
 }
 
 }  // namespace
@@ -1101,7 +1118,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_hull_kernel(void *ws, Lay
 cudaError_t launch_small_hull(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
 {
     probe_before(CH_K_CHAIN, st);
-    small_hull_kernel<<<1, kSmallThreads, 0, st>>>(ws, L, hull_idx, hull_count);
+    small_hull_kernel<<<1, kSmallHull, 0, st>>>(ws, L, hull_idx, hull_count);
     note_kernels(CH_K_CHAIN, 1);
     probe_after(CH_K_CHAIN, st);
     return cudaGetLastError();
