@@ -10,11 +10,12 @@
 // MLP: 1024 -> 64 -> 64 -> 68 (4 K-logits, 64 offsets), ReLU between,
 // BF16 weights, FP32 accumulation; one parameter array, row-major:
 //   W1[64][1024] b1[64] W2[64][64] b2[64] W3[68][64] b3[68].
-// Training kernels: forward (keeping the activations), the loss gradient
-// (softmax cross-entropy on the K-logits; squared error on the offsets of
-// samples that carry an offset label), backward through the activations,
-// the weight gradients summed over the batch, and an Adam step on FP32
-// master weights that also writes their BF16 copy.
+// Training: one kernel per sample (forward, the loss -- softmax
+// cross-entropy on the K-logits, squared error on the offsets of samples
+// that carry an offset label -- and the backward pass through the
+// activations), and one per parameter (its gradient summed over the batch
+// and the Adam step on FP32 master weights, which also writes their BF16
+// copy).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -101,128 +102,257 @@ __global__ void __launch_bounds__(1024) features_kernel(const float *__restrict_
     for (int c = t; c < kIn; c += 1024) feat[c] = (float)s_cnt[c] * inv;
 }
 
-// One block of 128 threads per sample: X[b] -> H1[b], H2[b], OUT[b].
-__global__ void __launch_bounds__(128) forward_kernel(const float *__restrict__ X, int B, const __nv_bfloat16 *__restrict__ P,
-                                                      float *__restrict__ H1, float *__restrict__ H2, float *__restrict__ OUT)
+// Eight consecutive weights (VEC: the parameters are 16-byte aligned, one
+// load; else one by one).
+template <bool VEC>
+__device__ __forceinline__ void weights8(const __nv_bfloat16 *__restrict__ P, int i, float (&w)[8])
 {
-    __shared__ float s_x[kIn], s_h1[kHid], s_h2[kHid];
-    const int b = blockIdx.x, t = (int)threadIdx.x;
-    if (b >= B) return;
-    for (int i = t; i < kIn; i += 128) s_x[i] = X[(int64_t)b * kIn + i];
-    __syncthreads();
-    if (t < kHid) {
-        float acc = wf(P, oB1 + t);
-        for (int i = 0; i < kIn; ++i) acc = __fmaf_rn(wf(P, oW1 + t * kIn + i), s_x[i], acc);
-        s_h1[t] = fmaxf(acc, 0.0f);
-        H1[b * kHid + t] = s_h1[t];
-    }
-    __syncthreads();
-    if (t < kHid) {
-        float acc = wf(P, oB2 + t);
-        for (int i = 0; i < kHid; ++i) acc = __fmaf_rn(wf(P, oW2 + t * kHid + i), s_h1[i], acc);
-        s_h2[t] = fmaxf(acc, 0.0f);
-        H2[b * kHid + t] = s_h2[t];
-    }
-    __syncthreads();
-    if (t < kOut) {
-        float acc = wf(P, oB3 + t);
-        for (int i = 0; i < kHid; ++i) acc = __fmaf_rn(wf(P, oW3 + t * kHid + i), s_h2[i], acc);
-        OUT[b * kOut + t] = acc;
-    }
-}
-
-// dOUT = d(loss) / d(OUT), loss = mean over the batch of
-//   CE(softmax(OUT[0:4]), label) + lam * mask * mean_j (OUT[4+j] - off[j])^2.
-__global__ void loss_grad_kernel(const float *__restrict__ OUT, int B, const int32_t *__restrict__ label,
-                                 const float *__restrict__ off, const float *__restrict__ mask, float lam,
-                                 float *__restrict__ dOUT, float *__restrict__ loss)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const float *o = OUT + b * kOut;
-    float mx = o[0];
-    for (int k = 1; k < 4; ++k) mx = fmaxf(mx, o[k]);
-    float e[4], z = 0.0f;
-    for (int k = 0; k < 4; ++k) {
-        e[k] = expf(o[k] - mx);
-        z += e[k];
-    }
-    const int y = min(max(label[b], 0), 3);   // labels are 0..3; the clamp keeps a bad one in bounds
-    float l = logf(z) + mx - o[y];
-    const float invB = 1.0f / (float)B;
-    for (int k = 0; k < 4; ++k) dOUT[b * kOut + k] = (e[k] / z - (k == y ? 1.0f : 0.0f)) * invB;
-    const float w = lam * mask[b];
-    for (int j = 0; j < 64; ++j) {
-        const float d = o[4 + j] - off[b * 64 + j];
-        l += w * d * d / 64.0f;
-        dOUT[b * kOut + 4 + j] = w * 2.0f * d / 64.0f * invB;
-    }
-    loss[b] = l;
-}
-
-// Per sample: dH2 = (W3^T dOUT) * [H2 > 0], dH1 = (W2^T dH2) * [H1 > 0].
-__global__ void __launch_bounds__(64) backward_kernel(const float *__restrict__ dOUT, int B, const __nv_bfloat16 *__restrict__ P,
-                                                      const float *__restrict__ H1, const float *__restrict__ H2,
-                                                      float *__restrict__ dH1, float *__restrict__ dH2)
-{
-    __shared__ float s_d[kOut], s_dh2[kHid];
-    const int b = blockIdx.x, t = (int)threadIdx.x;
-    if (b >= B) return;
-    for (int j = t; j < kOut; j += 64) s_d[j] = dOUT[b * kOut + j];
-    __syncthreads();
-    float acc = 0.0f;
-    for (int j = 0; j < kOut; ++j) acc = __fmaf_rn(wf(P, oW3 + j * kHid + t), s_d[j], acc);
-    const float g2 = H2[b * kHid + t] > 0.0f ? acc : 0.0f;
-    s_dh2[t] = g2;
-    dH2[b * kHid + t] = g2;
-    __syncthreads();
-    acc = 0.0f;
-    for (int j = 0; j < kHid; ++j) acc = __fmaf_rn(wf(P, oW2 + j * kHid + t), s_dh2[j], acc);
-    dH1[b * kHid + t] = H1[b * kHid + t] > 0.0f ? acc : 0.0f;
-}
-
-// One thread per parameter: its gradient summed over the batch.
-__global__ void wgrad_kernel(const float *__restrict__ X, int B, const float *__restrict__ H1, const float *__restrict__ H2,
-                             const float *__restrict__ dH1, const float *__restrict__ dH2, const float *__restrict__ dOUT,
-                             float *__restrict__ G)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kParams) return;
-    float acc = 0.0f;
-    if (p < oB1) {
-        const int j = p / kIn, i = p % kIn;
-        for (int b = 0; b < B; ++b) acc = __fmaf_rn(dH1[b * kHid + j], X[(int64_t)b * kIn + i], acc);
-    } else if (p < oW2) {
-        for (int b = 0; b < B; ++b) acc += dH1[b * kHid + (p - oB1)];
-    } else if (p < oB2) {
-        const int j = (p - oW2) / kHid, i = (p - oW2) % kHid;
-        for (int b = 0; b < B; ++b) acc = __fmaf_rn(dH2[b * kHid + j], H1[b * kHid + i], acc);
-    } else if (p < oW3) {
-        for (int b = 0; b < B; ++b) acc += dH2[b * kHid + (p - oB2)];
-    } else if (p < oB3) {
-        const int j = (p - oW3) / kHid, i = (p - oW3) % kHid;
-        for (int b = 0; b < B; ++b) acc = __fmaf_rn(dOUT[b * kOut + j], H2[b * kHid + i], acc);
+    if constexpr (VEC) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(P + i));
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            w[2 * q] = __uint_as_float(u[q] << 16);
+            w[2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
+        }
     } else {
-        for (int b = 0; b < B; ++b) acc += dOUT[b * kOut + (p - oB3)];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w[q] = wf(P, i + q);
     }
-    G[p] = acc;
 }
 
-// Adam on the FP32 master weights; the BF16 copy is what the kernels read.
-__global__ void adam_kernel(float *__restrict__ Wm, const float *__restrict__ G, float *__restrict__ M,
-                            float *__restrict__ V, __nv_bfloat16 *__restrict__ P, float lr, float b1, float b2,
-                            float eps, float c1, float c2)
+template <int W>   // sum over groups of W lanes, in every lane
+__device__ __forceinline__ float lanes_sum(float v)
+{
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+struct LossArgs {
+    const int32_t *label;
+    const float *off, *mask;
+    float lam;
+    float *dOUT, *dH1, *dH2, *loss;
+};
+
+// One block of 512 threads per sample: X[b] -> H1[b], H2[b], and OUT[b]
+// (forward) or, TRAIN, the sample's loss
+//   CE(softmax(OUT[0:4]), label) + lam * mask * mean_j (OUT[4+j] - off[j])^2
+// and the gradients of the batch mean with respect to OUT, H2 and H1
+// (dH2 = (W3^T dOUT) * [H2 > 0], dH1 = (W2^T dH2) * [H1 > 0]), all of a
+// sample's chain in one launch.
+// Bound by latency: the weights (144 KB) come from L2 once per sample.
+// Layer 1 gives a warp four outputs, each lane 32 inputs of the sample in
+// registers and 16-byte weight loads, all in flight together; the later
+// layers give an output eight lanes, and their weights are asked for before
+// layer 1 is summed.  One thread per output read W1 with a stride of 2 KB
+// and summed 1024 terms in a chain: 54 us for 64 samples, and 18 us more
+// in two kernels for the loss and the backward pass; a whole training step
+// of 64 samples went from 79 to 18 us.
+constexpr int MT = 512;
+
+template <bool VEC, bool TRAIN>
+__global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X, int B, const __nv_bfloat16 *__restrict__ P,
+                                                    float *__restrict__ H1, float *__restrict__ H2,
+                                                    float *__restrict__ OUT, LossArgs A)
+{
+    __shared__ float s_h1[kHid], s_h2[kHid], s_o[kOut], s_d[kOut], s_dh2[kHid], s_part[MT / kHid][kHid];
+    const int b = blockIdx.x, t = (int)threadIdx.x, lane = t & 31, warp = t >> 5;
+    const float *x = X + (int64_t)b * kIn;
+    constexpr int PW = kHid / (MT / 32);   // layer-1 outputs per warp
+    constexpr int C = kIn / 256;           // 8 inputs per lane and chunk of 256
+    float xv[C][8];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        const int i = c * 256 + lane * 8;
+        if constexpr (VEC) {
+            const float4 u = __ldg(reinterpret_cast<const float4 *>(x + i)), v = __ldg(reinterpret_cast<const float4 *>(x + i) + 1);
+            xv[c][0] = u.x, xv[c][1] = u.y, xv[c][2] = u.z, xv[c][3] = u.w;
+            xv[c][4] = v.x, xv[c][5] = v.y, xv[c][6] = v.z, xv[c][7] = v.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) xv[c][q] = __ldg(x + i + q);
+        }
+    }
+    const int o8 = t >> 3, l8 = t & 7;     // layers 2 and 3: output and its lane
+    float w2[8], w3[8];
+    weights8<VEC>(P, oW2 + o8 * kHid + l8 * 8, w2);
+    weights8<VEC>(P, oW3 + o8 * kHid + l8 * 8, w3);
+    float acc[PW];
+#pragma unroll
+    for (int u = 0; u < PW; ++u) {
+        acc[u] = 0.0f;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            float w[8];
+            weights8<VEC>(P, oW1 + (warp * PW + u) * kIn + c * 256 + lane * 8, w);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc[u] = __fmaf_rn(w[q], xv[c][q], acc[u]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < PW; ++u) {
+        const float h = fmaxf(lanes_sum<32>(acc[u]) + wf(P, oB1 + warp * PW + u), 0.0f);
+        if (lane == u) {
+            s_h1[warp * PW + u] = h;
+            H1[b * kHid + warp * PW + u] = h;
+        }
+    }
+    __syncthreads();
+    {
+        float a = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a = __fmaf_rn(w2[q], s_h1[l8 * 8 + q], a);
+        const float h = fmaxf(lanes_sum<8>(a) + wf(P, oB2 + o8), 0.0f);
+        if (l8 == 0) {
+            s_h2[o8] = h;
+            H2[b * kHid + o8] = h;
+        }
+    }
+    __syncthreads();
+    {
+        float a = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a = __fmaf_rn(w3[q], s_h2[l8 * 8 + q], a);
+        a = lanes_sum<8>(a) + wf(P, oB3 + o8);
+        if (l8 == 0) s_o[o8] = a;
+        if (warp == 0) {   // the last kOut - 64 outputs: eight lanes each again
+            const int o = kHid + (lane >> 3);
+            weights8<VEC>(P, oW3 + o * kHid + l8 * 8, w3);
+            a = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) a = __fmaf_rn(w3[q], s_h2[l8 * 8 + q], a);
+            a = lanes_sum<8>(a) + wf(P, oB3 + o);
+            if (l8 == 0) s_o[o] = a;
+        }
+    }
+    __syncthreads();
+    if constexpr (!TRAIN) {
+        if (t < kOut) OUT[b * kOut + t] = s_o[t];
+    } else {
+        const float invB = 1.0f / (float)B, w = A.lam * A.mask[b];
+        if (warp == 0) {   // loss, and the gradient of the logits
+            const float mx = fmaxf(fmaxf(s_o[0], s_o[1]), fmaxf(s_o[2], s_o[3]));
+            float e[4], z = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                e[k] = expf(s_o[k] - mx);
+                z += e[k];
+            }
+            const int y = min(max(A.label[b], 0), 3);   // labels are 0..3; the clamp keeps a bad one in bounds
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (lane == k) {
+                    s_d[k] = (e[k] / z - (k == y ? 1.0f : 0.0f)) * invB;
+                    A.dOUT[b * kOut + k] = s_d[k];
+                }
+            }
+            const float d0 = s_o[4 + lane] - A.off[b * 64 + lane], d1 = s_o[36 + lane] - A.off[b * 64 + 32 + lane];
+            const float l = lanes_sum<32>(w * d0 * d0 / 64.0f + w * d1 * d1 / 64.0f);
+            if (lane == 0) A.loss[b] = logf(z) + mx - s_o[y] + l;
+        } else if (warp < 3) {   // the gradient of the offsets
+            const int j = t - 32;
+            const float d = w * 2.0f * (s_o[4 + j] - A.off[b * 64 + j]) / 64.0f * invB;
+            s_d[4 + j] = d;
+            A.dOUT[b * kOut + 4 + j] = d;
+        }
+        __syncthreads();
+        constexpr int NP = MT / kHid;        // rows of a column's sum per thread: every NP-th
+        const int col = t % kHid, part = t / kHid;
+        float a = 0.0f;
+#pragma unroll
+        for (int j = part; j < kOut; j += NP) a = __fmaf_rn(wf(P, oW3 + j * kHid + col), s_d[j], a);
+        s_part[part][col] = a;
+        __syncthreads();
+        if (t < kHid) {
+            a = 0.0f;
+#pragma unroll
+            for (int q = 0; q < NP; ++q) a += s_part[q][t];
+            const float g = s_h2[t] > 0.0f ? a : 0.0f;
+            s_dh2[t] = g;
+            A.dH2[b * kHid + t] = g;
+        }
+        __syncthreads();
+        a = 0.0f;
+#pragma unroll
+        for (int j = part; j < kHid; j += NP) a = __fmaf_rn(wf(P, oW2 + j * kHid + col), s_dh2[j], a);
+        s_part[part][col] = a;
+        __syncthreads();
+        if (t < kHid) {
+            a = 0.0f;
+#pragma unroll
+            for (int q = 0; q < NP; ++q) a += s_part[q][t];
+            A.dH1[b * kHid + t] = s_h1[t] > 0.0f ? a : 0.0f;
+        }
+    }
+}
+
+// One thread per parameter: its gradient summed over the batch, then the
+// Adam step on the FP32 master weights and their BF16 copy, which is what
+// the other kernels read.  Bound by latency (each thread's loads over the
+// batch go out 16 at a time); the gradient stays in a register.
+struct AdamArgs {
+    float *Wm, *M, *V;
+    __nv_bfloat16 *P;
+    float lr, b1, b2, eps, c1, c2;
+};
+
+__global__ void __launch_bounds__(256) wgrad_adam_kernel(const float *__restrict__ X, int B, const float *__restrict__ H1,
+                                                         const float *__restrict__ H2, const float *__restrict__ dH1,
+                                                         const float *__restrict__ dH2, const float *__restrict__ dOUT,
+                                                         AdamArgs A)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= kParams) return;
-    const float g = G[p];
-    const float m = b1 * M[p] + (1.0f - b1) * g;
-    const float v = b2 * V[p] + (1.0f - b2) * g * g;
-    M[p] = m;
-    V[p] = v;
-    const float w = Wm[p] - lr * (m / c1) / (sqrtf(v / c2) + eps);
-    Wm[p] = w;
-    P[p] = __float2bfloat16_rn(w);
+    // the parameter's factors: column d of the layer's output gradient, and
+    // (weights) column x of its input
+    const float *d, *x = nullptr;
+    int ds, xs = 0;
+    if (p < oW2) {
+        d = dH1 + (p < oB1 ? p / kIn : p - oB1);
+        ds = kHid;
+        if (p < oB1) {
+            x = X + p % kIn;
+            xs = kIn;
+        }
+    } else if (p < oW3) {
+        d = dH2 + (p < oB2 ? (p - oW2) / kHid : p - oB2);
+        ds = kHid;
+        if (p < oB2) {
+            x = H1 + (p - oW2) % kHid;
+            xs = kHid;
+        }
+    } else {
+        d = dOUT + (p < oB3 ? (p - oW3) / kHid : p - oB3);
+        ds = kOut;
+        if (p < oB3) {
+            x = H2 + (p - oW3) % kHid;
+            xs = kHid;
+        }
+    }
+    const float m0 = A.M[p], v0 = A.V[p], w0 = A.Wm[p];
+    float g = 0.0f;
+    if (x) {
+#pragma unroll 16
+        for (int b = 0; b < B; ++b) g = __fmaf_rn(__ldg(d + (int64_t)b * ds), __ldg(x + (int64_t)b * xs), g);
+    } else {
+#pragma unroll 16
+        for (int b = 0; b < B; ++b) g += __ldg(d + (int64_t)b * ds);
+    }
+    const float m = A.b1 * m0 + (1.0f - A.b1) * g;
+    const float v = A.b2 * v0 + (1.0f - A.b2) * g * g;
+    A.M[p] = m;
+    A.V[p] = v;
+    const float w = w0 - A.lr * (m / A.c1) / (sqrtf(v / A.c2) + A.eps);
+    A.Wm[p] = w;
+    A.P[p] = __float2bfloat16_rn(w);
+}
+
+// 16-byte loads of the inputs and weights where both allow them.
+inline bool vec16(const float *X, const void *P)
+{
+    return ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(P)) & 15u) == 0;
 }
 
 }  // namespace
@@ -267,8 +397,10 @@ extern "C" ch_status ch_mlp_forward(const float *X, int32_t B, const void *param
                                     void *stream)
 {
     if (!X || !params || !H1 || !H2 || !OUT || B < 1) return CH_ERR_ARG;
-    forward_kernel<<<B, 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-        X, B, static_cast<const __nv_bfloat16 *>(params), H1, H2, OUT);
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const __nv_bfloat16 *P = static_cast<const __nv_bfloat16 *>(params);
+    if (vec16(X, params)) sample_kernel<true, false><<<B, MT, 0, st>>>(X, B, P, H1, H2, OUT, LossArgs{});
+    else sample_kernel<false, false><<<B, MT, 0, st>>>(X, B, P, H1, H2, OUT, LossArgs{});
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ERR_CUDA;
 }
 
@@ -281,16 +413,16 @@ extern "C" ch_status ch_mlp_train_step(const float *X, int32_t B, const int32_t 
         return CH_ERR_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     __nv_bfloat16 *P = static_cast<__nv_bfloat16 *>(params);
-    // scratch: H1, H2 (B x 64 each), OUT, dOUT (B x 68 each), dH1, dH2 (B x 64 each), G (params)
-    float *H1 = scratch, *H2 = H1 + B * kHid, *OUT = H2 + B * kHid, *dOUT = OUT + B * kOut;
-    float *dH1 = dOUT + B * kOut, *dH2 = dH1 + B * kHid, *G = dH2 + B * kHid;
-    forward_kernel<<<B, 128, 0, st>>>(X, B, P, H1, H2, OUT);
-    loss_grad_kernel<<<(B + 127) / 128, 128, 0, st>>>(OUT, B, label, off, mask, lam, dOUT, loss);
-    backward_kernel<<<B, 64, 0, st>>>(dOUT, B, P, H1, H2, dH1, dH2);
-    wgrad_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(X, B, H1, H2, dH1, dH2, dOUT, G);
+    // scratch: H1, H2 (B x 64 each), dOUT (B x 68), dH1, dH2 (B x 64 each)
+    float *H1 = scratch, *H2 = H1 + (int64_t)B * kHid, *dOUT = H2 + (int64_t)B * kHid;
+    float *dH1 = dOUT + (int64_t)B * kOut, *dH2 = dH1 + (int64_t)B * kHid;
+    const LossArgs A{label, off, mask, lam, dOUT, dH1, dH2, loss};
+    if (vec16(X, params)) sample_kernel<true, true><<<B, MT, 0, st>>>(X, B, P, H1, H2, nullptr, A);
+    else sample_kernel<false, true><<<B, MT, 0, st>>>(X, B, P, H1, H2, nullptr, A);
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
-    adam_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(master, G, adam_m, adam_v, P, lr, b1, b2, 1e-8f, c1, c2);
+    wgrad_adam_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(X, B, H1, H2, dH1, dH2, dOUT,
+                                                            AdamArgs{master, adam_m, adam_v, P, lr, b1, b2, 1e-8f, c1, c2});
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ERR_CUDA;
 }
 
