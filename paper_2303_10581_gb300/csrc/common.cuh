@@ -72,6 +72,7 @@ struct Octagon {
     float bxl, bxh, byl, byh;   // closed bounding box of the eight vertices
     uint32_t box_check;     // 1: points may lie outside that box (caller-supplied vertices)
     uint32_t pad2;
+    float tx[8], ty[8], tz[8];   // edge k's affine form (octtest.cuh)
 };
 
 // extremes reduction state: left zeroed by the last block of every sweep

@@ -87,6 +87,19 @@ __device__ __forceinline__ void combine(float &k, uint32_t &i, float ok, uint32_
 // their box; a point outside the box is never strictly inside.  The static
 // bound then holds for every point that reaches the edge test.
 //
+// The affine form of edge k (octtest.cuh), with c the box centre, u* = px -
+// cx, v* = py - cy exactly, (ex, ey) = b - a and K = ex (ay - cy) - ey (ax -
+// cx): the orientation is t = -ey u* + ex v* - K.  Let U >= |u*|, V >= |v*|
+// over the box, S = |ey| U + |ex| V + |K| and s = 2^21 / S.  The form has the
+// coefficients fl(-ey s), fl(ex s), fl(-K s) (binary64, rounded once) and
+// takes fl(u*), fl(v*) and two FMAs: each of its three terms gets at most
+// four relative errors of eps = 2^-24 (coefficient, difference, two FMAs),
+// so |T - s t| <= 4 eps s S (1 + 2^-20) < 0.51 < 1 for every point of the
+// box (underflows are below 2^-20: every term is at most 2^21 and the form
+// only decides values beyond 1).  An edge of zero length gets T = 2.  When
+// the box is not finite or a coefficient overflows, all forms are zero: T =
+// 0, undecided.
+//
 // A closed axis-aligned rectangle whose four corners are, exactly, strictly
 // left of every valid edge lies strictly inside the polygon (the region
 // "strictly left of every edge" is an intersection of open half-planes,
@@ -139,6 +152,21 @@ __device__ void build_octagon_warp(const float2 *pts, const uint32_t *ext8, Octa
     }
     const double cxd = 0.5 * ((double)xmin + (double)xmax);
     const double cyd = 0.5 * ((double)ymin + (double)ymax);
+    {
+        const double cx = (double)(float)cxd, cy = (double)(float)cyd;
+        const double ex = (double)b.x - a.x, ey = (double)b.y - a.y;
+        const double K = ex * ((double)a.y - cy) - ey * ((double)a.x - cx);
+        const double U = fmax((double)xmax - cx, cx - (double)xmin), V = fmax((double)ymax - cy, cy - (double)ymin);
+        const double sc = 0x1p21 / ((fabs(ey) * U + fabs(ex) * V + fabs(K)) * (1.0 + 0x1p-20));
+        const float tx = (float)(-ey * sc), ty = (float)(ex * sc), tz = (float)(-K * sc);
+        const bool fin = !valid || (fabsf(tx) <= 3.0e38f && fabsf(ty) <= 3.0e38f && fabsf(tz) <= 3.0e38f);
+        const bool on = __all_sync(0xffffffffu, fin && W <= 3.0e38f && H <= 3.0e38f);
+        if (lane < 8) {
+            out->tx[k] = on && valid ? tx : 0.0f;
+            out->ty[k] = on && valid ? ty : 0.0f;
+            out->tz[k] = on ? (valid ? tz : 2.0f) : 0.0f;
+        }
+    }
     const double hw = 0.5 * ((double)xmax - (double)xmin);
     const double hh = 0.5 * ((double)ymax - (double)ymin);
     // quick-discard rectangle: lane = (corner c = lane / 8, edge k)

@@ -20,11 +20,9 @@
 //    and writes its survivors; points are read once, but each tile waits on
 //    its predecessors.
 //
-// The test: the quick-discard rectangle, then the polygon edge facing the
-// point's octant; a point strictly left of that edge is likely inside and
-// needs every edge, so such points are queued per warp and tested 32 at a
-// time (spread over the lanes they would hold whole warps in the edge
-// loop).
+// The test: the quick-discard rectangle, then all edges at once by affine
+// forms with a proven error (octtest.cuh), exact signs for the few points
+// they leave undecided.
 //
 // In the hull step the fan test of kgon.cu runs between the two passes and
 // clears keep bits of points strictly inside the fan, so the scatter pass
@@ -38,163 +36,70 @@
 #include "common.cuh"
 #include "fan.cuh"
 #include "launch.h"
+#include "octtest.cuh"
 
 namespace ch {
 
 namespace {
 
-// Outside the closed bounding box of the polygon's vertices: never strictly
-// inside the polygon.  Only tested when the vertices were supplied by the
-// caller (BOX); the data's own extremes span a box holding every point.
-template <bool BOX>
-__device__ __forceinline__ bool outside_box(const Octagon &o, float x, float y)
-{
-    if constexpr (BOX) return x < o.bxl || x > o.bxh || y < o.byl || y > o.byh;
-    return false;
-}
-
-// keep(p) <=> NOT (p strictly left of every valid edge); see
-// build_octagon_warp for the error bound of the binary32 test, which holds
-// for points inside the vertices' bounding box.  The first edge tried is
-// the one facing p's octant around the box centre, which settles points
-// outside the polygon after one test; the order does not change the result.
-template <bool BOX>
-__device__ __forceinline__ bool keep_point(const Octagon &o, float x, float y)
-{
-    if (x >= o.xl && x <= o.xh && y >= o.yl && y <= o.yh) return false;
-    if (!o.has_edges || outside_box<BOX>(o, x, y)) return true;
-    const float ux = x - o.cx, uy = y - o.cy;
-    int s;
-    if (uy >= 0.0f) {
-        if (ux >= 0.0f) s = ux >= uy ? 0 : 1;
-        else s = uy >= -ux ? 2 : 3;
-    } else {
-        if (ux < 0.0f) s = -ux >= -uy ? 4 : 5;
-        else s = -uy >= ux ? 6 : 7;
-    }
-#pragma unroll 1
-    for (int j = 0; j < 8; ++j) {
-        const int e = (s + j) & 7;
-        if (!((o.valid >> e) & 1u)) continue;
-        const float u = __fsub_rn(x, o.ax[e]);
-        const float v = __fsub_rn(y, o.ay[e]);
-        const float t = __fsub_rn(__fmul_rn(o.dx[e], v), __fmul_rn(o.dy[e], u));
-        const float bnd = o.bound[e];
-        if (t > bnd) continue;
-        if (t < -bnd) return true;
-        if (orient_d(o.ax[e], o.ay[e], o.bx[e], o.by[e], x, y) <= 0) return true;
-    }
-    return false;
-}
-
 constexpr int NW = kFiltThreads / 32;
-
-// The polygon in shared memory, with the first look's per-edge data packed
-// (one 16-byte and one 4-byte load per point): (ax, ay, dx, dy) and the
-// bound of edge k; an edge of zero length gets zeros and +inf, which never
-// proves a point outside it.
-struct OctSmem : Octagon {
-    float4 e4[8];
-    float eb[8];
-};
-
-// Fills the packed edges of `so` from the polygon `o` (threads 0..7; the
-// caller synchronises before they are read).
-__device__ __forceinline__ void pack_edges(OctSmem &so, const Octagon &o)
-{
-    const uint32_t k = threadIdx.x;
-    if (k < 8) {
-        const bool v = (o.valid >> k) & 1u;
-        so.e4[k] = v ? make_float4(o.ax[k], o.ay[k], o.dx[k], o.dy[k]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        so.eb[k] = v ? o.bound[k] : __int_as_float(0x7f800000);
-    }
-}
-
-// A point's first look: 0 discard (inside the quick-discard rectangle), 1
-// keep (outside the vertices' box, or proven not strictly left of the edge
-// facing it), 2 deferred (likely strictly inside: every edge must be
-// tested).  The facing edge is the one of p's octant around the box centre,
-// picked without branches (on a circle the lanes of a warp face every
-// octant); any edge would give the same final decisions (a 1 is a proof, a
-// 2 is tested in full).
-template <bool BOX>
-__device__ __forceinline__ uint32_t first_look(const OctSmem &o, float x, float y)
-{
-    // the rectangle first, as an early exit: it holds nearly every point of
-    // a normal cloud (whole warps skip the rest) and none of a circle's
-    if (x >= o.xl && x <= o.xh && y >= o.yl && y <= o.yh) return 0u;
-    if (!o.has_edges || outside_box<BOX>(o, x, y)) return 1u;
-    const float ux = x - o.cx, uy = y - o.cy;
-    const float aux = fabsf(ux), auy = fabsf(uy);
-    const uint32_t q = uy < 0.0f ? (ux < 0.0f ? 2u : 3u) : (ux < 0.0f ? 1u : 0u);   // quadrant
-    const uint32_t e = 2u * q + ((q & 1u) ? (auy >= aux ? 0u : 1u) : (aux >= auy ? 0u : 1u));
-    const float4 d = o.e4[e];
-    const float u = __fsub_rn(x, d.x);
-    const float v = __fsub_rn(y, d.y);
-    const float t = __fsub_rn(__fmul_rn(d.z, v), __fmul_rn(d.w, u));
-    return t < -o.eb[e] ? 1u : 2u;
-}
-
-// Deferred points, spread over the lanes, would hold whole warps in the
-// edge loop; each warp queues them (lane, item) and tests them 32 at a
-// time after its items' first look, re-reading each point (an L2 hit).
-constexpr uint32_t kDeferCap = 32 * kFiltItems;   // every item of the warp
-
-struct FiltQueue {
-    uint16_t tag[kDeferCap];   // lane << 4 | item
-    uint32_t res[32];          // kept item bits, per lane
-};
-
-__device__ __forceinline__ void queue_reset(FiltQueue &q)
-{
-    q.res[lane_id()] = 0u;
-    __syncwarp();
-}
-
-// Tests this warp's deferred points (dm: this lane's deferred items, all
-// lanes call): they are queued in lane order (an exclusive scan of the
-// lanes' counts; the queue holds every item of the warp), tested 32 at a
-// time, and this lane's keep bits among them are returned.  load(lane,
-// item) reads a point of this warp.
-template <bool BOX, class LoadPoint>
-__device__ __forceinline__ uint32_t resolve_deferred(FiltQueue &q, const Octagon &so, uint32_t dm, LoadPoint load)
-{
-    const uint32_t c = __popc(dm);
-    if (!__any_sync(0xffffffffu, c != 0u)) return 0u;   // the common case: nothing deferred
-    const uint32_t lane = lane_id();
-    uint32_t incl = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += t;
-    }
-    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-    uint32_t slot = incl - c;
-    for (uint32_t m = dm; m; m &= m - 1u) q.tag[slot++] = (uint16_t)((lane << 4) | (uint32_t)(__ffs(m) - 1));
-    __syncwarp();
-    for (uint32_t i = lane; i < total; i += 32) {
-        const uint32_t tg = q.tag[i];
-        const float2 v = load(tg >> 4, tg & 15u);
-        if (keep_point<BOX>(so, v.x, v.y)) atomicOr(&q.res[tg >> 4], 1u << (tg & 15u));
-    }
-    __syncwarp();
-    const uint32_t r = q.res[lane];
-    q.res[lane] = 0u;   // only this lane touches its entry until the next call's barrier
-    __syncwarp();
-    return r;
-}
 
 // Copies the polygon to shared memory; false when the call was aborted
 // (non-finite input or a bad vertex index).
 __device__ __forceinline__ bool load_octagon(OctSmem &so, void *ws, const Layout &L)
 {
-    const Octagon *g = at<Octagon>(ws, L.oct);
-    const uint32_t *src = reinterpret_cast<const uint32_t *>(g);
-    uint32_t *dst = reinterpret_cast<uint32_t *>(static_cast<Octagon *>(&so));
-    for (uint32_t w = threadIdx.x; w < sizeof(Octagon) / 4; w += blockDim.x) dst[w] = src[w];
-    pack_edges(so, *g);
+    fill_octagon(so, at<Octagon>(ws, L.oct));
     __syncthreads();
     return !so.abort;
+}
+
+// Keep bits of this thread's 16 points: the quick-discard rectangle first
+// (it holds nearly every point of a normal cloud, and a warp whose points
+// are all in it is done), then the edges' affine forms, eight points at a
+// time, then the exact test of the few undecided ones (all_valid: bits of
+// the points that exist).  load(q) reads point q again: the exact test is a
+// call, and points kept in registers across it would be spilled.
+template <bool BOX, class Load>
+__device__ __forceinline__ uint32_t test_points(const OctSmem &so, const float (&px)[kFiltItems],
+                                                const float (&py)[kFiltItems], uint32_t all_valid, Load load)
+{
+    const float xl = so.xl, xh = so.xh, yl = so.yl, yh = so.yh;
+    uint32_t rect = 0;
+#pragma unroll
+    for (int q = 0; q < kFiltItems; ++q)
+        rect |= (((px[q] >= xl) & (px[q] <= xh) & (py[q] >= yl) & (py[q] <= yh)) ? 1u : 0u) << q;
+    uint32_t open = all_valid & ~rect;
+    if (!__any_sync(0xffffffffu, open != 0u)) return 0u;
+    if (!so.has_edges) return open;
+    uint32_t keep = 0;
+    if constexpr (BOX) {
+#pragma unroll
+        for (int q = 0; q < kFiltItems; ++q) keep |= (outside_box<true>(so, px[q], py[q]) ? 1u : 0u) << q;
+        keep &= open;
+        open &= ~keep;
+    }
+    uint32_t in = 0, und = 0;
+#pragma unroll
+    for (int h = 0; h < kFiltItems / 8; ++h) {
+        float qx[8], qy[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            qx[q] = px[8 * h + q];
+            qy[q] = py[8 * h + q];
+        }
+        uint32_t i8, u8;
+        oct_decide<8>(so, qx, qy, i8, u8);
+        in |= i8 << (8 * h);
+        und |= u8 << (8 * h);
+    }
+    keep |= open & ~in;
+    und &= open;
+#pragma unroll 1
+    for (; und; und &= und - 1u) {
+        const float2 p = load(__ffs(und) - 1);
+        if (!keep_point<BOX>(so, p.x, p.y)) keep &= ~(und & (0u - und));
+    }
+    return keep;
 }
 
 // Loads and tests one tile.  Thread t holds the points
@@ -203,12 +108,11 @@ __device__ __forceinline__ bool load_octagon(OctSmem &so, void *ws, const Layout
 // (bit r * G + h); positions past n are not kept.
 template <int G, bool BOX>
 __device__ __forceinline__ uint32_t load_test(const float *__restrict__ pts, int64_t n, int64_t base,
-                                              const OctSmem &so, float (&px)[kFiltItems], float (&py)[kFiltItems],
-                                              FiltQueue &fq)
+                                              const OctSmem &so, float (&px)[kFiltItems], float (&py)[kFiltItems])
 {
     constexpr int ROWS = kFiltItems / G;
     const uint32_t tid = threadIdx.x;
-    uint32_t keep = 0;
+    uint32_t valid = 0xffffu;
     if (base + kFiltTile <= n) {
         if constexpr (G == 2) {
             const float4 *p4 = reinterpret_cast<const float4 *>(pts) + base / 2;
@@ -233,37 +137,28 @@ __device__ __forceinline__ uint32_t load_test(const float *__restrict__ pts, int
                 py[r] = v[r].y;
             }
         }
-        uint32_t dm = 0;   // deferred items
-#pragma unroll
-        for (int q = 0; q < kFiltItems; ++q) {
-            const uint32_t c = first_look<BOX>(so, px[q], py[q]);
-            keep |= (c == 1u ? 1u : 0u) << q;
-            dm |= (c == 2u ? 1u : 0u) << q;
-        }
-        const uint32_t wbase = tid & ~31u;
-        keep |= resolve_deferred<BOX>(fq, so, dm, [&](uint32_t ln, uint32_t item) {
-            const int64_t i = base + (int64_t)((item / G) * kFiltThreads + wbase + ln) * G + item % G;
-            return reinterpret_cast<const float2 *>(pts)[i];
-        });
     } else {
         const float2 *p2 = reinterpret_cast<const float2 *>(pts);
+        valid = 0u;
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
 #pragma unroll
             for (int h = 0; h < G; ++h) {
                 const int64_t i = base + (int64_t)(r * kFiltThreads + tid) * G + h;
-                px[r * G + h] = 0.0f;
-                py[r * G + h] = 0.0f;
+                px[r * G + h] = so.cx;
+                py[r * G + h] = so.cy;
                 if (i < n) {
                     const float2 v = p2[i];
                     px[r * G + h] = v.x;
                     py[r * G + h] = v.y;
-                    if (keep_point<BOX>(so, v.x, v.y)) keep |= 1u << (r * G + h);
+                    valid |= 1u << (r * G + h);
                 }
             }
         }
     }
-    return keep;
+    return test_points<BOX>(so, px, py, valid, [&](int q) {
+        return reinterpret_cast<const float2 *>(pts)[base + (int64_t)((q / G) * kFiltThreads + tid) * G + q % G];
+    });
 }
 
 // Kept points per (row, warp), turned into exclusive offsets in row-major
@@ -471,8 +366,6 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
                                                               uint32_t *__restrict__ surv_count)
 {
     __shared__ OctSmem so;
-    __shared__ FiltQueue s_fq[NW];
-    queue_reset(s_fq[threadIdx.x >> 5]);
     __shared__ uint32_t s_off[kFiltItems / G][NW];
     __shared__ uint32_t s_tile;
     __shared__ unsigned long long s_excl;
@@ -493,7 +386,7 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
         if (tile >= ntiles) break;
         const int64_t base = tile * kFiltTile;
         float px[kFiltItems], py[kFiltItems];
-        const uint32_t keep = load_test<G, BOX>(pts, n, base, so, px, py, s_fq[threadIdx.x >> 5]);
+        const uint32_t keep = load_test<G, BOX>(pts, n, base, so, px, py);
         row_counts<G>(keep, s_off);
         __syncthreads();
         if (warp == 0) {
@@ -687,15 +580,13 @@ __device__ __forceinline__ uint32_t block_sum_to0(uint32_t v, uint32_t (&s_w)[NW
 // by atomicMax (read first: most points do not raise their bin), the
 // first level's farthest sampled point per bin without a pass of its own.
 template <int G, bool BOX>
-__global__ void __launch_bounds__(kFiltThreads, BOX ? 4 : 5) filter_count_kernel(const float *__restrict__ pts, int64_t n,
+__global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const float *__restrict__ pts, int64_t n,
                                                                     void *ws, Layout L,
                                                                     unsigned long long *fan_slots,
                                                                     int32_t fan_stride)
 {
     __shared__ OctSmem so;
-    __shared__ FiltQueue s_fq[NW];
     __shared__ uint32_t s_cnt[kCountRing];
-    queue_reset(s_fq[threadIdx.x >> 5]);
     __shared__ uint32_t s_w[NW];
     for (int i = threadIdx.x; i < kCountRing; i += kFiltThreads) s_cnt[i] = 0u;
     if (!load_octagon(so, ws, L)) return;   // (its barrier also covers s_cnt)
@@ -725,7 +616,7 @@ __global__ void __launch_bounds__(kFiltThreads, BOX ? 4 : 5) filter_count_kernel
                     bulk_prefetch_l2(pts + 2 * nb, (nn * 8u) & ~15u);
             }
             float px[kFiltItems], py[kFiltItems];
-            const uint32_t keep = load_test<G, BOX>(pts, n, tile * kFiltTile, so, px, py, s_fq[threadIdx.x >> 5]);
+            const uint32_t keep = load_test<G, BOX>(pts, n, tile * kFiltTile, so, px, py);
             bits[tile * kFiltThreads + threadIdx.x] = (uint16_t)keep;
             if (!BOX && fan_slots && tile % fan_stride == 0) {   // block-uniform (the hull step only)
                 // the kept points again from L2 (the tile was just read), so
@@ -884,27 +775,19 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
 // ---------------------------------------------------------------------------
 // Thread t tests points lo + r * 256 + t of the set (r < 16), below hi.
 __device__ __forceinline__ uint32_t bx_load_test(const float2 *__restrict__ p2, int64_t lo, int64_t hi,
-                                                 const OctSmem &so, float (&px)[kFiltItems],
-                                                 float (&py)[kFiltItems], FiltQueue &fq)
+                                                 const OctSmem &so)
 {
-    uint32_t keep = 0, dm = 0;
+    float px[kFiltItems], py[kFiltItems];
+    uint32_t valid = 0;
 #pragma unroll
     for (int r = 0; r < kFiltItems; ++r) {
         const int64_t i = lo + r * kFiltThreads + threadIdx.x;
-        px[r] = py[r] = 0.0f;
-        if (i < hi) {
-            const float2 v = __ldcs(p2 + i);
-            px[r] = v.x;
-            py[r] = v.y;
-            const uint32_t c = first_look<false>(so, v.x, v.y);
-            keep |= (c == 1u ? 1u : 0u) << r;
-            dm |= (c == 2u ? 1u : 0u) << r;
-        }
+        const float2 v = i < hi ? __ldcs(p2 + i) : make_float2(so.cx, so.cy);
+        px[r] = v.x;
+        py[r] = v.y;
+        valid |= (i < hi ? 1u : 0u) << r;
     }
-    const uint32_t wbase = threadIdx.x & ~31u;
-    return keep | resolve_deferred<false>(fq, so, dm, [&](uint32_t ln, uint32_t item) {
-               return p2[lo + (int64_t)item * kFiltThreads + wbase + ln];
-           });
+    return test_points<false>(so, px, py, valid, [&](int q) { return p2[lo + q * kFiltThreads + threadIdx.x]; });
 }
 
 // Copies set b's polygon to shared memory when the block moves to a new set.
@@ -912,21 +795,16 @@ __device__ __forceinline__ void bx_octagon_to_smem(OctSmem &so, int64_t &cur, in
 {
     if (b == cur) return;   // block-uniform
     __syncthreads();
-    const uint32_t *src = reinterpret_cast<const uint32_t *>(octs + b);
-    uint32_t *dst = reinterpret_cast<uint32_t *>(static_cast<Octagon *>(&so));
-    for (uint32_t w = threadIdx.x; w < sizeof(Octagon) / 4; w += blockDim.x) dst[w] = src[w];
-    pack_edges(so, octs[b]);
+    fill_octagon(so, octs + b);
     __syncthreads();
     cur = b;
 }
 
-__global__ void __launch_bounds__(kFiltThreads) bx_filter_count_kernel(const float *__restrict__ pts, void *ws,
+__global__ void __launch_bounds__(kFiltThreads, 4) bx_filter_count_kernel(const float *__restrict__ pts, void *ws,
                                                                        Layout L, BatchLayout BL)
 {
     __shared__ OctSmem so;
-    __shared__ FiltQueue s_fq[NW];
     __shared__ uint32_t s_cnt[kCountRing];
-    queue_reset(s_fq[threadIdx.x >> 5]);
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     for (int i = threadIdx.x; i < kCountRing; i += kFiltThreads) s_cnt[i] = 0u;   // (the first set's load syncs)
@@ -962,9 +840,7 @@ __global__ void __launch_bounds__(kFiltThreads) bx_filter_count_kernel(const flo
             if (!so.abort) {
                 const int64_t lo = (int64_t)(t - sets[b].tile_base) * kFiltTile;
                 const int64_t hi = min(lo + kFiltTile, sets[b].n);
-                float px[kFiltItems], py[kFiltItems];
-                keep = bx_load_test(reinterpret_cast<const float2 *>(pts) + sets[b].pt_begin, lo, hi, so, px, py,
-                                    s_fq[threadIdx.x >> 5]);
+                keep = bx_load_test(reinterpret_cast<const float2 *>(pts) + sets[b].pt_begin, lo, hi, so);
             }
             bits[(size_t)t * kFiltThreads + threadIdx.x] = (uint16_t)keep;
             uint32_t c = __popc(keep);
