@@ -102,7 +102,7 @@ extern "C" ch_status ch_filter(const float *pts, int64_t n, const uint32_t *ext8
     cudaError_t e = launch_octagon(pts, n, ext8, ws, L, at<unsigned long long>(ws, L.ctrl),
                                    (int64_t)L.zero_words, st);
     if (e != cudaSuccess) return CH_ERR_CUDA;
-    return cuda_status(launch_filter(pts, n, ws, L, surv_idx, surv_pts, surv_count, false, st));
+    return cuda_status(launch_filter(pts, n, ws, L, surv_idx, surv_pts, surv_count, st));
 }
 
 extern "C" ch_status ch_extremes_filter(const float *pts, int64_t n, uint32_t *ext8, uint32_t *surv_idx,
@@ -122,7 +122,7 @@ extern "C" ch_status ch_extremes_filter(const float *pts, int64_t n, uint32_t *e
     cudaError_t e = launch_extremes(pts, n, ws, L, ext8, true, at<unsigned long long>(ws, L.ctrl),
                                     (int64_t)L.zero_words, st, variant == 0);
     if (e == cudaSuccess)
-        e = launch_filter(pts, n, ws, L, surv_idx, surv_pts, surv_count, false, st, variant, false, true);
+        e = launch_filter(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, variant, true);
     return cuda_status(e);
 }
 
@@ -193,7 +193,8 @@ cudaError_t hull_pipeline(const float *pts, int64_t n, uint32_t *hull_idx, uint3
     cudaError_t e = launch_extremes(pts, n, ws, L, at<uint32_t>(ws, L.ext8), true,
                                     at<unsigned long long>(ws, L.ctrl), (int64_t)L.zero_words, st, variant == 0,
                                     learn_params, learn_dirs, learn_k);
-    if (e == cudaSuccess) e = launch_filter(pts, n, ws, L, nullptr, nullptr, nullptr, true, st, variant, true, true, kg);
+    if (e == cudaSuccess)
+        e = variant == 1 ? launch_filter_keys_single(pts, n, ws, L, st) : launch_hull_filter(pts, n, ws, L, kg, st);
     if (e == cudaSuccess) e = launch_small_hull(ws, L, hull_idx, hull_count, st);
     if (e == cudaSuccess) e = launch_sort(ws, L, st);
     if (e == cudaSuccess) e = launch_chain(ws, L, hull_idx, hull_count, st);

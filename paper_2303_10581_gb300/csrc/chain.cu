@@ -4,8 +4,7 @@
 // The paper copies the candidates to the host and calls CGAL; its
 // conclusion names a fully device-resident hull as the next step.  Here:
 //
-//  0. runs: the survivors arrive sorted by x (equal x in ascending index
-//     order).  In a run of equal x only the lowest point can be a vertex of
+//  0. runs: the survivors arrive sorted by x (equal x in any order).  In a run of equal x only the lowest point can be a vertex of
 //     the lower chain and only the highest one of the upper chain, because
 //     the others lie strictly above (below) it on the same vertical.  The
 //     exceptions are the first x, whose lowest point starts both chains and
@@ -184,8 +183,9 @@ struct ChainSmem {
     uint32_t wsum[LT / 32];
     uint32_t total;
     float red_y[2][LT / 32];      // look-ahead reduction scratch
-    uint32_t red_q[2][LT / 32];
+    unsigned long long red_q[2][LT / 32];
     uint32_t ext_pos[2];          // global positions of the look-ahead lowest / highest
+    uint32_t ext_idx[2];          // and their point indices
     float prev_x;
     int has_prev;
     int seq_len;
@@ -414,22 +414,23 @@ __device__ void climb(const ChainPtrs &P, int64_t c, int64_t nsc, int64_t coff, 
     }
 }
 
-// Block reduction of (y, position) pairs: the lowest (highest) y, ties to the
-// lowest position.  Contains two barriers.
-__device__ __forceinline__ void block_extreme_y(ChainSmem &s, float ylo, uint32_t qlo, float yhi, uint32_t qhi,
-                                                float &out_ylo, uint32_t &out_qlo, float &out_yhi, uint32_t &out_qhi)
+// Block reduction of (y, index << 32 | position) pairs: the lowest (highest)
+// y, ties to the lowest index.  Contains two barriers.
+__device__ __forceinline__ void block_extreme_y(ChainSmem &s, float ylo, unsigned long long qlo, float yhi,
+                                                unsigned long long qhi, float &out_ylo, unsigned long long &out_qlo,
+                                                float &out_yhi, unsigned long long &out_qhi)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float y1 = __shfl_xor_sync(0xffffffffu, ylo, o);
-        const uint32_t q1 = __shfl_xor_sync(0xffffffffu, qlo, o);
+        const unsigned long long q1 = __shfl_xor_sync(0xffffffffu, qlo, o);
         if (y1 < ylo || (y1 == ylo && q1 < qlo)) {
             ylo = y1;
             qlo = q1;
         }
         const float y2 = __shfl_xor_sync(0xffffffffu, yhi, o);
-        const uint32_t q2 = __shfl_xor_sync(0xffffffffu, qhi, o);
+        const unsigned long long q2 = __shfl_xor_sync(0xffffffffu, qhi, o);
         if (y2 > yhi || (y2 == yhi && q2 < qhi)) {
             yhi = y2;
             qhi = q2;
@@ -500,19 +501,20 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
         int64_t run_end = base + m;
         if (ext) {
             float ylo = kInf, yhi = -kInf;
-            uint32_t qlo = 0xffffffffu, qhi = 0xffffffffu;
+            unsigned long long qlo = ~0ull, qhi = ~0ull;   // index << 32 | position
             for (int64_t q0 = base + m;; q0 += LT) {
                 const int64_t q = q0 + t;
                 const bool in_run = q < send && key_float(__ldg(P.keys + q)) == xr;
                 if (in_run) {
-                    const float y = key_float((uint32_t)(__ldg(P.pay + q) >> 32));
-                    if (y < ylo || (y == ylo && (uint32_t)q < qlo)) {
+                    const unsigned long long pv = __ldg(P.pay + q), iq = (pv << 32) | (uint32_t)q;
+                    const float y = key_float((uint32_t)(pv >> 32));
+                    if (y < ylo || (y == ylo && iq < qlo)) {
                         ylo = y;
-                        qlo = (uint32_t)q;
+                        qlo = iq;
                     }
-                    if (y > yhi || (y == yhi && (uint32_t)q < qhi)) {
+                    if (y > yhi || (y == yhi && iq < qhi)) {
                         yhi = y;
-                        qhi = (uint32_t)q;
+                        qhi = iq;
                     }
                 }
                 // the keys are sorted, so the run's positions are contiguous
@@ -523,13 +525,15 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
                 }
             }
             float oyl, oyh;
-            uint32_t oql, oqh;
+            unsigned long long oql, oqh;
             block_extreme_y(sm, ylo, qlo, yhi, qhi, oyl, oql, oyh, oqh);
             if (t == 0) {
                 sm.pts[SC] = make_float2(xr, oyl);
                 sm.pts[SC + 1] = make_float2(xr, oyh);
-                sm.ext_pos[0] = oql;
-                sm.ext_pos[1] = oqh;
+                sm.ext_pos[0] = (uint32_t)oql;
+                sm.ext_pos[1] = (uint32_t)oqh;
+                sm.ext_idx[0] = (uint32_t)(oql >> 32);
+                sm.ext_idx[1] = (uint32_t)(oqh >> 32);
             }
         }
         const bool holds_last = run_end == send;
@@ -540,20 +544,22 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
             const int r1 = k + 1 < R ? sm.list[2][k + 1] : m;
             int lo = r0, hi = r0;
             float ylo = sm.pts[r0].y, yhi = ylo;
+            // equal points (the sort does not order a run): the lowest index
+            const auto before = [&](uint32_t a, int b) { return a < (uint32_t)__ldg(P.pay + base + b); };
             for (int i = r0 + 1; i < r1; ++i) {
                 const float y = sm.pts[i].y;
-                if (y < ylo) {
+                if (y < ylo || (y == ylo && before((uint32_t)__ldg(P.pay + base + i), lo))) {
                     ylo = y;
                     lo = i;
                 }
-                if (y > yhi) {
+                if (y > yhi || (y == yhi && before((uint32_t)__ldg(P.pay + base + i), hi))) {
                     yhi = y;
                     hi = i;
                 }
             }
             if (k == R - 1 && ext) {
-                if (sm.pts[SC].y < ylo) lo = SC;
-                if (sm.pts[SC + 1].y > yhi) hi = SC + 1;
+                if (sm.pts[SC].y < ylo || (sm.pts[SC].y == ylo && before(sm.ext_idx[0], lo))) lo = SC;
+                if (sm.pts[SC + 1].y > yhi || (sm.pts[SC + 1].y == yhi && before(sm.ext_idx[1], hi))) hi = SC + 1;
             }
             sm.list[0][k] = (uint16_t)lo;
             sm.list[1][k] = (uint16_t)hi;

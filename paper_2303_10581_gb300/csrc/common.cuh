@@ -90,9 +90,13 @@ constexpr int kFanBins = 28672;
 
 struct KgonCtrl {                          // zeroed with the control block
     unsigned long long slot[kFanBins];     // packed (far_key << 32 | ~index): farthest sampled input point per bin
-    uint32_t sample, inside;               // the estimate's sample and how much of it is inside the fan
-    uint32_t s_oct;                        // octagon survivors (0: the fan kernels did not run)
-    uint32_t pad;
+    uint32_t sample, inside;               // points sampled for the bins, octagon survivors among them
+    uint32_t s_oct;                        // octagon survivors
+    uint32_t bad;                          // 1: consecutive vertices not proven counter-clockwise around c
+    uint32_t rho_inv;                      // ~bits of a lower bound (binary32) on the squared distance from
+                                           // c to the fan's boundary, the largest so far
+    uint32_t edges;                        // consecutive vertex pairs with v != w
+    uint32_t pad[2];
 };
 
 // second fan level (kgon.cu): over the first level's survivors, kFan2Sub
@@ -105,17 +109,16 @@ constexpr int64_t kFan2MinN = 1 << 19;           // smaller sets get no tables
 struct Fan2Ctrl {                          // zeroed with the control block
     uint32_t on;                           // 1: the second level runs this call
     uint32_t count_in;                     // survivors of the first level, its input
-    uint32_t bad;                          // 1: no vertices (nothing is dropped)
-    uint32_t pad;
+    uint32_t bad;                          // 1: no usable vertices (nothing is dropped)
+    uint32_t kept;                         // survivors of the second level
+    uint32_t done;                         // test blocks finished
+    uint32_t edges;                        // consecutive vertex pairs with v != w
+    uint32_t pad[2];
 };
 
 struct Kgon {
-    float cx, cy;                          // fan centre, strictly inside the hull
+    float cx, cy;                          // fan centre
     uint32_t ok;                           // 0: no fan this call
-    uint32_t disk_bad;                     // 1: no disk around the centre is proven inside the fan
-    unsigned long long rho2;               // bits of a lower bound on the squared distance from
-                                           // the centre to the fan's boundary (binary64 >= 0)
-    uint32_t disk_edges;                   // consecutive vertex pairs with v != w
     uint32_t pad;
     float2 v[kFanBins];                    // vertex of every bin (input points)
 };
@@ -229,7 +232,7 @@ struct Layout {
     size_t utmp;          // u32[n]
     size_t spec, p0;        // SpecCtrl, the speculative sweep's test region (SpecBox, extremes.cu)
     size_t learn;           // the learned proposal's scratch (LearnScratch)
-    size_t fan2_v;          // float2[fan2_bins]: the second fan level's vertices
+    size_t fan2_v;          // float2[fan2_bins + 2]: the second fan level's vertices, the ends repeated
     size_t total;
     int64_t n, filt_tiles, sort_tiles, n_chunks, n_nodes, emit_tiles;
     int64_t fan2_bins;      // kFan2Bins for sets of at least kFan2MinN points, else 0 (no second level)
@@ -368,7 +371,7 @@ __host__ __device__ inline Layout make_layout(int64_t n, int64_t sets = 0)
     L.spec = take(sizeof(SpecCtrl));
     L.p0 = take(256);
     L.learn = take(sizeof(LearnScratch));
-    L.fan2_v = take((size_t)L.fan2_bins * 8);
+    L.fan2_v = take((size_t)(L.fan2_bins + 2) * 8);
     L.total = o;
     return L;
 }

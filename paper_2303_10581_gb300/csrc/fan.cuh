@@ -1,7 +1,5 @@
 // fan.cuh -- the hull step's fan: angular bins around the centre and the
-// order key of the farthest-point choice, shared by the filter's count
-// pass (which gathers the first level's bin maxima on its sampled tiles)
-// and the fan kernels (kgon.cu).
+// order key of the farthest-point choice (kgon.cu).
 #pragma once
 
 #include "common.cuh"
@@ -17,12 +15,10 @@ __host__ __device__ inline int64_t fan_sample_stride(int64_t tiles)
     return s < 1 ? 1 : (s > 8 ? 8 : s);
 }
 
-// Bin of the direction (dx, dy): a pseudo-angle in [0, 4) that grows with
-// the angle counter-clockwise from +x, scaled to the bins.  Any value is
-// safe (it only picks a triangle); the conversion saturates and the result
-// is clamped.
+// Scaled pseudo-angle of the direction (dx, dy): in [0, NB], growing with
+// the angle counter-clockwise from +x; bin b holds [b, b + 1).
 template <int NB = kFanBins>
-__device__ __forceinline__ int fan_bin(float dx, float dy)
+__device__ __forceinline__ float fan_phi(float dx, float dy)
 {
     const float s = fabsf(dx) + fabsf(dy);
     float a = 0.0f;
@@ -30,10 +26,15 @@ __device__ __forceinline__ int fan_bin(float dx, float dy)
         const float t = __fdividef(dy, s);
         a = dx >= 0.0f ? (dy >= 0.0f ? t : 4.0f + t) : 2.0f - t;
     }
-    // a is in [0, 4] (t in [-1, 1]; a NaN from an overflowed difference
-    // converts to 0): only the top needs a clamp
-    const int b = __float2int_rz(a * (NB / 4.0f));
-    return min(b, NB - 1);
+    return a * (NB / 4.0f);
+}
+
+// Its bin (phi is in [0, NB], a NaN from an overflowed difference converts
+// to 0: only the top needs a clamp).
+template <int NB = kFanBins>
+__device__ __forceinline__ int fan_bin(float dx, float dy)
+{
+    return min(__float2int_rz(fan_phi<NB>(dx, dy)), NB - 1);
 }
 
 template <int NB = kFanBins>
@@ -87,22 +88,5 @@ __device__ __forceinline__ float far_ref(const Octagon &o)
     const float ux = __fsub_rn(o.ax[0], o.cx), uy = __fsub_rn(o.ay[0], o.cy);
     return __fmaf_rn(ux, ux, __fmul_rn(uy, uy));
 }
-
-// Strictly inside a fan triangle (exact signs).  V: kFanBins vertices.
-// With o = orient(c, v, p) = +1 the triangle is (c, v, w), w the next
-// vertex, and p is inside iff orient(v, w, p) = orient(w, c, p) = +1; with
-// o = -1 it is (c, w, v), w the previous vertex, and p is inside iff
-// orient(w, v, p) = orient(c, w, p) = +1, i.e. orient(v, w, p) =
-// orient(w, c, p) = -1.
-//
-// fan_signs_f32 takes the three signs in binary32 (branch-free, so a
-// thread's items interleave): 1 inside, 0 outside, 2 undecided (a sign the
-// binary32 bound does not prove, and that matters); fan_inside_exact
-// settles the undecided ones.
-// The two signs with c as a vertex are taken with c as the reference point
-// (a cyclic shift of a triple keeps its orientation): orient(c, v, p) as
-// orient(v, p, c) and orient(w, c, p) as orient(p, w, c), so that both use
-// the differences p - c of the bin; orient_f32 certifies the sign of either
-// form with the same bound.
 
 }  // namespace ch

@@ -24,9 +24,9 @@
 // forms with a proven error (octtest.cuh), exact signs for the few points
 // they leave undecided.
 //
-// In the hull step the fan test of kgon.cu runs between the two passes and
-// clears keep bits of points strictly inside the fan, so the scatter pass
-// writes only the points that survive both tests.
+// ch_hull runs neither pass (kgon.cu tests and writes the survivors of the
+// octagon and of its fan in one), unless a second polygon reads the count
+// pass's keep bits in between.
 //
 // Memory traffic: 8 bytes per point read (twice for tiles with survivors in
 // the two-pass variant), 12 bytes per kept point written.
@@ -34,7 +34,6 @@
 #include <atomic>
 
 #include "common.cuh"
-#include "fan.cuh"
 #include "launch.h"
 #include "octtest.cuh"
 
@@ -575,20 +574,18 @@ __device__ __forceinline__ uint32_t block_sum_to0(uint32_t v, uint32_t (&s_w)[NW
     return t;
 }
 
-// fan_slots (the hull step, else NULL): on every fan_stride-th tile the
-// kept points' packed (far_key << 32 | ~index) go into the fan's bin slots
-// by atomicMax (read first: most points do not raise their bin), the
-// first level's farthest sampled point per bin without a pass of its own.
+// kdev (ch_hull_learned, else NULL): the device's choice of K; 8 means that
+// no second polygon will read the keep bits, and the pass is not needed.
 template <int G, bool BOX>
 __global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const float *__restrict__ pts, int64_t n,
                                                                     void *ws, Layout L,
-                                                                    unsigned long long *fan_slots,
-                                                                    int32_t fan_stride)
+                                                                    const int32_t *kdev)
 {
     __shared__ OctSmem so;
     __shared__ uint32_t s_cnt[kCountRing];
     __shared__ uint32_t s_w[NW];
     for (int i = threadIdx.x; i < kCountRing; i += kFiltThreads) s_cnt[i] = 0u;
+    if (kdev && *kdev == 8) return;
     if (!load_octagon(so, ws, L)) return;   // (its barrier also covers s_cnt)
     if constexpr (!BOX) {
         if (so.spec) {   // the speculative sweep proved all but its candidates inside
@@ -618,21 +615,6 @@ __global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const flo
             float px[kFiltItems], py[kFiltItems];
             const uint32_t keep = load_test<G, BOX>(pts, n, tile * kFiltTile, so, px, py);
             bits[tile * kFiltThreads + threadIdx.x] = (uint16_t)keep;
-            if (!BOX && fan_slots && tile % fan_stride == 0) {   // block-uniform (the hull step only)
-                // the kept points again from L2 (the tile was just read), so
-                // that the test's registers are free here
-                const float r2ref = far_ref(so);
-#pragma unroll 1
-                for (uint32_t m = keep; m; m &= m - 1u) {
-                    const int q = __ffs(m) - 1;
-                    const uint32_t i = (uint32_t)(tile * kFiltTile + ((q / G) * kFiltThreads + threadIdx.x) * G + q % G);
-                    const float2 p = __ldcg(reinterpret_cast<const float2 *>(pts) + i);
-                    const int b = fan_bin(__fsub_rn(p.x, so.cx), __fsub_rn(p.y, so.cy));
-                    const unsigned long long v =
-                        ((unsigned long long)far_key(p.x, p.y, so.cx, so.cy, r2ref) << 32) | (uint32_t)~i;
-                    if (v > __ldcg(fan_slots + b)) atomicMax(fan_slots + b, v);
-                }
-            }
             uint32_t c = __popc(keep);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
@@ -1004,46 +986,30 @@ cudaError_t launch_single(const float *pts, int64_t n, void *ws, const Layout &L
     return cudaGetLastError();
 }
 
+template <int G, bool BOX>
+int64_t count_blocks(int64_t n)
+{
+    static const int per_sm = occupancy(filter_count_kernel<G, BOX>, kFiltThreads);
+    return std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>((int64_t)sm_count() * per_sm, kFiltMaxBlocks),
+                                                  ceil_div(n, kFiltTile)));
+}
+
 // BOX: the polygon's vertices were supplied by the caller (ch_filter), so
 // points outside their box must be kept first; otherwise they are the
 // data's extremes, and the scatter may take the speculative sweep's
 // candidates (Octagon::spec)
-template <int G, bool KEYS, bool BOX>
+template <int G, bool BOX>
 cudaError_t launch_two_pass(const float *pts, int64_t n, void *ws, const Layout &L, uint32_t *surv_idx,
-                            float *surv_pts, uint32_t *surv_count, cudaStream_t st, bool fan, const KgonStage *kg)
+                            float *surv_pts, uint32_t *surv_count, cudaStream_t st)
 {
     // both passes use the same grid (block b owns the same tile range),
     // the count pass's resident blocks (the scatter pass's warps take
     // tiles on their own, so a second partial wave of it costs little)
-    static const int per_sm = occupancy(filter_count_kernel<G, BOX>, kFiltThreads);
-    const int64_t ntiles = ceil_div(n, kFiltTile);
-    const int64_t bc = std::max<int64_t>(
-        1, std::min<int64_t>(std::min<int64_t>((int64_t)sm_count() * per_sm, kFiltMaxBlocks), ntiles));
-    // the hull step's fan gathers its bin maxima in this pass
-    unsigned long long *fan_slots = (fan && !BOX) ? at<KgonCtrl>(ws, L.kgon_ctrl)->slot : nullptr;
-    filter_count_kernel<G, BOX><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, fan_slots,
-                                                                       (int32_t)fan_sample_stride(ntiles));
-    if (kg && (kg->kdev || kg->K != 8)) {   // the second polygon, over the octagon's survivors
-        probe_after(CH_K_FILTER, st);
-        const cudaError_t e = launch_kx_sv(pts, n, kg->dirs, kg->kdev, kg->K, kg->ext_out, ws, L, bc, st);
-        if (e != cudaSuccess) return e;
-        probe_before(CH_K_FILTER, st);
-    }
-    if (fan) {   // timed as its own group, between the filter's two
-        probe_after(CH_K_FILTER, st);
-        const cudaError_t e = launch_fan(pts, n, G == 2, bc, ws, L, st);
-        if (e != cudaSuccess) return e;
-        probe_before(CH_K_FILTER, st);
-    }
-    filter_scatter_kernel<G, KEYS><<<(unsigned)bc, kFiltThreads, 0, st>>>(
+    const int64_t bc = count_blocks<G, BOX>(n);
+    filter_count_kernel<G, BOX><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, nullptr);
+    filter_scatter_kernel<G, false><<<(unsigned)bc, kFiltThreads, 0, st>>>(
         pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count, BOX ? 0 : 1);
     note_kernels(CH_K_FILTER, 2);
-    if (fan && KEYS) {   // the hull step: the fan's second level over the survivors just written
-        probe_after(CH_K_FILTER, st);
-        const cudaError_t e = launch_fan2(n, ws, L, st);
-        if (e != cudaSuccess) return e;
-        probe_before(CH_K_FILTER, st);
-    }
     return cudaGetLastError();
 }
 
@@ -1052,19 +1018,13 @@ cudaError_t launch_two_pass(const float *pts, int64_t n, void *ws, const Layout 
 // host thread is not a data race)
 std::atomic<int> g_filter_variant{0};
 
-template <int G, bool KEYS>
+template <int G>
 cudaError_t launch_variant(const float *pts, int64_t n, void *ws, const Layout &L, uint32_t *surv_idx,
-                           float *surv_pts, uint32_t *surv_count, cudaStream_t st, int variant, bool fan,
-                           bool data_extremes, const KgonStage *kg)
+                           float *surv_pts, uint32_t *surv_count, cudaStream_t st, int variant, bool data_extremes)
 {
-    probe_before(CH_K_FILTER, st);
-    cudaError_t e;
-    if (variant == 1) e = launch_single<G, KEYS>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st);
-    else if (KEYS || data_extremes)
-        e = launch_two_pass<G, KEYS, false>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, fan, kg);
-    else e = launch_two_pass<G, false, true>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, fan, nullptr);
-    probe_after(CH_K_FILTER, st);
-    return e;
+    if (variant == 1) return launch_single<G, false>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st);
+    if (data_extremes) return launch_two_pass<G, false>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st);
+    return launch_two_pass<G, true>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st);
 }
 
 }  // namespace
@@ -1072,18 +1032,39 @@ cudaError_t launch_variant(const float *pts, int64_t n, void *ws, const Layout &
 int filter_variant() { return g_filter_variant.load(std::memory_order_relaxed); }
 
 cudaError_t launch_filter(const float *pts, int64_t n, void *ws, const Layout &L, uint32_t *surv_idx,
-                          float *surv_pts, uint32_t *surv_count, bool keys_mode, cudaStream_t st, int variant,
-                          bool fan, bool data_extremes, const KgonStage *kg)
+                          float *surv_pts, uint32_t *surv_count, cudaStream_t st, int variant, bool data_extremes)
 {
     const int v = variant < 0 ? g_filter_variant.load(std::memory_order_relaxed) : variant;
     const bool vec = (reinterpret_cast<uintptr_t>(pts) & 15u) == 0;
-    if (keys_mode)
-        return vec ? launch_variant<2, true>(pts, n, ws, L, nullptr, nullptr, nullptr, st, v, fan, true, kg)
-                   : launch_variant<1, true>(pts, n, ws, L, nullptr, nullptr, nullptr, st, v, fan, true, kg);
-    return vec ? launch_variant<2, false>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, v, false, data_extremes,
-                                          nullptr)
-               : launch_variant<1, false>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, v, false, data_extremes,
-                                          nullptr);
+    probe_before(CH_K_FILTER, st);
+    const cudaError_t e = vec ? launch_variant<2>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, v, data_extremes)
+                              : launch_variant<1>(pts, n, ws, L, surv_idx, surv_pts, surv_count, st, v, data_extremes);
+    probe_after(CH_K_FILTER, st);
+    return e;
+}
+
+cudaError_t launch_filter_keys_single(const float *pts, int64_t n, void *ws, const Layout &L, cudaStream_t st)
+{
+    const bool vec = (reinterpret_cast<uintptr_t>(pts) & 15u) == 0;
+    probe_before(CH_K_FILTER, st);
+    const cudaError_t e = vec ? launch_single<2, true>(pts, n, ws, L, nullptr, nullptr, nullptr, st)
+                              : launch_single<1, true>(pts, n, ws, L, nullptr, nullptr, nullptr, st);
+    probe_after(CH_K_FILTER, st);
+    return e;
+}
+
+cudaError_t launch_filter_count(const float *pts, int64_t n, const int32_t *kdev, void *ws, const Layout &L,
+                                int64_t *grid, cudaStream_t st)
+{
+    const bool vec = (reinterpret_cast<uintptr_t>(pts) & 15u) == 0;
+    const int64_t bc = vec ? count_blocks<2, false>(n) : count_blocks<1, false>(n);
+    *grid = bc;
+    probe_before(CH_K_FILTER, st);
+    if (vec) filter_count_kernel<2, false><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, kdev);
+    else filter_count_kernel<1, false><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, kdev);
+    note_kernels(CH_K_FILTER, 1);
+    probe_after(CH_K_FILTER, st);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_filter_scatter(const float *pts, int64_t n, int64_t grid, void *ws, const Layout &L,

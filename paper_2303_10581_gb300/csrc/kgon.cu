@@ -1,63 +1,802 @@
-// kgon.cu -- a second throw-away step inside the device hull: a fan of
-// triangles around an interior point, applied to the octagon filter's keep
-// decisions before its survivors are written.
+// kgon.cu -- the hull step's filter: the octagon test of Sec. 3.2 and a
+// second throw-away test against a fan of triangles around an interior
+// point, in one pass that writes the survivors of both.
 //
 // The octagon filter (Sec. 3.1-3.2) removes almost nothing from points near
 // a circle, and on a displaced circle 95 % survive it, although the hulls
 // have a small fraction of the points as vertices.  The hull step repeats
 // the throw-away idea of Sec. 3.1 on a much finer scale.  Let c be the
-// centre of the bounding box, checked with exact signs to lie strictly
-// inside the octagon, hence strictly inside the hull.  The plane around c
-// is cut into kFanBins angular bins; the vertex of a bin is the input point
-// farthest from c among a sample (the octagon survivors of about
-// kFanBinTiles evenly spaced 4096-point tiles of the input, fan.cuh), and a
-// bin the sample missed repeats the vertex before it.  For
-// consecutive vertices v, w every point strictly inside the triangle
-// (c, v, w) is a combination of c, v and w with positive weights, so it
-// lies strictly inside the hull and is no vertex of it: it is dropped.
-// This holds whatever the vertices are (they are input points), so nothing
-// needs to be exact but the three orientation signs of the final test, and
-// a triangle that comes out clockwise or flat drops nothing.
+// centre of the bounding box.  The plane around c is cut into kFanBins
+// angular bins (a pseudo-angle, fan.cuh); the vertex of a bin is the input
+// point farthest from c among a sample (the octagon survivors of about
+// kFanBinTiles evenly spaced 4096-point tiles of the input), and a bin the
+// sample missed repeats the vertex before it.
 //
-// The kernels run between the filter's count pass (which leaves keep bits,
-// per-tile counts and per-block totals) and its scatter pass, so the
-// scatter writes only the points that survive both tests:
+// The test of a point p in bin b, with P, Q, N the vertices of the bins
+// b - 1, b, b + 1: p is dropped when it is strictly left of P -> Q (unless P
+// == Q: bin b has no sample) and strictly left of Q -> N, both signs proven
+// by the binary32 bound of orient_f32.  Then p lies strictly inside the
+// hull:
+//  - the pseudo-angle grows with the angle, and its binary32 value is off by
+//    less than 0.0049 bins (0.0386 with the second level's eight times as
+//    many): in units of eps = 2^-24, t = dy / (|dx| + |dy|) gets 7 |t| (two
+//    differences, the sum, at most 2 ulp for the quotient), 2 - t or 4 + t
+//    half an ulp of at most 4, i.e. 2, and the product with NB / 4 half an
+//    ulp of at most NB.  A vertex is taken only where its value is at least
+//    a margin (1/32; 1/8) away from both ends of its bin, so as directions P
+//    comes strictly before p and N strictly after it, and Q, too, is before
+//    p where bin b has no sample;
+//  - consecutive vertices v, w were proven strictly counter-clockwise around
+//    c (v != w), less than half a turn apart, so p is in the wedge of (P, Q)
+//    or of (Q, N), where strictly left of the edge and inside the wedge is
+//    the triangle (c, P, Q) or (c, Q, N).  The triangles wind around c once,
+//    so c and the triangles' interiors (and the rays between them) are in
+//    the interior of a polygon of input points;
+//  - the quotient needs |dx| + |dy| within [2^-126, 2^126]: the set's box is
+//    checked for the upper end, and a point closer to c than 2^-126 is
+//    inside the disk around c that is proven inside the fan (the fan is off
+//    unless its radius exceeds 2^-60).
+// Nothing else is exact: a vertex only has to be an input point, a sign that
+// is not proven keeps the point, and what is kept only costs the sort time.
+// (Sets so small or large that the products of the signs under- or overflow,
+// below 10^-15 or above 10^18, keep all their points.)
 //
-//  (count pass)         per bin, the farthest sampled octagon survivor
-//                       (atomicMax of (far_key << 32 | ~index) into global
-//                       slots, on the sampled tiles, filter.cu)
-//  fan_build_kernel     octagon survivor count; exact centre check against
-//                       the octagon; the vertex of every bin
-//  fan_estimate_kernel  exact test of an input sample: whether the fan drops
-//                       at least an eighth of the octagon's survivors
-//  fan_refine_kernel    per tile of the filter: the kept points' exact fan
-//                       test, then new keep bits, tile counts and block totals
+// The disk around c proven inside the fan (a lower bound on the distance
+// from c to every fan edge) lets most points of a displaced circle pass
+// with one compare.
 //
-// Test of a point p: its bin b from a binary32 pseudo-angle (a hint only),
-// v the vertex of b.  p strictly left of the ray c -> v: the triangle
-// (c, v, next vertex); strictly right: (c, previous vertex, v); on it: kept.
+//  fan_bins_kernel    per bin, the farthest sampled octagon survivor
+//                     (atomicMax of (far_key << 32 | ~index) into global
+//                     slots), and how many of the sample survived
+//  fan_build_kernel   whether there is a fan; the vertex of every bin; the
+//                     proofs that need consecutive vertices; the disk
+//  hull_filter_kernel both tests of every point; the survivors' sort keys and
+//                     payloads, in no particular order (the chain breaks
+//                     ties by the index in the payload)
 #include <algorithm>
 
 #include "common.cuh"
 #include "fan.cuh"
 #include "launch.h"
+#include "octtest.cuh"
 
 namespace ch {
 namespace {
 
-constexpr int FT = 512;                  // threads per block of the bins pass
-constexpr int FITEMS = 8;                // points per thread per tile there
-constexpr int CT = 1024;                 // threads per block of the refine pass: four
+constexpr int CT = 1024;                 // threads per block of the filter pass: four
 constexpr int CG = CT / kFiltThreads;    // groups of kFiltThreads, each with its own tiles
 constexpr uint32_t kKgonMinS = 1u << 16; // fewer octagon survivors: not worth a pass
-constexpr int kFanSmem = kFanBins * 8;   // bins or vertices, 224 KB
-static_assert(kFiltItems == 16 && CT % kFiltThreads == 0, "refine pass: 16 keep bits per filter thread");
+constexpr int kFanSmem = (kFanBins + 2) * 8;   // vertices, the last one again before the first and the first after the last
+constexpr float kFanMargin = 1.0f / 32.0f;     // of a vertex's pseudo-angle from its bin's ends
+constexpr float kFan2Margin = 1.0f / 8.0f;     // second level
+static_assert(kFiltItems == 16 && CT % kFiltThreads == 0, "16 items per filter thread");
+static_assert(kFanSmem <= 227 * 1024 - 2048, "the table fits a block's shared memory");
 
 __device__ __forceinline__ float2 input_point(const float *pts, int64_t i)
 {
     return __ldg(reinterpret_cast<const float2 *>(pts) + i);
 }
 
+// Whether (ax, ay) x (bx, by) is proven positive (orient_f32's bound, on the
+// rounded differences a - c and b - c).
+__device__ __forceinline__ bool left_of(float acx, float acy, float bcx, float bcy)
+{
+    const float detleft = __fmul_rn(acx, bcy);
+    const float detright = __fmul_rn(acy, bcx);
+    const float det = __fsub_rn(detleft, detright);
+    const float detsum = __fadd_rn(fabsf(detleft), fabsf(detright));
+    // (an overflowed product makes the bound infinite or NaN: not proven)
+    return det > __fmaf_ru(detsum, 2.384185791015625e-07f /* 2^-22 */, 7.174648137343064e-43f /* 2^-140 */);
+}
+
+// Strictly inside the fan, proven (see the top of the file).  V[-1] and
+// V[NB] are the last and the first vertex again; (dx, dy) = fl(p - c).
+template <int NB>
+__device__ __forceinline__ bool fan_inside(const float2 *V, float dx, float dy, float px, float py)
+{
+    const float2 *v = V + fan_bin<NB>(dx, dy);
+    const float2 P = v[-1], Q = v[0], N = v[1];
+    const float ux = __fsub_rn(px, Q.x), uy = __fsub_rn(py, Q.y);
+    const bool qn = left_of(__fsub_rn(N.x, Q.x), __fsub_rn(N.y, Q.y), ux, uy);
+    const bool pq = left_of(ux, uy, __fsub_rn(P.x, Q.x), __fsub_rn(P.y, Q.y));
+    return qn && (pq || (P.x == Q.x && P.y == Q.y));
+}
+
+// The bin a point may be the vertex of, -1 when its pseudo-angle is within
+// `margin` of the bin's ends.
+template <int NB>
+__device__ __forceinline__ int vertex_bin(float dx, float dy, float margin)
+{
+    const float phi = fan_phi<NB>(dx, dy);
+    const int b = min(__float2int_rz(phi), NB - 1);
+    const float f = phi - (float)b;
+    return f >= margin && f <= 1.0f - margin ? b : -1;
+}
+
+// Whether this call has a fan whose proofs hold (after fan_build_kernel).
+__device__ __forceinline__ float fan_rho2(const KgonCtrl *kc) { return __uint_as_float(~kc->rho_inv); }
+__device__ __forceinline__ bool fan_ready(const KgonCtrl *kc, const Kgon *g)
+{
+    return g->ok && !kc->bad && kc->edges >= 3u && fan_rho2(kc) > 0x1p-120f;
+}
+
+// Point of item q (of this thread's 16) of a 4096-point tile; the layout is
+// the count pass's: item q = r * G + h is point base + (r * kFiltThreads + t) * G + h.
+template <int G>
+__device__ __forceinline__ int64_t item_point(int64_t base, uint32_t t, int q)
+{
+    return base + (int64_t)((q / G) * kFiltThreads + t) * G + q % G;
+}
+
+// Items 8 half .. 8 half + 7 of a thread's 16 in the tile at `base`, all of
+// them below n (G = 2: 16-byte loads).
+template <int G>
+__device__ __forceinline__ void load8(const float *__restrict__ pts, int64_t base, uint32_t t, int half, float (&px)[8],
+                                      float (&py)[8])
+{
+    if constexpr (G == 2) {
+        const float4 *p4 = reinterpret_cast<const float4 *>(pts) + base / 2 + half * 4 * kFiltThreads + t;
+        float4 v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = __ldg(p4 + r * kFiltThreads);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            px[2 * r] = v[r].x;
+            py[2 * r] = v[r].y;
+            px[2 * r + 1] = v[r].z;
+            py[2 * r + 1] = v[r].w;
+        }
+    } else {
+        const float2 *p2 = reinterpret_cast<const float2 *>(pts) + base + half * 8 * kFiltThreads + t;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const float2 v = __ldg(p2 + r * kFiltThreads);
+            px[r] = v.x;
+            py[r] = v.y;
+        }
+    }
+}
+
+// The same where the tile ends before them: the centre stands in for the
+// missing points; returns the bits of those that exist.
+template <int G>
+__device__ __forceinline__ uint32_t load8_ragged(const float *__restrict__ pts, int64_t n, int64_t base, uint32_t t,
+                                                 int half, float cx, float cy, float (&px)[8], float (&py)[8])
+{
+    uint32_t live = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int64_t i = item_point<G>(base, t, 8 * half + k);
+        const float2 v = i < n ? input_point(pts, i) : make_float2(cx, cy);
+        px[k] = v.x;
+        py[k] = v.y;
+        live |= (i < n ? 1u : 0u) << k;
+    }
+    return live;
+}
+
+// ---------------------------------------------------------------------------
+// first level: bins and vertices
+// ---------------------------------------------------------------------------
+// Every stride-th tile, a block each: the octagon survivors' bins.  Bound by
+// the slots' L2 reads and the key's arithmetic (about 90 instructions per
+// sampled survivor); inside the count pass, where an eighth of the tiles
+// held their block up while the others waited for it, the same work took
+// 90 to 180 us of 10^8 points on a circle and a displaced circle.
+template <int G>
+__global__ void __launch_bounds__(kFiltThreads) fan_bins_kernel(const float *__restrict__ pts, int64_t n, void *ws,
+                                                                Layout L, int32_t stride, int use_bits,
+                                                                const int32_t *kdev)
+{
+    __shared__ OctSmem so;
+    const Octagon *oct = at<Octagon>(ws, L.oct);
+    if (oct->abort || oct->spec || !oct->has_edges) return;
+    fill_octagon(so, oct);
+    __syncthreads();
+    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
+    const bool bits_mode = use_bits && (!kdev || *kdev != 8);
+    const uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
+    unsigned long long *slot = kc->slot;
+    const float cx = so.cx, cy = so.cy, r2ref = far_ref(so);
+    const uint32_t t = threadIdx.x;
+    uint32_t seen = 0, kept = 0;
+    for (int64_t tile = (int64_t)blockIdx.x * stride; tile * kFiltTile < n; tile += (int64_t)gridDim.x * stride) {
+        const int64_t base = tile * kFiltTile;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            float px[8], py[8];
+            uint32_t live = 0xffu;
+            if (base + kFiltTile <= n) load8<G>(pts, base, t, half, px, py);
+            else live = load8_ragged<G>(pts, n, base, t, half, cx, cy, px, py);
+            seen += __popc(live);
+            if (bits_mode) {
+                live &= (uint32_t)bits[tile * kFiltThreads + t] >> (8 * half);
+            } else {
+                uint32_t in, und;
+                oct_decide<8>(so, px, py, in, und);
+                live &= ~in;   // (undecided points are input points all the same)
+            }
+            kept += __popc(live);
+            if (!__any_sync(0xffffffffu, live != 0u)) continue;
+            int b[8];
+            uint32_t key[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                b[k] = ((live >> k) & 1u) ? vertex_bin<kFanBins>(__fsub_rn(px[k], cx), __fsub_rn(py[k], cy), kFanMargin) : -1;
+                key[k] = far_key(px[k], py[k], cx, cy, r2ref);
+            }
+            uint32_t top[8];   // the slots' keys: most points do not raise their bin's
+#pragma unroll
+            for (int k = 0; k < 8; ++k) top[k] = b[k] >= 0 ? __ldcg(reinterpret_cast<const uint32_t *>(slot + b[k]) + 1) : ~0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (b[k] >= 0 && key[k] >= top[k]) {
+                    const uint32_t i = (uint32_t)item_point<G>(base, t, 8 * half + k);
+                    atomicMax(slot + b[k], ((unsigned long long)key[k] << 32) | (uint32_t)~i);
+                }
+            }
+        }
+    }
+    seen = __reduce_add_sync(0xffffffffu, seen);
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if (lane_id() == 0 && seen) {
+        atomicAdd(&kc->sample, seen);
+        if (kept) atomicAdd(&kc->inside, kept);
+    }
+}
+
+// One thread per bin (kFanBins / BT blocks).  The vertex of bin b is the
+// sampled point of the last non-empty bin at or before b, cyclically: a
+// max-scan of "non-empty bin index" inside the block, and for the bins
+// before the block's first non-empty one, the last non-empty bin of the
+// nearest earlier range of BT bins that has one (searched range by range).
+constexpr int BT = 1024;
+static_assert(kFanBins % BT == 0, "bins split evenly over the blocks");
+
+__device__ __forceinline__ int block_max(int v, int *s_w)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();   // s_w may still be read from an earlier call
+    if (lane_id() == 0) s_w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int m = -1;
+    for (int w = 0; w < BT / 32; ++w) m = max(m, s_w[w]);
+    return m;
+}
+
+// The bin whose point is the vertex of bin blockIdx.x * BT + threadIdx.x (-1:
+// every bin is empty; block-uniform then).  Every thread of the block calls.
+__device__ __forceinline__ int vertex_source(const unsigned long long *slot, int *s_w, int *s_scan)
+{
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const int b = (int)(blockIdx.x * BT + tid);
+    int incl = slot[b] != 0ull ? b : -1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl = max(incl, u);
+    }
+    if (lane == 31) s_scan[warp] = incl;
+    __syncthreads();
+    for (int w = 0; w < (int)warp; ++w) incl = max(incl, s_scan[w]);
+    if (!__syncthreads_or(incl < 0)) return incl;
+    int prev = -1;
+    for (uint32_t k = 1; k <= gridDim.x && prev < 0; ++k) {   // prev is block-uniform
+        const uint32_t rb = (blockIdx.x + gridDim.x - k) % gridDim.x;
+        const int j = (int)(rb * BT + tid);
+        prev = block_max(slot[j] != 0ull ? j : -1, s_w);
+    }
+    return prev < 0 ? -1 : (incl >= 0 ? incl : prev);
+}
+
+// Lower bound on the squared distance from c to the segment [v, w] (v != w),
+// or -1 when (c, v, w) is not proven strictly counter-clockwise.  The
+// distance is the one to the nearer end when the foot of the perpendicular
+// provably falls outside the segment, else at least the one to the line.
+// T: the arithmetic; its rounding (half an ulp) is U.  Sums of two products
+// lose at most 4 U of the sum of their magnitudes, squares and the quotient
+// 16 U.
+template <class T>
+__device__ __forceinline__ T edge_bound(float cx, float cy, float2 v, float2 w, T U)
+{
+    const T ux = (T)cx - (T)v.x, uy = (T)cy - (T)v.y;   // c - v
+    const T dv = (ux * ux + uy * uy) * ((T)1 - (T)16 * U);
+    const T ex = (T)w.x - (T)v.x, ey = (T)w.y - (T)v.y;   // w - v
+    const T t1 = ex * uy, t2 = ey * ux;
+    const T lo = (t1 - t2) - (fabs(t1) + fabs(t2)) * ((T)8 * U);   // c strictly left of v -> w
+    if (!(lo > (T)0)) return (T)-1;
+    const T len2 = ex * ex + ey * ey;
+    const T d1 = ex * ux, d2 = ey * uy;
+    const T dot = d1 + d2, derr = (fabs(d1) + fabs(d2)) * ((T)8 * U);   // (c - v) . (w - v)
+    if (dot < -derr) return dv;   // the foot lies before v
+    if (dot > len2 * ((T)1 + (T)16 * U) + derr) {   // after w
+        const T zx = (T)cx - (T)w.x, zy = (T)cy - (T)w.y;
+        return (zx * zx + zy * zy) * ((T)1 - (T)16 * U);
+    }
+    return lo * lo / (len2 * ((T)1 + (T)16 * U)) * ((T)1 - (T)16 * U);
+}
+
+// In binary32 first (28672 binary64 quotients on 28 SMs would take 15 us),
+// in binary64 where that proves nothing: a value in binary32, rounded down.
+__device__ __forceinline__ float disk_bound(float cx, float cy, float2 v, float2 w)
+{
+    const float f = edge_bound<float>(cx, cy, v, w, 0x1p-24f);
+    if (f >= 0x1p-100f && f <= 0x1p100f) return f;
+    const double d = edge_bound<double>(cx, cy, v, w, 0x1p-53);
+    return d < 0.0 ? -1.0f : (d <= 3.0e38 ? __double2float_rd(d) : 3.0e38f);
+}
+
+__global__ void __launch_bounds__(BT) fan_build_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L)
+{
+    __shared__ int s_w[BT / 32];
+    __shared__ int s_scan[BT / 32];
+    const Octagon *oct = at<Octagon>(ws, L.oct);
+    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
+    Kgon *g = at<Kgon>(ws, L.kgon);
+    const uint32_t tid = threadIdx.x;
+    // (an aborted call, the speculative sweep's candidates, a polygon without
+    // edges: the bins pass left no sample)
+    const uint32_t sample = kc->sample;
+    const float box = __fadd_rn(__fsub_rn(oct->bxh, oct->bxl), __fsub_rn(oct->byh, oct->byl));
+    const bool live = sample != 0u && (double)kc->inside / sample * (double)n >= (double)kKgonMinS && box < 4.0e37f;
+    if (!live) {
+        if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
+        return;
+    }
+    const float cx = oct->cx, cy = oct->cy;
+    const int b = (int)(blockIdx.x * BT + tid);
+    const int src = vertex_source(kc->slot, s_w, s_scan);
+    if (src < 0) {
+        if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
+        return;
+    }
+    const auto point_of = [&](unsigned long long packed) {
+        const uint32_t i = ~(uint32_t)packed;
+        return input_point(pts, (int64_t)i < n ? i : 0u);
+    };
+    const unsigned long long nextp = kc->slot[next_bin(b)];
+    const float2 v = point_of(kc->slot[src]);
+    g->v[b] = v;
+    // the next bin's vertex: its own point, or this one's again
+    const float2 w = nextp != 0ull ? point_of(nextp) : v;
+    float r = __int_as_float(0x7f800000);
+    const bool edge = v.x != w.x || v.y != w.y;
+    bool bad = false;
+    if (edge) {
+        r = disk_bound(cx, cy, v, w);
+        bad = r < 0.0f;
+    }
+    uint32_t inv = ~__float_as_uint(fmaxf(r, 0.0f));
+    inv = __reduce_max_sync(0xffffffffu, inv);
+    const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge));
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane_id() == 0) {
+        atomicMax(&kc->rho_inv, inv);
+        if (edges) atomicAdd(&kc->edges, edges);
+        if (bad) atomicOr(&kc->bad, 1u);
+    }
+    if (blockIdx.x == 0 && tid == 0) {
+        g->cx = cx;
+        g->cy = cy;
+        g->ok = 1u;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// the filter pass
+// ---------------------------------------------------------------------------
+// The warp's kept points (mask: this lane's items; get(q): the point and its
+// index) to the end of the survivor list.
+template <class Get>
+__device__ __forceinline__ void append_survivors(uint32_t mask, uint32_t *count, uint32_t *keys, unsigned long long *pay,
+                                                 Get get)
+{
+    const uint32_t lane = lane_id(), c = __popc(mask);
+    if (!__any_sync(0xffffffffu, c != 0u)) return;
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += u;
+    }
+    uint32_t pos = 0;
+    if (lane == 31) pos = atomicAdd(count, incl);
+    pos = __shfl_sync(0xffffffffu, pos, 31) + incl - c;
+#pragma unroll 1
+    for (; mask; mask &= mask - 1u, ++pos) {
+        uint32_t i;
+        const float2 p = get(__ffs(mask) - 1, i);
+        keys[pos] = ord_key(p.x);
+        pay[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
+    }
+}
+
+// The speculative sweep's candidates (extremes.cu; every other point is
+// proven inside the octagon): a warp per slice, the exact test.
+__device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *ws, const Layout &L, uint32_t *count,
+                                                      uint32_t *keys, unsigned long long *pay)
+{
+    const SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
+    const uint32_t *cidx = at<uint32_t>(ws, L.keys[1]);
+    const float2 *cpt = at<float2>(ws, L.pay[1]);
+    const uint32_t slices = sc->nseg * kSpecWarps, cap = sc->cap, lane = lane_id();
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    uint32_t mine = 0;
+    for (uint32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < slices; j += warps) {
+        const uint32_t c = min(sc->scnt[j], cap);
+        const size_t s0 = (size_t)j * cap;
+        for (uint32_t e0 = 0; e0 < c; e0 += 32) {   // warp-uniform
+            float2 p = make_float2(0.0f, 0.0f);
+            bool keep = e0 + lane < c;
+            if (keep) {
+                p = cpt[s0 + e0 + lane];
+                keep = keep_point<false>(so, p.x, p.y);
+            }
+            mine += keep ? 1u : 0u;
+            append_survivors(keep ? 1u : 0u, count, keys, pay, [&](int, uint32_t &i) {
+                i = cidx[s0 + e0 + lane];
+                return p;
+            });
+        }
+    }
+    return mine;
+}
+
+// The tiles go in contiguous ranges to groups of kFiltThreads threads; a
+// thread takes its 16 points of a tile eight at a time: the octagon's affine
+// forms, then (fan) the disk and the fan test, branch-free.  The few points
+// the octagon's forms leave undecided and those that are written are read
+// again (L2), so that eight points are all the registers hold.  bits_mode: a
+// second polygon has refined the count pass's keep bits, which then stand
+// for the octagon test.
+// One block of 1024 threads per SM: the 28672 vertices take its shared
+// memory.  Bound by issue on circle-like sets (two differences, 23
+// instructions for the octagon, about 35 for the fan and two three-vertex
+// reads of shared memory per point) and by HBM on others.  Testing and
+// writing in one pass replaces a count pass, a fan pass and a scatter that
+// each read the points again: 274 + 455 + 214 us on 10^8 points of the unit
+// circle.
+template <int G>
+__global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L,
+                                                            int has_fan, int use_bits, const int32_t *kdev)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ OctSmem so;
+    __shared__ uint32_t s_oct;
+    const Octagon *oct = at<Octagon>(ws, L.oct);
+    if (oct->abort) return;
+    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
+    Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
+    uint32_t *keys = at<uint32_t>(ws, L.keys[0]), *count = &ctrl->surv_count;
+    unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
+    fill_octagon(so, oct);
+    if (threadIdx.x == 0) s_oct = 0u;
+    const Kgon *g = at<Kgon>(ws, L.kgon);
+    const bool fan = has_fan && !oct->spec && fan_ready(kc, g);
+    const float2 *V = reinterpret_cast<const float2 *>(smem_raw) + 1;
+    if (fan) {
+        float2 *sv = reinterpret_cast<float2 *>(smem_raw) + 1;
+        for (int i = threadIdx.x; i < kFanBins; i += CT) sv[i] = __ldg(g->v + i);
+        if (threadIdx.x == 0) {
+            sv[-1] = __ldg(g->v + kFanBins - 1);
+            sv[kFanBins] = __ldg(g->v);
+        }
+    }
+    __syncthreads();
+    uint32_t octs = 0;   // octagon survivors of this thread
+    if (oct->spec) {
+        octs = filter_candidates(so, ws, L, count, keys, pay);
+    } else {
+        const bool bits_mode = use_bits && (!kdev || *kdev != 8);
+        const uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
+        const float cx = so.cx, cy = so.cy;
+        // r2 < rho2t proves |p - c|^2 < rho^2 (2^-20 covers the rounding of r2)
+        const float rho2t = fan ? __fmul_rd(fan_rho2(kc), 1.0f - 0x1p-20f) : 0.0f;
+        bool use_disk = fan;
+        const int64_t ntiles = ceil_div(n, kFiltTile);
+        const uint32_t grp = threadIdx.x / kFiltThreads, t = threadIdx.x % kFiltThreads;
+        const int64_t groups = (int64_t)gridDim.x * CG, gi = (int64_t)blockIdx.x * CG + grp;
+        const int64_t per = ceil_div(ntiles, groups);
+        const int64_t t1 = std::min<int64_t>(ntiles, (gi + 1) * per);
+        for (int64_t tile = gi * per; tile < t1; ++tile) {
+            const int64_t base = tile * kFiltTile;
+            if (t == 0 && tile + 1 < t1) {   // the next tile streams into L2 meanwhile
+                const uint32_t nn = (uint32_t)std::min<int64_t>(kFiltTile, n - base - kFiltTile);
+                if (((reinterpret_cast<uintptr_t>(pts + 2 * (base + kFiltTile))) & 15u) == 0)
+                    bulk_prefetch_l2(pts + 2 * (base + kFiltTile), (nn * 8u) & ~15u);
+            }
+            uint32_t keep = 0, und = 0, drop = 0;
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                float px[8], py[8];
+                uint32_t live = 0xffu;
+                if (base + kFiltTile <= n) load8<G>(pts, base, t, half, px, py);
+                else live = load8_ragged<G>(pts, n, base, t, half, cx, cy, px, py);
+                if (bits_mode) {
+                    live &= (uint32_t)bits[tile * kFiltThreads + t] >> (8 * half);
+                } else if (!so.has_edges) {
+                } else {
+                    uint32_t in8, und8;
+                    oct_decide<8>(so, px, py, in8, und8);
+                    live &= ~in8;
+                    und |= (live & und8) << (8 * half);
+                }
+                keep |= live << (8 * half);
+                if (!fan || !__any_sync(0xffffffffu, live != 0u)) continue;
+                uint32_t in = 0;
+                if (use_disk) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float dx = __fsub_rn(px[k], cx), dy = __fsub_rn(py[k], cy);
+                        in |= (__fmaf_rn(dx, dx, __fmul_rn(dy, dy)) < rho2t ? 1u : 0u) << k;
+                    }
+                    in &= live;
+                    // a warp that finds under a quarter of its points in the
+                    // disk stops testing it
+                    const unsigned hits = __reduce_add_sync(0xffffffffu, (unsigned)__popc(in));
+                    const unsigned tried = __reduce_add_sync(0xffffffffu, (unsigned)__popc(live));
+                    if (4u * hits < tried) use_disk = false;
+                }
+                uint32_t out = live & ~in;   // to test against the fan
+                if (__reduce_max_sync(0xffffffffu, (unsigned)__popc(out)) <= 2u) {
+#pragma unroll 1
+                    for (; out; out &= out - 1u) {
+                        const float2 p = input_point(pts, item_point<G>(base, t, 8 * half + __ffs(out) - 1));
+                        if (fan_inside<kFanBins>(V, __fsub_rn(p.x, cx), __fsub_rn(p.y, cy), p.x, p.y))
+                            in |= out & (0u - out);
+                    }
+                } else {
+                    uint32_t f = 0;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        f |= (fan_inside<kFanBins>(V, __fsub_rn(px[k], cx), __fsub_rn(py[k], cy), px[k], py[k]) ? 1u : 0u) << k;
+                    in |= f & out;
+                }
+                drop |= in << (8 * half);
+            }
+#pragma unroll 1
+            for (; und; und &= und - 1u) {
+                const float2 p = input_point(pts, item_point<G>(base, t, __ffs(und) - 1));
+                if (!keep_point<false>(so, p.x, p.y)) keep &= ~(und & (0u - und));
+            }
+            octs += __popc(keep);
+            append_survivors(keep & ~drop, count, keys, pay, [&](int q, uint32_t &i) {
+                const int64_t j = item_point<G>(base, t, q);
+                i = (uint32_t)j;
+                return input_point(pts, j);
+            });
+        }
+    }
+    octs = __reduce_add_sync(0xffffffffu, octs);
+    if (lane_id() == 0 && octs) atomicAdd(&s_oct, octs);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_oct) atomicAdd(&kc->s_oct, s_oct);
+}
+
+// ---------------------------------------------------------------------------
+// second level, over the first level's survivors.  On the unit circle the
+// binary32 points scatter about 10^-7 around the circle while a chord of
+// the first fan sags 6 10^-9 below it, so a fan vertex, the farthest
+// sampled point of its bin, leaves the points near the top of that scatter
+// outside its triangles: about a sixteenth of 10^8 points.  The same test
+// with kFan2Sub times as many bins, each vertex the farthest survivor of
+// its sub-bin (every survivor, not a sample), drops most of those.
+//
+//  fan2_max_kernel      whether the level runs (a fan whose proofs hold, and
+//                       at least kFan2MinS points, or the tuned minimum,
+//                       survived); per sub-bin the farthest survivor
+//  fan2_build_kernel    the vertex of every sub-bin (the previous non-empty
+//                       one for an empty sub-bin, cyclically); the proof
+//                       that consecutive ones are counter-clockwise
+//  fan2_test_kernel     the test of every survivor; the kept ones go to the
+//                       sort's second buffers, which the sort then reads
+// ---------------------------------------------------------------------------
+constexpr int F2T = 256;
+constexpr int F2I = 8;   // survivors per thread and step of the test
+static_assert(kFan2Bins % BT == 0, "sub-bins split evenly over the build blocks");
+
+__device__ __forceinline__ float2 surv_point(const uint32_t *keys, const unsigned long long *pay, uint32_t i)
+{
+    return make_float2(key_float(keys[i]), key_float((uint32_t)(pay[i] >> 32)));
+}
+
+__global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint32_t min_s)
+{
+    const Octagon *oct = at<Octagon>(ws, L.oct);
+    const Kgon *g = at<Kgon>(ws, L.kgon);
+    const uint32_t m = at<Ctrl>(ws, L.ctrl)->surv_count;
+    const bool on = !oct->abort && !oct->spec && m >= min_s && fan_ready(at<KgonCtrl>(ws, L.kgon_ctrl), g);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
+        f2->on = on ? 1u : 0u;
+        f2->count_in = on ? m : 0u;
+    }
+    if (!on) return;
+    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
+    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
+    unsigned long long *slot = at<unsigned long long>(ws, L.fan2_slot);
+    const float cx = g->cx, cy = g->cy, r2ref = far_ref(*oct);
+    for (uint32_t i = blockIdx.x * F2T + threadIdx.x; i < m; i += gridDim.x * F2T) {
+        const float2 p = surv_point(keys, pay, i);
+        const int b = vertex_bin<kFan2Bins>(__fsub_rn(p.x, cx), __fsub_rn(p.y, cy), kFan2Margin);
+        if (b < 0) continue;
+        const unsigned long long v = ((unsigned long long)far_key(p.x, p.y, cx, cy, r2ref) << 32) | (uint32_t)~i;
+        if (v > __ldcg(&slot[b])) atomicMax(&slot[b], v);   // the read only saves atomics
+    }
+}
+
+// One thread per sub-bin, as fan_build_kernel; the table's ends are repeated
+// at V[-1] and V[kFan2Bins].
+__global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
+{
+    __shared__ int s_w[BT / 32];
+    __shared__ int s_scan[BT / 32];
+    Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
+    if (!f2->on) return;
+    const unsigned long long *slot = at<unsigned long long>(ws, L.fan2_slot);
+    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
+    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
+    const Kgon *g = at<Kgon>(ws, L.kgon);
+    float2 *V = at<float2>(ws, L.fan2_v) + 1;
+    const int b = (int)(blockIdx.x * BT + threadIdx.x);
+    const int src = vertex_source(slot, s_w, s_scan);
+    if (src < 0) {   // no survivor reached a slot: keep everything
+        if (threadIdx.x == 0) f2->bad = 1u;
+        return;
+    }
+    const float2 v = surv_point(keys, pay, ~(uint32_t)slot[src]);
+    V[b] = v;
+    if (b == 0) V[kFan2Bins] = v;
+    if (b == kFan2Bins - 1) V[-1] = v;
+    const unsigned long long nextp = slot[next_bin<kFan2Bins>(b)];
+    const float2 w = nextp != 0ull ? surv_point(keys, pay, ~(uint32_t)nextp) : v;
+    const bool edge = v.x != w.x || v.y != w.y;
+    // c strictly left of v -> w, proven in binary32 or exactly
+    const bool bad = edge && orient(v.x, v.y, w.x, w.y, g->cx, g->cy) <= 0;
+    const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge));
+    if (lane_id() == 0 && edges) atomicAdd(&f2->edges, edges);
+    if (bad) f2->bad = 1u;
+}
+
+// Bound by the latency of the 1.8 MB table in L2: eight survivors per thread
+// keep their reads in flight together, and only binary32 signs are taken.
+// The order of the survivors is not kept, so the kept ones are appended and
+// need no second pass (test and ordered compaction took 105 + 39 us for the
+// 6.4 M first-level survivors of 10^8 circle points).
+__global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
+{
+    Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
+    if (!f2->on) return;
+    const uint32_t m = f2->count_in;
+    const bool test = !f2->bad && f2->edges >= 3u;
+    const Kgon *g = at<Kgon>(ws, L.kgon);
+    const float cx = g->cx, cy = g->cy;
+    const float2 *V = at<float2>(ws, L.fan2_v) + 1;
+    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
+    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
+    uint32_t *okeys = at<uint32_t>(ws, L.keys[1]);
+    unsigned long long *opay = at<unsigned long long>(ws, L.pay[1]);
+    const uint32_t lane = lane_id();
+    for (uint32_t base = blockIdx.x * (F2T * F2I); base < m; base += gridDim.x * (F2T * F2I)) {
+        uint32_t kv[F2I];
+        unsigned long long pv[F2I];
+        uint32_t keep = 0;
+#pragma unroll
+        for (int k = 0; k < F2I; ++k) {
+            const uint32_t i = base + k * F2T + threadIdx.x;
+            kv[k] = 0u;
+            pv[k] = 0ull;
+            if (i < m) {
+                kv[k] = __ldcs(keys + i);
+                pv[k] = __ldcs(pay + i);
+                keep |= 1u << k;
+            }
+        }
+        if (test) {
+            uint32_t in = 0;
+#pragma unroll
+            for (int k = 0; k < F2I; ++k) {
+                const float x = key_float(kv[k]), y = key_float((uint32_t)(pv[k] >> 32));
+                in |= (fan_inside<kFan2Bins>(V, __fsub_rn(x, cx), __fsub_rn(y, cy), x, y) ? 1u : 0u) << k;
+            }
+            keep &= ~in;
+        }
+        uint32_t incl = __popc(keep);
+        const uint32_t c = incl;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += u;
+        }
+        uint32_t pos = 0;
+        if (lane == 31 && incl) pos = atomicAdd(&f2->kept, incl);
+        pos = __shfl_sync(0xffffffffu, pos, 31) + incl - c;
+#pragma unroll
+        for (int k = 0; k < F2I; ++k) {
+            if ((keep >> k) & 1u) {
+                okeys[pos] = kv[k];
+                opay[pos] = pv[k];
+                ++pos;
+            }
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (atomicAdd(&f2->done, 1u) == gridDim.x - 1) {   // every block's survivors are counted
+            Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
+            ctrl->surv_count = atomicAdd(&f2->kept, 0u);
+            ctrl->sort_in = 1u;
+        }
+    }
+}
+
+template <int G>
+cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const Layout &L, int use_bits,
+                                 const int32_t *kdev, cudaStream_t st)
+{
+    const int sms = sm_count();
+    static const bool attr = [] {   // thread-safe one-time initialisation
+        cudaFuncSetAttribute(hull_filter_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFanSmem);
+        return true;
+    }();
+    (void)attr;
+    const int64_t ntiles = ceil_div(n, kFiltTile);
+    const int has_fan = n >= (int64_t)kKgonMinS ? 1 : 0;   // (fewer points: fewer survivors)
+    if (has_fan) {
+        const int64_t stride = fan_sample_stride(ntiles);
+        const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride), (int64_t)sms * 4);
+        probe_before(CH_K_KGON, st);
+        fan_bins_kernel<G><<<(unsigned)bb, kFiltThreads, 0, st>>>(pts, n, ws, L, (int32_t)stride, use_bits, kdev);
+        fan_build_kernel<<<kFanBins / BT, BT, 0, st>>>(pts, n, ws, L);
+        note_kernels(CH_K_KGON, 2);
+        probe_after(CH_K_KGON, st);
+    }
+    probe_before(CH_K_FILTER, st);
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(ntiles, (int64_t)CG), sms));
+    hull_filter_kernel<G><<<(unsigned)grid, CT, has_fan ? kFanSmem : 0, st>>>(pts, n, ws, L, has_fan, use_bits, kdev);
+    note_kernels(CH_K_FILTER, 1);
+    probe_after(CH_K_FILTER, st);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || L.fan2_bins == 0) return e;   // (a set too small for the second level)
+    probe_before(CH_K_KGON, st);
+    const int lg = tune_value(CH_TUNE_FAN2_MIN_LOG2);
+    fan2_max_kernel<<<sms * 8, F2T, 0, st>>>(ws, L, lg ? (uint32_t)(1ull << lg) : kFan2MinS);
+    fan2_build_kernel<<<kFan2Bins / BT, BT, 0, st>>>(ws, L);
+    const int64_t tb = std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, (int64_t)F2T * F2I), (int64_t)sms * 8));
+    fan2_test_kernel<<<(unsigned)tb, F2T, 0, st>>>(ws, L);
+    note_kernels(CH_K_KGON, 3);
+    probe_after(CH_K_KGON, st);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_hull_filter(const float *pts, int64_t n, void *ws, const Layout &L, const KgonStage *kg,
+                               cudaStream_t st)
+{
+    const bool bits = kg && (kg->kdev || kg->K != 8);   // the second polygon's keep bits
+    if (bits) {
+        int64_t bc = 0;
+        cudaError_t e = launch_filter_count(pts, n, kg->kdev, ws, L, &bc, st);
+        if (e == cudaSuccess) e = launch_kx_sv(pts, n, kg->dirs, kg->kdev, kg->K, kg->ext_out, ws, L, bc, st);
+        if (e != cudaSuccess) return e;
+    }
+    const int32_t *kdev = bits ? kg->kdev : nullptr;
+    return (reinterpret_cast<uintptr_t>(pts) & 15u) == 0
+               ? launch_hull_filter_g<2>(pts, n, ws, L, bits ? 1 : 0, kdev, st)
+               : launch_hull_filter_g<1>(pts, n, ws, L, bits ? 1 : 0, kdev, st);
+}
+
+namespace {
+
+// ---------------------------------------------------------------------------
+// many sets (ch_hull_batched): the same fan for every set with at least
+// kKgonMinS octagon survivors, between the batched count pass and its scan
+// ---------------------------------------------------------------------------
+constexpr int FT = 512;                  // threads per block of the bins pass
+constexpr int FITEMS = 8;                // points per thread per tile there
 // The signs orient_f32 certifies, as two flags (det > bound, -det > bound;
 // neither when undecided or when the terms may have overflowed): the same
 // arithmetic on the rounded differences a - c and b - c, without turning
@@ -104,781 +843,6 @@ __device__ __noinline__ bool fan_inside_exact(const float2 *V, float cx, float c
     return orient(v.x, v.y, w.x, w.y, px, py) == o && orient(w.x, w.y, cx, cy, px, py) == o;
 }
 
-template <int NB = kFanBins>
-__device__ __forceinline__ bool fan_inside(const float2 *V, float cx, float cy, float2 p)
-{
-    const int f = fan_signs_f32<NB>(V, cx, cy, p.x, p.y);
-    return f != 2 ? f == 1 : fan_inside_exact<NB>(V, cx, cy, p.x, p.y);
-}
-
-// The fan runs when the octagon left at least kKgonMinS survivors and has
-// an edge (otherwise it does nothing).
-__device__ __forceinline__ bool fan_live(const KgonCtrl *kc, const Octagon *oct, uint32_t &s)
-{
-    s = oct->abort ? 0u : kc->s_oct;
-    return s >= kKgonMinS && oct->has_edges && !oct->spec;   // spec: no keep bits to refine
-}
-
-// One thread per bin (kFanBins / BT blocks).  The vertex of bin b is the
-// sampled point of the last non-empty bin at or before b, cyclically: a
-// max-scan of "non-empty bin index" inside the block, and for the bins
-// before the block's first non-empty one, the last non-empty bin of the
-// nearest earlier range of BT bins that has one (searched range by range).
-constexpr int BT = 1024;
-static_assert(kFanBins % BT == 0, "bins split evenly over the blocks");
-
-__device__ __forceinline__ int block_max(int v, int *s_w)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    __syncthreads();   // s_w may still be read from an earlier call
-    if (lane_id() == 0) s_w[threadIdx.x >> 5] = v;
-    __syncthreads();
-    int m = -1;
-    for (int w = 0; w < BT / 32; ++w) m = max(m, s_w[w]);
-    return m;
-}
-
-// bc: the grid of the filter's count pass (its block totals are in
-// filt_bsum[0, bc)); the count pass gathered the bins' farthest sampled
-// points (filter.cu).
-__global__ void __launch_bounds__(BT) fan_build_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L,
-                                                       int32_t bc)
-{
-    __shared__ int s_w[BT / 32];
-    __shared__ int s_scan[BT / 32];
-    __shared__ int s_ok;
-    __shared__ uint32_t s_sum[BT / 32];
-    const Octagon *oct = at<Octagon>(ws, L.oct);
-    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
-    Kgon *g = at<Kgon>(ws, L.kgon);
-    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    // octagon survivors: the sum of the count pass's block totals (none
-    // when the call was aborted: the count pass left no totals)
-    uint32_t s = 0;
-    if (!oct->abort) {
-        const uint32_t *bsum = at<uint32_t>(ws, L.filt_bsum);
-        uint32_t t = 0;
-        for (int i = (int)tid; i < bc; i += BT) t += bsum[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) s_sum[warp] = t;
-        __syncthreads();
-        for (int w = 0; w < BT / 32; ++w) s += s_sum[w];
-    }
-    if (blockIdx.x == 0 && tid == 0) kc->s_oct = s;   // read by the later fan kernels
-    if (!(s >= kKgonMinS && oct->has_edges && !oct->spec)) {   // (fan_live, before s_oct is visible)
-        if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
-        return;
-    }
-    const float cx = oct->cx, cy = oct->cy;
-    // c strictly left of every edge of non-zero length: the edges turn once
-    // around c with every step counter-clockwise, so c lies strictly inside
-    // the hull of the octagon's vertices
-    if (tid == 0) s_ok = 1;
-    __syncthreads();
-    if (tid < 8 && ((oct->valid >> tid) & 1u) &&
-        orient(oct->ax[tid], oct->ay[tid], oct->bx[tid], oct->by[tid], cx, cy) <= 0)
-        s_ok = 0;
-    const int b = (int)(blockIdx.x * BT + tid);
-    const unsigned long long mine = kc->slot[b];
-    int incl = mine != 0ull ? b : -1;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl = max(incl, u);
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    for (int w = 0; w < (int)warp; ++w) incl = max(incl, s_scan[w]);
-    // the nearest earlier range with a non-empty bin (the block's own range
-    // last, for the wrap-around)
-    int prev = -1;
-    for (uint32_t k = 1; k <= gridDim.x && prev < 0; ++k) {   // prev is block-uniform
-        const uint32_t rb = (blockIdx.x + gridDim.x - k) % gridDim.x;
-        const int j = (int)(rb * BT + tid);
-        prev = block_max(kc->slot[j] != 0ull ? j : -1, s_w);
-    }
-    if (prev < 0 || !s_ok) {   // no sampled point at all, or c not inside
-        if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
-        return;
-    }
-    const int cur = incl >= 0 ? incl : prev;
-    const uint32_t i = ~(uint32_t)(cur == b ? mine : kc->slot[cur]);
-    g->v[b] = input_point(pts, (int64_t)i < n ? i : 0u);
-    if (blockIdx.x == 0 && tid == 0) {
-        g->cx = cx;
-        g->cy = cy;
-        g->ok = 1u;
-        g->disk_bad = 0u;
-        g->disk_edges = 0u;
-        g->rho2 = 0x7ff0000000000000ull;   // +inf until the estimate kernel bounds it
-    }
-}
-
-// A disk around the centre inside the fan: the fan's triangles (c, v, w) of
-// consecutive vertices turn counter-clockwise around c (bins in angular
-// order), so when every triangle with v != w is proven strictly
-// counter-clockwise their union is a polygon winding once around c, and
-// the open disk of radius rho < the distance from c to each of its edges
-// (segments [v, w], or the point v when v == w) lies in its interior,
-// hence strictly inside the hull.  The distance to a segment is the
-// distance to its nearer end when the foot of the perpendicular from c
-// provably falls outside it, else at least the distance to its line.
-// Binary64 with slack: cross and dot products lose at most 2^-50 of the
-// sum of their terms' magnitudes, squares and the quotient 2^-40.  Returns
-// the lower bound on the squared distance to edge (v, w), or -1 when the
-// triangle is not proven counter-clockwise.
-__device__ __forceinline__ double disk_bound(float cx, float cy, float2 v, float2 w)
-{
-    const double ux = (double)cx - v.x, uy = (double)cy - v.y;   // c - v
-    const double dv = (ux * ux + uy * uy) * (1.0 - 0x1p-40);
-    if (v.x == w.x && v.y == w.y) return dv;
-    const double ex = (double)w.x - v.x, ey = (double)w.y - v.y;   // w - v
-    const double t1 = ex * uy, t2 = ey * ux;
-    const double lo = (t1 - t2) - (fabs(t1) + fabs(t2)) * 0x1p-50;   // c strictly left of v -> w
-    if (!(lo > 0.0)) return -1.0;
-    const double len2 = ex * ex + ey * ey;
-    const double d1 = ex * ux, d2 = ey * uy;
-    const double dot = d1 + d2, derr = (fabs(d1) + fabs(d2)) * 0x1p-50;   // (c - v) . (w - v)
-    if (dot < -derr) return dv;   // the foot lies before v: v is the nearest point
-    if (dot > len2 * (1.0 + 0x1p-40) + derr) {   // after w
-        const double zx = (double)cx - w.x, zy = (double)cy - w.y;
-        return (zx * zx + zy * zy) * (1.0 - 0x1p-40);
-    }
-    return lo * lo / (len2 * (1.0 + 0x1p-40)) * (1.0 - 0x1p-40);
-}
-
-// About 2^16 evenly spaced input points.  With f the share of them inside
-// the fan and s of n points surviving the octagon, the fan drops at least
-// f n - (n - s) of the survivors; the refine pass runs when that is at
-// least s / 8.
-__global__ void __launch_bounds__(256) fan_estimate_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L)
-{
-    __shared__ uint32_t s_in[8], s_tot[8];
-    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
-    uint32_t s;
-    if (!fan_live(kc, at<Octagon>(ws, L.oct), s)) return;
-    const Kgon *g = at<Kgon>(ws, L.kgon);
-    if (!g->ok) return;
-    const int64_t stride = std::max<int64_t>(1, n >> 16);
-    const int64_t nsamp = (n - stride / 2 + stride - 1) / stride;
-    uint32_t in = 0, tot = 0;
-    for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < nsamp; k += (int64_t)gridDim.x * 256) {
-        in += fan_inside(g->v, g->cx, g->cy, input_point(pts, k * stride + stride / 2)) ? 1u : 0u;
-        ++tot;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        in += __shfl_xor_sync(0xffffffffu, in, o);
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    const uint32_t warp = threadIdx.x >> 5;
-    if (lane_id() == 0) {
-        s_in[warp] = in;
-        s_tot[warp] = tot;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t a = 0, b = 0;
-        for (int w = 0; w < 8; ++w) {
-            a += s_in[w];
-            b += s_tot[w];
-        }
-        atomicAdd(&kc->inside, a);
-        atomicAdd(&kc->sample, b);
-    }
-    // the disk around the centre (disk_bound), min over all bins
-    Kgon *gw = at<Kgon>(ws, L.kgon);
-    double mn = __longlong_as_double(0x7ff0000000000000ll);
-    bool bad = false;
-    uint32_t edges = 0;
-    for (int b = (int)(blockIdx.x * 256 + threadIdx.x); b < kFanBins; b += (int)(gridDim.x * 256)) {
-        const float2 v = g->v[b], w = g->v[next_bin(b)];
-        const double d = disk_bound(g->cx, g->cy, v, w);
-        if (d < 0.0) bad = true;
-        else mn = fmin(mn, d);
-        edges += (v.x != w.x || v.y != w.y) ? 1u : 0u;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        edges += __shfl_xor_sync(0xffffffffu, edges, o);
-    }
-    bad = __any_sync(0xffffffffu, bad);
-    if (lane_id() == 0) {
-        atomicMin(&gw->rho2, (unsigned long long)__double_as_longlong(mn));   // >= 0: bits order as values
-        if (bad) atomicOr(&gw->disk_bad, 1u);
-        if (edges) atomicAdd(&gw->disk_edges, edges);
-    }
-}
-
-__device__ __forceinline__ bool fan_worth(const KgonCtrl *kc, int64_t n, uint32_t s)
-{
-    const double f = kc->sample ? (double)kc->inside / (double)kc->sample : 0.0;
-    return kc->sample > 0u && f * (double)n - (double)(n - s) >= (double)s / 8.0;
-}
-
-// Point of item q (of this thread's 16) of a filter tile; the layout is the
-// count pass's: item q = r * G + h is point base + (r * kFiltThreads + t) * G + h.
-template <int G>
-__device__ __forceinline__ int64_t item_point(int64_t base, uint32_t t, int q)
-{
-    return base + (int64_t)((q / G) * kFiltThreads + t) * G + q % G;
-}
-
-// Fan test of one half (items 8 half .. 8 half + 7) of a filter thread's
-// kept points.  Returns the bits (at item positions) of kept points strictly
-// inside the fan.  The coordinates of the few undecided points are read
-// again for the exact test, so none stay live across it.  Called by every
-// lane of the warp (a warp-wide reduction picks the path).
-template <int G>
-__device__ __forceinline__ uint32_t refine_half(const float *__restrict__ pts, int64_t n, int64_t base, uint32_t t,
-                                                uint32_t kb, int half, const float2 *sv, float cx, float cy,
-                                                float rho2t, bool &use_disk)
-{
-    float px[8], py[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) px[k] = py[k] = 0.0f;
-    if constexpr (G == 2) {
-#pragma unroll
-        for (int r4 = 0; r4 < 4; ++r4) {
-            const int r = half * 4 + r4;
-            if ((kb >> (2 * r)) & 3u) {
-                const int64_t i = base + (int64_t)(r * kFiltThreads + t) * 2;
-                float4 v;
-                if (i + 1 < n) {
-                    v = __ldcs(reinterpret_cast<const float4 *>(pts) + i / 2);
-                } else {
-                    const float2 a = reinterpret_cast<const float2 *>(pts)[i];
-                    v = make_float4(a.x, a.y, 0.0f, 0.0f);
-                }
-                px[2 * r4] = v.x;
-                py[2 * r4] = v.y;
-                px[2 * r4 + 1] = v.z;
-                py[2 * r4 + 1] = v.w;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int r = half * 8 + k;
-            if ((kb >> r) & 1u) {
-                const float2 v = __ldcs(reinterpret_cast<const float2 *>(pts) + base + r * kFiltThreads + t);
-                px[k] = v.x;
-                py[k] = v.y;
-            }
-        }
-    }
-    const uint32_t live = (kb >> (8 * half)) & 0xffu;
-    // the disk around the centre first: r2 < rho2t proves |p - c|^2 < rho^2
-    // (rho2t is rho^2 less 2^-20 of it, rounded down, which covers the
-    // rounding of r2); when few of a lane's points lie outside the disk the
-    // fan test visits only those
-    // (use_disk, warp-uniform: a warp whose first half-tile finds fewer than
-    // a quarter of its kept points in the disk stops testing it)
-    uint32_t outd = live;
-    if (use_disk) {
-        outd = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float dx = __fsub_rn(px[k], cx), dy = __fsub_rn(py[k], cy);
-            const float r2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
-            outd |= (r2 < rho2t ? 0u : 1u) << k;
-        }
-        outd &= live;
-        const unsigned hits = __reduce_add_sync(0xffffffffu, (unsigned)__popc(live & ~outd));
-        const unsigned tried = __reduce_add_sync(0xffffffffu, (unsigned)__popc(live));
-        if (4u * hits < tried) use_disk = false;
-    }
-    uint32_t in = live & ~outd;
-    if (__reduce_max_sync(0xffffffffu, (unsigned)__popc(outd)) <= 2u) {
-        for (uint32_t b = outd; b; b &= b - 1u) {
-            const int k = __ffs(b) - 1;
-            const float2 p = reinterpret_cast<const float2 *>(pts)[item_point<G>(base, t, 8 * half + k)];
-            if (fan_inside(sv, cx, cy, p)) in |= 1u << k;
-        }
-        return in << (8 * half);
-    }
-    uint32_t und = 0;
-    in = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int f = fan_signs_f32(sv, cx, cy, px[k], py[k]);
-        in |= (f == 1 ? 1u : 0u) << k;
-        und |= (f == 2 ? 1u : 0u) << k;
-    }
-    in = (in & live) | (live & ~outd);
-    und &= outd;
-    while (und) {
-        const int k = __ffs(und) - 1;
-        und &= und - 1u;
-        const float2 p = reinterpret_cast<const float2 *>(pts)[item_point<G>(base, t, 8 * half + k)];
-        if (fan_inside_exact(sv, cx, cy, p.x, p.y)) in |= 1u << k;
-    }
-    return in << (8 * half);
-}
-
-// The tiles of the filter go in contiguous ranges to groups of
-// kFiltThreads threads (four per block); thread t of a group holds the 16
-// keep bits of filter thread t.  Kept points strictly inside the fan lose
-// their keep bit, and the tile's count and its count block's total drop by
-// the number removed (atomics: no barrier in the loop), so the filter's
-// scatter pass writes only the points that survive both tests.
-template <int G>
-__global__ void __launch_bounds__(CT, 1) fan_refine_kernel(const float *__restrict__ pts, int64_t n, void *ws,
-                                                          Layout L, int32_t bc)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *sv = reinterpret_cast<float2 *>(smem_raw);   // kFanBins vertices
-    const Octagon *oct = at<Octagon>(ws, L.oct);
-    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
-    uint32_t s;
-    if (!fan_live(kc, oct, s)) return;
-    const Kgon *g = at<Kgon>(ws, L.kgon);
-    if (!g->ok || !fan_worth(kc, n, s)) return;
-    {
-        const float4 *src = reinterpret_cast<const float4 *>(g->v);
-        float4 *dst = reinterpret_cast<float4 *>(sv);
-        for (int i = threadIdx.x; i < kFanBins / 2; i += CT) dst[i] = __ldg(src + i);
-    }
-    const float cx = g->cx, cy = g->cy;
-    // -1: no disk (the test never passes for r2 >= 0)
-    // (the triangles wind around c only with three distinct vertices or more)
-    const float rho2t = (g->disk_bad || g->disk_edges < 3u)
-                            ? -1.0f
-                            : __double2float_rd(__longlong_as_double((long long)g->rho2) * (1.0 - 0x1p-20));
-    bool use_disk = rho2t > 0.0f;
-    __syncthreads();
-    uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    uint32_t *bsum = at<uint32_t>(ws, L.filt_bsum);
-    const int64_t ntiles = ceil_div(n, kFiltTile);
-    const int64_t per_block = ceil_div(ntiles, (int64_t)bc);   // tiles per count block
-    const uint32_t grp = threadIdx.x / kFiltThreads, t = threadIdx.x % kFiltThreads, lane = lane_id();
-    const int64_t groups = (int64_t)gridDim.x * CG, gi = (int64_t)blockIdx.x * CG + grp;
-    const int64_t per = ceil_div(ntiles, groups);
-    const int64_t t1 = std::min<int64_t>(ntiles, (gi + 1) * per);
-    for (int64_t tile = gi * per; tile < t1; ++tile) {
-        const int64_t base = tile * kFiltTile;
-        if (t == 0 && tile + 1 < t1) {   // the next tile streams into L2 meanwhile
-            const uint32_t nn = (uint32_t)std::min<int64_t>(kFiltTile, n - base - kFiltTile);
-            if (((reinterpret_cast<uintptr_t>(pts + 2 * (base + kFiltTile))) & 15u) == 0)
-                bulk_prefetch_l2(pts + 2 * (base + kFiltTile), (nn * 8u) & ~15u);
-        }
-        const uint32_t kb = bits[tile * kFiltThreads + t];
-        uint32_t in = 0;
-        // every lane takes both halves (refine_half has a warp-wide
-        // reduction; a half without kept points costs little)
-#pragma unroll 1
-        for (int half = 0; half < 2; ++half)
-            in |= refine_half<G>(pts, n, base, t, kb, half, sv, cx, cy, rho2t, use_disk);
-        if (in) bits[tile * kFiltThreads + t] = (uint16_t)(kb & ~in);
-        uint32_t removed = __popc(in);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, o);
-        if (lane == 0 && removed) {
-            atomicAdd(&status[tile], 0ull - (unsigned long long)removed);   // count - removed >= 0
-            atomicSub(&bsum[tile / per_block], removed);
-        }
-    }
-}
-
-}  // namespace
-
-cudaError_t launch_fan(const float *pts, int64_t n, bool vec, int64_t filter_blocks, void *ws, const Layout &L,
-                       cudaStream_t st)
-{
-    const int sms = sm_count();
-    static const bool attrs = [] {
-        cudaFuncSetAttribute(fan_refine_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFanSmem);
-        cudaFuncSetAttribute(fan_refine_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFanSmem);
-        return true;
-    }();
-    (void)attrs;
-    const int32_t bc = (int32_t)filter_blocks;
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(sms, filter_blocks));
-    probe_before(CH_K_KGON, st);
-    fan_build_kernel<<<kFanBins / BT, BT, 0, st>>>(pts, n, ws, L, bc);
-    fan_estimate_kernel<<<sms, 256, 0, st>>>(pts, n, ws, L);
-    if (vec) fan_refine_kernel<2><<<(unsigned)grid, CT, kFanSmem, st>>>(pts, n, ws, L, bc);
-    else fan_refine_kernel<1><<<(unsigned)grid, CT, kFanSmem, st>>>(pts, n, ws, L, bc);
-    note_kernels(CH_K_KGON, 3);
-    probe_after(CH_K_KGON, st);
-    return cudaGetLastError();
-}
-
-namespace {
-
-// ---------------------------------------------------------------------------
-// second level, over the first level's survivors (the filter's scatter
-// output: sort keys and payloads in point order).  On the unit circle the
-// binary32 points scatter about 10^-7 around the circle while a chord of
-// the first fan sags 6 10^-9 below it, so a fan vertex, the farthest
-// sampled point of its bin, leaves the points near the top of that scatter
-// outside its triangles: about a sixth of the points reach the sort.  The
-// same test with kFan2Sub times as many bins, each vertex the farthest
-// survivor of its sub-bin (every survivor, not a sample), drops most of
-// those.  The vertices are again input points and the centre is the
-// first level's, so the same argument holds: a survivor strictly inside a
-// triangle (c, v, w) is no hull vertex.  Kernels (grid-wide passes, after
-// the scatter):
-//
-//  fan2_max_kernel      whether the level runs (the first level's centre
-//                       was proven inside and at least kFan2MinS points,
-//                       or the tuned minimum, survived); per sub-bin the
-//                       farthest survivor
-//  fan2_build_kernel    the vertex of every sub-bin (the previous
-//                       non-empty one for an empty sub-bin, cyclically)
-//  fan2_test_kernel     per tile of 4096 survivors the exact test, keep bits
-//                       and counts (in the filter's keep-bit, tile-count and
-//                       block-total buffers, free by then)
-//  fan2_scatter_kernel  the kept survivors, in their order, into the sort's
-//                       second buffers; the sort then reads those
-// ---------------------------------------------------------------------------
-constexpr int F2T = 256;
-static_assert(kFan2Bins % BT == 0, "sub-bins split evenly over the build blocks");
-static_assert(F2T == kFiltThreads, "the test pass keeps the filter's keep-bit layout");
-
-__device__ __forceinline__ float2 surv_point(const uint32_t *keys, const unsigned long long *pay, uint32_t i)
-{
-    return make_float2(key_float(keys[i]), key_float((uint32_t)(pay[i] >> 32)));
-}
-
-__global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint32_t min_s)
-{
-    const Octagon *oct = at<Octagon>(ws, L.oct);
-    const Kgon *g = at<Kgon>(ws, L.kgon);
-    const uint32_t m = at<Ctrl>(ws, L.ctrl)->surv_count;
-    // g->ok is this call's: the fan kernels ran before (they clear it when
-    // the fan does not run)
-    const bool on = !oct->abort && g->ok && m >= min_s;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
-        f2->on = on ? 1u : 0u;
-        f2->count_in = on ? m : 0u;
-    }
-    if (!on) return;
-    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
-    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
-    unsigned long long *slot = at<unsigned long long>(ws, L.fan2_slot);
-    const float cx = g->cx, cy = g->cy, r2ref = far_ref(*oct);
-    for (uint32_t i = blockIdx.x * F2T + threadIdx.x; i < m; i += gridDim.x * F2T) {
-        const float2 p = surv_point(keys, pay, i);
-        const float dx = __fsub_rn(p.x, cx), dy = __fsub_rn(p.y, cy);
-        const int b = fan_bin<kFan2Bins>(dx, dy);
-        const unsigned long long v = ((unsigned long long)far_key(p.x, p.y, cx, cy, r2ref) << 32) | (uint32_t)~i;
-        if (v > __ldcg(&slot[b])) atomicMax(&slot[b], v);   // the read only saves atomics
-    }
-}
-
-// One thread per sub-bin, as fan_build_kernel.
-__global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
-{
-    __shared__ int s_w[BT / 32];
-    __shared__ int s_scan[BT / 32];
-    Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
-    if (!f2->on) return;
-    const unsigned long long *slot = at<unsigned long long>(ws, L.fan2_slot);
-    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
-    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
-    float2 *V = at<float2>(ws, L.fan2_v);
-    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    const int b = (int)(blockIdx.x * BT + tid);
-    const unsigned long long mine = slot[b];
-    int incl = mine != 0ull ? b : -1;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl = max(incl, u);
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    for (int w = 0; w < (int)warp; ++w) incl = max(incl, s_scan[w]);
-    int prev = -1;
-    for (uint32_t k = 1; k <= gridDim.x && prev < 0; ++k) {   // prev is block-uniform
-        const uint32_t rb = (blockIdx.x + gridDim.x - k) % gridDim.x;
-        const int j = (int)(rb * BT + tid);
-        prev = block_max(slot[j] != 0ull ? j : -1, s_w);
-    }
-    if (prev < 0) {   // no survivor reached a slot: keep everything
-        if (tid == 0) f2->bad = 1u;
-        return;
-    }
-    const int cur = incl >= 0 ? incl : prev;
-    const uint32_t i = ~(uint32_t)(cur == b ? mine : slot[cur]);
-    V[b] = surv_point(keys, pay, i);
-}
-
-// Per-tile survivor counts of a window of tiles, added up in shared memory
-// as the warps finish each tile (as in the filter's count pass).
-constexpr int kF2Ring = 256;
-
-__global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
-{
-    __shared__ uint32_t s_cnt[kF2Ring];
-    __shared__ uint32_t s_w[F2T / 32];
-    const Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
-    if (!f2->on) return;
-    const uint32_t m = f2->count_in;
-    const bool none = f2->bad != 0u;
-    const Kgon *g = at<Kgon>(ws, L.kgon);
-    const float cx = g->cx, cy = g->cy;
-    const float2 *V = at<float2>(ws, L.fan2_v);
-    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
-    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
-    uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    for (int i = threadIdx.x; i < kF2Ring; i += F2T) s_cnt[i] = 0u;
-    __syncthreads();
-    const int64_t ntiles = ceil_div((int64_t)m, kFiltTile);
-    const int64_t per = ceil_div(ntiles, (int64_t)gridDim.x);
-    const int64_t t1 = std::min<int64_t>(ntiles, (int64_t)(blockIdx.x + 1) * per);
-    uint32_t part = 0;
-    for (int64_t w0 = (int64_t)blockIdx.x * per; w0 < t1; w0 += kF2Ring) {
-        const int64_t w1 = std::min<int64_t>(t1, w0 + kF2Ring);
-        for (int64_t tile = w0; tile < w1; ++tile) {
-            const uint32_t base = (uint32_t)(tile * kFiltTile);
-            uint32_t keep = 0;
-            // eight survivors at a time: binary32 signs without branches (the
-            // table loads of the eight overlap), then the exact tiers for
-            // the undecided ones
-#pragma unroll 1
-            for (int h = 0; h < kFiltItems / 8; ++h) {
-                float2 q[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const uint32_t i = base + (8 * h + k) * F2T + threadIdx.x;
-                    q[k] = i < m ? surv_point(keys, pay, i) : make_float2(cx, cy);
-                }
-                uint32_t live = 0, in = 0, und = 0;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    live |= (base + (8 * h + k) * F2T + threadIdx.x < m ? 1u : 0u) << k;
-                    const int f = fan_signs_f32<kFan2Bins>(V, cx, cy, q[k].x, q[k].y);
-                    in |= (f == 1 ? 1u : 0u) << k;
-                    und |= (f == 2 ? 1u : 0u) << k;
-                }
-                und &= live;   // (positions past the list hold the centre: never read again)
-                while (und) {
-                    const int k = __ffs(und) - 1;
-                    und &= und - 1u;
-                    const float2 p = surv_point(keys, pay, base + (8 * h + k) * F2T + threadIdx.x);
-                    if (fan_inside_exact<kFan2Bins>(V, cx, cy, p.x, p.y)) in |= 1u << k;
-                }
-                keep |= (live & (none ? 0xffu : ~in)) << (8 * h);
-            }
-            bits[tile * F2T + threadIdx.x] = (uint16_t)keep;
-            uint32_t c = __popc(keep);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-            if (lane_id() == 0 && c) atomicAdd(&s_cnt[tile - w0], c);
-        }
-        __syncthreads();
-        for (int64_t i = threadIdx.x; i < w1 - w0; i += F2T) {
-            const uint32_t v = s_cnt[i];
-            status[w0 + i] = v;
-            s_cnt[i] = 0u;
-            part += v;
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if (lane_id() == 0) s_w[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (int w = 0; w < F2T / 32; ++w) t += s_w[w];
-        at<uint32_t>(ws, L.filt_bsum)[blockIdx.x] = t;
-    }
-}
-
-// One warp writes the kept survivors of one tile in order (thread t of the
-// test pass held items base + r * 256 + t, r < 16: eight groups of 32
-// threads, each row's first output position from the warp's row counts).
-__device__ __forceinline__ void fan2_scatter_tile(const uint32_t *__restrict__ keys,
-                                                  const unsigned long long *__restrict__ pay,
-                                                  const uint16_t *__restrict__ tbits, uint32_t base, uint32_t out_off,
-                                                  uint32_t *out_keys, unsigned long long *out_pay)
-{
-    const uint32_t lane = lane_id(), lt = (1u << lane) - 1u;
-    uint32_t kb[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) kb[k] = tbits[k * 32 + lane];
-    uint32_t racc[kFiltItems];
-    {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = kb[2 * j] | (kb[2 * j + 1] << 16);
-        uint32_t run = out_off;
-#pragma unroll
-        for (int r = 0; r < kFiltItems; ++r) {
-            uint32_t c = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) c += __popc(w[j] & (0x10001u << r));
-            racc[r] = run;
-            run += __reduce_add_sync(0xffffffffu, c);
-        }
-    }
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-        const uint32_t kbk = tbits[k * 32 + lane];
-        if (!__any_sync(0xffffffffu, kbk != 0u)) continue;
-        const uint32_t t = k * 32 + lane;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t kv[8];
-            unsigned long long pv[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int r = 8 * h + q;
-                kv[q] = 0u;
-                pv[q] = 0ull;
-                if ((kbk >> r) & 1u) {
-                    kv[q] = keys[base + r * F2T + t];
-                    pv[q] = pay[base + r * F2T + t];
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int r = 8 * h + q;
-                const uint32_t mk = (kbk >> r) & 1u;
-                const uint32_t b0 = __ballot_sync(0xffffffffu, mk);
-                if (!b0) continue;
-                const uint32_t pos = racc[r] + __popc(b0 & lt);
-                racc[r] += __popc(b0);
-                if (mk) {
-                    out_keys[pos] = kv[q];
-                    out_pay[pos] = pv[q];
-                }
-            }
-        }
-    }
-}
-
-// Launched with the test pass's grid: block b owns the same tile range, its
-// output offset the earlier blocks' totals.  Block 0 hands the kept list to
-// the sort (count, buffer 1).
-__global__ void __launch_bounds__(F2T) fan2_scatter_kernel(void *ws, Layout L)
-{
-    __shared__ uint32_t s_red[2][F2T / 32];
-    __shared__ uint32_t s_list[F2T];
-    __shared__ uint32_t s_loff[F2T];
-    __shared__ uint32_t s_nlist;
-    const Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
-    if (!f2->on) return;
-    const uint32_t m = f2->count_in;
-    const unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    const uint32_t *bsum = at<uint32_t>(ws, L.filt_bsum);
-    const uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
-    const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
-    uint32_t *out_keys = at<uint32_t>(ws, L.keys[1]);
-    unsigned long long *out_pay = at<unsigned long long>(ws, L.pay[1]);
-    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
-    constexpr int NWF = F2T / 32;
-    uint32_t before = 0, total = 0;
-    for (uint32_t i = tid; i < gridDim.x; i += F2T) {
-        const uint32_t v = bsum[i];
-        total += v;
-        if (i < blockIdx.x) before += v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        before += __shfl_xor_sync(0xffffffffu, before, o);
-        total += __shfl_xor_sync(0xffffffffu, total, o);
-    }
-    if (lane == 0) {
-        s_red[0][warp] = before;
-        s_red[1][warp] = total;
-    }
-    __syncthreads();
-    before = total = 0;
-#pragma unroll
-    for (int w = 0; w < NWF; ++w) {
-        before += s_red[0][w];
-        total += s_red[1][w];
-    }
-    if (blockIdx.x == 0 && tid == 0) {
-        Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
-        ctrl->surv_count = total;
-        ctrl->sort_in = 1u;
-    }
-    __syncthreads();   // s_red is reused below
-    const int64_t ntiles = ceil_div((int64_t)m, kFiltTile);
-    const int64_t per = ceil_div(ntiles, (int64_t)gridDim.x);
-    const int64_t r0 = (int64_t)blockIdx.x * per, r1 = std::min<int64_t>(ntiles, r0 + per);
-    uint32_t run = before;
-    for (int64_t c0 = r0; c0 < r1; c0 += F2T) {
-        const int64_t t = c0 + tid;
-        const uint32_t cnt = t < r1 ? (uint32_t)(status[t] & 0xffffffffull) : 0u;
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= (uint32_t)o) incl += u;
-        }
-        const uint32_t nz = __ballot_sync(0xffffffffu, cnt != 0u);
-        if (lane == 31) {
-            s_red[0][warp] = incl;
-            s_red[1][warp] = __popc(nz);
-        }
-        __syncthreads();
-        uint32_t wbefore = 0, chunk_total = 0, lbefore = 0, nlist = 0;
-#pragma unroll
-        for (int w = 0; w < NWF; ++w) {
-            if (w < (int)warp) {
-                wbefore += s_red[0][w];
-                lbefore += s_red[1][w];
-            }
-            chunk_total += s_red[0][w];
-            nlist += s_red[1][w];
-        }
-        if (cnt != 0u) {
-            const uint32_t slot = lbefore + __popc(nz & ((1u << lane) - 1u));
-            s_list[slot] = tid;
-            s_loff[slot] = run + wbefore + incl - cnt;
-        }
-        if (tid == 0) s_nlist = nlist;
-        __syncthreads();
-        const uint32_t nl = s_nlist;
-        for (uint32_t li = warp; li < nl; li += NWF) {
-            const int64_t tile = c0 + s_list[li];
-            fan2_scatter_tile(keys, pay, bits + tile * F2T, (uint32_t)(tile * kFiltTile), s_loff[li], out_keys,
-                              out_pay);
-        }
-        __syncthreads();   // s_list, s_loff and s_red are rebuilt for the next chunk
-        run += chunk_total;
-    }
-}
-
-}  // namespace
-
-cudaError_t launch_fan2(int64_t n, void *ws, const Layout &L, cudaStream_t st)
-{
-    if (L.fan2_bins == 0) return cudaSuccess;   // a set too small for the second level
-    const int sms = sm_count();
-    const int64_t tiles = ceil_div(n, kFiltTile);   // survivor tiles at most
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>((int64_t)sms * 4, kFiltMaxBlocks), tiles));
-    probe_before(CH_K_KGON, st);
-    const int lg = tune_value(CH_TUNE_FAN2_MIN_LOG2);
-    const uint32_t min_s = lg ? (uint32_t)(1ull << lg) : kFan2MinS;
-    fan2_max_kernel<<<sms * 8, F2T, 0, st>>>(ws, L, min_s);
-    fan2_build_kernel<<<kFan2Bins / BT, BT, 0, st>>>(ws, L);
-    fan2_test_kernel<<<(unsigned)grid, F2T, 0, st>>>(ws, L);
-    fan2_scatter_kernel<<<(unsigned)grid, F2T, 0, st>>>(ws, L);
-    note_kernels(CH_K_KGON, 4);
-    probe_after(CH_K_KGON, st);
-    return cudaGetLastError();
-}
-
-namespace {
-
-// ---------------------------------------------------------------------------
-// many sets (ch_hull_batched): the same fan for every set with at least
-// kKgonMinS octagon survivors, between the batched count pass and its scan
-// ---------------------------------------------------------------------------
 constexpr int kBxBinStride = 2;   // built-in: the bins see every 2nd tile of a set (1 and 4 measured slower overall)
 
 // One block: numbers the sets that get a fan and lays out the refine's

@@ -31,26 +31,30 @@ cudaError_t launch_extremes(const float *pts, int64_t n, void *ws, const Layout 
 cudaError_t launch_octagon(const float *pts, int64_t n, const uint32_t *ext8, void *ws, const Layout &L,
                            unsigned long long *zero_ptr, int64_t zero_words, cudaStream_t st);
 
-// point test + stable compaction.  keys_mode: write (x key, (y key, index))
-// pairs into the sort buffers of ws instead of (index, point) outputs.
-// variant: 0 two passes (needs keep_bits in L), 1 single pass, -1 the
-// process-wide choice of ch_filter_variant.  fan (hull step, two passes
-// only): launch_fan between the count and the scatter pass.  data_extremes:
-// the polygon was built from the data's own extremes (ch_hull,
-// ch_extremes_filter; always so in keys mode), which allows the speculative
-// sweep's candidates; otherwise the vertices are the caller's (ch_filter).
-// A second polygon between the count pass and the fan (two passes only):
-// the K-direction polygon over the octagon's survivors (launch_kx_sv).
+// point test + stable compaction.  variant: 0 two passes (needs keep_bits in
+// L), 1 single pass, -1 the process-wide choice of ch_filter_variant.
+// data_extremes: the polygon was built from the data's own extremes
+// (ch_extremes_filter), which allows the speculative sweep's candidates;
+// otherwise the vertices are the caller's (ch_filter).
+cudaError_t launch_filter(const float *pts, int64_t n, void *ws, const Layout &L, uint32_t *surv_idx,
+                          float *surv_pts, uint32_t *surv_count, cudaStream_t st, int variant = -1,
+                          bool data_extremes = false);
+// the hull step's survivors (sort keys and payloads in buffer 0) with the
+// single-pass schedule
+cudaError_t launch_filter_keys_single(const float *pts, int64_t n, void *ws, const Layout &L, cudaStream_t st);
+// the count pass alone (the data's own extremes), its grid in *grid; kdev:
+// the device's choice of K, 8: the pass returns at once
+cudaError_t launch_filter_count(const float *pts, int64_t n, const int32_t *kdev, void *ws, const Layout &L,
+                                int64_t *grid, cudaStream_t st);
+
+// A second polygon of ch_hull (two passes only): the K-direction polygon
+// over the octagon's survivors (launch_kx_sv).
 struct KgonStage {
     const float *dirs;       // device, K directions (cos, sin)
     const int32_t *kdev;     // device choice of K, or NULL: K below
     int K;                   // 16, 32 or 64 (8: no stage) when kdev is NULL
     uint32_t *ext_out;       // device, K vertex indices, or NULL
 };
-cudaError_t launch_filter(const float *pts, int64_t n, void *ws, const Layout &L, uint32_t *surv_idx,
-                          float *surv_pts, uint32_t *surv_count, bool keys_mode, cudaStream_t st,
-                          int variant = -1, bool fan = false, bool data_extremes = false,
-                          const KgonStage *kgon = nullptr);
 
 // the process-wide compaction schedule (ch_filter_variant)
 int filter_variant();
@@ -82,16 +86,11 @@ cudaError_t launch_kx_sv(const float *pts, int64_t n, const float *dirs, const i
 cudaError_t launch_learned_choice(const float *pts, int64_t n, const void *params, void *ws, const Layout &L,
                                   cudaStream_t st);
 
-// hull step: the fan test applied to the keep bits, tile counts and block
-// totals that the filter's count pass (filter_blocks blocks) left in ws;
-// may do nothing.  vec: the count pass used 16-byte point pairs.
-// The second fan level over the survivors the filter's scatter wrote (sort
-// keys and payloads in buffer 0): when it runs, the kept ones go to buffer 1
-// and the sort reads those (Ctrl::sort_in).  After launch_fan and the
-// scatter of the same call; does nothing for sets without its tables.
-cudaError_t launch_fan2(int64_t n, void *ws, const Layout &L, cudaStream_t st);
-cudaError_t launch_fan(const float *pts, int64_t n, bool vec, int64_t filter_blocks, void *ws, const Layout &L,
-                       cudaStream_t st);
+// hull step: the survivors of the octagon (or of the second polygon kg),
+// less the points inside a fan of triangles around the centre where that
+// pays, as sort keys and payloads; their number in Ctrl::surv_count
+cudaError_t launch_hull_filter(const float *pts, int64_t n, void *ws, const Layout &L, const KgonStage *kg,
+                               cudaStream_t st);
 
 // the whole hull in one block when few points survived the filter (the
 // sort and chain kernels then stop at once); otherwise nothing

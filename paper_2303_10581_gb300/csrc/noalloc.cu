@@ -115,7 +115,7 @@ extern "C" ch_status ch_filter_noalloc(const float *pts, int64_t n, const uint32
                                    (int64_t)L.zero_words, st);
     if (e != cudaSuccess) return CH_ERR_CUDA;
     // the single-pass schedule: its only scratch is the look-back status
-    e = launch_filter(pts, n, scratch, L, surv_idx, surv_pts, surv_count, false, st, 1);
+    e = launch_filter(pts, n, scratch, L, surv_idx, surv_pts, surv_count, st, 1);
     if (e != cudaSuccess) return CH_ERR_CUDA;
     noalloc_status_kernel<<<1, 1, 0, st>>>(scratch, L, surv_count);
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ERR_CUDA;
