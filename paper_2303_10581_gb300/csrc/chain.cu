@@ -61,6 +61,7 @@ constexpr int SC = kChainC;         // points per super-chunk
 constexpr int CS = kChainStride;    // chain slots per super-chunk
 constexpr int NL = SC + 2;          // sequence capacity: SC points + 2 look-ahead slots
 constexpr int NWB = LT / 32;        // warps per block
+constexpr int kLongRun = 32;        // a longer run of equal x is reduced by a warp
 constexpr int LWMAX = ((NL + NWB - 1) / NWB + 31) / 32;   // longest leaf (17)
 
 // pop / advance test: lower chains drop a vertex when the turn is not
@@ -190,6 +191,8 @@ struct ChainSmem {
     int has_prev;
     int seq_len;
     int wcur, wdone;              // single-warp passes: buffer and convergence
+    int nlong;                    // runs longer than kLongRun, and which
+    uint16_t lrun[SC / (kLongRun + 1) + 1];
 };
 
 // leaf c's entries start at flat[lb[c]]; its stack holds offsets from there
@@ -538,31 +541,83 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
         }
         const bool holds_last = run_end == send;
         __syncthreads();
-        // ---- representatives: lowest (list[0]) and highest (list[1]) point of each run
+        // ---- representatives: lowest (list[0]) and highest (list[1]) point of
+        // each run; equal points (the sort does not order a run): the lowest
+        // index.  A thread takes a short run, a warp a long one (the extreme
+        // x of a circle holds thousands of points: 120 us for one thread).
+        const auto index_of = [&](int e) {
+            return e < SC ? (uint32_t)__ldg(P.pay + base + e) : sm.ext_idx[e - SC];
+        };
+        const auto lower = [&](float y, int e, float y0, int e0) {
+            return y < y0 || (y == y0 && e != e0 && index_of(e) < index_of(e0));
+        };
+        const auto higher = [&](float y, int e, float y0, int e0) {
+            return y > y0 || (y == y0 && e != e0 && index_of(e) < index_of(e0));
+        };
+        const auto put = [&](int k, int lo, float ylo, int hi, float yhi) {
+            if (k == R - 1 && ext) {
+                if (lower(sm.pts[SC].y, SC, ylo, lo)) lo = SC;
+                if (higher(sm.pts[SC + 1].y, SC + 1, yhi, hi)) hi = SC + 1;
+            }
+            sm.list[0][k] = (uint16_t)lo;
+            sm.list[1][k] = (uint16_t)hi;
+        };
+        if (t == 0) sm.nlong = 0;
+        __syncthreads();
         for (int k = t; k < R; k += LT) {
             const int r0 = sm.list[2][k];
             const int r1 = k + 1 < R ? sm.list[2][k + 1] : m;
+            if (r1 - r0 > kLongRun) {
+                sm.lrun[atomicAdd(&sm.nlong, 1)] = (uint16_t)k;
+                continue;
+            }
             int lo = r0, hi = r0;
             float ylo = sm.pts[r0].y, yhi = ylo;
-            // equal points (the sort does not order a run): the lowest index
-            const auto before = [&](uint32_t a, int b) { return a < (uint32_t)__ldg(P.pay + base + b); };
             for (int i = r0 + 1; i < r1; ++i) {
                 const float y = sm.pts[i].y;
-                if (y < ylo || (y == ylo && before((uint32_t)__ldg(P.pay + base + i), lo))) {
+                if (lower(y, i, ylo, lo)) {
                     ylo = y;
                     lo = i;
                 }
-                if (y > yhi || (y == yhi && before((uint32_t)__ldg(P.pay + base + i), hi))) {
+                if (higher(y, i, yhi, hi)) {
                     yhi = y;
                     hi = i;
                 }
             }
-            if (k == R - 1 && ext) {
-                if (sm.pts[SC].y < ylo || (sm.pts[SC].y == ylo && before(sm.ext_idx[0], lo))) lo = SC;
-                if (sm.pts[SC + 1].y > yhi || (sm.pts[SC + 1].y == yhi && before(sm.ext_idx[1], hi))) hi = SC + 1;
+            put(k, lo, ylo, hi, yhi);
+        }
+        __syncthreads();
+        for (int q = warp; q < sm.nlong; q += NWB) {
+            const int k = sm.lrun[q];
+            const int r0 = sm.list[2][k];
+            const int r1 = k + 1 < R ? sm.list[2][k + 1] : m;
+            int lo = r0 + lane, hi = lo;   // (a long run has a point for every lane)
+            float ylo = sm.pts[lo].y, yhi = ylo;
+            for (int i = lo + 32; i < r1; i += 32) {
+                const float y = sm.pts[i].y;
+                if (lower(y, i, ylo, lo)) {
+                    ylo = y;
+                    lo = i;
+                }
+                if (higher(y, i, yhi, hi)) {
+                    yhi = y;
+                    hi = i;
+                }
             }
-            sm.list[0][k] = (uint16_t)lo;
-            sm.list[1][k] = (uint16_t)hi;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float y1 = __shfl_xor_sync(0xffffffffu, ylo, o), y2 = __shfl_xor_sync(0xffffffffu, yhi, o);
+                const int e1 = __shfl_xor_sync(0xffffffffu, lo, o), e2 = __shfl_xor_sync(0xffffffffu, hi, o);
+                if (lower(y1, e1, ylo, lo)) {
+                    ylo = y1;
+                    lo = e1;
+                }
+                if (higher(y2, e2, yhi, hi)) {
+                    yhi = y2;
+                    hi = e2;
+                }
+            }
+            if (lane == 0) put(k, lo, ylo, hi, yhi);
         }
         __syncthreads();
         const uint16_t first_lo = sm.list[0][0];

@@ -84,15 +84,16 @@ struct ExtCtrl {
 
 // second throw-away step of the hull step (kgon.cu): a fan of triangles
 // around the bounding-box centre, one vertex per angular bin
-// (28672 vertices of 8 bytes fill 224 KB: as many as one block's shared
-// memory holds)
-constexpr int kFanBins = 28672;
+// (27648 vertices of 8 bytes are 216 KB: with the filter pass's queues beside
+// them, as many as one block's shared memory holds)
+constexpr int kFanBins = 27648;
 
 struct KgonCtrl {                          // zeroed with the control block
     unsigned long long slot[kFanBins];     // packed (far_key << 32 | ~index): farthest sampled input point per bin
     uint32_t sample, inside;               // points sampled for the bins, octagon survivors among them
     uint32_t s_oct;                        // octagon survivors
-    uint32_t bad;                          // 1: consecutive vertices not proven counter-clockwise around c
+    uint32_t bad;                          // bit 0: samples in one place only; bit 1: consecutive vertices not
+                                           // proven counter-clockwise around c
     uint32_t rho_inv;                      // ~bits of a lower bound (binary32) on the squared distance from
                                            // c to the fan's boundary, the largest so far
     uint32_t edges;                        // consecutive vertex pairs with v != w
@@ -102,7 +103,7 @@ struct KgonCtrl {                          // zeroed with the control block
 // second fan level (kgon.cu): over the first level's survivors, kFan2Sub
 // sub-bins per bin, each vertex the farthest survivor of its sub-bin
 constexpr int kFan2Sub = 8;
-constexpr int kFan2Bins = kFanBins * kFan2Sub;   // 229376
+constexpr int kFan2Bins = kFanBins * kFan2Sub;   // 221184
 constexpr uint32_t kFan2MinS = 1u << 19;         // fewer survivors of the first level: the sort takes them
 constexpr int64_t kFan2MinN = 1 << 19;           // smaller sets get no tables
 
@@ -120,7 +121,8 @@ struct Kgon {
     float cx, cy;                          // fan centre
     uint32_t ok;                           // 0: no fan this call
     uint32_t pad;
-    float2 v[kFanBins];                    // vertex of every bin (input points)
+    float2 v[kFanBins];                    // vertex of every bin
+    float2 raw[kFanBins];                  // the same before empty bins are filled (x = NaN: none)
 };
 
 // K-direction filter polygon (kfilter.cu; the learned proposal's filter)
@@ -232,7 +234,7 @@ struct Layout {
     size_t utmp;          // u32[n]
     size_t spec, p0;        // SpecCtrl, the speculative sweep's test region (SpecBox, extremes.cu)
     size_t learn;           // the learned proposal's scratch (LearnScratch)
-    size_t fan2_v;          // float2[fan2_bins + 2]: the second fan level's vertices, the ends repeated
+    size_t fan2_v;          // float2[fan2_bins + 3]: the second fan level's vertices, the ends repeated
     size_t total;
     int64_t n, filt_tiles, sort_tiles, n_chunks, n_nodes, emit_tiles;
     int64_t fan2_bins;      // kFan2Bins for sets of at least kFan2MinN points, else 0 (no second level)
@@ -371,7 +373,7 @@ __host__ __device__ inline Layout make_layout(int64_t n, int64_t sets = 0)
     L.spec = take(sizeof(SpecCtrl));
     L.p0 = take(256);
     L.learn = take(sizeof(LearnScratch));
-    L.fan2_v = take((size_t)(L.fan2_bins + 2) * 8);
+    L.fan2_v = take((size_t)(L.fan2_bins + 3) * 8);
     L.total = o;
     return L;
 }
@@ -599,6 +601,49 @@ __device__ __forceinline__ int orient(float ax, float ay, float bx, float by, fl
 {
     const int o = orient_f32(ax, ay, bx, by, cx, cy);
     return o != 2 ? o : orient_rest(ax, ay, bx, by, cx, cy);
+}
+
+// ---------------------------------------------------------------------------
+// packed binary32 pairs and three-operand minima (sm_100 and later): one
+// instruction for two differences or FMAs, each rounded as on its own
+// ---------------------------------------------------------------------------
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a.x, a.y)), "l"(pack2(b.x, b.y)));
+    return unpack2(r);
+}
+// NaN-propagating minima
+__device__ __forceinline__ float min_nan(float a, float b)
+{
+    float d;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ float min_nan(float a, float b, float c)
+{
+    float d;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
 // ---------------------------------------------------------------------------

@@ -16,25 +16,47 @@ __host__ __device__ inline int64_t fan_sample_stride(int64_t tiles)
 }
 
 // Scaled pseudo-angle of the direction (dx, dy): in [0, NB], growing with
-// the angle counter-clockwise from +x; bin b holds [b, b + 1).
+// the angle counter-clockwise from -y; bin b holds [b, b + 1).  With t = dy /
+// (|dx| + |dy|) it is (1 + t) NB / 4 on the right and (3 - t) NB / 4 on the
+// left: one test and one FMA.  (dx = dy = 0 gives a NaN.)
+__device__ __forceinline__ float fan_turn(float dx, float dy)   // t on the right, -t on the left
+{
+    float r;   // (at most 1 ulp off; a subnormal sum counts as zero)
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__fadd_rn(fabsf(dx), fabsf(dy))));
+    return __uint_as_float(__float_as_uint(__fmul_rn(dy, r)) ^ (__float_as_uint(dx) & 0x80000000u));
+}
+
 template <int NB = kFanBins>
 __device__ __forceinline__ float fan_phi(float dx, float dy)
 {
-    const float s = fabsf(dx) + fabsf(dy);
-    float a = 0.0f;
-    if (s > 0.0f) {
-        const float t = __fdividef(dy, s);
-        a = dx >= 0.0f ? (dy >= 0.0f ? t : 4.0f + t) : 2.0f - t;
-    }
-    return a * (NB / 4.0f);
+    const bool left = (int)__float_as_uint(dx) < 0;
+    return __fmaf_rn(fan_turn(dx, dy), NB / 4.0f, left ? 3.0f * NB / 4.0f : NB / 4.0f);
 }
 
-// Its bin (phi is in [0, NB], a NaN from an overflowed difference converts
-// to 0: only the top needs a clamp).
+// kBinBias + its bin, the bin in [0, NB] (a NaN: kBinBias + NB): the same FMA
+// shifted by 2^23 and rounded down leaves the bin in the low mantissa bits.
+constexpr uint32_t kBinBias = 0x4b000000u;
 template <int NB = kFanBins>
-__device__ __forceinline__ int fan_bin(float dx, float dy)
+__device__ __forceinline__ uint32_t fan_bin_biased(float dx, float dy)
 {
-    return min(__float2int_rz(fan_phi<NB>(dx, dy)), NB - 1);
+    static_assert(NB % 4 == 0 && NB < (1 << 22), "the shifted offsets are exact");
+    const bool left = (int)__float_as_uint(dx) < 0;
+    const float f = __fmaf_rd(fan_turn(dx, dy), NB / 4.0f, left ? 0x1p23f + 3.0f * NB / 4.0f : 0x1p23f + NB / 4.0f);
+    return min(__float_as_uint(f), kBinBias + (uint32_t)NB);
+}
+template <int NB = kFanBins>
+__device__ __forceinline__ uint32_t fan_bin(float dx, float dy)
+{
+    return fan_bin_biased<NB>(dx, dy) - kBinBias;
+}
+
+// The direction of pseudo-angle a / NB of the full turn (|x| + |y| = 1).
+template <int NB = kFanBins>
+__device__ __forceinline__ float2 fan_direction(float a)
+{
+    const float q = a * (4.0f / NB);
+    const float t = q < 2.0f ? q - 1.0f : 3.0f - q;
+    return make_float2(q < 2.0f ? 1.0f - fabsf(t) : fabsf(t) - 1.0f, t);
 }
 
 template <int NB = kFanBins>

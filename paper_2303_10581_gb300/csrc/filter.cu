@@ -52,112 +52,66 @@ __device__ __forceinline__ bool load_octagon(OctSmem &so, void *ws, const Layout
     return !so.abort;
 }
 
-// Keep bits of this thread's 16 points: the quick-discard rectangle first
-// (it holds nearly every point of a normal cloud, and a warp whose points
-// are all in it is done), then the edges' affine forms, eight points at a
-// time, then the exact test of the few undecided ones (all_valid: bits of
-// the points that exist).  load(q) reads point q again: the exact test is a
-// call, and points kept in registers across it would be spilled.
-template <bool BOX, class Load>
-__device__ __forceinline__ uint32_t test_points(const OctSmem &so, const float (&px)[kFiltItems],
-                                                const float (&py)[kFiltItems], uint32_t all_valid, Load load)
+// Of eight points (live: bits of those that exist), the ones to keep; those
+// the affine forms left undecided are among them, and the result says
+// whether there may be any.  The quick-discard rectangle comes first: it
+// holds nearly every point of a normal cloud, and a warp whose points are
+// all in it is done.
+template <bool BOX>
+__device__ __forceinline__ bool test8(const OctSmem &so, const float (&px)[8], const float (&py)[8], uint32_t live,
+                                      uint32_t &keep)
 {
     const float xl = so.xl, xh = so.xh, yl = so.yl, yh = so.yh;
     uint32_t rect = 0;
 #pragma unroll
-    for (int q = 0; q < kFiltItems; ++q)
-        rect |= (((px[q] >= xl) & (px[q] <= xh) & (py[q] >= yl) & (py[q] <= yh)) ? 1u : 0u) << q;
-    uint32_t open = all_valid & ~rect;
-    if (!__any_sync(0xffffffffu, open != 0u)) return 0u;
-    if (!so.has_edges) return open;
-    uint32_t keep = 0;
+    for (int q = 0; q < 8; ++q)
+        if ((px[q] >= xl) & (px[q] <= xh) & (py[q] >= yl) & (py[q] <= yh)) rect |= 1u << q;
+    keep = live & ~rect;
+    if (!__any_sync(0xffffffffu, keep != 0u) || !so.has_edges) return false;
+    uint32_t outside = 0;
     if constexpr (BOX) {
 #pragma unroll
-        for (int q = 0; q < kFiltItems; ++q) keep |= (outside_box<true>(so, px[q], py[q]) ? 1u : 0u) << q;
-        keep &= open;
-        open &= ~keep;
+        for (int q = 0; q < 8; ++q)
+            if (outside_box<true>(so, px[q], py[q])) outside |= 1u << q;
     }
-    uint32_t in = 0, und = 0;
-#pragma unroll
-    for (int h = 0; h < kFiltItems / 8; ++h) {
-        float qx[8], qy[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            qx[q] = px[8 * h + q];
-            qy[q] = py[8 * h + q];
-        }
-        uint32_t i8, u8;
-        oct_decide<8>(so, qx, qy, i8, u8);
-        in |= i8 << (8 * h);
-        und |= u8 << (8 * h);
-    }
-    keep |= open & ~in;
-    und &= open;
+    uint32_t k8;
+    const bool near = oct_decide<8>(so, px, py, k8);
+    keep &= k8 | outside;
+    return near;
+}
+
+// Exact decisions for the kept ones (load(q) reads point q) that the affine
+// forms left undecided.
+template <bool BOX, class Load>
+__device__ __forceinline__ uint32_t settle_near(const OctSmem &so, uint32_t keep, Load load)
+{
 #pragma unroll 1
-    for (; und; und &= und - 1u) {
-        const float2 p = load(__ffs(und) - 1);
-        if (!keep_point<BOX>(so, p.x, p.y)) keep &= ~(und & (0u - und));
+    for (uint32_t m = keep; m; m &= m - 1u) {
+        const float2 p = load(__ffs(m) - 1);
+        if (oct_undecided(so, p.x, p.y) && !keep_point<BOX>(so, p.x, p.y)) keep &= ~(m & (0u - m));
     }
     return keep;
 }
 
-// Loads and tests one tile.  Thread t holds the points
-// base + (r * 256 + t) * G + h, r < kFiltItems / G, h < G (G = 2: one
-// 16-byte load per row; G = 1: one 8-byte load).  Returns the keep bits
-// (bit r * G + h); positions past n are not kept.
+// Loads and tests one tile, eight of the thread's 16 points at a time (all
+// 16 at once would spill).  Returns the keep bits; positions past n are not
+// kept.
 template <int G, bool BOX>
-__device__ __forceinline__ uint32_t load_test(const float *__restrict__ pts, int64_t n, int64_t base,
-                                              const OctSmem &so, float (&px)[kFiltItems], float (&py)[kFiltItems])
+__device__ __forceinline__ uint32_t load_test(const float *__restrict__ pts, int64_t n, int64_t base, const OctSmem &so)
 {
-    constexpr int ROWS = kFiltItems / G;
     const uint32_t tid = threadIdx.x;
-    uint32_t valid = 0xffffu;
-    if (base + kFiltTile <= n) {
-        if constexpr (G == 2) {
-            const float4 *p4 = reinterpret_cast<const float4 *>(pts) + base / 2;
-            float4 v[ROWS];
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) v[r] = __ldcs(p4 + r * kFiltThreads + tid);
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                px[2 * r] = v[r].x;
-                py[2 * r] = v[r].y;
-                px[2 * r + 1] = v[r].z;
-                py[2 * r + 1] = v[r].w;
-            }
-        } else {
-            const float2 *p2 = reinterpret_cast<const float2 *>(pts) + base;
-            float2 v[ROWS];
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) v[r] = __ldcs(p2 + r * kFiltThreads + tid);
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                px[r] = v[r].x;
-                py[r] = v[r].y;
-            }
-        }
-    } else {
-        const float2 *p2 = reinterpret_cast<const float2 *>(pts);
-        valid = 0u;
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-#pragma unroll
-            for (int h = 0; h < G; ++h) {
-                const int64_t i = base + (int64_t)(r * kFiltThreads + tid) * G + h;
-                px[r * G + h] = so.cx;
-                py[r * G + h] = so.cy;
-                if (i < n) {
-                    const float2 v = p2[i];
-                    px[r * G + h] = v.x;
-                    py[r * G + h] = v.y;
-                    valid |= 1u << (r * G + h);
-                }
-            }
-        }
+    uint32_t keep = 0;
+    bool near = false;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        float px[8], py[8];
+        uint32_t live = 0xffu, k8;
+        if (base + kFiltTile <= n) load_part<G, 8>(pts, base, tid, half, px, py);
+        else live = load_part_ragged<G, 8>(pts, n, base, tid, half, so.cx, so.cy, px, py);
+        near |= test8<BOX>(so, px, py, live, k8);
+        keep |= k8 << (8 * half);
     }
-    return test_points<BOX>(so, px, py, valid, [&](int q) {
-        return reinterpret_cast<const float2 *>(pts)[base + (int64_t)((q / G) * kFiltThreads + tid) * G + q % G];
-    });
+    return near ? settle_near<BOX>(so, keep, [&](int q) { return input_point(pts, item_point<G>(base, tid, q)); }) : keep;
 }
 
 // Kept points per (row, warp), turned into exclusive offsets in row-major
@@ -208,9 +162,9 @@ __device__ __forceinline__ uint32_t scan_rows_warp0(uint32_t (&s_off)[kFiltItems
 // Writes the kept points of one tile; excl is the tile's output offset.
 template <int G, bool KEYS>
 __device__ __forceinline__ void scatter_tile(uint32_t keep, int64_t base, uint64_t excl,
-                                             const uint32_t (&s_off)[kFiltItems / G][NW], const float (&px)[kFiltItems],
-                                             const float (&py)[kFiltItems], uint32_t *surv_idx, float2 *surv_pts,
-                                             uint32_t *out_keys, unsigned long long *out_pay)
+                                             const uint32_t (&s_off)[kFiltItems / G][NW], const float *__restrict__ pts,
+                                             uint32_t *surv_idx, float2 *surv_pts, uint32_t *out_keys,
+                                             unsigned long long *out_pay)
 {
     constexpr int ROWS = kFiltItems / G;
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
@@ -224,13 +178,15 @@ __device__ __forceinline__ void scatter_tile(uint32_t keep, int64_t base, uint64
         for (int h = 0; h < G; ++h) {
             if ((keep >> (r * G + h)) & 1u) {
                 const int64_t pos = (int64_t)excl + pre;
-                const uint32_t idx = (uint32_t)(base + (int64_t)(r * kFiltThreads + tid) * G + h);
+                const int64_t i = item_point<G>(base, tid, r * G + h);
+                const uint32_t idx = (uint32_t)i;
+                const float2 p = input_point(pts, i);
                 if constexpr (KEYS) {
-                    out_keys[pos] = ord_key(px[r * G + h]);
-                    out_pay[pos] = ((unsigned long long)ord_key(py[r * G + h]) << 32) | idx;
+                    out_keys[pos] = ord_key(p.x);
+                    out_pay[pos] = ((unsigned long long)ord_key(p.y) << 32) | idx;
                 } else {
                     surv_idx[pos] = idx;
-                    if (surv_pts) surv_pts[pos] = make_float2(px[r * G + h], py[r * G + h]);
+                    if (surv_pts) surv_pts[pos] = p;
                 }
                 ++pre;
             }
@@ -384,8 +340,7 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
         const int64_t tile = s_tile;
         if (tile >= ntiles) break;
         const int64_t base = tile * kFiltTile;
-        float px[kFiltItems], py[kFiltItems];
-        const uint32_t keep = load_test<G, BOX>(pts, n, base, so, px, py);
+        const uint32_t keep = load_test<G, BOX>(pts, n, base, so);
         row_counts<G>(keep, s_off);
         __syncthreads();
         if (warp == 0) {
@@ -406,7 +361,7 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
         }
         __syncthreads();
         if (s_total != 0)
-            scatter_tile<G, KEYS>(keep, base, s_excl, s_off, px, py, surv_idx, surv_pts, at<uint32_t>(ws, L.keys[0]),
+            scatter_tile<G, KEYS>(keep, base, s_excl, s_off, pts, surv_idx, surv_pts, at<uint32_t>(ws, L.keys[0]),
                                   at<unsigned long long>(ws, L.pay[0]));
         __syncthreads();
     }
@@ -612,8 +567,7 @@ __global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const flo
                 if (((reinterpret_cast<uintptr_t>(pts + 2 * nb)) & 15u) == 0)
                     bulk_prefetch_l2(pts + 2 * nb, (nn * 8u) & ~15u);
             }
-            float px[kFiltItems], py[kFiltItems];
-            const uint32_t keep = load_test<G, BOX>(pts, n, tile * kFiltTile, so, px, py);
+            const uint32_t keep = load_test<G, BOX>(pts, n, tile * kFiltTile, so);
             bits[tile * kFiltThreads + threadIdx.x] = (uint16_t)keep;
             uint32_t c = __popc(keep);
 #pragma unroll
@@ -755,21 +709,12 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
 // many sets (ch_hull_batched): the two passes over set-aligned 4096-point
 // tiles, with 8-byte loads (sets start anywhere); indices are set-local
 // ---------------------------------------------------------------------------
-// Thread t tests points lo + r * 256 + t of the set (r < 16), below hi.
+// Thread t tests points lo + r * 256 + t of the set p2 (r < 16), below hi.
 __device__ __forceinline__ uint32_t bx_load_test(const float2 *__restrict__ p2, int64_t lo, int64_t hi,
                                                  const OctSmem &so)
 {
-    float px[kFiltItems], py[kFiltItems];
-    uint32_t valid = 0;
-#pragma unroll
-    for (int r = 0; r < kFiltItems; ++r) {
-        const int64_t i = lo + r * kFiltThreads + threadIdx.x;
-        const float2 v = i < hi ? __ldcs(p2 + i) : make_float2(so.cx, so.cy);
-        px[r] = v.x;
-        py[r] = v.y;
-        valid |= (i < hi ? 1u : 0u) << r;
-    }
-    return test_points<false>(so, px, py, valid, [&](int q) { return p2[lo + q * kFiltThreads + threadIdx.x]; });
+    // (the tile in 8-byte loads is load_test's with one point per row)
+    return load_test<1, false>(reinterpret_cast<const float *>(p2), hi, lo, so);
 }
 
 // Copies set b's polygon to shared memory when the block moves to a new set.

@@ -7,39 +7,38 @@
 // have a small fraction of the points as vertices.  The hull step repeats
 // the throw-away idea of Sec. 3.1 on a much finer scale.  Let c be the
 // centre of the bounding box.  The plane around c is cut into kFanBins
-// angular bins (a pseudo-angle, fan.cuh); the vertex of a bin is the input
+// angular bins (a pseudo-angle, fan.cuh).  The vertex of a bin is the input
 // point farthest from c among a sample (the octagon survivors of about
-// kFanBinTiles evenly spaced 4096-point tiles of the input), and a bin the
-// sample missed repeats the vertex before it.
+// kFanBinTiles evenly spaced 4096-point tiles of the input), or, where that
+// lies well inside the chord of samples to either side of the bin, a point on
+// that chord, rounded a little inwards; a bin with neither repeats the vertex
+// before it.  Every vertex is a point of the hull.
 //
 // The test of a point p in bin b, with P, Q, N the vertices of the bins
-// b - 1, b, b + 1: p is dropped when it is strictly left of P -> Q (unless P
-// == Q: bin b has no sample) and strictly left of Q -> N, both signs proven
-// by the binary32 bound of orient_f32.  Then p lies strictly inside the
-// hull:
+// b - 1, b, b + 1: if p is proven strictly after Q (left of c -> Q) and
+// strictly left of Q -> N, or strictly before Q and strictly left of P -> Q,
+// it is dropped.  Signs are proven in binary32 (proven_sign).  Then p lies
+// strictly inside the hull:
 //  - the pseudo-angle grows with the angle, and its binary32 value is off by
 //    less than 0.0049 bins (0.0386 with the second level's eight times as
 //    many): in units of eps = 2^-24, t = dy / (|dx| + |dy|) gets 7 |t| (two
-//    differences, the sum, at most 2 ulp for the quotient), 2 - t or 4 + t
-//    half an ulp of at most 4, i.e. 2, and the product with NB / 4 half an
-//    ulp of at most NB.  A vertex is taken only where its value is at least
-//    a margin (1/32; 1/8) away from both ends of its bin, so as directions P
-//    comes strictly before p and N strictly after it, and Q, too, is before
-//    p where bin b has no sample;
+//    differences, the sum, at most 2 ulp for the quotient); the scaling is
+//    one FMA, which rounds by at most half an ulp of NB, or down to the bin.  A vertex is taken only where its value is at least a margin (1/32;
+//    1/8) away from both ends of its bin, so as directions P comes strictly
+//    before p and N strictly after it (or N == Q, whose sign is never proven);
 //  - consecutive vertices v, w were proven strictly counter-clockwise around
-//    c (v != w), less than half a turn apart, so p is in the wedge of (P, Q)
-//    or of (Q, N), where strictly left of the edge and inside the wedge is
-//    the triangle (c, P, Q) or (c, Q, N).  The triangles wind around c once,
-//    so c and the triangles' interiors (and the rays between them) are in
-//    the interior of a polygon of input points;
+//    c (v != w), less than half a turn apart, so p is in the wedge of (Q, N)
+//    or of (P, Q), where strictly left of the edge is the triangle (c, Q, N)
+//    or (c, P, Q).  The triangles wind around c once, so c and the
+//    triangles' interiors are in the interior of a polygon of hull points;
 //  - the quotient needs |dx| + |dy| within [2^-126, 2^126]: the set's box is
 //    checked for the upper end, and a point closer to c than 2^-126 is
 //    inside the disk around c that is proven inside the fan (the fan is off
 //    unless its radius exceeds 2^-60).
-// Nothing else is exact: a vertex only has to be an input point, a sign that
-// is not proven keeps the point, and what is kept only costs the sort time.
-// (Sets so small or large that the products of the signs under- or overflow,
-// below 10^-15 or above 10^18, keep all their points.)
+// Nothing else is exact: a sign that is not proven keeps the point, and what
+// is kept only costs the sort time.  (Sets so small that the products of the
+// signs underflow, below 10^-15, or with a box above 2^62 keep all their
+// points.)
 //
 // The disk around c proven inside the fan (a lower bound on the distance
 // from c to every fan edge) lets most points of a displaced circle pass
@@ -48,8 +47,9 @@
 //  fan_bins_kernel    per bin, the farthest sampled octagon survivor
 //                     (atomicMax of (far_key << 32 | ~index) into global
 //                     slots), and how many of the sample survived
-//  fan_build_kernel   whether there is a fan; the vertex of every bin; the
-//                     proofs that need consecutive vertices; the disk
+//  fan_vertex_kernel  whether there is a fan; the bins' vertices
+//  fan_build_kernel   empty bins filled; the proofs that need consecutive
+//                     vertices; the disk
 //  hull_filter_kernel both tests of every point; the survivors' sort keys and
 //                     payloads, in no particular order (the chain breaks
 //                     ties by the index in the payload)
@@ -63,43 +63,68 @@
 namespace ch {
 namespace {
 
-constexpr int CT = 1024;                 // threads per block of the filter pass: four
+constexpr int CT = 768;                  // threads per block of the filter pass: groups
 constexpr int CG = CT / kFiltThreads;    // groups of kFiltThreads, each with its own tiles
 constexpr uint32_t kKgonMinS = 1u << 16; // fewer octagon survivors: not worth a pass
-constexpr int kFanSmem = (kFanBins + 2) * 8;   // vertices, the last one again before the first and the first after the last
+constexpr int kFanTable = (kFanBins + 4) * 8;  // vertices, the last again before them and the first two after them (and padding)
+constexpr int kQueue = 96;                     // points a warp of the filter pass queues
+constexpr int kQueueSmem = CT / 32 * kQueue * 4;
 constexpr float kFanMargin = 1.0f / 32.0f;     // of a vertex's pseudo-angle from its bin's ends
 constexpr float kFan2Margin = 1.0f / 8.0f;     // second level
 static_assert(kFiltItems == 16 && CT % kFiltThreads == 0, "16 items per filter thread");
-static_assert(kFanSmem <= 227 * 1024 - 2048, "the table fits a block's shared memory");
+static_assert(kFanTable + kQueueSmem <= 227 * 1024 - 1024, "table and queues fit a block's shared memory");
 
-__device__ __forceinline__ float2 input_point(const float *pts, int64_t i)
+// det = (a - c) x (b - c) from the rounded differences, and a bound: a det
+// beyond it in magnitude has the exact sign.  Shewchuk's orient2d error
+// (orient_f32) is below 2^-22 (|l| + |r|) with l, r the products; |r| <= |l| +
+// |det|, so |det| > 2^-20 |l| implies |det| > 2^-22 (|l| + |r|) (2^-140 for
+// products that underflow; the fan's box rules out overflow).
+__device__ __forceinline__ float det_bound(float2 ac, float2 bc, float &bound)
 {
-    return __ldg(reinterpret_cast<const float2 *>(pts) + i);
+    const float l = __fmul_rn(ac.x, bc.y), r = __fmul_rn(ac.y, bc.x);
+    bound = __fmaf_ru(fabsf(l), 0x1p-20f, 0x1p-140f);
+    return __fsub_rn(l, r);
 }
 
-// Whether (ax, ay) x (bx, by) is proven positive (orient_f32's bound, on the
-// rounded differences a - c and b - c).
-__device__ __forceinline__ bool left_of(float acx, float acy, float bcx, float bcy)
-{
-    const float detleft = __fmul_rn(acx, bcy);
-    const float detright = __fmul_rn(acy, bcx);
-    const float det = __fsub_rn(detleft, detright);
-    const float detsum = __fadd_rn(fabsf(detleft), fabsf(detright));
-    // (an overflowed product makes the bound infinite or NaN: not proven)
-    return det > __fmaf_ru(detsum, 2.384185791015625e-07f /* 2^-22 */, 7.174648137343064e-43f /* 2^-140 */);
-}
+// The vertices in shared memory, at their bins' biased indices.
+struct SharedFan {
+    uint32_t base;
+    __device__ __forceinline__ explicit SharedFan(const float2 *V)
+        : base((uint32_t)__cvta_generic_to_shared(V) - kBinBias * 8u)
+    {
+    }
+    __device__ __forceinline__ uint32_t at(uint32_t biased) const { return base + biased * 8u; }
+    __device__ __forceinline__ float2 get(uint32_t a, int d) const   // the vertex d entries on
+    {
+        float2 v;
+        asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a + (uint32_t)(8 * d)));
+        return v;
+    }
+};
 
-// Strictly inside the fan, proven (see the top of the file).  V[-1] and
-// V[NB] are the last and the first vertex again; (dx, dy) = fl(p - c).
-template <int NB>
-__device__ __forceinline__ bool fan_inside(const float2 *V, float dx, float dy, float px, float py)
+// The same in global memory.
+struct GlobalFan {
+    const float2 *V;
+    __device__ __forceinline__ const float2 *at(uint32_t biased) const { return V + (biased - kBinBias); }
+    __device__ __forceinline__ float2 get(const float2 *a, int d) const { return __ldg(a + d); }
+};
+
+// Strictly inside the fan, proven (see the top of the file).  F: the
+// vertices; before the first comes the last, after the last the first two
+// again; d = fl(p - c).  Two vertices are read: in shared memory the reads of
+// 32 random bins conflict (six wavefronts each), and a third would bound the
+// pass.
+template <int NB, class Fan>
+__device__ __forceinline__ bool fan_inside(const Fan &F, float2 c, float2 d, float2 p)
 {
-    const float2 *v = V + fan_bin<NB>(dx, dy);
-    const float2 P = v[-1], Q = v[0], N = v[1];
-    const float ux = __fsub_rn(px, Q.x), uy = __fsub_rn(py, Q.y);
-    const bool qn = left_of(__fsub_rn(N.x, Q.x), __fsub_rn(N.y, Q.y), ux, uy);
-    const bool pq = left_of(ux, uy, __fsub_rn(P.x, Q.x), __fsub_rn(P.y, Q.y));
-    return qn && (pq || (P.x == Q.x && P.y == Q.y));
+    const auto a = F.at(fan_bin_biased<NB>(d.x, d.y));   // (a NaN: any vertex; such a point is next to c)
+    const float2 Q = F.get(a, 0);
+    float e1, e2;
+    const float side = det_bound(sub2(Q, c), d, e1);
+    const float2 W = F.get(a, side > 0.0f ? 1 : -1);
+    const float det = det_bound(sub2(W, Q), sub2(p, Q), e2);
+    const float turned = __uint_as_float(__float_as_uint(det) ^ (__float_as_uint(side) & 0x80000000u));
+    return (fabsf(side) > e1) & (turned > e2);   // (no branches: the points of a thread interleave)
 }
 
 // The bin a point may be the vertex of, -1 when its pseudo-angle is within
@@ -108,9 +133,9 @@ template <int NB>
 __device__ __forceinline__ int vertex_bin(float dx, float dy, float margin)
 {
     const float phi = fan_phi<NB>(dx, dy);
-    const int b = min(__float2int_rz(phi), NB - 1);
+    const int b = __float2int_rd(phi);
     const float f = phi - (float)b;
-    return f >= margin && f <= 1.0f - margin ? b : -1;
+    return f >= margin && f <= 1.0f - margin && b >= 0 && b < NB ? b : -1;
 }
 
 // Whether this call has a fan whose proofs hold (after fan_build_kernel).
@@ -120,69 +145,11 @@ __device__ __forceinline__ bool fan_ready(const KgonCtrl *kc, const Kgon *g)
     return g->ok && !kc->bad && kc->edges >= 3u && fan_rho2(kc) > 0x1p-120f;
 }
 
-// Point of item q (of this thread's 16) of a 4096-point tile; the layout is
-// the count pass's: item q = r * G + h is point base + (r * kFiltThreads + t) * G + h.
-template <int G>
-__device__ __forceinline__ int64_t item_point(int64_t base, uint32_t t, int q)
-{
-    return base + (int64_t)((q / G) * kFiltThreads + t) * G + q % G;
-}
-
-// Items 8 half .. 8 half + 7 of a thread's 16 in the tile at `base`, all of
-// them below n (G = 2: 16-byte loads).
-template <int G>
-__device__ __forceinline__ void load8(const float *__restrict__ pts, int64_t base, uint32_t t, int half, float (&px)[8],
-                                      float (&py)[8])
-{
-    if constexpr (G == 2) {
-        const float4 *p4 = reinterpret_cast<const float4 *>(pts) + base / 2 + half * 4 * kFiltThreads + t;
-        float4 v[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = __ldg(p4 + r * kFiltThreads);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            px[2 * r] = v[r].x;
-            py[2 * r] = v[r].y;
-            px[2 * r + 1] = v[r].z;
-            py[2 * r + 1] = v[r].w;
-        }
-    } else {
-        const float2 *p2 = reinterpret_cast<const float2 *>(pts) + base + half * 8 * kFiltThreads + t;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const float2 v = __ldg(p2 + r * kFiltThreads);
-            px[r] = v.x;
-            py[r] = v.y;
-        }
-    }
-}
-
-// The same where the tile ends before them: the centre stands in for the
-// missing points; returns the bits of those that exist.
-template <int G>
-__device__ __forceinline__ uint32_t load8_ragged(const float *__restrict__ pts, int64_t n, int64_t base, uint32_t t,
-                                                 int half, float cx, float cy, float (&px)[8], float (&py)[8])
-{
-    uint32_t live = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int64_t i = item_point<G>(base, t, 8 * half + k);
-        const float2 v = i < n ? input_point(pts, i) : make_float2(cx, cy);
-        px[k] = v.x;
-        py[k] = v.y;
-        live |= (i < n ? 1u : 0u) << k;
-    }
-    return live;
-}
-
 // ---------------------------------------------------------------------------
 // first level: bins and vertices
 // ---------------------------------------------------------------------------
 // Every stride-th tile, a block each: the octagon survivors' bins.  Bound by
-// the slots' L2 reads and the key's arithmetic (about 90 instructions per
-// sampled survivor); inside the count pass, where an eighth of the tiles
-// held their block up while the others waited for it, the same work took
-// 90 to 180 us of 10^8 points on a circle and a displaced circle.
+// the latency of the points' and then the slots' reads.
 template <int G>
 __global__ void __launch_bounds__(kFiltThreads) fan_bins_kernel(const float *__restrict__ pts, int64_t n, void *ws,
                                                                 Layout L, int32_t stride, int use_bits,
@@ -206,15 +173,15 @@ __global__ void __launch_bounds__(kFiltThreads) fan_bins_kernel(const float *__r
         for (int half = 0; half < 2; ++half) {
             float px[8], py[8];
             uint32_t live = 0xffu;
-            if (base + kFiltTile <= n) load8<G>(pts, base, t, half, px, py);
-            else live = load8_ragged<G>(pts, n, base, t, half, cx, cy, px, py);
+            if (base + kFiltTile <= n) load_part<G, 8>(pts, base, t, half, px, py);
+            else live = load_part_ragged<G, 8>(pts, n, base, t, half, cx, cy, px, py);
             seen += __popc(live);
             if (bits_mode) {
                 live &= (uint32_t)bits[tile * kFiltThreads + t] >> (8 * half);
             } else {
-                uint32_t in, und;
-                oct_decide<8>(so, px, py, in, und);
-                live &= ~in;   // (undecided points are input points all the same)
+                uint32_t out;
+                oct_decide<8>(so, px, py, out);   // (undecided points are input points all the same)
+                live &= out;
             }
             kept += __popc(live);
             if (!__any_sync(0xffffffffu, live != 0u)) continue;
@@ -245,10 +212,9 @@ __global__ void __launch_bounds__(kFiltThreads) fan_bins_kernel(const float *__r
     }
 }
 
-// One thread per bin (kFanBins / BT blocks).  The vertex of bin b is the
-// sampled point of the last non-empty bin at or before b, cyclically: a
-// max-scan of "non-empty bin index" inside the block, and for the bins
-// before the block's first non-empty one, the last non-empty bin of the
+// One thread per bin (kFanBins / BT blocks).  An empty bin repeats the last
+// vertex before it, cyclically: a max-scan of the bins that have one inside
+// the block, and for the bins before the block's first, the last one of the
 // nearest earlier range of BT bins that has one (searched range by range).
 constexpr int BT = 1024;
 static_assert(kFanBins % BT == 0, "bins split evenly over the blocks");
@@ -265,13 +231,15 @@ __device__ __forceinline__ int block_max(int v, int *s_w)
     return m;
 }
 
-// The bin whose point is the vertex of bin blockIdx.x * BT + threadIdx.x (-1:
-// every bin is empty; block-uniform then).  Every thread of the block calls.
-__device__ __forceinline__ int vertex_source(const unsigned long long *slot, int *s_w, int *s_scan)
+// The last bin with a vertex of its own at or before bin blockIdx.x * BT +
+// threadIdx.x, cyclically (-1: no bin has one; block-uniform then).  Every
+// thread of the block calls; has(j): bin j has one.
+template <class Has>
+__device__ __forceinline__ int vertex_source(Has has, int *s_w, int *s_scan)
 {
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const int b = (int)(blockIdx.x * BT + tid);
-    int incl = slot[b] != 0ull ? b : -1;
+    int incl = has(b) ? b : -1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int u = __shfl_up_sync(0xffffffffu, incl, o);
@@ -285,7 +253,7 @@ __device__ __forceinline__ int vertex_source(const unsigned long long *slot, int
     for (uint32_t k = 1; k <= gridDim.x && prev < 0; ++k) {   // prev is block-uniform
         const uint32_t rb = (blockIdx.x + gridDim.x - k) % gridDim.x;
         const int j = (int)(rb * BT + tid);
-        prev = block_max(slot[j] != 0ull ? j : -1, s_w);
+        prev = block_max(has(j) ? j : -1, s_w);
     }
     return prev < 0 ? -1 : (incl >= 0 ? incl : prev);
 }
@@ -317,7 +285,7 @@ __device__ __forceinline__ T edge_bound(float cx, float cy, float2 v, float2 w, 
     return lo * lo / (len2 * ((T)1 + (T)16 * U)) * ((T)1 - (T)16 * U);
 }
 
-// In binary32 first (28672 binary64 quotients on 28 SMs would take 15 us),
+// In binary32 first (27648 binary64 quotients on 28 SMs would take 15 us),
 // in binary64 where that proves nothing: a value in binary32, rounded down.
 __device__ __forceinline__ float disk_bound(float cx, float cy, float2 v, float2 w)
 {
@@ -327,7 +295,156 @@ __device__ __forceinline__ float disk_bound(float cx, float cy, float2 v, float2
     return d < 0.0 ? -1.0f : (d <= 3.0e38 ? __double2float_rd(d) : 3.0e38f);
 }
 
-__global__ void __launch_bounds__(BT) fan_build_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L)
+__device__ __forceinline__ bool fan_live(const KgonCtrl *kc, const Octagon *oct, int64_t n)
+{
+    // (an aborted call, the speculative sweep's candidates, a polygon without
+    // edges: the bins pass left no sample)
+    const uint32_t sample = kc->sample;
+    const float box = __fadd_rn(__fsub_rn(oct->bxh, oct->bxl), __fsub_rn(oct->byh, oct->byl));
+    return sample != 0u && (double)kc->inside / sample * (double)n >= (double)kKgonMinS && box < 0x1p62f;
+}
+
+// The vertices of 64 consecutive bins, a warp: the samples of the bins and of
+// the nearest non-empty bins to either side, then strict-turn elimination
+// passes leave their (nearly) convex chain.  A bin whose sample was
+// eliminated and lies more than 2^-18 inside the chord over it, or that has
+// none, gets the point of the chord in the direction of its middle, moved
+// inwards by 2^-20 and rounded; it is used only when it is proven inside the
+// triangle of c and the chord's ends (exact signs, its bin's margins), hence
+// in the hull.  On a displaced circle with few samples per bin the farthest
+// sample of a bin lies deep: of 10^8 points 338428 reached the sort with the
+// samples alone, and the disk around c missed a fourteenth of the points.
+constexpr int VB = 64;                   // bins per warp
+constexpr int VT = 256;                  // threads per block
+constexpr int kVertexPasses = 16;
+static_assert(kFanBins % (VB * VT / 32) == 0, "bins split evenly over the warps");
+
+struct VertexSmem {
+    float2 p[2][VB + 2];
+    int bin[2][VB + 2];                  // unwrapped: below 0 / beyond NB across the ends
+};
+
+// The nearest non-empty bin before `from` (dir = -1) or from `from` on (dir =
+// 1), unwrapped; from -+ NB when there is none.
+template <int NB>
+__device__ __forceinline__ int nearest_bin(const unsigned long long *slot, int from, int dir)
+{
+    const int lane = (int)lane_id();
+    for (int k = 0; k < NB; k += 32) {
+        const int j = dir > 0 ? from + k + lane : from - 1 - k - lane;
+        const int w = j < 0 ? j + NB : (j >= NB ? j - NB : j);
+        const uint32_t m = __ballot_sync(0xffffffffu, __ldcg(slot + w) != 0ull);
+        if (m) return dir > 0 ? from + k + __ffs(m) - 1 : from - k - __ffs(m);
+    }
+    return dir > 0 ? from + NB : from - NB;
+}
+
+// Bins [b0, b0 + VB) of a fan with NB bins; point(i) reads input point i
+// (clamped to the input); V receives the vertices, x = NaN for none.  False
+// when there are no samples outside the range (no fan).
+template <int NB, class Point>
+__device__ __forceinline__ bool make_vertices(VertexSmem &sm, const unsigned long long *slot, int b0, float2 c, Point point,
+                                              float2 *V)
+{
+    const int lane = (int)lane_id();
+    const uint32_t lt = (1u << lane) - 1u;
+    const int pb = nearest_bin<NB>(slot, b0, -1), nb = nearest_bin<NB>(slot, b0 + VB, 1);
+    if (pb <= b0 + VB - 1 - NB || nb >= b0 + NB) return false;   // (only this range has samples)
+    bool has[VB / 32];
+    float2 own[VB / 32];
+    int len = 1;
+#pragma unroll
+    for (int h = 0; h < VB / 32; ++h) {
+        const unsigned long long v = __ldcg(slot + b0 + 32 * h + lane);
+        has[h] = v != 0ull;
+        own[h] = has[h] ? point(~(uint32_t)v) : c;
+        const uint32_t m = __ballot_sync(0xffffffffu, has[h]);
+        if (has[h]) {
+            sm.p[0][len + __popc(m & lt)] = own[h];
+            sm.bin[0][len + __popc(m & lt)] = b0 + 32 * h + lane;
+        }
+        len += __popc(m);
+    }
+    if (lane < 2) {
+        const int j = lane ? nb : pb;
+        const int w = j < 0 ? j + NB : (j >= NB ? j - NB : j);
+        const int at = lane ? len : 0;
+        sm.p[0][at] = point(~(uint32_t)__ldcg(slot + w));
+        sm.bin[0][at] = j;
+    }
+    ++len;
+    __syncwarp();
+    int cur = 0;
+    for (int pass = 0; pass < kVertexPasses; ++pass) {
+        int kept = 0;
+        for (int i0 = 0; i0 < len; i0 += 32) {
+            const int i = i0 + lane;
+            bool keep = i < len;
+            if (keep && i > 0 && i < len - 1) {
+                const float2 a = sm.p[cur][i - 1], q = sm.p[cur][i], d = sm.p[cur][i + 1];
+                keep = (a.x - q.x) * (d.y - q.y) - (a.y - q.y) * (d.x - q.x) < 0.0f;   // right of the chord
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                sm.p[cur ^ 1][kept + __popc(m & lt)] = sm.p[cur][i];
+                sm.bin[cur ^ 1][kept + __popc(m & lt)] = sm.bin[cur][i];
+            }
+            kept += __popc(m);
+        }
+        __syncwarp();
+        cur ^= 1;
+        const bool done = kept == len;
+        len = kept;
+        if (done) break;
+    }
+#pragma unroll
+    for (int h = 0; h < VB / 32; ++h) {
+        const int b = b0 + 32 * h + lane;
+        int lo = 0, hi = len - 1;   // last entry at or before bin b (entry 0 is before the range, the last after it)
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (sm.bin[cur][mid] <= b) lo = mid;
+            else hi = mid;
+        }
+        const float2 Lp = sm.p[cur][lo], Rp = sm.p[cur][lo + 1];
+        float2 v = own[h];
+        bool ok = has[h];
+        if (sm.bin[cur][lo] != b) {
+            const float lx = Lp.x - c.x, ly = Lp.y - c.y, ex = Rp.x - Lp.x, ey = Rp.y - Lp.y;
+            const float num = lx * ey - ly * ex;
+            const float own_den = (v.x - c.x) * ey - (v.y - c.y) * ex;
+            if (!ok || num > own_den * (1.0f + 0x1p-18f)) {   // (own_den > 0: the sample is on the chord's side of c)
+                const float2 d = fan_direction<NB>((float)b + 0.5f);
+                const float s = num / (d.x * ey - d.y * ex) * (1.0f - 0x1p-20f);
+                const float2 q = make_float2(__fmaf_rn(s, d.x, c.x), __fmaf_rn(s, d.y, c.y));
+                if (fabsf(q.x) <= 3.0e38f && fabsf(q.y) <= 3.0e38f &&
+                    vertex_bin<NB>(__fsub_rn(q.x, c.x), __fsub_rn(q.y, c.y), kFanMargin) == b &&
+                    orient(Lp.x, Lp.y, Rp.x, Rp.y, q.x, q.y) > 0 && orient(Lp.x, Lp.y, Rp.x, Rp.y, c.x, c.y) > 0) {
+                    v = q;
+                    ok = true;
+                }
+            }
+        }
+        V[b] = ok ? v : make_float2(__int_as_float(0x7fc00000), 0.0f);
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L)
+{
+    __shared__ VertexSmem sm[VT / 32];
+    const Octagon *oct = at<Octagon>(ws, L.oct);
+    KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
+    if (!fan_live(kc, oct, n)) return;
+    const int warp = (int)(threadIdx.x >> 5);
+    const int b0 = (int)(blockIdx.x * (VT / 32) + warp) * VB;
+    const bool ok = make_vertices<kFanBins>(
+        sm[warp], kc->slot, b0, make_float2(oct->cx, oct->cy),
+        [&](uint32_t i) { return input_point(pts, (int64_t)i < n ? i : 0u); }, at<Kgon>(ws, L.kgon)->raw);
+    if (!ok && lane_id() == 0) kc->bad = 1u;
+}
+
+__global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layout L)
 {
     __shared__ int s_w[BT / 32];
     __shared__ int s_scan[BT / 32];
@@ -335,31 +452,19 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(const float *__restrict__
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     Kgon *g = at<Kgon>(ws, L.kgon);
     const uint32_t tid = threadIdx.x;
-    // (an aborted call, the speculative sweep's candidates, a polygon without
-    // edges: the bins pass left no sample)
-    const uint32_t sample = kc->sample;
-    const float box = __fadd_rn(__fsub_rn(oct->bxh, oct->bxl), __fsub_rn(oct->byh, oct->byl));
-    const bool live = sample != 0u && (double)kc->inside / sample * (double)n >= (double)kKgonMinS && box < 4.0e37f;
-    if (!live) {
-        if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
-        return;
-    }
-    const float cx = oct->cx, cy = oct->cy;
+    const bool live = fan_live(kc, oct, n) && !(kc->bad & 1u);   // (bit 1 is set below)
     const int b = (int)(blockIdx.x * BT + tid);
-    const int src = vertex_source(kc->slot, s_w, s_scan);
+    int src = -1;
+    if (live) src = vertex_source([&](int j) { return g->raw[j].x == g->raw[j].x; }, s_w, s_scan);   // block-uniform
     if (src < 0) {
         if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
         return;
     }
-    const auto point_of = [&](unsigned long long packed) {
-        const uint32_t i = ~(uint32_t)packed;
-        return input_point(pts, (int64_t)i < n ? i : 0u);
-    };
-    const unsigned long long nextp = kc->slot[next_bin(b)];
-    const float2 v = point_of(kc->slot[src]);
+    const float cx = oct->cx, cy = oct->cy;
+    const float2 v = g->raw[src], next = g->raw[next_bin(b)];
     g->v[b] = v;
     // the next bin's vertex: its own point, or this one's again
-    const float2 w = nextp != 0ull ? point_of(nextp) : v;
+    const float2 w = next.x == next.x ? next : v;
     float r = __int_as_float(0x7f800000);
     const bool edge = v.x != w.x || v.y != w.y;
     bool bad = false;
@@ -374,7 +479,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(const float *__restrict__
     if (lane_id() == 0) {
         atomicMax(&kc->rho_inv, inv);
         if (edges) atomicAdd(&kc->edges, edges);
-        if (bad) atomicOr(&kc->bad, 1u);
+        if (bad) atomicOr(&kc->bad, 2u);
     }
     if (blockIdx.x == 0 && tid == 0) {
         g->cx = cx;
@@ -389,8 +494,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(const float *__restrict__
 // The warp's kept points (mask: this lane's items; get(q): the point and its
 // index) to the end of the survivor list.
 template <class Get>
-__device__ __forceinline__ void append_survivors(uint32_t mask, uint32_t *count, uint32_t *keys, unsigned long long *pay,
-                                                 Get get)
+__device__ __forceinline__ void append_survivors(uint32_t mask, void *ws, const Layout &L, Get get)
 {
     const uint32_t lane = lane_id(), c = __popc(mask);
     if (!__any_sync(0xffffffffu, c != 0u)) return;
@@ -401,21 +505,20 @@ __device__ __forceinline__ void append_survivors(uint32_t mask, uint32_t *count,
         if (lane >= (uint32_t)o) incl += u;
     }
     uint32_t pos = 0;
-    if (lane == 31) pos = atomicAdd(count, incl);
+    if (lane == 31) pos = atomicAdd(&at<Ctrl>(ws, L.ctrl)->surv_count, incl);
     pos = __shfl_sync(0xffffffffu, pos, 31) + incl - c;
 #pragma unroll 1
     for (; mask; mask &= mask - 1u, ++pos) {
         uint32_t i;
         const float2 p = get(__ffs(mask) - 1, i);
-        keys[pos] = ord_key(p.x);
-        pay[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
+        at<uint32_t>(ws, L.keys[0])[pos] = ord_key(p.x);
+        at<unsigned long long>(ws, L.pay[0])[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
     }
 }
 
 // The speculative sweep's candidates (extremes.cu; every other point is
 // proven inside the octagon): a warp per slice, the exact test.
-__device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *ws, const Layout &L, uint32_t *count,
-                                                      uint32_t *keys, unsigned long long *pay)
+__device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *ws, const Layout &L)
 {
     const SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const uint32_t *cidx = at<uint32_t>(ws, L.keys[1]);
@@ -434,7 +537,7 @@ __device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *w
                 keep = keep_point<false>(so, p.x, p.y);
             }
             mine += keep ? 1u : 0u;
-            append_survivors(keep ? 1u : 0u, count, keys, pay, [&](int, uint32_t &i) {
+            append_survivors(keep ? 1u : 0u, ws, L, [&](int, uint32_t &i) {
                 i = cidx[s0 + e0 + lane];
                 return p;
             });
@@ -443,22 +546,75 @@ __device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *w
     return mine;
 }
 
+// A warp's queue of point indices (shared memory): survivors on their way to
+// the list, or (candidates) points outside the disk that still need the fan
+// test.  Full batches of 32 leave it, read their points again (L2) and do the
+// fan test of scattered points and the list's atomics and writes as a whole
+// warp.
+struct PointQueue {
+    uint32_t *i;
+    uint32_t n;   // warp-uniform
+};
+
+struct FanView {
+    bool test;   // candidates
+    SharedFan F;
+    float2 c;
+};
+
+// An index with this bit (n < 2^30) is a point the octagon's forms may have
+// left undecided: the exact test first, and then the fan test.
+constexpr uint32_t kUnsettled = 0x80000000u;
+
+// Whether point p (i: its index and kUnsettled) survives; octs counts the
+// octagon survivors among the unsettled ones.
+__device__ __forceinline__ bool settle(const OctSmem &so, const FanView &f, bool fan, uint32_t i, float2 p, uint32_t &octs)
+{
+    bool keep = true;
+    if (i & kUnsettled) {
+        keep = keep_point<false>(so, p.x, p.y);
+        octs += keep ? 1u : 0u;
+    }
+    if (f.test || ((i & kUnsettled) && fan)) keep = keep && !fan_inside<kFanBins>(f.F, f.c, sub2(p, f.c), p);
+    return keep;
+}
+
+// The last (up to) 32 points of the queue: the survivors to the list.
+__device__ __forceinline__ void queue_drain(PointQueue &q, const OctSmem &so, const FanView &f, bool fan,
+                                            const float *__restrict__ pts, void *ws, const Layout &L, uint32_t &octs)
+{
+    const uint32_t lane = lane_id(), m = min(q.n, 32u);
+    q.n -= m;
+    bool keep = lane < m;
+    const uint32_t e = q.i[q.n + (keep ? lane : 0u)], i = e & ~kUnsettled;
+    const float2 p = input_point(pts, i);
+    __syncwarp();   // the slots may be filled again
+    if (keep) keep = settle(so, f, fan, e, p, octs);
+    const uint32_t b = __ballot_sync(0xffffffffu, keep);
+    if (!b) return;
+    uint32_t pos = 0;
+    if (lane == 0) pos = atomicAdd(&at<Ctrl>(ws, L.ctrl)->surv_count, (uint32_t)__popc(b));
+    pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(b & ((1u << lane) - 1u));
+    if (keep) {
+        at<uint32_t>(ws, L.keys[0])[pos] = ord_key(p.x);
+        at<unsigned long long>(ws, L.pay[0])[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
+    }
+}
+
 // The tiles go in contiguous ranges to groups of kFiltThreads threads; a
-// thread takes its 16 points of a tile eight at a time: the octagon's affine
-// forms, then (fan) the disk and the fan test, branch-free.  The few points
-// the octagon's forms leave undecided and those that are written are read
-// again (L2), so that eight points are all the registers hold.  bits_mode: a
-// second polygon has refined the count pass's keep bits, which then stand
-// for the octagon test.
-// One block of 1024 threads per SM: the 28672 vertices take its shared
-// memory.  Bound by issue on circle-like sets (two differences, 23
-// instructions for the octagon, about 35 for the fan and two three-vertex
-// reads of shared memory per point) and by HBM on others.  Testing and
-// writing in one pass replaces a count pass, a fan pass and a scatter that
-// each read the points again: 274 + 455 + 214 us on 10^8 points of the unit
-// circle.
+// thread tests its 16 points of a tile eight at a time: the octagon's affine
+// forms, then (fan) the fan test, branch-free -- or, in a warp where the disk
+// holds most points, the disk test, the others going to the queue.
+// bits_mode: a second polygon has refined the count pass's keep bits, which
+// then stand for the octagon test.
+// One block of 1024 threads per SM: the vertices and the queues take its
+// shared memory.  Bound by issue and the vertices' bank conflicts on
+// circle-like sets (about 18 instructions for the octagon, 27 for the fan and
+// two vertex reads per point) and by HBM on others.  Testing and writing in
+// one pass replaces a count pass, a fan pass and a scatter that each read the
+// points again: 274 + 455 + 214 us on 10^8 points of the unit circle.
 template <int G>
-__global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L,
+__global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restrict__ pts, uint32_t n, void *ws, Layout L,
                                                             int has_fan, int use_bits, const int32_t *kdev)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -467,106 +623,124 @@ __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restr
     const Octagon *oct = at<Octagon>(ws, L.oct);
     if (oct->abort) return;
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
-    Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
-    uint32_t *keys = at<uint32_t>(ws, L.keys[0]), *count = &ctrl->surv_count;
-    unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
     fill_octagon(so, oct);
     if (threadIdx.x == 0) s_oct = 0u;
     const Kgon *g = at<Kgon>(ws, L.kgon);
     const bool fan = has_fan && !oct->spec && fan_ready(kc, g);
-    const float2 *V = reinterpret_cast<const float2 *>(smem_raw) + 1;
+    float2 *sv = reinterpret_cast<float2 *>(smem_raw + kQueueSmem) + 1;
     if (fan) {
-        float2 *sv = reinterpret_cast<float2 *>(smem_raw) + 1;
         for (int i = threadIdx.x; i < kFanBins; i += CT) sv[i] = __ldg(g->v + i);
         if (threadIdx.x == 0) {
             sv[-1] = __ldg(g->v + kFanBins - 1);
             sv[kFanBins] = __ldg(g->v);
+            sv[kFanBins + 1] = __ldg(g->v + 1);
         }
     }
     __syncthreads();
     uint32_t octs = 0;   // octagon survivors of this thread
     if (oct->spec) {
-        octs = filter_candidates(so, ws, L, count, keys, pay);
+        octs = filter_candidates(so, ws, L);
     } else {
         const bool bits_mode = use_bits && (!kdev || *kdev != 8);
-        const uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-        const float cx = so.cx, cy = so.cy;
+        const float2 c = make_float2(so.cx, so.cy);
+        const SharedFan F(sv);
+        const uint32_t warp = threadIdx.x >> 5, lt = (1u << lane_id()) - 1u;
+        PointQueue q{reinterpret_cast<uint32_t *>(smem_raw) + warp * kQueue, 0u};
         // r2 < rho2t proves |p - c|^2 < rho^2 (2^-20 covers the rounding of r2)
         const float rho2t = fan ? __fmul_rd(fan_rho2(kc), 1.0f - 0x1p-20f) : 0.0f;
-        bool use_disk = fan;
-        const int64_t ntiles = ceil_div(n, kFiltTile);
-        const uint32_t grp = threadIdx.x / kFiltThreads, t = threadIdx.x % kFiltThreads;
-        const int64_t groups = (int64_t)gridDim.x * CG, gi = (int64_t)blockIdx.x * CG + grp;
-        const int64_t per = ceil_div(ntiles, groups);
-        const int64_t t1 = std::min<int64_t>(ntiles, (gi + 1) * per);
-        for (int64_t tile = gi * per; tile < t1; ++tile) {
-            const int64_t base = tile * kFiltTile;
+        bool use_disk = fan;   // (then the queue holds candidates)
+        const bool edges = !bits_mode && so.has_edges;
+        const uint32_t ntiles = (n + kFiltTile - 1) / kFiltTile;   // (n < 2^30)
+        const uint32_t t = threadIdx.x % kFiltThreads, gi = blockIdx.x * CG + threadIdx.x / kFiltThreads;
+        const uint32_t per = (ntiles + gridDim.x * CG - 1) / (gridDim.x * CG);
+        const uint32_t t1 = min(ntiles, (gi + 1) * per);
+        for (uint32_t tile = gi * per; tile < t1; ++tile) {
+            const uint32_t base = tile * kFiltTile;
             if (t == 0 && tile + 1 < t1) {   // the next tile streams into L2 meanwhile
-                const uint32_t nn = (uint32_t)std::min<int64_t>(kFiltTile, n - base - kFiltTile);
-                if (((reinterpret_cast<uintptr_t>(pts + 2 * (base + kFiltTile))) & 15u) == 0)
-                    bulk_prefetch_l2(pts + 2 * (base + kFiltTile), (nn * 8u) & ~15u);
+                const float *next = pts + 2 * (size_t)(base + kFiltTile);
+                if ((reinterpret_cast<uintptr_t>(next) & 15u) == 0)
+                    bulk_prefetch_l2(next, (min((uint32_t)kFiltTile, n - base - kFiltTile) * 8u) & ~15u);
             }
-            uint32_t keep = 0, und = 0, drop = 0;
+            // kept: octagon survivors; drop: those of them inside the disk or
+            // the fan; near: some may be undecided, and all of this lane's are
+            // settled when they leave the queue (rare: next to the octagon)
+            uint32_t kept = 0xffffu, drop = 0;
+            bool near = false;
+            if (bits_mode) kept = at<uint16_t>(ws, L.keep_bits)[tile * kFiltThreads + t];
 #pragma unroll 1
             for (int half = 0; half < 2; ++half) {
                 float px[8], py[8];
-                uint32_t live = 0xffu;
-                if (base + kFiltTile <= n) load8<G>(pts, base, t, half, px, py);
-                else live = load8_ragged<G>(pts, n, base, t, half, cx, cy, px, py);
-                if (bits_mode) {
-                    live &= (uint32_t)bits[tile * kFiltThreads + t] >> (8 * half);
-                } else if (!so.has_edges) {
-                } else {
-                    uint32_t in8, und8;
-                    oct_decide<8>(so, px, py, in8, und8);
-                    live &= ~in8;
-                    und |= (live & und8) << (8 * half);
+                if (base + kFiltTile <= n) load_part<G, 8>(pts, base, t, half, px, py);
+                else kept &= ~(0xffu << (8 * half)) |
+                             load_part_ragged<G, 8>(pts, n, base, t, half, c.x, c.y, px, py) << (8 * half);
+                if (edges) {
+                    uint32_t out8;
+                    near |= oct_decide<8>(so, px, py, out8);
+                    kept &= ~(0xffu << (8 * half)) | out8 << (8 * half);
                 }
-                keep |= live << (8 * half);
-                if (!fan || !__any_sync(0xffffffffu, live != 0u)) continue;
+                if (!fan) continue;
                 uint32_t in = 0;
                 if (use_disk) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
-                        const float dx = __fsub_rn(px[k], cx), dy = __fsub_rn(py[k], cy);
-                        in |= (__fmaf_rn(dx, dx, __fmul_rn(dy, dy)) < rho2t ? 1u : 0u) << k;
+                        const float dx = __fsub_rn(px[k], c.x), dy = __fsub_rn(py[k], c.y);
+                        if (__fmaf_rn(dx, dx, __fmul_rn(dy, dy)) < rho2t) in |= 1u << k;
                     }
-                    in &= live;
-                    // a warp that finds under a quarter of its points in the
-                    // disk stops testing it
-                    const unsigned hits = __reduce_add_sync(0xffffffffu, (unsigned)__popc(in));
-                    const unsigned tried = __reduce_add_sync(0xffffffffu, (unsigned)__popc(live));
-                    if (4u * hits < tried) use_disk = false;
-                }
-                uint32_t out = live & ~in;   // to test against the fan
-                if (__reduce_max_sync(0xffffffffu, (unsigned)__popc(out)) <= 2u) {
-#pragma unroll 1
-                    for (; out; out &= out - 1u) {
-                        const float2 p = input_point(pts, item_point<G>(base, t, 8 * half + __ffs(out) - 1));
-                        if (fan_inside<kFanBins>(V, __fsub_rn(p.x, cx), __fsub_rn(p.y, cy), p.x, p.y))
-                            in |= out & (0u - out);
-                    }
-                } else {
-                    uint32_t f = 0;
+                } else if (__any_sync(0xffffffffu, ((kept >> (8 * half)) & 0xffu) != 0u)) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        f |= (fan_inside<kFanBins>(V, __fsub_rn(px[k], cx), __fsub_rn(py[k], cy), px[k], py[k]) ? 1u : 0u) << k;
-                    in |= f & out;
+                    for (int k = 0; k < 8; ++k) {
+                        if (k % 4 == 0) asm volatile("" ::: "memory");   // four points at a time (more would spill)
+                        const float2 p = make_float2(px[k], py[k]);
+                        if (fan_inside<kFanBins>(F, c, sub2(p, c), p)) in |= 1u << k;
+                    }
                 }
                 drop |= in << (8 * half);
             }
-#pragma unroll 1
-            for (; und; und &= und - 1u) {
-                const float2 p = input_point(pts, item_point<G>(base, t, __ffs(und) - 1));
-                if (!keep_point<false>(so, p.x, p.y)) keep &= ~(und & (0u - und));
+            uint32_t live = near ? kept : kept & ~drop;
+            if (!near) octs += __popc(kept);
+            const uint32_t total = __reduce_add_sync(0xffffffffu, __popc(live));
+            if (use_disk) {   // a warp that finds under a quarter of a tile's points in the disk stops testing it
+                const uint32_t tried = __reduce_add_sync(0xffffffffu, __popc(kept));
+                if (4u * total > 3u * tried) {
+                    while (q.n) queue_drain(q, so, FanView{true, F, c}, fan, pts, ws, L, octs);
+                    if (!near) octs -= __popc(kept);
+                    use_disk = false;
+                    --tile;   // once more, with the fan
+                    continue;
+                }
             }
-            octs += __popc(keep);
-            append_survivors(keep & ~drop, count, keys, pay, [&](int q, uint32_t &i) {
-                const int64_t j = item_point<G>(base, t, q);
-                i = (uint32_t)j;
-                return input_point(pts, j);
-            });
+            if (total == 0u) continue;
+            const FanView f{use_disk, F, c};
+            if (q.n + total <= (uint32_t)kQueue) {
+                uint32_t at = q.n;
+                q.n += total;
+                // (a ballot per round: a lane has few points)
+                while (at < q.n) {
+                    const uint32_t m = __ballot_sync(0xffffffffu, live != 0u);
+                    if (live)
+                        q.i[at + __popc(m & lt)] = (uint32_t)item_point<G>(base, t, __ffs(live) - 1) | (near ? kUnsettled : 0u);
+                    live &= live - 1u;
+                    at += __popc(m);
+                }
+                __syncwarp();
+                while (q.n >= 32u) queue_drain(q, so, f, fan, pts, ws, L, octs);
+            } else {   // many at once: each lane its own, the points read again
+                if (f.test || near) {
+#pragma unroll 1
+                    for (uint32_t m = live; m; m &= m - 1u) {
+                        const uint32_t i = (uint32_t)item_point<G>(base, t, __ffs(m) - 1);
+                        if (!settle(so, f, fan, i | (near ? kUnsettled : 0u), input_point(pts, i), octs))
+                            live &= ~(m & (0u - m));
+                    }
+                }
+                append_survivors(live, ws, L, [&](int k, uint32_t &i) {
+                    const int64_t j = item_point<G>(base, t, k);
+                    i = (uint32_t)j;
+                    return input_point(pts, j);
+                });
+            }
         }
+        while (q.n) queue_drain(q, so, FanView{use_disk, F, c}, fan, pts, ws, L, octs);
     }
     octs = __reduce_add_sync(0xffffffffu, octs);
     if (lane_id() == 0 && octs) atomicAdd(&s_oct, octs);
@@ -627,7 +801,7 @@ __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint3
 }
 
 // One thread per sub-bin, as fan_build_kernel; the table's ends are repeated
-// at V[-1] and V[kFan2Bins].
+// at V[-1] and V[kFan2Bins], V[kFan2Bins + 1].
 __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
 {
     __shared__ int s_w[BT / 32];
@@ -640,14 +814,14 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
     const Kgon *g = at<Kgon>(ws, L.kgon);
     float2 *V = at<float2>(ws, L.fan2_v) + 1;
     const int b = (int)(blockIdx.x * BT + threadIdx.x);
-    const int src = vertex_source(slot, s_w, s_scan);
+    const int src = vertex_source([&](int j) { return slot[j] != 0ull; }, s_w, s_scan);
     if (src < 0) {   // no survivor reached a slot: keep everything
         if (threadIdx.x == 0) f2->bad = 1u;
         return;
     }
     const float2 v = surv_point(keys, pay, ~(uint32_t)slot[src]);
     V[b] = v;
-    if (b == 0) V[kFan2Bins] = v;
+    if (b < 2) V[kFan2Bins + b] = v;
     if (b == kFan2Bins - 1) V[-1] = v;
     const unsigned long long nextp = slot[next_bin<kFan2Bins>(b)];
     const float2 w = nextp != 0ull ? surv_point(keys, pay, ~(uint32_t)nextp) : v;
@@ -671,8 +845,8 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
     const uint32_t m = f2->count_in;
     const bool test = !f2->bad && f2->edges >= 3u;
     const Kgon *g = at<Kgon>(ws, L.kgon);
-    const float cx = g->cx, cy = g->cy;
-    const float2 *V = at<float2>(ws, L.fan2_v) + 1;
+    const float2 c = make_float2(g->cx, g->cy);
+    const GlobalFan F{at<float2>(ws, L.fan2_v) + 1};
     const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
     const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
     uint32_t *okeys = at<uint32_t>(ws, L.keys[1]);
@@ -697,13 +871,13 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
             uint32_t in = 0;
 #pragma unroll
             for (int k = 0; k < F2I; ++k) {
-                const float x = key_float(kv[k]), y = key_float((uint32_t)(pv[k] >> 32));
-                in |= (fan_inside<kFan2Bins>(V, __fsub_rn(x, cx), __fsub_rn(y, cy), x, y) ? 1u : 0u) << k;
+                const float2 p = make_float2(key_float(kv[k]), key_float((uint32_t)(pv[k] >> 32)));
+                if (fan_inside<kFan2Bins>(F, c, sub2(p, c), p)) in |= 1u << k;
             }
             keep &= ~in;
         }
         uint32_t incl = __popc(keep);
-        const uint32_t c = incl;
+        const uint32_t cnt = incl;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
@@ -711,7 +885,7 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
         }
         uint32_t pos = 0;
         if (lane == 31 && incl) pos = atomicAdd(&f2->kept, incl);
-        pos = __shfl_sync(0xffffffffu, pos, 31) + incl - c;
+        pos = __shfl_sync(0xffffffffu, pos, 31) + incl - cnt;
 #pragma unroll
         for (int k = 0; k < F2I; ++k) {
             if ((keep >> k) & 1u) {
@@ -738,7 +912,7 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
 {
     const int sms = sm_count();
     static const bool attr = [] {   // thread-safe one-time initialisation
-        cudaFuncSetAttribute(hull_filter_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFanSmem);
+        cudaFuncSetAttribute(hull_filter_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kQueueSmem + kFanTable);
         return true;
     }();
     (void)attr;
@@ -746,16 +920,17 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
     const int has_fan = n >= (int64_t)kKgonMinS ? 1 : 0;   // (fewer points: fewer survivors)
     if (has_fan) {
         const int64_t stride = fan_sample_stride(ntiles);
-        const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride), (int64_t)sms * 4);
+        const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride), 1 << 16);
         probe_before(CH_K_KGON, st);
         fan_bins_kernel<G><<<(unsigned)bb, kFiltThreads, 0, st>>>(pts, n, ws, L, (int32_t)stride, use_bits, kdev);
-        fan_build_kernel<<<kFanBins / BT, BT, 0, st>>>(pts, n, ws, L);
-        note_kernels(CH_K_KGON, 2);
+        fan_vertex_kernel<<<kFanBins / (VB * VT / 32), VT, 0, st>>>(pts, n, ws, L);
+        fan_build_kernel<<<kFanBins / BT, BT, 0, st>>>(n, ws, L);
+        note_kernels(CH_K_KGON, 3);
         probe_after(CH_K_KGON, st);
     }
     probe_before(CH_K_FILTER, st);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(ntiles, (int64_t)CG), sms));
-    hull_filter_kernel<G><<<(unsigned)grid, CT, has_fan ? kFanSmem : 0, st>>>(pts, n, ws, L, has_fan, use_bits, kdev);
+    hull_filter_kernel<G><<<(unsigned)grid, CT, kQueueSmem + (has_fan ? kFanTable : 0), st>>>(pts, (uint32_t)n, ws, L, has_fan, use_bits, kdev);
     note_kernels(CH_K_FILTER, 1);
     probe_after(CH_K_FILTER, st);
     cudaError_t e = cudaGetLastError();
@@ -795,6 +970,7 @@ namespace {
 // many sets (ch_hull_batched): the same fan for every set with at least
 // kKgonMinS octagon survivors, between the batched count pass and its scan
 // ---------------------------------------------------------------------------
+constexpr int kFanSmem = kFanBins * 8;
 constexpr int FT = 512;                  // threads per block of the bins pass
 constexpr int FITEMS = 8;                // points per thread per tile there
 // The signs orient_f32 certifies, as two flags (det > bound, -det > bound;
@@ -819,7 +995,7 @@ template <int NB = kFanBins>
 __device__ __forceinline__ int fan_signs_f32(const float2 *V, float cx, float cy, float px, float py)
 {
     const float dx = __fsub_rn(px, cx), dy = __fsub_rn(py, cy);
-    const int b = fan_bin<NB>(dx, dy);
+    const int b = (int)min(fan_bin<NB>(dx, dy), NB - 1u);
     const float2 v = V[b];
     const Sgn o = sgn_ref(__fsub_rn(v.x, cx), __fsub_rn(v.y, cy), dx, dy);                   // (v, p, c)
     const float2 w = V[o.pos ? next_bin<NB>(b) : prev_bin<NB>(b)];
@@ -835,7 +1011,7 @@ __device__ __forceinline__ int fan_signs_f32(const float2 *V, float cx, float cy
 template <int NB = kFanBins>
 __device__ __noinline__ bool fan_inside_exact(const float2 *V, float cx, float cy, float px, float py)
 {
-    const int b = fan_bin<NB>(px - cx, py - cy);
+    const int b = (int)min(fan_bin<NB>(px - cx, py - cy), NB - 1u);
     const float2 v = V[b];
     const int o = orient(cx, cy, v.x, v.y, px, py);
     if (o == 0) return false;
@@ -948,7 +1124,7 @@ __global__ void __launch_bounds__(FT) bx_fan_bins_kernel(const float *__restrict
                 const int64_t i = lo + r * FT + threadIdx.x;
                 if (i < hi) {
                     const float dx = p[r].x - cx, dy = p[r].y - cy;
-                    const int bin = fan_bin(dx, dy);
+                    const int bin = (int)min(fan_bin(dx, dy), kFanBins - 1u);
                     const unsigned long long v =
                         ((unsigned long long)far_key(p[r].x, p[r].y, cx, cy, r2ref) << 32) | (uint32_t)~(uint32_t)i;
                     if (v > __ldcg(sl + bin)) atomicMax(sl + bin, v);
@@ -1045,7 +1221,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
     }
 }
 
-// Persistent blocks take work items by ticket; the 28672 vertices of the
+// Persistent blocks take work items by ticket; the 27648 vertices of the
 // item's fan are loaded into shared memory when the fan changes (items of
 // one fan are consecutive).  The four groups of kFiltThreads threads share
 // the item's tiles; thread t holds the 16 keep bits of count-pass thread t

@@ -9,8 +9,9 @@
 // point of the polygon's box (build_octagon_warp, which has the proof):
 // min_k T_k > 1 proves the point strictly inside, min_k T_k < -1 proves it
 // kept, anything else (a band of relative width 2^-20 around the boundary)
-// is decided exactly by keep_point.  Two differences, 16 FMAs and 7 minima
-// decide nearly every point, whatever the polygon's shape.  Testing the edge
+// is decided exactly by keep_point.  Two differences, 16 FMAs (8
+// instructions: two points at once) and 4 three-operand minima decide nearly
+// every point, whatever the polygon's shape.  Testing the edge
 // of the point's octant first and the other seven in a second, queued step
 // took 46 instructions for a circle's points and sent most points of a thin
 // rotated ellipse to the second step: the hull of 10^8 such points took 2167
@@ -53,9 +54,11 @@ __device__ __noinline__ bool keep_point(const Octagon &o, float x, float y)
     return false;
 }
 
-// The polygon in shared memory, the edges' affine forms packed.
+// The polygon in shared memory, the edges' affine forms twice over for the
+// packed arithmetic.
 struct OctSmem : Octagon {
-    float4 t4[8];   // (tx, ty, tz, -)
+    float4 txy[8];   // tx, tx, ty, ty
+    float2 tzz[8];   // tz, tz
 };
 
 // Copies the polygon `g` to shared memory; the caller synchronises before
@@ -65,49 +68,124 @@ __device__ __forceinline__ void fill_octagon(OctSmem &so, const Octagon *g)
     const uint32_t *src = reinterpret_cast<const uint32_t *>(g);
     uint32_t *dst = reinterpret_cast<uint32_t *>(static_cast<Octagon *>(&so));
     for (uint32_t w = threadIdx.x; w < sizeof(Octagon) / 4; w += blockDim.x) dst[w] = src[w];
-    if (threadIdx.x < 8)
-        so.t4[threadIdx.x] = make_float4(g->tx[threadIdx.x], g->ty[threadIdx.x], g->tz[threadIdx.x], 0.0f);
+    if (threadIdx.x < 8) {
+        const float tx = g->tx[threadIdx.x], ty = g->ty[threadIdx.x], tz = g->tz[threadIdx.x];
+        so.txy[threadIdx.x] = make_float4(tx, tx, ty, ty);
+        so.tzz[threadIdx.x] = make_float2(tz, tz);
+    }
 }
 
-// NaN-propagating minimum: an overflowed difference (or edge forms that are
-// switched off) must leave a point undecided, not inside.
-__device__ __forceinline__ float min_nan(float a, float b)
-{
-    float d;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
-    return d;
-}
-
-// N points at once: bit q of `in` when point q is proven strictly inside,
-// of `und` when it is undecided.  The edges are the outer loop, so their
-// forms are read once for the N points.
+// N points at once: bit q of `keep` unless point q is proven strictly inside
+// the polygon; the result says whether any of them is undecided
+// (oct_undecided then tells which; the NaN-propagating minima leave a point
+// undecided whose difference overflowed).  The edges are the outer loop, so
+// their forms are read once for the N points, and two points share an FMA
+// instruction.
 template <int N>
-__device__ __forceinline__ void oct_decide(const OctSmem &o, const float (&px)[N], const float (&py)[N], uint32_t &in,
-                                           uint32_t &und)
+__device__ __forceinline__ bool oct_decide(const OctSmem &o, const float (&px)[N], const float (&py)[N], uint32_t &keep)
 {
-    float u[N], v[N], m[N];
+    f32x2 u[N / 2], v[N / 2];
+    float m[N];
     const float cx = o.cx, cy = o.cy;
 #pragma unroll
-    for (int q = 0; q < N; ++q) {
-        u[q] = __fsub_rn(px[q], cx);
-        v[q] = __fsub_rn(py[q], cy);
+    for (int q = 0; q < N / 2; ++q) {
+        u[q] = pack2(__fsub_rn(px[2 * q], cx), __fsub_rn(px[2 * q + 1], cx));
+        v[q] = pack2(__fsub_rn(py[2 * q], cy), __fsub_rn(py[2 * q + 1], cy));
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const float4 t = o.t4[k];
+    for (int k = 0; k < 8; k += 2) {
+        asm volatile("" ::: "memory");   // (two edges' forms in registers at a time)
+        const float4 ta = o.txy[k], tb = o.txy[k + 1];
+        const float2 za = o.tzz[k], zb = o.tzz[k + 1];
+        const f32x2 xa = pack2(ta.x, ta.y), ya = pack2(ta.z, ta.w), xb = pack2(tb.x, tb.y), yb = pack2(tb.z, tb.w);
+        const f32x2 z0 = pack2(za.x, za.y), z1 = pack2(zb.x, zb.y);
 #pragma unroll
-        for (int q = 0; q < N; ++q) {
-            const float T = __fmaf_rn(t.x, u[q], __fmaf_rn(t.y, v[q], t.z));
-            m[q] = k == 0 ? T : min_nan(m[q], T);
+        for (int q = 0; q < N / 2; ++q) {
+            const float2 a = unpack2(fma2(xa, u[q], fma2(ya, v[q], z0)));
+            const float2 b = unpack2(fma2(xb, u[q], fma2(yb, v[q], z1)));
+            m[2 * q] = k == 0 ? min_nan(a.x, b.x) : min_nan(m[2 * q], a.x, b.x);
+            m[2 * q + 1] = k == 0 ? min_nan(a.y, b.y) : min_nan(m[2 * q + 1], a.y, b.y);
         }
     }
-    in = und = 0u;
+    keep = 0u;
+    float near = 2.0f;
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-        const bool i = m[q] > 1.0f;
-        in |= (i ? 1u : 0u) << q;
-        und |= (!i && !(m[q] < -1.0f) ? 1u : 0u) << q;
+        if (!(m[q] > 1.0f)) keep |= 1u << q;
+        near = min_nan(near, fabsf(m[q]));
     }
+    return !(near > 1.0f);
+}
+
+// Whether point (x, y) is undecided by the same forms.
+static __device__ __noinline__ bool oct_undecided(const OctSmem &o, float x, float y)
+{
+    const float u = __fsub_rn(x, o.cx), v = __fsub_rn(y, o.cy);
+    float m = 2.0f;
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) m = min_nan(m, __fmaf_rn(o.txy[k].x, u, __fmaf_rn(o.txy[k].z, v, o.tzz[k].x)));
+    return !(fabsf(m) > 1.0f);
+}
+
+// Point of item q of the 16 that thread t (of kFiltThreads) has in the
+// 4096-point tile at `base`: item q = r * G + h is point base + (r *
+// kFiltThreads + t) * G + h (G = 2: pairs of points, read 16 bytes at once).
+template <int G>
+__device__ __forceinline__ int64_t item_point(int64_t base, uint32_t t, int q)
+{
+    return base + (int64_t)((q / G) * kFiltThreads + t) * G + q % G;
+}
+
+__device__ __forceinline__ float2 input_point(const float *pts, int64_t i)
+{
+    return __ldg(reinterpret_cast<const float2 *>(pts) + i);
+}
+
+// Items N part .. N part + N - 1 of a thread's 16 in the tile at `base`, all of
+// them below n (G = 2: 16-byte loads).
+template <int G, int N>
+__device__ __forceinline__ void load_part(const float *__restrict__ pts, int64_t base, uint32_t t, int part,
+                                          float (&px)[N], float (&py)[N])
+{
+    if constexpr (G == 2) {
+        const float4 *p4 = reinterpret_cast<const float4 *>(pts) + base / 2 + part * (N / 2) * kFiltThreads + t;
+        float4 v[N / 2];
+#pragma unroll
+        for (int r = 0; r < N / 2; ++r) v[r] = __ldg(p4 + r * kFiltThreads);
+#pragma unroll
+        for (int r = 0; r < N / 2; ++r) {
+            px[2 * r] = v[r].x;
+            py[2 * r] = v[r].y;
+            px[2 * r + 1] = v[r].z;
+            py[2 * r + 1] = v[r].w;
+        }
+    } else {
+        const float2 *p2 = reinterpret_cast<const float2 *>(pts) + base + part * N * kFiltThreads + t;
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+            const float2 v = __ldg(p2 + r * kFiltThreads);
+            px[r] = v.x;
+            py[r] = v.y;
+        }
+    }
+}
+
+// The same where the tile ends before them: the centre stands in for the
+// missing points; returns the bits of those that exist.
+template <int G, int N>
+__device__ __forceinline__ uint32_t load_part_ragged(const float *__restrict__ pts, int64_t n, int64_t base, uint32_t t,
+                                                     int part, float cx, float cy, float (&px)[N], float (&py)[N])
+{
+    uint32_t live = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int64_t i = item_point<G>(base, t, N * part + k);
+        const float2 v = i < n ? input_point(pts, i) : make_float2(cx, cy);
+        px[k] = v.x;
+        py[k] = v.y;
+        live |= (i < n ? 1u : 0u) << k;
+    }
+    return live;
 }
 
 }  // namespace ch
