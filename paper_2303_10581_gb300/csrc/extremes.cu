@@ -105,7 +105,7 @@ __device__ __forceinline__ void combine(float &k, uint32_t &i, float ok, uint32_
 // "strictly left of every edge" is an intersection of open half-planes,
 // hence convex); points in it are discarded with four comparisons.  The
 // largest of a few concentric candidates that passes is kept.
-__device__ void build_octagon_warp(const float2 *pts, const uint32_t *ext8, Octagon *out, bool data_extremes)
+__device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_t *ext8, Octagon *out, bool data_extremes)
 {
     const uint32_t lane = lane_id();
     const uint32_t k = lane & 7u;
@@ -511,28 +511,51 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
     if constexpr (SPEC)
         if (lane == 0) sc->scnt[blockIdx.x * kSpecWarps + warp] = min(wcnt, cap);
 
-    // the full tiles' winners: per slot, the lanes holding the warp's
-    // largest key re-read their tile and take its first point with that key
+    // the full tiles' winners: per slot, the lanes holding the warp's largest
+    // key; their tiles are read again for the first point with that key, four
+    // lanes per slot (one per pair of points a thread has in a tile), so that
+    // all slots' reads are one latency (one slot after the other took 8 us)
+    static_assert(U == 4, "four lanes re-read a thread's pairs of a tile");
+    uint32_t wmask = 0;   // of this lane's slot: the lanes holding the largest key
+    float wkey = 0.0f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        float m = bk[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         const int32_t bt = s_btile[j][threadIdx.x];
-        if (bt >= 0 && bk[j] == m) {
-            const int64_t q0 = (int64_t)bt * kExtPairs;
-            uint32_t idx = 0xffffffffu;
-#pragma unroll
-            for (int u = U - 1; u >= 0; --u) {   // backwards: the last match is the first point
-                const float4 w = p4[q0 + u * kExtThreads + threadIdx.x];
-                float k[8];
-                slot_keys(w.z, w.w, k);
-                if (k[j] == bk[j]) idx = (uint32_t)(head + 2 * (q0 + u * kExtThreads + threadIdx.x) + 1);
-                slot_keys(w.x, w.y, k);
-                if (k[j] == bk[j]) idx = (uint32_t)(head + 2 * (q0 + u * kExtThreads + threadIdx.x));
-            }
-            if (idx != 0xffffffffu) combine(b.k[j], b.i[j], bk[j], idx);
+        // (ordered keys: unsigned maxima over the warp are one instruction; 0: no tile)
+        const uint32_t m = __reduce_max_sync(0xffffffffu, bt >= 0 ? ord_key(bk[j]) : 0u);
+        const uint32_t w = __ballot_sync(0xffffffffu, bt >= 0 && ord_key(bk[j]) == m);
+        if ((int)(lane >> 2) == j) {
+            wmask = w;
+            wkey = key_float(m);
         }
+    }
+    __syncwarp();   // the other lanes' tiles
+    const int wslot = (int)(lane >> 2);
+    uint32_t widx = 0xffffffffu;
+    for (uint32_t m = wmask; m; m &= m - 1u) {   // ties: every holder
+        const uint32_t th = (warp << 5) + (uint32_t)(__ffs(m) - 1);
+        const int64_t q = (int64_t)s_btile[wslot][th] * kExtPairs + (lane & 3u) * kExtThreads + th;
+        const float4 v = p4[q];
+        float ka[8], kb[8];
+        slot_keys(v.x, v.y, ka);
+        slot_keys(v.z, v.w, kb);
+        float a = ka[0], d = kb[0];
+#pragma unroll
+        for (int j = 1; j < 8; ++j) {
+            a = wslot == j ? ka[j] : a;
+            d = wslot == j ? kb[j] : d;
+        }
+        const uint32_t i0 = (uint32_t)(head + 2 * q);
+        if (d == wkey) widx = min(widx, i0 + 1u);
+        if (a == wkey) widx = min(widx, i0);
+    }
+    __syncwarp();
+    widx = min(widx, __shfl_xor_sync(0xffffffffu, widx, 1));
+    widx = min(widx, __shfl_xor_sync(0xffffffffu, widx, 2));
+    if ((lane & 3u) == 0u) {   // lane 4 j: slot j's candidate joins its own of the ragged ends
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (wslot == j) combine(b.k[j], b.i[j], wkey, widx);
     }
     // warp reduction
 #pragma unroll
@@ -636,67 +659,68 @@ constexpr int kSampleRun = kSampleThreads * 8;
 constexpr double kP0Shrink = 0.9;
 constexpr int kSpecProbe = 1024;   // points tested against A before the sweep
 
-__device__ void build_spec_box(const float (&kmax)[8], SpecBox *out)
+// Run by one full warp: lanes 0..7 (and their copies) each take one bound, so
+// the binary64 chain is one bound's (one thread for all eight took 6 us).
+// kmax: the slot key maximum of lane & 7, in slot order max x, max s, max y,
+// max -d, max -x, max -s, max -y, max d.
+__device__ void build_spec_box(float kmax, SpecBox *out)
 {
-    // kmax in slot order: max x, max s, max y, max -d, max -x, max -s, max -y, max d
-    double xh = kmax[0], sh = kmax[1], yh = kmax[2], dl = -(double)kmax[3];
-    double xl = -(double)kmax[4], sl = -(double)kmax[5], yl = -(double)kmax[6], dh = kmax[7];
-    SpecBox b{};
-    b.ok = 0;
+    const uint32_t k = lane_id() & 7u;
+    const bool lower = k >= 3u && k <= 6u;   // dl, xl, sl, yl: minima
+    const double e = lower ? -(double)kmax : (double)kmax;
+    const auto of = [&](double v, int j) { return __shfl_sync(0xffffffffu, v, j); };
+    double xh = of(e, 0), yh = of(e, 2), xl = of(e, 4), yl = of(e, 6);
     const double M = fmax(fabs(xl), fabs(xh)) + fmax(fabs(yl), fabs(yh));
-    bool ok = xl < xh && yl < yh && M < 1e37 && M > 1e-30;
-    if (ok) {
-        const double cx = 0.5 * (xl + xh), cy = 0.5 * (yl + yh), cs = cx + cy, cd = cx - cy;
-        const double f = kP0Shrink;
-        xh = cx + f * (xh - cx);
-        xl = cx + f * (xl - cx);
-        yh = cy + f * (yh - cy);
-        yl = cy + f * (yl - cy);
-        sh = cs + f * (sh - cs);
-        sl = cs + f * (sl - cs);
-        dh = cd + f * (dh - cd);
-        dl = cd + f * (dl - cd);
-        // grid: the smallest power of two >= 2^-21 M
-        int ge = 0;
-        frexp(M * 0x1p-21, &ge);   // M 2^-21 < 2^ge
-        const double g = ldexp(1.0, ge);
-        xh = floor(xh / g) * g;
-        yh = floor(yh / g) * g;
-        sh = floor(sh / g) * g;
-        dh = floor(dh / g) * g;
-        xl = ceil(xl / g) * g;
-        yl = ceil(yl / g) * g;
-        sl = ceil(sl / g) * g;
-        dl = ceil(dl / g) * g;
-        // each diagonal cuts its corner of the box, within the box's edges
-        sh = fmax(fmin(sh, xh + yh), fmax(xh + yl, xl + yh));
-        sl = fmin(fmax(sl, xl + yl), fmin(xh + yl, xl + yh));
-        dh = fmax(fmin(dh, xh - yl), fmax(xh - yh, xl - yl));
-        dl = fmin(fmax(dl, xl - yh), fmin(xh - yh, xl - yl));
-        const double vx[8] = {xh, sh - yh, dl + yh, xl, xl, sl - yl, dh + yl, xh};
-        const double vy[8] = {sh - xh, yh, yh, xl - dl, sl - xl, yl, yl, xh - dh};
-        // in order around the box: right, top, left, bottom edges not inverted
-        ok = xl < xh && yl < yh && vy[7] <= vy[0] && vx[2] <= vx[1] && vy[4] <= vy[3] && vx[5] <= vx[6];
-        // the test's diagonal bounds, moved in by m = 2^-23 M' (M' = |x| + |y|
-        // bound inside the snapped box), rounded inwards
-        const double Mb = fmax(fabs(xl), fabs(xh)) + fmax(fabs(yl), fabs(yh));
-        const double m = Mb * 0x1p-23;
-        b.xl = (float)xl;
-        b.xh = (float)xh;
-        b.yl = (float)yl;
-        b.yh = (float)yh;
-        b.slb = __double2float_ru(sl + m);
-        b.shb = __double2float_rd(sh - m);
-        b.dlb = __double2float_ru(dl + m);
-        b.dhb = __double2float_rd(dh - m);
-        ok = ok && b.slb <= b.shb && b.dlb <= b.dhb;
-        for (int k = 0; k < 8; ++k) {
-            b.vx[k] = (float)vx[k];
-            b.vy[k] = (float)vy[k];
-        }
+    bool ok = xl < xh && yl < yh && M < 1e37 && M > 1e-30;   // warp-uniform
+    if (!ok) {
+        if (lane_id() == 0) out->ok = 0u;
+        return;
     }
-    b.ok = ok ? 1u : 0u;
-    *out = b;
+    const double cx = 0.5 * (xl + xh), cy = 0.5 * (yl + yh);
+    // this bound's centre: x, s = x + y, y, d = x - y, x, s, y, d
+    const double c = (k & 3u) == 0u ? cx : ((k & 3u) == 2u ? cy : ((k == 1u || k == 5u) ? cx + cy : cx - cy));
+    // grid: the smallest power of two > 2^-21 M
+    int ge = 0;
+    frexp(M * 0x1p-21, &ge);   // M 2^-21 < 2^ge
+    const double g = ldexp(1.0, ge), gi = ldexp(1.0, -ge);
+    const double v = (c + kP0Shrink * (e - c)) * gi;   // (a power of two: exact, as the product below)
+    const double snapped = (lower ? ceil(v) : floor(v)) * g;
+    xh = of(snapped, 0);
+    double sh = of(snapped, 1);
+    yh = of(snapped, 2);
+    double dl = of(snapped, 3);
+    xl = of(snapped, 4);
+    double sl = of(snapped, 5);
+    yl = of(snapped, 6);
+    double dh = of(snapped, 7);
+    // each diagonal cuts its corner of the box, within the box's edges
+    sh = fmax(fmin(sh, xh + yh), fmax(xh + yl, xl + yh));
+    sl = fmin(fmax(sl, xl + yl), fmin(xh + yl, xl + yh));
+    dh = fmax(fmin(dh, xh - yl), fmax(xh - yh, xl - yl));
+    dl = fmin(fmax(dl, xl - yh), fmin(xh - yh, xl - yl));
+    if (lane_id() != 0) return;
+    const double vx[8] = {xh, sh - yh, dl + yh, xl, xl, sl - yl, dh + yl, xh};
+    const double vy[8] = {sh - xh, yh, yh, xl - dl, sl - xl, yl, yl, xh - dh};
+    // in order around the box: right, top, left, bottom edges not inverted
+    ok = xl < xh && yl < yh && vy[7] <= vy[0] && vx[2] <= vx[1] && vy[4] <= vy[3] && vx[5] <= vx[6];
+    // the test's diagonal bounds, moved in by m = 2^-23 M' (M' = |x| + |y|
+    // bound inside the snapped box), rounded inwards
+    const double Mb = fmax(fabs(xl), fabs(xh)) + fmax(fabs(yl), fabs(yh));
+    const double m = Mb * 0x1p-23;
+    out->xl = (float)xl;
+    out->xh = (float)xh;
+    out->yl = (float)yl;
+    out->yh = (float)yh;
+    out->slb = __double2float_ru(sl + m);
+    out->shb = __double2float_rd(sh - m);
+    out->dlb = __double2float_ru(dl + m);
+    out->dhb = __double2float_rd(dh - m);
+    ok = ok && out->slb <= out->shb && out->dlb <= out->dhb;
+    for (int j = 0; j < 8; ++j) {
+        out->vx[j] = (float)vx[j];
+        out->vy[j] = (float)vy[j];
+    }
+    out->ok = ok ? 1u : 0u;
 }
 
 __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float *__restrict__ pts, int64_t n, void *ws,
@@ -705,6 +729,9 @@ __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float
     SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const float2 *p2 = reinterpret_cast<const float2 *>(pts);
     const int64_t start = (n - kSampleRun) * (int64_t)blockIdx.x / (gridDim.x - 1);
+    // the probe's points into L2 (the last block reads them at the end)
+    if (threadIdx.x < kSpecProbe / kSampleBlocks)
+        prefetch_l2(p2 + (int64_t)(blockIdx.x * (kSpecProbe / kSampleBlocks) + threadIdx.x) * (n / kSpecProbe));
     float km[8];
     float2 pv[kSampleRun / kSampleThreads];
 #pragma unroll
@@ -740,15 +767,16 @@ __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float
     if (!s_last) return;
     __threadfence();
     __shared__ SpecBox s_box;
+    float kmax = 0.0f;
+    if (lane < 8) kmax = key_float(atomicExch(&sc->kmax[lane], 0u));
+    kmax = __shfl_sync(0xffffffffu, kmax, (int)(lane & 7u));
     if (lane == 0) {
-        float kmax[8];
-        for (int j = 0; j < 8; ++j) kmax[j] = key_float(atomicExch(&sc->kmax[j], 0u));
         sc->sample_done = 0u;
         sc->fail = 0u;
         sc->nseg = nseg;
         sc->cap = cap;
-        build_spec_box(kmax, &s_box);
     }
+    build_spec_box(kmax, &s_box);
     __syncwarp();
     // the share of kSpecProbe evenly spaced points outside A predicts the
     // candidates' share: above half the segments' capacity (1 / kSpecCapDiv
@@ -757,8 +785,9 @@ __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float
     uint32_t out = 0;
     if (s_box.ok) {
         const int64_t stride = n / kSpecProbe;
-        for (int k = (int)lane; k < kSpecProbe; k += 32) {
-            const float2 v = __ldg(p2 + (int64_t)k * stride);
+#pragma unroll 32
+        for (int r = 0; r < kSpecProbe / 32; ++r) {   // (the reads go out together)
+            const float2 v = __ldg(p2 + (int64_t)(r * 32 + (int)lane) * stride);
             out += spec_inside(s_box, v.x, v.y, __fadd_rn(v.x, v.y), __fsub_rn(v.x, v.y)) ? 0u : 1u;
         }
     }

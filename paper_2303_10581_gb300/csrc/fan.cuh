@@ -7,12 +7,14 @@
 namespace ch {
 
 // The first level's sample: every fan_sample_stride(tiles)-th 4096-point
-// tile (at least every tile; about kFanBinTiles tiles, at most every 8th).
+// tile (at least every tile; about kFanBinTiles tiles, at most every 16th).
+// Of 10^8 circle points 7.5 M reach the second level with every 16th tile and
+// 7.0 M with every 8th, whose bins take 40 us more.
 constexpr int64_t kFanBinTiles = 1536;
 __host__ __device__ inline int64_t fan_sample_stride(int64_t tiles)
 {
     const int64_t s = tiles / kFanBinTiles;
-    return s < 1 ? 1 : (s > 8 ? 8 : s);
+    return s < 1 ? 1 : (s > 16 ? 16 : s);
 }
 
 // Scaled pseudo-angle of the direction (dx, dy): in [0, NB], growing with

@@ -128,14 +128,14 @@ __device__ __forceinline__ bool fan_inside(const Fan &F, float2 c, float2 d, flo
 }
 
 // The bin a point may be the vertex of, -1 when its pseudo-angle is within
-// `margin` of the bin's ends.
+// `margin` of the bin's ends (or undefined).
 template <int NB>
 __device__ __forceinline__ int vertex_bin(float dx, float dy, float margin)
 {
     const float phi = fan_phi<NB>(dx, dy);
-    const int b = __float2int_rd(phi);
-    const float f = phi - (float)b;
-    return f >= margin && f <= 1.0f - margin && b >= 0 && b < NB ? b : -1;
+    const float f = __fadd_rd(phi, 0x1p23f);   // 2^23 + the bin
+    const float mid = phi - (f - 0x1p23f) - 0.5f;
+    return fabsf(mid) <= 0.5f - margin ? (int)(__float_as_uint(f) - kBinBias) : -1;
 }
 
 // Whether this call has a fan whose proofs hold (after fan_build_kernel).
@@ -148,12 +148,20 @@ __device__ __forceinline__ bool fan_ready(const KgonCtrl *kc, const Kgon *g)
 // ---------------------------------------------------------------------------
 // first level: bins and vertices
 // ---------------------------------------------------------------------------
-// Every stride-th tile, a block each: the octagon survivors' bins.  Bound by
-// the latency of the points' and then the slots' reads.
+// Every stride-th tile, in quarters (1024 points, four a thread) over a
+// persistent grid: the bins' farthest points.  The first quarter's points
+// take the octagon test as well: it tells how many points survive it (a point
+// inside the octagon is an input point all the same, and rarely the
+// farthest).  A point whose binary32 distance is clearly below its slot's
+// needs no exact key.  Bound by the latency of the points' and then the
+// slots' reads, so the next quarter's points are read while this one is
+// binned, and few registers keep five blocks on an SM.
+constexpr int BI = 4;   // points per thread and step
+
 template <int G>
-__global__ void __launch_bounds__(kFiltThreads) fan_bins_kernel(const float *__restrict__ pts, int64_t n, void *ws,
-                                                                Layout L, int32_t stride, int use_bits,
-                                                                const int32_t *kdev)
+__global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *__restrict__ pts, uint32_t n, void *ws,
+                                                                   Layout L, uint32_t stride, int use_bits,
+                                                                   const int32_t *kdev)
 {
     __shared__ OctSmem so;
     const Octagon *oct = at<Octagon>(ws, L.oct);
@@ -162,44 +170,65 @@ __global__ void __launch_bounds__(kFiltThreads) fan_bins_kernel(const float *__r
     __syncthreads();
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     const bool bits_mode = use_bits && (!kdev || *kdev != 8);
-    const uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    unsigned long long *slot = kc->slot;
     const float cx = so.cx, cy = so.cy, r2ref = far_ref(so);
     const uint32_t t = threadIdx.x;
-    uint32_t seen = 0, kept = 0;
-    for (int64_t tile = (int64_t)blockIdx.x * stride; tile * kFiltTile < n; tile += (int64_t)gridDim.x * stride) {
-        const int64_t base = tile * kFiltTile;
-#pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
-            float px[8], py[8];
-            uint32_t live = 0xffu;
-            if (base + kFiltTile <= n) load_part<G, 8>(pts, base, t, half, px, py);
-            else live = load_part_ragged<G, 8>(pts, n, base, t, half, cx, cy, px, py);
-            seen += __popc(live);
-            if (bits_mode) {
-                live &= (uint32_t)bits[tile * kFiltThreads + t] >> (8 * half);
-            } else {
-                uint32_t out;
-                oct_decide<8>(so, px, py, out);   // (undecided points are input points all the same)
-                live &= out;
-            }
-            kept += __popc(live);
-            if (!__any_sync(0xffffffffu, live != 0u)) continue;
-            int b[8];
-            uint32_t key[8];
+    constexpr uint32_t parts = kFiltItems / BI;
+    const uint32_t ntiles = (n + kFiltTile - 1) / kFiltTile, steps = (ntiles + stride - 1) / stride * parts;
+    uint32_t seen = 0, kept = 0;   // (n < 2^30)
+    float px[BI], py[BI];
+    uint32_t live = 0;
+    const auto fetch = [&](uint32_t w) {
+        const uint32_t base = w / parts * stride * kFiltTile;
+        const int part = (int)(w % parts);
+        if (base + kFiltTile <= n) {
+            load_part<G, BI>(pts, base, t, part, px, py);
+            live = (1u << BI) - 1u;
+        } else {
+            live = load_part_ragged<G, BI>(pts, n, base, t, part, cx, cy, px, py);
+        }
+    };
+    if (blockIdx.x < steps) fetch(blockIdx.x);
+    for (uint32_t w = blockIdx.x; w < steps; w += gridDim.x) {
+        const uint32_t tile = w / parts * stride, part = w % parts;
+        float qx[BI], qy[BI];
+        uint32_t mine = live;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                b[k] = ((live >> k) & 1u) ? vertex_bin<kFanBins>(__fsub_rn(px[k], cx), __fsub_rn(py[k], cy), kFanMargin) : -1;
-                key[k] = far_key(px[k], py[k], cx, cy, r2ref);
-            }
-            uint32_t top[8];   // the slots' keys: most points do not raise their bin's
+        for (int k = 0; k < BI; ++k) {
+            qx[k] = px[k];
+            qy[k] = py[k];
+        }
+        if (w + gridDim.x < steps) fetch(w + gridDim.x);
+        if (bits_mode) {
+            seen += __popc(mine);
+            mine &= (uint32_t)at<uint16_t>(ws, L.keep_bits)[tile * kFiltThreads + t] >> (BI * part);
+            kept += __popc(mine);
+        } else if (part == 0u) {
+            seen += __popc(mine);
+            uint32_t out;
+            oct_decide<BI>(so, qx, qy, out);   // (undecided points count)
+            mine &= out;
+            kept += __popc(mine);
+        }
+        if (!__any_sync(0xffffffffu, mine != 0u)) continue;
+        uint32_t top[BI];   // the slots' keys (most points do not raise their bin's); ~0: no bin
+        int b[BI];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) top[k] = b[k] >= 0 ? __ldcg(reinterpret_cast<const uint32_t *>(slot + b[k]) + 1) : ~0u;
+        for (int k = 0; k < BI; ++k) {
+            b[k] = vertex_bin<kFanBins>(__fsub_rn(qx[k], cx), __fsub_rn(qy[k], cy), kFanMargin);
+            top[k] = 0u;
+            if (!((mine >> k) & 1u)) b[k] = -1;
+            if (b[k] >= 0) top[k] = __ldcg(reinterpret_cast<const uint32_t *>(kc->slot + b[k]) + 1);
+        }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (b[k] >= 0 && key[k] >= top[k]) {
-                    const uint32_t i = (uint32_t)item_point<G>(base, t, 8 * half + k);
-                    atomicMax(slot + b[k], ((unsigned long long)key[k] << 32) | (uint32_t)~i);
+        for (int k = 0; k < BI; ++k) {
+            const float dx = __fsub_rn(qx[k], cx), dy = __fsub_rn(qy[k], cy);
+            const float r2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
+            // (an empty slot's key is a NaN: not below)
+            if (b[k] >= 0 && !(r2 - r2ref < __fmaf_rn(r2, -0x1p-20f, key_float(top[k])))) {
+                const uint32_t key = far_key(qx[k], qy[k], cx, cy, r2ref);
+                if (key >= top[k]) {
+                    const uint32_t i = (uint32_t)item_point<G>(tile * kFiltTile, t, BI * part + k);
+                    atomicMax(kc->slot + b[k], ((unsigned long long)key << 32) | (uint32_t)~i);
                 }
             }
         }
@@ -920,9 +949,9 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
     const int has_fan = n >= (int64_t)kKgonMinS ? 1 : 0;   // (fewer points: fewer survivors)
     if (has_fan) {
         const int64_t stride = fan_sample_stride(ntiles);
-        const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride), 1 << 16);
+        const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride) * (kFiltItems / BI), (int64_t)sms * 5);
         probe_before(CH_K_KGON, st);
-        fan_bins_kernel<G><<<(unsigned)bb, kFiltThreads, 0, st>>>(pts, n, ws, L, (int32_t)stride, use_bits, kdev);
+        fan_bins_kernel<G><<<(unsigned)bb, kFiltThreads, 0, st>>>(pts, (uint32_t)n, ws, L, (uint32_t)stride, use_bits, kdev);
         fan_vertex_kernel<<<kFanBins / (VB * VT / 32), VT, 0, st>>>(pts, n, ws, L);
         fan_build_kernel<<<kFanBins / BT, BT, 0, st>>>(n, ws, L);
         note_kernels(CH_K_KGON, 3);
