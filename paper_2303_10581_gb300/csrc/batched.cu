@@ -19,6 +19,7 @@ constexpr uint32_t kSiteOffsets = 40;
 __global__ void __launch_bounds__(kSetupThreads) bx_setup_kernel(const int64_t *__restrict__ offsets, void *ws,
                                                                  Layout L, BatchLayout BL, int64_t n_cap)
 {
+    kernel_entry();
     __shared__ uint64_t s_w[kSetupThreads / 32];
     __shared__ int s_bad;
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -91,6 +92,7 @@ __device__ __forceinline__ int64_t last_le(int64_t count, uint64_t v, F key)
 
 __global__ void __launch_bounds__(256) bx_tileset_kernel(void *ws, BatchLayout BL)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -118,6 +120,7 @@ __device__ __forceinline__ void set_chain_sizes(const SetInfo &S, const uint32_t
 // One block: hull sizes and their exclusive scan into hull_offsets[0..B].
 __global__ void __launch_bounds__(kSetupThreads) bx_hullsize_kernel(void *ws, BatchLayout BL, int64_t *hull_offsets)
 {
+    kernel_entry();
     __shared__ uint64_t s_w[kSetupThreads / 32];
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -163,7 +166,7 @@ cudaError_t launch_bx_setup(const int64_t *offsets, void *ws, const Layout &L, c
 {
     bx_setup_kernel<<<1, kSetupThreads, 0, st>>>(offsets, ws, L, BL, n_cap);
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(ceil_div(BL.tiles_max, 256), sm_count() * 4));
-    bx_tileset_kernel<<<(unsigned)blocks, 256, 0, st>>>(ws, BL);
+    launch_next(bx_tileset_kernel, (unsigned)blocks, 256, 0, st, ws, BL);
     note_kernels(CH_K_EXTREMES, 2);
     return cudaGetLastError();
 }
@@ -172,7 +175,7 @@ cudaError_t launch_bx_finish(void *ws, const Layout &L, const BatchLayout &BL, u
                              int64_t *hull_offsets, cudaStream_t st)
 {
     probe_before(CH_K_FINISH, st);
-    bx_hullsize_kernel<<<1, kSetupThreads, 0, st>>>(ws, BL, hull_offsets);
+    launch_next(bx_hullsize_kernel, 1, kSetupThreads, 0, st, ws, BL, hull_offsets);
     const cudaError_t e = launch_bx_assemble(ws, L, BL, hull_offsets, hull_idx, st);
     if (e != cudaSuccess) return e;
     note_kernels(CH_K_FINISH, 2);

@@ -807,6 +807,7 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
 
 __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L)
 {
+    kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ChainSmem &sm = *reinterpret_cast<ChainSmem *>(smem_raw);
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
@@ -831,6 +832,7 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L)
 // climbs; the second child to reach a node merges the pair.
 __global__ void __launch_bounds__(32) chain_merge_kernel(void *ws, Layout L)
 {
+    kernel_entry();
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
@@ -845,6 +847,7 @@ __global__ void __launch_bounds__(32) chain_merge_kernel(void *ws, Layout L)
 // merge tree; the sorted arrays end up in buffer 0 (four passes)
 __global__ void __launch_bounds__(LT) bx_chain_kernel(void *ws, Layout L, BatchLayout BL)
 {
+    kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ChainSmem &sm = *reinterpret_cast<ChainSmem *>(smem_raw);
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -863,6 +866,7 @@ __global__ void __launch_bounds__(LT) bx_chain_kernel(void *ws, Layout L, BatchL
 
 __global__ void __launch_bounds__(32) bx_merge_kernel(void *ws, Layout L, BatchLayout BL)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -993,6 +997,7 @@ __device__ __forceinline__ void copy_chain_part(const ChainPtrs &P, int side, in
 
 __global__ void __launch_bounds__(kEmitThreads) emit_kernel(void *ws, Layout L)
 {
+    kernel_entry();
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
@@ -1010,6 +1015,7 @@ __global__ void __launch_bounds__(kEmitThreads) emit_kernel(void *ws, Layout L)
 __global__ void __launch_bounds__(kEmitThreads) hull_copy_kernel(void *ws, Layout L, uint32_t *hull_idx,
                                                                  uint32_t *hull_count)
 {
+    kernel_entry();
     const Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     if (ctrl->small_done) return;
     const uint32_t hl = ctrl->h_lower, hu = ctrl->h_upper;
@@ -1030,6 +1036,7 @@ __global__ void __launch_bounds__(kEmitThreads) hull_copy_kernel(void *ws, Layou
 // all sets at once: the offsets of every super-chunk's ranges
 __global__ void __launch_bounds__(kEmitThreads) bx_emit_kernel(void *ws, Layout L, BatchLayout BL)
 {
+    kernel_entry();
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const int64_t nc = bc->nsc;
@@ -1048,6 +1055,7 @@ __global__ void __launch_bounds__(kEmitThreads) bx_assemble_kernel(void *ws, Lay
                                                                    const int64_t *__restrict__ hull_offsets,
                                                                    uint32_t *hull_idx)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -1093,6 +1101,7 @@ struct SmallSmem {
 __global__ void __launch_bounds__(kSmallHull) small_hull_kernel(void *ws, Layout L, uint32_t *hull_idx,
                                                                 uint32_t *hull_count)
 {
+    kernel_entry();
     __shared__ SmallSmem sm;
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
@@ -1179,7 +1188,7 @@ __global__ void __launch_bounds__(kSmallHull) small_hull_kernel(void *ws, Layout
 cudaError_t launch_small_hull(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
 {
     probe_before(CH_K_CHAIN, st);
-    small_hull_kernel<<<1, kSmallHull, 0, st>>>(ws, L, hull_idx, hull_count);
+    launch_next(small_hull_kernel, 1, kSmallHull, 0, st, ws, L, hull_idx, hull_count);
     note_kernels(CH_K_CHAIN, 1);
     probe_after(CH_K_CHAIN, st);
     return cudaGetLastError();
@@ -1198,8 +1207,8 @@ cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t
     if (cb > (int64_t)sms * per_sm) cb = (int64_t)sms * per_sm;
     if (cb < 1) cb = 1;
     probe_before(CH_K_CHAIN, st);
-    chain_kernel<<<(unsigned)cb, LT, sizeof(ChainSmem), st>>>(ws, L);
-    chain_merge_kernel<<<(unsigned)ceil_div(L.n_chunks, 32), 32, 0, st>>>(ws, L);
+    launch_next(chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L);
+    launch_next(chain_merge_kernel, (unsigned)ceil_div(L.n_chunks, 32), 32, 0, st, ws, L);
     note_kernels(CH_K_CHAIN, 2);
     probe_after(CH_K_CHAIN, st);
     cudaError_t e = cudaGetLastError();
@@ -1208,14 +1217,14 @@ cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t
     if (eb > (int64_t)sms * 4) eb = (int64_t)sms * 4;
     if (eb < 1) eb = 1;
     probe_before(CH_K_EMIT, st);
-    emit_kernel<<<(unsigned)eb, kEmitThreads, 0, st>>>(ws, L);
+    launch_next(emit_kernel, (unsigned)eb, kEmitThreads, 0, st, ws, L);
     note_kernels(CH_K_EMIT, 1);
     probe_after(CH_K_EMIT, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t fb = std::min<int64_t>(ceil_div(L.n_chunks * 2 * kCopyParts, kEmitThreads / 32), (int64_t)sms * 4);
     probe_before(CH_K_FINISH, st);
-    hull_copy_kernel<<<(unsigned)fb, kEmitThreads, 0, st>>>(ws, L, hull_idx, hull_count);
+    launch_next(hull_copy_kernel, (unsigned)fb, kEmitThreads, 0, st, ws, L, hull_idx, hull_count);
     note_kernels(CH_K_FINISH, 1);
     probe_after(CH_K_FINISH, st);
     return cudaGetLastError();
@@ -1234,8 +1243,8 @@ cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cu
     if (cb > (int64_t)sms * per_sm) cb = (int64_t)sms * per_sm;
     if (cb < 1) cb = 1;
     probe_before(CH_K_CHAIN, st);
-    bx_chain_kernel<<<(unsigned)cb, LT, sizeof(ChainSmem), st>>>(ws, L, BL);
-    bx_merge_kernel<<<(unsigned)ceil_div(BL.tiles_max, 32), 32, 0, st>>>(ws, L, BL);
+    launch_next(bx_chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L, BL);
+    launch_next(bx_merge_kernel, (unsigned)ceil_div(BL.tiles_max, 32), 32, 0, st, ws, L, BL);
     note_kernels(CH_K_CHAIN, 2);
     probe_after(CH_K_CHAIN, st);
     cudaError_t e = cudaGetLastError();
@@ -1245,7 +1254,7 @@ cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cu
     if (eb > (int64_t)sms * emit_per_sm) eb = (int64_t)sms * emit_per_sm;
     if (eb < 1) eb = 1;
     probe_before(CH_K_EMIT, st);
-    bx_emit_kernel<<<(unsigned)eb, kEmitThreads, 0, st>>>(ws, L, BL);
+    launch_next(bx_emit_kernel, (unsigned)eb, kEmitThreads, 0, st, ws, L, BL);
     note_kernels(CH_K_EMIT, 1);
     probe_after(CH_K_EMIT, st);
     return cudaGetLastError();
@@ -1256,7 +1265,7 @@ cudaError_t launch_bx_assemble(void *ws, const Layout &L, const BatchLayout &BL,
 {
     const int64_t blocks =
         std::min<int64_t>(ceil_div(BL.tiles_max * 2 * kCopyParts, kEmitThreads / 32), (int64_t)sm_count() * 8);
-    bx_assemble_kernel<<<(unsigned)blocks, kEmitThreads, 0, st>>>(ws, L, BL, hull_offsets, hull_idx);
+    launch_next(bx_assemble_kernel, (unsigned)blocks, kEmitThreads, 0, st, ws, L, BL, hull_offsets, hull_idx);
     return cudaGetLastError();
 }
 

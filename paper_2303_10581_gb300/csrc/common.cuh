@@ -663,6 +663,26 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
 }
 
 // ---------------------------------------------------------------------------
+// programmatic dependent launch
+// ---------------------------------------------------------------------------
+// First statement of every kernel: waits until the kernels before this one
+// have completed and their writes are visible.  A kernel launched with
+// launch_next (launch.h) is put on the SMs when the blocks of the kernel before
+// it have left them, without waiting for its end to be signalled to the front
+// end first.  Every thread passes here, before any return, so a kernel's
+// completion implies that of all kernels before it.  A call's pipeline holds
+// up to a dozen kernels that find nothing to do for a given set, each 2.8 us
+// when launched the ordinary way: ch_hull of 1000 points 62 -> 40 us, of 2^20
+// normal points 105 -> 68, of 10^8 circle points 970 -> 919.  No kernel lets the
+// next one in earlier (launch_dependents): its blocks would then fill the
+// first SMs to become free, and grids of fewer blocks than the chip holds
+// would run on half of it (circle 1057, 2^20 normal points 75).
+__device__ __forceinline__ void kernel_entry()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // error reporting and bounded waits
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void set_error(void *ws, const Layout &L, uint32_t code, uint32_t site)

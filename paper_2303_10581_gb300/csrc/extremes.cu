@@ -338,6 +338,7 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
                                                                   const __nv_bfloat16 *learn, float *learn_dirs,
                                                                   int32_t *learn_k)
 {
+    kernel_entry();
     static_assert(kExtThreads == mlp::LT, "the learned block has the sweep's block size");
     const uint32_t nsweep = gridDim.x - (learn ? 1u : 0u);   // blocks of the sweep
     if (learn && blockIdx.x == nsweep) {
@@ -726,6 +727,7 @@ __device__ void build_spec_box(float kmax, SpecBox *out)
 __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float *__restrict__ pts, int64_t n, void *ws,
                                                                      Layout L, uint32_t nseg, uint32_t cap)
 {
+    kernel_entry();
     SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const float2 *p2 = reinterpret_cast<const float2 *>(pts);
     const int64_t start = (n - kSampleRun) * (int64_t)blockIdx.x / (gridDim.x - 1);
@@ -805,6 +807,7 @@ __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float
 __global__ void octagon_kernel(const float *__restrict__ pts, int64_t n, const uint32_t *ext8, void *ws,
                                Layout L, unsigned long long *zero_ptr, int64_t zero_words)
 {
+    kernel_entry();
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
     for (int64_t w = gtid; w < zero_words; w += gthreads) zero_ptr[w] = 0ull;
@@ -881,6 +884,7 @@ template <int T>   // threads per block: each holds kFiltTile / T points of a ti
 __global__ void __launch_bounds__(T) bx_extremes_kernel(const float *__restrict__ pts, void *ws, Layout L,
                                                         BatchLayout BL)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -941,6 +945,7 @@ __global__ void __launch_bounds__(T) bx_extremes_kernel(const float *__restrict_
 __global__ void __launch_bounds__(256) bx_octagon_kernel(const float *__restrict__ pts, void *ws, Layout L,
                                                          BatchLayout BL)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
     const unsigned long long *slots = at<unsigned long long>(ws, BL.ext_slot);
@@ -974,10 +979,10 @@ cudaError_t launch_bx_extremes(const float *pts, void *ws, const Layout &L, cons
     int64_t blocks = std::min<int64_t>(BL.tiles_max, (int64_t)sm_count() * per_sm);
     const unsigned g = (unsigned)std::max<int64_t>(blocks, 1);
     probe_before(CH_K_EXTREMES, st);
-    if (items == 4) bx_extremes_kernel<1024><<<g, 1024, 0, st>>>(pts, ws, L, BL);
-    else if (items == 8) bx_extremes_kernel<512><<<g, 512, 0, st>>>(pts, ws, L, BL);
-    else bx_extremes_kernel<256><<<g, 256, 0, st>>>(pts, ws, L, BL);
-    bx_octagon_kernel<<<(unsigned)ceil_div(BL.num_sets, 8), 256, 0, st>>>(pts, ws, L, BL);
+    if (items == 4) launch_next(bx_extremes_kernel<1024>, g, 1024, 0, st, pts, ws, L, BL);
+    else if (items == 8) launch_next(bx_extremes_kernel<512>, g, 512, 0, st, pts, ws, L, BL);
+    else launch_next(bx_extremes_kernel<256>, g, 256, 0, st, pts, ws, L, BL);
+    launch_next(bx_octagon_kernel, (unsigned)ceil_div(BL.num_sets, 8), 256, 0, st, pts, ws, L, BL);
     note_kernels(CH_K_EXTREMES, 2);
     probe_after(CH_K_EXTREMES, st);
     return cudaGetLastError();
@@ -1034,7 +1039,7 @@ cudaError_t launch_extremes(const float *pts, int64_t n, void *ws, const Layout 
             probe_before(CH_K_EXTREMES, st);
             spec_sample_kernel<<<kSampleBlocks, kSampleThreads, 0, st>>>(pts, n, ws, L, (uint32_t)blocks,
                                                                          (uint32_t)cap);
-            extremes_kernel<true><<<(unsigned)blocks + extra, kExtThreads, 0, st>>>(pts, n, ws, L, ext8, 1, zero_ptr,
+            launch_next(extremes_kernel<true>, (unsigned)blocks + extra, kExtThreads, 0, st, pts, n, ws, L, ext8, 1, zero_ptr,
                                                                                    zero_words, (uint32_t)cap, learn,
                                                                                    learn_dirs, learn_k);
             note_kernels(CH_K_EXTREMES, 2);

@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
                                                               float2 *__restrict__ surv_pts,
                                                               uint32_t *__restrict__ surv_count)
 {
+    kernel_entry();
     __shared__ OctSmem so;
     __shared__ uint32_t s_off[kFiltItems / G][NW];
     __shared__ uint32_t s_tile;
@@ -536,6 +537,7 @@ __global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const flo
                                                                     void *ws, Layout L,
                                                                     const int32_t *kdev)
 {
+    kernel_entry();
     __shared__ OctSmem so;
     __shared__ uint32_t s_cnt[kCountRing];
     __shared__ uint32_t s_w[NW];
@@ -605,6 +607,7 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
                                                                       float2 *__restrict__ surv_pts,
                                                                       uint32_t *surv_count, int allow_spec)
 {
+    kernel_entry();
     __shared__ uint32_t s_abort;
     __shared__ uint32_t s_red[2][NW];
     __shared__ uint32_t s_list[kFiltThreads];    // non-empty tiles of a chunk: offset in chunk
@@ -730,6 +733,7 @@ __device__ __forceinline__ void bx_octagon_to_smem(OctSmem &so, int64_t &cur, in
 __global__ void __launch_bounds__(kFiltThreads, 4) bx_filter_count_kernel(const float *__restrict__ pts, void *ws,
                                                                        Layout L, BatchLayout BL)
 {
+    kernel_entry();
     __shared__ OctSmem so;
     __shared__ uint32_t s_cnt[kCountRing];
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -791,6 +795,7 @@ __global__ void __launch_bounds__(kFiltThreads, 4) bx_filter_count_kernel(const 
 // super-chunks (4096 survivors, also the sort tiles) and merge-tree nodes.
 __global__ void __launch_bounds__(1024) bx_filter_scan_kernel(void *ws, Layout L, BatchLayout BL)
 {
+    kernel_entry();
     __shared__ uint64_t s_w[32];
     __shared__ uint64_t s_w2[32];
     __shared__ uint64_t s_total;
@@ -887,6 +892,7 @@ __global__ void __launch_bounds__(1024) bx_filter_scan_kernel(void *ws, Layout L
 __global__ void __launch_bounds__(kFiltThreads, 3) bx_filter_scatter_kernel(const float *__restrict__ pts, void *ws,
                                                                             Layout L, BatchLayout BL)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -925,8 +931,7 @@ cudaError_t launch_single(const float *pts, int64_t n, void *ws, const Layout &L
     static int per_sm = occupancy(filter_kernel<G, KEYS, !KEYS>, kFiltThreads);
     const int64_t ntiles = ceil_div(n, kFiltTile);
     int64_t blocks = std::min<int64_t>((int64_t)sm_count() * per_sm, ntiles);
-    filter_kernel<G, KEYS, !KEYS><<<(unsigned)std::max<int64_t>(blocks, 1), kFiltThreads, 0, st>>>(
-        pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count);
+    launch_next(filter_kernel<G, KEYS, !KEYS>, (unsigned)std::max<int64_t>(blocks, 1), kFiltThreads, 0, st, pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count);
     note_kernels(CH_K_FILTER, 1);
     return cudaGetLastError();
 }
@@ -951,9 +956,8 @@ cudaError_t launch_two_pass(const float *pts, int64_t n, void *ws, const Layout 
     // the count pass's resident blocks (the scatter pass's warps take
     // tiles on their own, so a second partial wave of it costs little)
     const int64_t bc = count_blocks<G, BOX>(n);
-    filter_count_kernel<G, BOX><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, nullptr);
-    filter_scatter_kernel<G, false><<<(unsigned)bc, kFiltThreads, 0, st>>>(
-        pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count, BOX ? 0 : 1);
+    launch_next(filter_count_kernel<G, BOX>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, nullptr);
+    launch_next(filter_scatter_kernel<G, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count, BOX ? 0 : 1);
     note_kernels(CH_K_FILTER, 2);
     return cudaGetLastError();
 }
@@ -1005,8 +1009,8 @@ cudaError_t launch_filter_count(const float *pts, int64_t n, const int32_t *kdev
     const int64_t bc = vec ? count_blocks<2, false>(n) : count_blocks<1, false>(n);
     *grid = bc;
     probe_before(CH_K_FILTER, st);
-    if (vec) filter_count_kernel<2, false><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, kdev);
-    else filter_count_kernel<1, false><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L, kdev);
+    if (vec) launch_next(filter_count_kernel<2, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, kdev);
+    else launch_next(filter_count_kernel<1, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, kdev);
     note_kernels(CH_K_FILTER, 1);
     probe_after(CH_K_FILTER, st);
     return cudaGetLastError();
@@ -1020,11 +1024,11 @@ cudaError_t launch_filter_scatter(const float *pts, int64_t n, int64_t grid, voi
     float2 *sp = reinterpret_cast<float2 *>(surv_pts);
     const unsigned g = (unsigned)std::max<int64_t>(1, grid);
     if (keys_mode) {
-        if (vec) filter_scatter_kernel<2, true><<<g, kFiltThreads, 0, st>>>(pts, n, ws, L, nullptr, nullptr, nullptr, 0);
-        else filter_scatter_kernel<1, true><<<g, kFiltThreads, 0, st>>>(pts, n, ws, L, nullptr, nullptr, nullptr, 0);
+        if (vec) launch_next(filter_scatter_kernel<2, true>, g, kFiltThreads, 0, st, pts, n, ws, L, nullptr, nullptr, nullptr, 0);
+        else launch_next(filter_scatter_kernel<1, true>, g, kFiltThreads, 0, st, pts, n, ws, L, nullptr, nullptr, nullptr, 0);
     } else {
-        if (vec) filter_scatter_kernel<2, false><<<g, kFiltThreads, 0, st>>>(pts, n, ws, L, surv_idx, sp, surv_count, 0);
-        else filter_scatter_kernel<1, false><<<g, kFiltThreads, 0, st>>>(pts, n, ws, L, surv_idx, sp, surv_count, 0);
+        if (vec) launch_next(filter_scatter_kernel<2, false>, g, kFiltThreads, 0, st, pts, n, ws, L, surv_idx, sp, surv_count, 0);
+        else launch_next(filter_scatter_kernel<1, false>, g, kFiltThreads, 0, st, pts, n, ws, L, surv_idx, sp, surv_count, 0);
     }
     note_kernels(CH_K_FILTER, 1);
     return cudaGetLastError();
@@ -1038,15 +1042,15 @@ cudaError_t launch_bx_filter(const float *pts, void *ws, const Layout &L, const 
     const int64_t bc = std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * (tuned ? tuned : per_sm_c), BL.tiles_max));
     const int64_t bs = std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * (tuned ? tuned : per_sm_s), BL.tiles_max));
     probe_before(CH_K_FILTER, st);
-    bx_filter_count_kernel<<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, ws, L, BL);
+    launch_next(bx_filter_count_kernel, (unsigned)bc, kFiltThreads, 0, st, pts, ws, L, BL);
     // the hull step's fan for the sets with many octagon survivors, timed
     // as its own group between the count pass and the scan
     probe_after(CH_K_FILTER, st);
     const cudaError_t e = launch_bx_fan(pts, ws, L, BL, st);
     if (e != cudaSuccess) return e;
     probe_before(CH_K_FILTER, st);
-    bx_filter_scan_kernel<<<1, 1024, 0, st>>>(ws, L, BL);
-    bx_filter_scatter_kernel<<<(unsigned)bs, kFiltThreads, 0, st>>>(pts, ws, L, BL);
+    launch_next(bx_filter_scan_kernel, 1, 1024, 0, st, ws, L, BL);
+    launch_next(bx_filter_scatter_kernel, (unsigned)bs, kFiltThreads, 0, st, pts, ws, L, BL);
     note_kernels(CH_K_FILTER, 3);
     probe_after(CH_K_FILTER, st);
     return cudaGetLastError();

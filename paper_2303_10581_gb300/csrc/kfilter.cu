@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(XT) kx_extremes_kernel(const float *__restrict
                                                          const float *__restrict__ dirs, uint32_t *ext_out, void *ws,
                                                          Layout L, unsigned long long *zero_ptr, int64_t zero_words)
 {
+    kernel_entry();
     static_assert(K >= 8 && K <= kMaxDirs && XT % K == 0, "directions split the block evenly");
     constexpr int PARTS = XT / K;
     __shared__ float2 s_p[XTILE];
@@ -297,6 +298,7 @@ template <int G>
 __global__ void __launch_bounds__(kFiltThreads) kx_count_kernel(const float *__restrict__ pts, int64_t n, void *ws,
                                                                Layout L)
 {
+    kernel_entry();
     constexpr int ROWS = kFiltItems / G;
     __shared__ KPoly sp;
     __shared__ uint32_t s_w[kFiltThreads / 32];
@@ -520,6 +522,7 @@ __global__ void __launch_bounds__(ST) kx_sv_extremes_kernel(const float *__restr
                                                             const float *__restrict__ dirs, const int32_t *kdev,
                                                             uint32_t *ext_out, void *ws, Layout L)
 {
+    kernel_entry();
     __shared__ SvSmem sm;
     if constexpr (KT == 0) {
         const int K = *kdev;   // uniform
@@ -538,6 +541,7 @@ template <int G>
 __global__ void __launch_bounds__(ST) kx_sv_refine_kernel(const float *__restrict__ pts, int64_t n,
                                                           const int32_t *kdev, int K, void *ws, Layout L, int32_t bc)
 {
+    kernel_entry();
     __shared__ KPoly sp;
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const int Kr = kdev ? *kdev : K;
@@ -584,11 +588,11 @@ cudaError_t launch_kx_sv_stage(const float *pts, int64_t n, const float *dirs, c
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)sm_count() * (kdev ? 1 : 4)));
     const unsigned g = (unsigned)grid;
     probe_before(CH_K_KGON, st);
-    if (kdev) kx_sv_extremes_kernel<0, G><<<g, ST, 0, st>>>(pts, n, dirs, kdev, ext_out, ws, L);
-    else if (K == 16) kx_sv_extremes_kernel<16, G><<<g, ST, 0, st>>>(pts, n, dirs, kdev, ext_out, ws, L);
-    else if (K == 32) kx_sv_extremes_kernel<32, G><<<g, ST, 0, st>>>(pts, n, dirs, kdev, ext_out, ws, L);
-    else kx_sv_extremes_kernel<64, G><<<g, ST, 0, st>>>(pts, n, dirs, kdev, ext_out, ws, L);
-    kx_sv_refine_kernel<G><<<g, ST, 0, st>>>(pts, n, kdev, K, ws, L, (int32_t)bc);
+    if (kdev) launch_next(kx_sv_extremes_kernel<0, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
+    else if (K == 16) launch_next(kx_sv_extremes_kernel<16, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
+    else if (K == 32) launch_next(kx_sv_extremes_kernel<32, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
+    else launch_next(kx_sv_extremes_kernel<64, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
+    launch_next(kx_sv_refine_kernel<G>, g, ST, 0, st, pts, n, kdev, K, ws, L, (int32_t)bc);
     note_kernels(CH_K_KGON, 2);
     probe_after(CH_K_KGON, st);
     return cudaGetLastError();
@@ -644,8 +648,8 @@ cudaError_t launch_kx_count(const float *pts, int64_t n, int K, void *ws, const 
         1, std::min<int64_t>({ntiles, (int64_t)sm_count() * (vec ? per_sm2 : per_sm1), (int64_t)kFiltMaxBlocks}));
     *grid = bc;
     probe_before(CH_K_FILTER, st);
-    if (vec) kx_count_kernel<2><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L);
-    else kx_count_kernel<1><<<(unsigned)bc, kFiltThreads, 0, st>>>(pts, n, ws, L);
+    if (vec) launch_next(kx_count_kernel<2>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L);
+    else launch_next(kx_count_kernel<1>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L);
     note_kernels(CH_K_FILTER, 1);
     probe_after(CH_K_FILTER, st);
     return cudaGetLastError();

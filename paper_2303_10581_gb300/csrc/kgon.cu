@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *
                                                                    Layout L, uint32_t stride, int use_bits,
                                                                    const int32_t *kdev)
 {
+    kernel_entry();
     __shared__ OctSmem so;
     const Octagon *oct = at<Octagon>(ws, L.oct);
     if (oct->abort || oct->spec || !oct->has_edges) return;
@@ -461,6 +462,7 @@ __device__ __forceinline__ bool make_vertices(VertexSmem &sm, const unsigned lon
 
 __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L)
 {
+    kernel_entry();
     __shared__ VertexSmem sm[VT / 32];
     const Octagon *oct = at<Octagon>(ws, L.oct);
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
@@ -475,6 +477,7 @@ __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict_
 
 __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layout L)
 {
+    kernel_entry();
     __shared__ int s_w[BT / 32];
     __shared__ int s_scan[BT / 32];
     const Octagon *oct = at<Octagon>(ws, L.oct);
@@ -646,6 +649,7 @@ template <int G>
 __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restrict__ pts, uint32_t n, void *ws, Layout L,
                                                             int has_fan, int use_bits, const int32_t *kdev)
 {
+    kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ OctSmem so;
     __shared__ uint32_t s_oct;
@@ -806,6 +810,7 @@ __device__ __forceinline__ float2 surv_point(const uint32_t *keys, const unsigne
 
 __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint32_t min_s)
 {
+    kernel_entry();
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const Kgon *g = at<Kgon>(ws, L.kgon);
     const uint32_t m = at<Ctrl>(ws, L.ctrl)->surv_count;
@@ -833,6 +838,7 @@ __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint3
 // at V[-1] and V[kFan2Bins], V[kFan2Bins + 1].
 __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
 {
+    kernel_entry();
     __shared__ int s_w[BT / 32];
     __shared__ int s_scan[BT / 32];
     Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
@@ -869,6 +875,7 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
 // 6.4 M first-level survivors of 10^8 circle points).
 __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
 {
+    kernel_entry();
     Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
     if (!f2->on) return;
     const uint32_t m = f2->count_in;
@@ -951,25 +958,25 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
         const int64_t stride = fan_sample_stride(ntiles);
         const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride) * (kFiltItems / BI), (int64_t)sms * 5);
         probe_before(CH_K_KGON, st);
-        fan_bins_kernel<G><<<(unsigned)bb, kFiltThreads, 0, st>>>(pts, (uint32_t)n, ws, L, (uint32_t)stride, use_bits, kdev);
-        fan_vertex_kernel<<<kFanBins / (VB * VT / 32), VT, 0, st>>>(pts, n, ws, L);
-        fan_build_kernel<<<kFanBins / BT, BT, 0, st>>>(n, ws, L);
+        launch_next(fan_bins_kernel<G>, (unsigned)bb, kFiltThreads, 0, st, pts, (uint32_t)n, ws, L, (uint32_t)stride, use_bits, kdev);
+        launch_next(fan_vertex_kernel, kFanBins / (VB * VT / 32), VT, 0, st, pts, n, ws, L);
+        launch_next(fan_build_kernel, kFanBins / BT, BT, 0, st, n, ws, L);
         note_kernels(CH_K_KGON, 3);
         probe_after(CH_K_KGON, st);
     }
     probe_before(CH_K_FILTER, st);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(ntiles, (int64_t)CG), sms));
-    hull_filter_kernel<G><<<(unsigned)grid, CT, kQueueSmem + (has_fan ? kFanTable : 0), st>>>(pts, (uint32_t)n, ws, L, has_fan, use_bits, kdev);
+    launch_next(hull_filter_kernel<G>, (unsigned)grid, CT, kQueueSmem + (has_fan ? kFanTable : 0), st, pts, (uint32_t)n, ws, L, has_fan, use_bits, kdev);
     note_kernels(CH_K_FILTER, 1);
     probe_after(CH_K_FILTER, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || L.fan2_bins == 0) return e;   // (a set too small for the second level)
     probe_before(CH_K_KGON, st);
     const int lg = tune_value(CH_TUNE_FAN2_MIN_LOG2);
-    fan2_max_kernel<<<sms * 8, F2T, 0, st>>>(ws, L, lg ? (uint32_t)(1ull << lg) : kFan2MinS);
-    fan2_build_kernel<<<kFan2Bins / BT, BT, 0, st>>>(ws, L);
+    launch_next(fan2_max_kernel, sms * 8, F2T, 0, st, ws, L, lg ? (uint32_t)(1ull << lg) : kFan2MinS);
+    launch_next(fan2_build_kernel, kFan2Bins / BT, BT, 0, st, ws, L);
     const int64_t tb = std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, (int64_t)F2T * F2I), (int64_t)sms * 8));
-    fan2_test_kernel<<<(unsigned)tb, F2T, 0, st>>>(ws, L);
+    launch_next(fan2_test_kernel, (unsigned)tb, F2T, 0, st, ws, L);
     note_kernels(CH_K_KGON, 3);
     probe_after(CH_K_KGON, st);
     return cudaGetLastError();
@@ -1054,6 +1061,7 @@ constexpr int kBxBinStride = 2;   // built-in: the bins see every 2nd tile of a 
 // work items (runs of up to kBxFanChunk tiles of one such set).
 __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, Layout L, BatchLayout BL, uint32_t chunk)
 {
+    kernel_entry();
     __shared__ uint32_t s_w[2][32];
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -1124,6 +1132,7 @@ __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, Layout L,
 __global__ void __launch_bounds__(FT) bx_fan_bins_kernel(const float *__restrict__ pts, void *ws, Layout L,
                                                          BatchLayout BL, uint32_t chunk, uint32_t stride)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
     const Octagon *octs = at<Octagon>(ws, BL.octs);
@@ -1175,6 +1184,7 @@ static_assert(kFanBins % BT == 0, "bins split evenly over the threads");
 __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restrict__ pts, void *ws, Layout L,
                                                           BatchLayout BL)
 {
+    kernel_entry();
     __shared__ int s_w[BT / 32];
     __shared__ int s_ok;
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -1259,6 +1269,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
 __global__ void __launch_bounds__(CT, 1) bx_fan_refine_kernel(const float *__restrict__ pts, void *ws, Layout L,
                                                               BatchLayout BL, uint32_t chunk)
 {
+    kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *sv = reinterpret_cast<float2 *>(smem_raw);   // kFanBins vertices
     __shared__ uint32_t s_item;
@@ -1341,10 +1352,10 @@ cudaError_t launch_bx_fan(const float *pts, void *ws, const Layout &L, const Bat
     const uint32_t stride = tune_value(CH_TUNE_BX_FAN_STRIDE) ? (uint32_t)tune_value(CH_TUNE_BX_FAN_STRIDE)
                                                               : kBxBinStride;
     probe_before(CH_K_KGON, st);
-    bx_fan_select_kernel<<<1, 1024, 0, st>>>(ws, L, BL, chunk);
-    bx_fan_bins_kernel<<<(unsigned)(sms * 4), FT, 0, st>>>(pts, ws, L, BL, chunk, stride);
-    bx_fan_build_kernel<<<(unsigned)(sms * 2), BT, 0, st>>>(pts, ws, L, BL);
-    bx_fan_refine_kernel<<<(unsigned)sms, CT, kFanSmem, st>>>(pts, ws, L, BL, chunk);
+    launch_next(bx_fan_select_kernel, 1, 1024, 0, st, ws, L, BL, chunk);
+    launch_next(bx_fan_bins_kernel, (unsigned)(sms * 4), FT, 0, st, pts, ws, L, BL, chunk, stride);
+    launch_next(bx_fan_build_kernel, (unsigned)(sms * 2), BT, 0, st, pts, ws, L, BL);
+    launch_next(bx_fan_refine_kernel, (unsigned)sms, CT, kFanSmem, st, pts, ws, L, BL, chunk);
     note_kernels(CH_K_KGON, 4);
     probe_after(CH_K_KGON, st);
     return cudaGetLastError();

@@ -5,11 +5,32 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include <utility>
+
 #include "common.cuh"
 
 namespace ch {
 
 int sm_count();
+
+// Launches a kernel that may be put on the SMs before the kernel before it in
+// the stream has been retired (kernel_entry waits for it).  The first kernel of
+// a call is launched the ordinary way.
+template <class... P, class... A>
+inline void launch_next(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);   // (errors: cudaGetLastError)
+}
 
 // instrumentation around every launch (probe.cu)
 void probe_before(int kid, cudaStream_t st);

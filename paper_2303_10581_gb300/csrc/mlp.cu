@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
                                                     float *__restrict__ H1, float *__restrict__ H2,
                                                     float *__restrict__ OUT, LossArgs A)
 {
+    kernel_entry();
     __shared__ float s_h1[kHid], s_h2[kHid], s_o[kOut], s_d[kOut], s_dh2[kHid], s_part[MT / kHid][kHid];
     const int b = blockIdx.x, t = (int)threadIdx.x, lane = t & 31, warp = t >> 5;
     const float *x = X + (int64_t)b * kIn;
@@ -303,6 +304,7 @@ __global__ void __launch_bounds__(256) wgrad_adam_kernel(const float *__restrict
                                                          const float *__restrict__ dH2, const float *__restrict__ dOUT,
                                                          AdamArgs A)
 {
+    kernel_entry();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= kParams) return;
     // the parameter's factors: column d of the layer's output gradient, and
@@ -421,7 +423,7 @@ extern "C" ch_status ch_mlp_train_step(const float *X, int32_t B, const int32_t 
     else sample_kernel<false, true><<<B, MT, 0, st>>>(X, B, P, H1, H2, nullptr, A);
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
-    wgrad_adam_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(X, B, H1, H2, dH1, dH2, dOUT,
+    launch_next(wgrad_adam_kernel, (kParams + 255) / 256, 256, 0, st, X, B, H1, H2, dH1, dH2, dOUT,
                                                             AdamArgs{master, adam_m, adam_v, P, lr, b1, b2, 1e-8f, c1, c2});
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ERR_CUDA;
 }

@@ -73,6 +73,7 @@ __device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t &exc
 
 __global__ void __launch_bounds__(256) sort_hist_kernel(void *ws, Layout L)
 {
+    kernel_entry();
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
@@ -290,6 +291,7 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
 
 __global__ void __launch_bounds__(kSortThreads, 3) sort_pass_kernel(void *ws, Layout L, int p)
 {
+    kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
@@ -349,6 +351,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) sort_pass_kernel(void *ws, La
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) bx_sort_hist_kernel(void *ws, Layout L, BatchLayout BL)
 {
+    kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -385,6 +388,7 @@ __global__ void __launch_bounds__(256) bx_sort_hist_kernel(void *ws, Layout L, B
 
 __global__ void __launch_bounds__(kSortThreads, 3) bx_sort_pass_kernel(void *ws, Layout L, BatchLayout BL, int p)
 {
+    kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -455,7 +459,7 @@ cudaError_t launch_bx_sort(void *ws, const Layout &L, const BatchLayout &BL, cud
     const int64_t cap = BL.tiles_max;
     const int64_t hb = std::max<int64_t>(1, std::min<int64_t>(cap, (int64_t)sm_count() * 4));
     probe_before(CH_K_SORT_HIST, st);
-    bx_sort_hist_kernel<<<(unsigned)hb, 256, 0, st>>>(ws, L, BL);
+    launch_next(bx_sort_hist_kernel, (unsigned)hb, 256, 0, st, ws, L, BL);
     note_kernels(CH_K_SORT_HIST, 1);
     probe_after(CH_K_SORT_HIST, st);
     cudaError_t e = cudaGetLastError();
@@ -465,7 +469,7 @@ cudaError_t launch_bx_sort(void *ws, const Layout &L, const BatchLayout &BL, cud
         1, std::min<int64_t>(cap, (int64_t)sm_count() * (tuned ? tuned : bx_pass_blocks_per_sm())));
     for (int p = 0; p < kSortPasses; ++p) {
         probe_before(CH_K_SORT_PASS, st);
-        bx_sort_pass_kernel<<<(unsigned)pb, kSortThreads, sizeof(SortSmem), st>>>(ws, L, BL, p);
+        launch_next(bx_sort_pass_kernel, (unsigned)pb, kSortThreads, sizeof(SortSmem), st, ws, L, BL, p);
         note_kernels(CH_K_SORT_PASS, 1);
         probe_after(CH_K_SORT_PASS, st);
         e = cudaGetLastError();
@@ -481,7 +485,7 @@ cudaError_t launch_sort(void *ws, const Layout &L, cudaStream_t st)
     if (hb > cap) hb = cap;
     if (hb < 1) hb = 1;
     probe_before(CH_K_SORT_HIST, st);
-    sort_hist_kernel<<<(unsigned)hb, 256, 0, st>>>(ws, L);
+    launch_next(sort_hist_kernel, (unsigned)hb, 256, 0, st, ws, L);
     note_kernels(CH_K_SORT_HIST, 1);
     probe_after(CH_K_SORT_HIST, st);
     cudaError_t e = cudaGetLastError();
@@ -491,7 +495,7 @@ cudaError_t launch_sort(void *ws, const Layout &L, cudaStream_t st)
     if (pb < 1) pb = 1;
     for (int p = 0; p < kSortPasses; ++p) {
         probe_before(CH_K_SORT_PASS, st);
-        sort_pass_kernel<<<(unsigned)pb, kSortThreads, sizeof(SortSmem), st>>>(ws, L, p);
+        launch_next(sort_pass_kernel, (unsigned)pb, kSortThreads, sizeof(SortSmem), st, ws, L, p);
         note_kernels(CH_K_SORT_PASS, 1);
         probe_after(CH_K_SORT_PASS, st);
         e = cudaGetLastError();
