@@ -217,11 +217,12 @@ ch_status ch_hull_learned(const float *pts, int64_t n, const void *params, float
  * workload and caches the best in JSON. */
 typedef enum {
     CH_TUNE_BX_EXTREMES = 0,    /* extremes sweep, blocks per SM 1..64 (default 8)          */
-    CH_TUNE_BX_FILTER = 1,      /* filter count and scatter, blocks per SM (default: occupancy) */
+    CH_TUNE_BX_FILTER = 1,      /* filter of the sets without a fan, blocks per SM (default 3) */
     CH_TUNE_BX_SORT_PASS = 2,   /* radix-sort passes, blocks per SM (default: occupancy)     */
     CH_TUNE_BX_EMIT = 3,        /* chain compaction, blocks per SM (default 4)              */
-    CH_TUNE_BX_FAN_STRIDE = 4,  /* the fan's bins sample every k-th tile of a set, 1..64 (default 2) */
-    CH_TUNE_BX_FAN_CHUNK = 5,   /* tiles per work item of the fan refine: 8, 16, 32 or 64 (default 64) */
+    CH_TUNE_BX_FAN_STRIDE = 4,  /* the fan's bins sample every k-th tile of a set, 1..64 (default: by
+                                   the set's size and shape, 1 to 8) */
+    CH_TUNE_BX_FAN_CHUNK = 5,   /* tiles per work item of the fan sets' filter: 8, 16, 32 or 64 (default 32) */
     CH_TUNE_BX_EXT_ITEMS = 6,   /* points per thread per 4096-point tile of the extremes sweep:
                                    4, 8 or 16, i.e. blocks of 1024, 512 or 256 threads (default 16) */
     CH_TUNE_FAN2_MIN_LOG2 = 7,  /* single-set hull step: the fan's second level runs when the first
@@ -308,9 +309,8 @@ typedef enum {
     CH_K_CHAIN = 5,      /* Sec. 3.3 chunk chains + tree merges                 */
     CH_K_EMIT = 6,       /* compaction of the chain ranges                      */
     CH_K_FINISH = 7,     /* hull assembly                                       */
-    CH_K_KGON = 8,       /* hull step: fan test of the octagon survivors
-                            (runs between FILTER's count and scatter passes;
-                            its second level after the scatter) */
+    CH_K_KGON = 8,       /* hull step: the fan's vertices (the test itself is
+                            FILTER's); its second level after the filter */
     CH_K_COUNT = 9
 } ch_kernel_id;
 
@@ -319,12 +319,11 @@ typedef enum {
  * launch stream, for at most max_launches groups per id.  A group is the
  * kernels one step launches back to back under that id: one for
  * EXTREMES, OCTAGON, SORT_HIST, SORT_PASS (one per pass), EMIT (the chain
- * ranges' output offsets), FINISH (their copy); two for FILTER with the two-pass schedule (count,
- * scatter; in ch_hull each is its own group, KGON runs between them), one
- * with the single pass; two for CHAIN (chains, tree merge); for KGON three
- * (fan vertices, estimate, refine of the keep decisions; the count pass
- * gathers the bins) and four for its second level (sub-bin maxima,
- * vertices, test, compaction).  Kernel-launch
+ * ranges' output offsets), FINISH (their copy); two for FILTER with the
+ * two-pass schedule (count, scatter), one with the single pass and in
+ * ch_hull (octagon and fan test in one pass); two for CHAIN (chains, tree
+ * merge); for KGON three (the fan's bins, vertices, proofs; before FILTER)
+ * and three for its second level (sub-bin maxima, vertices, test).  Kernel-launch
  * counting for all ids restarts at zero.  Host-only bookkeeping; creates
  * the events.  Process-wide: one probe at a time, driven from one host
  * thread (see "Host threads" above). */

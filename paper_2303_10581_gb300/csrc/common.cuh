@@ -278,13 +278,25 @@ struct BatchCtrl {
     uint32_t filt_ticket, emit_ticket, pad0;
     uint32_t sort_ticket[kSortPasses];
     uint32_t h_lower, h_upper;
-    uint32_t nfan;        // sets that get the fan test (kgon.cu)
-    uint32_t nitems;      // the fan refine's work items (a set's run of up to kBxFanChunk tiles)
-    uint32_t fan_ticket;  // next work item of the fan refine
-    uint32_t pad;
+    uint32_t nfan;        // sets that get a fan (kgon.cu)
+    uint32_t nfan_items, nplain_items, nbin_items;   // work items
+    uint32_t fan_ticket, plain_ticket;               // next work item of the filter passes
 };
-constexpr int kBxFanChunk = 64;       // tiles per work item of the batched fan refine (built-in)
-constexpr int kBxFanChunkMin = 8;     // the smallest tunable one (sizes the work-item list)
+constexpr int kBxFanChunk = 32;       // tiles per work item of the fan sets' filter pass (built-in)
+constexpr int kBxFanChunkMin = 8;     // the smallest tunable one (sizes the work-item lists)
+constexpr int kBxTileBins = 1024;     // a set has up to this many bins per tile of 4096 points (kFanBins at most)
+constexpr int kBxBinRun = 512;        // bins per block of the vertex kernel
+
+// The fan of a set of ch_hull_batched.
+struct FanInfo {
+    uint32_t want;        // enough octagon survivors (an estimate) for a fan
+    uint32_t tight;       // the points' distances from the centre differ by rounding only (a circle)
+    uint32_t nb;          // bins
+    uint32_t bad;         // no usable vertices
+    uint32_t ready;       // the fan's proofs hold and it drops enough points
+    float rho2;           // lower bound on the squared distance from the centre to the fan's boundary
+    uint32_t pad[2];
+};
 
 // Extra workspace of ch_hull_batched, after the single-set regions.
 struct BatchLayout {
@@ -301,16 +313,17 @@ struct BatchLayout {
     size_t sc_off[2];     // u32[tiles_max + 1]: lower / upper chain offset of each super-chunk
     size_t lower;         // keys[1] again: free for the stages after the sort, which ends in buffer 0
     // the fan of the hull step, per set with many octagon survivors (kgon.cu)
-    size_t soct;          // u32[B]: octagon survivors per set (in the zeroed range)
-    size_t fan_id;        // i32[B]: the set's fan number, -1: none
-    size_t fan_set;       // u32[max_fan]: set of each fan
-    size_t fan_ok;        // u32[max_fan]: the fan has vertices and its centre is inside
-    size_t fan_c;         // float2[max_fan]: centre
-    size_t fan_slot;      // u64[max_fan * kFanBins]: farthest sampled point per bin (left zeroed)
-    size_t fan_v;         // float2[max_fan * kFanBins]: vertices
-    size_t fan_items;     // uint2[max_items]: (fan, first tile) of each refine work item
+    size_t soct;          // u32[B]: survivors per set (in the zeroed range)
+    size_t fan;           // FanInfo[B]
+    size_t fan_set;       // u32[B]: the sets with a fan
+    size_t fan_slot;      // u64[tiles_max * kBxTileBins]: farthest sampled point per bin, a set's bins from its
+                          // first tile's; later its vertices
+    size_t fan_raw;       // float2[tiles_max * kBxTileBins]: the vertices before empty bins are filled
+    size_t fan_items;     // uint2[max_items]: (set, first tile in the set) of each work item of the fan sets
+    size_t plain_items;   // uint2[max_items]: the same of the other sets
+    size_t bin_items;     // uint2[max_bin_items]: (set, first bin) of each run of kBxBinRun bins
     size_t total;
-    int64_t num_sets, tiles_max, max_fan, max_items;
+    int64_t num_sets, tiles_max, max_items, max_bin_items;
 };
 
 __host__ __device__ inline Layout make_layout(int64_t n, int64_t sets = 0)
@@ -403,16 +416,15 @@ __host__ __device__ inline BatchLayout make_batch_layout(const Layout &L, int64_
     B.sc_off[0] = take((size_t)(B.tiles_max + 1) * 4);
     B.sc_off[1] = take((size_t)(B.tiles_max + 1) * 4);
     B.lower = L.keys[1];
-    // a set with a fan has at least 2^16 points
-    B.max_fan = sets < L.n / 65536 + 1 ? sets : L.n / 65536 + 1;
-    B.max_items = B.tiles_max / kBxFanChunkMin + B.max_fan + 1;
-    B.fan_id = take((size_t)sets * 4);
-    B.fan_set = take((size_t)B.max_fan * 4);
-    B.fan_ok = take((size_t)B.max_fan * 4);
-    B.fan_c = take((size_t)B.max_fan * 8);
-    B.fan_slot = take((size_t)B.max_fan * kFanBins * 8);
-    B.fan_v = take((size_t)B.max_fan * kFanBins * 8);
+    B.max_items = B.tiles_max / kBxFanChunkMin + sets + 1;
+    B.max_bin_items = B.tiles_max * (kBxTileBins / kBxBinRun) + 1;
+    B.fan = take((size_t)sets * sizeof(FanInfo));
+    B.fan_set = take((size_t)sets * 4);
+    B.fan_slot = take((size_t)B.tiles_max * kBxTileBins * 8);
+    B.fan_raw = take((size_t)B.tiles_max * kBxTileBins * 8);
     B.fan_items = take((size_t)B.max_items * 8);
+    B.plain_items = take((size_t)B.max_items * 8);
+    B.bin_items = take((size_t)B.max_bin_items * 8);
     B.total = o;
     return B;
 }

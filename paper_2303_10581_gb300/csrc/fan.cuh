@@ -17,6 +17,20 @@ __host__ __device__ inline int64_t fan_sample_stride(int64_t tiles)
     return s < 1 ? 1 : (s > 16 ? 16 : s);
 }
 
+// A fan's number of bins NB (a multiple of 4, below 2^22): known at compile
+// time, or a set's own.
+template <int NB>
+struct FixedBins {
+    static_assert(NB % 4 == 0 && NB < (1 << 22), "the shifted offsets are exact");
+    __device__ static constexpr float quarter() { return NB / 4.0f; }
+    __device__ static constexpr uint32_t count() { return NB; }
+};
+struct SetBins {
+    uint32_t n;
+    __device__ float quarter() const { return (float)(n / 4u); }
+    __device__ uint32_t count() const { return n; }
+};
+
 // Scaled pseudo-angle of the direction (dx, dy): in [0, NB], growing with
 // the angle counter-clockwise from -y; bin b holds [b, b + 1).  With t = dy /
 // (|dx| + |dy|) it is (1 + t) NB / 4 on the right and (3 - t) NB / 4 on the
@@ -28,43 +42,33 @@ __device__ __forceinline__ float fan_turn(float dx, float dy)   // t on the righ
     return __uint_as_float(__float_as_uint(__fmul_rn(dy, r)) ^ (__float_as_uint(dx) & 0x80000000u));
 }
 
-template <int NB = kFanBins>
-__device__ __forceinline__ float fan_phi(float dx, float dy)
+template <class Bins>
+__device__ __forceinline__ float fan_phi(Bins nb, float dx, float dy)
 {
     const bool left = (int)__float_as_uint(dx) < 0;
-    return __fmaf_rn(fan_turn(dx, dy), NB / 4.0f, left ? 3.0f * NB / 4.0f : NB / 4.0f);
+    return __fmaf_rn(fan_turn(dx, dy), nb.quarter(), left ? 3.0f * nb.quarter() : nb.quarter());
 }
 
 // kBinBias + its bin, the bin in [0, NB] (a NaN: kBinBias + NB): the same FMA
 // shifted by 2^23 and rounded down leaves the bin in the low mantissa bits.
 constexpr uint32_t kBinBias = 0x4b000000u;
-template <int NB = kFanBins>
-__device__ __forceinline__ uint32_t fan_bin_biased(float dx, float dy)
+template <class Bins>
+__device__ __forceinline__ uint32_t fan_bin_biased(Bins nb, float dx, float dy)
 {
-    static_assert(NB % 4 == 0 && NB < (1 << 22), "the shifted offsets are exact");
     const bool left = (int)__float_as_uint(dx) < 0;
-    const float f = __fmaf_rd(fan_turn(dx, dy), NB / 4.0f, left ? 0x1p23f + 3.0f * NB / 4.0f : 0x1p23f + NB / 4.0f);
-    return min(__float_as_uint(f), kBinBias + (uint32_t)NB);
-}
-template <int NB = kFanBins>
-__device__ __forceinline__ uint32_t fan_bin(float dx, float dy)
-{
-    return fan_bin_biased<NB>(dx, dy) - kBinBias;
+    const float f = __fmaf_rd(fan_turn(dx, dy), nb.quarter(),
+                              left ? 0x1p23f + 3.0f * nb.quarter() : 0x1p23f + nb.quarter());
+    return min(__float_as_uint(f), kBinBias + nb.count());
 }
 
-// The direction of pseudo-angle a / NB of the full turn (|x| + |y| = 1).
-template <int NB = kFanBins>
-__device__ __forceinline__ float2 fan_direction(float a)
+// The direction of pseudo-angle a (|x| + |y| = 1).
+template <class Bins>
+__device__ __forceinline__ float2 fan_direction(Bins nb, float a)
 {
-    const float q = a * (4.0f / NB);
+    const float q = a / nb.quarter();
     const float t = q < 2.0f ? q - 1.0f : 3.0f - q;
     return make_float2(q < 2.0f ? 1.0f - fabsf(t) : fabsf(t) - 1.0f, t);
 }
-
-template <int NB = kFanBins>
-__device__ __forceinline__ int next_bin(int b) { return b + 1 == NB ? 0 : b + 1; }
-template <int NB = kFanBins>
-__device__ __forceinline__ int prev_bin(int b) { return b == 0 ? NB - 1 : b - 1; }
 
 // a - b = s + e and a + b = s + e exactly (Knuth's two-sum, binary32
 // round to nearest; the intrinsics are never contracted into an FMA)

@@ -708,212 +708,6 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
     }
 }
 
-// ---------------------------------------------------------------------------
-// many sets (ch_hull_batched): the two passes over set-aligned 4096-point
-// tiles, with 8-byte loads (sets start anywhere); indices are set-local
-// ---------------------------------------------------------------------------
-// Thread t tests points lo + r * 256 + t of the set p2 (r < 16), below hi.
-__device__ __forceinline__ uint32_t bx_load_test(const float2 *__restrict__ p2, int64_t lo, int64_t hi,
-                                                 const OctSmem &so)
-{
-    // (the tile in 8-byte loads is load_test's with one point per row)
-    return load_test<1, false>(reinterpret_cast<const float *>(p2), hi, lo, so);
-}
-
-// Copies set b's polygon to shared memory when the block moves to a new set.
-__device__ __forceinline__ void bx_octagon_to_smem(OctSmem &so, int64_t &cur, int64_t b, const Octagon *octs)
-{
-    if (b == cur) return;   // block-uniform
-    __syncthreads();
-    fill_octagon(so, octs + b);
-    __syncthreads();
-    cur = b;
-}
-
-__global__ void __launch_bounds__(kFiltThreads, 4) bx_filter_count_kernel(const float *__restrict__ pts, void *ws,
-                                                                       Layout L, BatchLayout BL)
-{
-    kernel_entry();
-    __shared__ OctSmem so;
-    __shared__ uint32_t s_cnt[kCountRing];
-    const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    if (bc->abort) return;
-    for (int i = threadIdx.x; i < kCountRing; i += kFiltThreads) s_cnt[i] = 0u;   // (the first set's load syncs)
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const uint32_t *tile_set = at<uint32_t>(ws, BL.tile_set);
-    const Octagon *octs = at<Octagon>(ws, BL.octs);
-    unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    uint32_t *soct = at<uint32_t>(ws, BL.soct);
-    const uint32_t lane = lane_id();
-    // a contiguous range of tiles per block: the polygon is loaded once per
-    // set the range touches (a block-wide step; between two, the warps run
-    // free and add their tile counts up in s_cnt)
-    const int64_t T = bc->tiles;
-    const int64_t per = ceil_div(T, (int64_t)gridDim.x);
-    const int64_t t0 = (int64_t)blockIdx.x * per, t1 = min(T, t0 + per);
-    int64_t cur = -1;
-    for (int64_t w0 = t0; w0 < t1; w0 += kCountRing) {
-        const int64_t w1 = min(t1, w0 + kCountRing);
-        for (int64_t t = w0; t < w1; ++t) {
-            const int64_t b = tile_set[t];
-            bx_octagon_to_smem(so, cur, b, octs);
-            if (threadIdx.x == 0 && t + 1 < t1) {   // the next tile streams into L2 meanwhile
-                const int64_t nb = tile_set[t + 1];
-                const int64_t nlo = (t + 1 - sets[nb].tile_base) * (int64_t)kFiltTile;
-                const int64_t nhi = min(nlo + kFiltTile, sets[nb].n);
-                const float2 *np = reinterpret_cast<const float2 *>(pts) + sets[nb].pt_begin;
-                const uintptr_t a0 = (reinterpret_cast<uintptr_t>(np + nlo) + 15) & ~(uintptr_t)15;
-                const uintptr_t a1 = reinterpret_cast<uintptr_t>(np + nhi) & ~(uintptr_t)15;
-                if (a1 > a0) bulk_prefetch_l2(reinterpret_cast<const void *>(a0), (uint32_t)(a1 - a0));
-            }
-            uint32_t keep = 0;
-            if (!so.abort) {
-                const int64_t lo = (int64_t)(t - sets[b].tile_base) * kFiltTile;
-                const int64_t hi = min(lo + kFiltTile, sets[b].n);
-                keep = bx_load_test(reinterpret_cast<const float2 *>(pts) + sets[b].pt_begin, lo, hi, so);
-            }
-            bits[(size_t)t * kFiltThreads + threadIdx.x] = (uint16_t)keep;
-            uint32_t c = __popc(keep);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-            if (lane == 0 && c) atomicAdd(&s_cnt[t - w0], c);
-        }
-        __syncthreads();
-        for (int64_t i = threadIdx.x; i < w1 - w0; i += kFiltThreads) {
-            const uint32_t v = s_cnt[i];
-            status[w0 + i] = v;
-            s_cnt[i] = 0u;
-            if (v) atomicAdd(&soct[tile_set[w0 + i]], v);
-        }
-        __syncthreads();
-    }
-}
-
-// One block: tile offsets (exclusive scan of the counts), each set's
-// survivor range, and the layout of the later stages: each set's
-// super-chunks (4096 survivors, also the sort tiles) and merge-tree nodes.
-__global__ void __launch_bounds__(1024) bx_filter_scan_kernel(void *ws, Layout L, BatchLayout BL)
-{
-    kernel_entry();
-    __shared__ uint64_t s_w[32];
-    __shared__ uint64_t s_w2[32];
-    __shared__ uint64_t s_total;
-    BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    if (bc->abort) return;
-    SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    uint32_t *sc_set = at<uint32_t>(ws, BL.sc_set);
-    unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, nthr = blockDim.x;
-    // ---- 1. tiles
-    {
-        const int64_t T = bc->tiles;
-        const int64_t per = ceil_div(T, (int64_t)nthr);
-        const int64_t t0 = threadIdx.x * per, t1 = min(t0 + per, T);
-        uint64_t sum = 0;
-        for (int64_t t = t0; t < t1; ++t) sum += status[t] & 0xffffffffull;
-        uint64_t incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= (uint32_t)o) incl += u;
-        }
-        if (lane == 31) s_w[warp] = incl;
-        __syncthreads();
-        uint64_t before = 0, total = 0;
-        for (uint32_t w = 0; w < nthr / 32; ++w) {
-            if (w < warp) before += s_w[w];
-            total += s_w[w];
-        }
-        uint64_t run = before + incl - sum;
-        for (int64_t t = t0; t < t1; ++t) {
-            const uint64_t c = status[t] & 0xffffffffull;
-            status[t] = (run << 32) | c;
-            run += c;
-        }
-        if (threadIdx.x == 0) s_total = total;
-        __syncthreads();
-    }
-    // ---- 2. sets: survivors, super-chunks, tree nodes
-    const int64_t B = BL.num_sets;
-    const int64_t T = bc->tiles;
-    const uint64_t total = s_total;
-    auto off = [&](int64_t t) -> uint64_t { return t < T ? (status[t] >> 32) : total; };
-    const int64_t per = ceil_div(B, (int64_t)nthr);
-    const int64_t b0 = threadIdx.x * per, b1 = min(b0 + per, B);
-    uint64_t sc_sum = 0, nd_sum = 0;
-    for (int64_t b = b0; b < b1; ++b) {
-        const uint64_t sb = off(sets[b].tile_base);
-        const uint32_t s = (uint32_t)(off(sets[b].tile_base + sets[b].ntiles) - sb);
-        sets[b].surv_base = sb;
-        sets[b].s = s;
-        const int64_t nsc = ceil_div((int64_t)s, kChainC);
-        sets[b].nsc = (uint32_t)nsc;
-        sc_sum += nsc;
-        nd_sum += nsc > 0 ? tree_nodes(nsc) + 1 : 0;
-    }
-    uint64_t i1 = sc_sum, i2 = nd_sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t u1 = __shfl_up_sync(0xffffffffu, i1, o);
-        const uint64_t u2 = __shfl_up_sync(0xffffffffu, i2, o);
-        if (lane >= (uint32_t)o) {
-            i1 += u1;
-            i2 += u2;
-        }
-    }
-    __syncthreads();
-    if (lane == 31) {
-        s_w[warp] = i1;
-        s_w2[warp] = i2;
-    }
-    __syncthreads();
-    uint64_t bsc = 0, bnd = 0, tsc = 0;
-    for (uint32_t w = 0; w < nthr / 32; ++w) {
-        if (w < warp) {
-            bsc += s_w[w];
-            bnd += s_w2[w];
-        }
-        tsc += s_w[w];
-    }
-    uint64_t rsc = bsc + i1 - sc_sum, rnd = bnd + i2 - nd_sum;
-    for (int64_t b = b0; b < b1; ++b) {
-        sets[b].sc_base = (uint32_t)rsc;
-        sets[b].node_base = (uint32_t)rnd;
-        for (uint32_t k = 0; k < sets[b].nsc; ++k) sc_set[rsc + k] = (uint32_t)b;
-        rsc += sets[b].nsc;
-        rnd += sets[b].nsc > 0 ? tree_nodes(sets[b].nsc) + 1 : 0;
-    }
-    if (threadIdx.x == 0) bc->nsc = (uint32_t)tsc;
-}
-
-// One warp per tile with survivors (warps of the whole grid in turn); the
-// scan left each tile's output offset in the high half of filt_status.
-__global__ void __launch_bounds__(kFiltThreads, 3) bx_filter_scatter_kernel(const float *__restrict__ pts, void *ws,
-                                                                            Layout L, BatchLayout BL)
-{
-    kernel_entry();
-    const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    if (bc->abort) return;
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const uint32_t *tile_set = at<uint32_t>(ws, BL.tile_set);
-    const unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    const uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    uint32_t *out_keys = at<uint32_t>(ws, L.keys[0]);
-    unsigned long long *out_pay = at<unsigned long long>(ws, L.pay[0]);
-    const uint32_t T = bc->tiles;
-    const uint32_t nwarps = gridDim.x * NW;
-    for (uint32_t t = blockIdx.x * NW + (threadIdx.x >> 5); t < T; t += nwarps) {
-        const unsigned long long st = status[t];
-        if ((st & 0xffffffffull) == 0) continue;   // warp-uniform
-        const int64_t b = tile_set[t];
-        const int64_t lo = (int64_t)(t - sets[b].tile_base) * kFiltTile;
-        const float *p = pts + 2 * sets[b].pt_begin;
-        scatter_tile_warp<1, true>(p, sets[b].n, bits + (size_t)t * kFiltThreads, lo, (uint32_t)(st >> 32), nullptr,
-                                   nullptr, out_keys, out_pay);
-    }
-}
-
 template <class K>
 int occupancy(K kernel, int threads)
 {
@@ -1031,28 +825,6 @@ cudaError_t launch_filter_scatter(const float *pts, int64_t n, int64_t grid, voi
         else launch_next(filter_scatter_kernel<1, false>, g, kFiltThreads, 0, st, pts, n, ws, L, surv_idx, sp, surv_count, 0);
     }
     note_kernels(CH_K_FILTER, 1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_bx_filter(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st)
-{
-    static int per_sm_c = occupancy(bx_filter_count_kernel, kFiltThreads);
-    static int per_sm_s = occupancy(bx_filter_scatter_kernel, kFiltThreads);
-    const int tuned = tune_value(CH_TUNE_BX_FILTER);
-    const int64_t bc = std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * (tuned ? tuned : per_sm_c), BL.tiles_max));
-    const int64_t bs = std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * (tuned ? tuned : per_sm_s), BL.tiles_max));
-    probe_before(CH_K_FILTER, st);
-    launch_next(bx_filter_count_kernel, (unsigned)bc, kFiltThreads, 0, st, pts, ws, L, BL);
-    // the hull step's fan for the sets with many octagon survivors, timed
-    // as its own group between the count pass and the scan
-    probe_after(CH_K_FILTER, st);
-    const cudaError_t e = launch_bx_fan(pts, ws, L, BL, st);
-    if (e != cudaSuccess) return e;
-    probe_before(CH_K_FILTER, st);
-    launch_next(bx_filter_scan_kernel, 1, 1024, 0, st, ws, L, BL);
-    launch_next(bx_filter_scatter_kernel, (unsigned)bs, kFiltThreads, 0, st, pts, ws, L, BL);
-    note_kernels(CH_K_FILTER, 3);
-    probe_after(CH_K_FILTER, st);
     return cudaGetLastError();
 }
 

@@ -67,12 +67,15 @@ constexpr int CT = 768;                  // threads per block of the filter pass
 constexpr int CG = CT / kFiltThreads;    // groups of kFiltThreads, each with its own tiles
 constexpr uint32_t kKgonMinS = 1u << 16; // fewer octagon survivors: not worth a pass
 constexpr int kFanTable = (kFanBins + 4) * 8;  // vertices, the last again before them and the first two after them (and padding)
-constexpr int kQueue = 96;                     // points a warp of the filter pass queues
+constexpr int kQueue = 64;                     // points a warp of the filter pass queues (under 32, and 32 more)
+constexpr uint32_t kMany = 128;                // a warp's survivors of a tile that go straight to the list
 constexpr int kQueueSmem = CT / 32 * kQueue * 4;
+using Level1 = FixedBins<kFanBins>;
+using Level2 = FixedBins<kFan2Bins>;
 constexpr float kFanMargin = 1.0f / 32.0f;     // of a vertex's pseudo-angle from its bin's ends
 constexpr float kFan2Margin = 1.0f / 8.0f;     // second level
 static_assert(kFiltItems == 16 && CT % kFiltThreads == 0, "16 items per filter thread");
-static_assert(kFanTable + kQueueSmem <= 227 * 1024 - 1024, "table and queues fit a block's shared memory");
+static_assert(kQueueSmem % 16 == 0 && kFanTable + kQueueSmem <= 227 * 1024 - 1024, "table and queues fit a block's shared memory");
 
 // det = (a - c) x (b - c) from the rounded differences, and a bound: a det
 // beyond it in magnitude has the exact sign.  Shewchuk's orient2d error
@@ -114,10 +117,10 @@ struct GlobalFan {
 // again; d = fl(p - c).  Two vertices are read: in shared memory the reads of
 // 32 random bins conflict (six wavefronts each), and a third would bound the
 // pass.
-template <int NB, class Fan>
-__device__ __forceinline__ bool fan_inside(const Fan &F, float2 c, float2 d, float2 p)
+template <class Bins, class Fan>
+__device__ __forceinline__ bool fan_inside(Bins nb, const Fan &F, float2 c, float2 d, float2 p)
 {
-    const auto a = F.at(fan_bin_biased<NB>(d.x, d.y));   // (a NaN: any vertex; such a point is next to c)
+    const auto a = F.at(fan_bin_biased(nb, d.x, d.y));   // (a NaN: any vertex; such a point is next to c)
     const float2 Q = F.get(a, 0);
     float e1, e2;
     const float side = det_bound(sub2(Q, c), d, e1);
@@ -129,10 +132,10 @@ __device__ __forceinline__ bool fan_inside(const Fan &F, float2 c, float2 d, flo
 
 // The bin a point may be the vertex of, -1 when its pseudo-angle is within
 // `margin` of the bin's ends (or undefined).
-template <int NB>
-__device__ __forceinline__ int vertex_bin(float dx, float dy, float margin)
+template <class Bins>
+__device__ __forceinline__ int vertex_bin(Bins nb, float dx, float dy, float margin)
 {
-    const float phi = fan_phi<NB>(dx, dy);
+    const float phi = fan_phi(nb, dx, dy);
     const float f = __fadd_rd(phi, 0x1p23f);   // 2^23 + the bin
     const float mid = phi - (f - 0x1p23f) - 0.5f;
     return fabsf(mid) <= 0.5f - margin ? (int)(__float_as_uint(f) - kBinBias) : -1;
@@ -148,16 +151,43 @@ __device__ __forceinline__ bool fan_ready(const KgonCtrl *kc, const Kgon *g)
 // ---------------------------------------------------------------------------
 // first level: bins and vertices
 // ---------------------------------------------------------------------------
+constexpr int BI = 4;   // points per thread and step of the bins passes
+
+// The bins' slots raised by a thread's points (live: those that count;
+// index(k): point k's index).  A point whose binary32 distance is clearly below
+// its slot's needs no exact key.
+template <class Bins, class Index>
+__device__ __forceinline__ void raise_bins(Bins nb, unsigned long long *slot, const float (&qx)[BI], const float (&qy)[BI],
+                                           uint32_t live, float2 c, float r2ref, Index index)
+{
+    uint32_t top[BI];   // the slots' keys (most points do not raise their bin's)
+    int b[BI];
+#pragma unroll
+    for (int k = 0; k < BI; ++k) {
+        b[k] = vertex_bin(nb, __fsub_rn(qx[k], c.x), __fsub_rn(qy[k], c.y), kFanMargin);
+        top[k] = 0u;
+        if (!((live >> k) & 1u)) b[k] = -1;
+        if (b[k] >= 0) top[k] = __ldcg(reinterpret_cast<const uint32_t *>(slot + b[k]) + 1);
+    }
+#pragma unroll
+    for (int k = 0; k < BI; ++k) {
+        const float dx = __fsub_rn(qx[k], c.x), dy = __fsub_rn(qy[k], c.y);
+        const float r2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
+        // (an empty slot's key is a NaN: not below)
+        if (b[k] >= 0 && !(r2 - r2ref < __fmaf_rn(r2, -0x1p-20f, key_float(top[k])))) {
+            const uint32_t key = far_key(qx[k], qy[k], c.x, c.y, r2ref);
+            if (key >= top[k]) atomicMax(slot + b[k], ((unsigned long long)key << 32) | (uint32_t)~index(k));
+        }
+    }
+}
+
 // Every stride-th tile, in quarters (1024 points, four a thread) over a
 // persistent grid: the bins' farthest points.  The first quarter's points
 // take the octagon test as well: it tells how many points survive it (a point
 // inside the octagon is an input point all the same, and rarely the
-// farthest).  A point whose binary32 distance is clearly below its slot's
-// needs no exact key.  Bound by the latency of the points' and then the
+// farthest).  Bound by the latency of the points' and then the
 // slots' reads, so the next quarter's points are read while this one is
 // binned, and few registers keep five blocks on an SM.
-constexpr int BI = 4;   // points per thread and step
-
 template <int G>
 __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *__restrict__ pts, uint32_t n, void *ws,
                                                                    Layout L, uint32_t stride, int use_bits,
@@ -211,28 +241,9 @@ __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *
             kept += __popc(mine);
         }
         if (!__any_sync(0xffffffffu, mine != 0u)) continue;
-        uint32_t top[BI];   // the slots' keys (most points do not raise their bin's); ~0: no bin
-        int b[BI];
-#pragma unroll
-        for (int k = 0; k < BI; ++k) {
-            b[k] = vertex_bin<kFanBins>(__fsub_rn(qx[k], cx), __fsub_rn(qy[k], cy), kFanMargin);
-            top[k] = 0u;
-            if (!((mine >> k) & 1u)) b[k] = -1;
-            if (b[k] >= 0) top[k] = __ldcg(reinterpret_cast<const uint32_t *>(kc->slot + b[k]) + 1);
-        }
-#pragma unroll
-        for (int k = 0; k < BI; ++k) {
-            const float dx = __fsub_rn(qx[k], cx), dy = __fsub_rn(qy[k], cy);
-            const float r2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
-            // (an empty slot's key is a NaN: not below)
-            if (b[k] >= 0 && !(r2 - r2ref < __fmaf_rn(r2, -0x1p-20f, key_float(top[k])))) {
-                const uint32_t key = far_key(qx[k], qy[k], cx, cy, r2ref);
-                if (key >= top[k]) {
-                    const uint32_t i = (uint32_t)item_point<G>(tile * kFiltTile, t, BI * part + k);
-                    atomicMax(kc->slot + b[k], ((unsigned long long)key << 32) | (uint32_t)~i);
-                }
-            }
-        }
+        raise_bins(Level1{}, kc->slot, qx, qy, mine, make_float2(cx, cy), r2ref, [&](int k) {
+            return (uint32_t)item_point<G>(tile * kFiltTile, t, (int)(BI * part) + k);
+        });
     }
     seen = __reduce_add_sync(0xffffffffu, seen);
     kept = __reduce_add_sync(0xffffffffu, kept);
@@ -356,8 +367,7 @@ struct VertexSmem {
 
 // The nearest non-empty bin before `from` (dir = -1) or from `from` on (dir =
 // 1), unwrapped; from -+ NB when there is none.
-template <int NB>
-__device__ __forceinline__ int nearest_bin(const unsigned long long *slot, int from, int dir)
+__device__ __forceinline__ int nearest_bin(int NB, const unsigned long long *slot, int from, int dir)
 {
     const int lane = (int)lane_id();
     for (int k = 0; k < NB; k += 32) {
@@ -369,17 +379,18 @@ __device__ __forceinline__ int nearest_bin(const unsigned long long *slot, int f
     return dir > 0 ? from + NB : from - NB;
 }
 
-// Bins [b0, b0 + VB) of a fan with NB bins; point(i) reads input point i
+// Bins [b0, b0 + VB) of a fan; point(i) reads input point i
 // (clamped to the input); V receives the vertices, x = NaN for none.  False
 // when there are no samples outside the range (no fan).
-template <int NB, class Point>
-__device__ __forceinline__ bool make_vertices(VertexSmem &sm, const unsigned long long *slot, int b0, float2 c, Point point,
-                                              float2 *V)
+template <class Bins, class Point>
+__device__ __forceinline__ bool make_vertices(Bins nb, VertexSmem &sm, const unsigned long long *slot, int b0, float2 c,
+                                              Point point, float2 *V)
 {
+    const int NB = (int)nb.count();
     const int lane = (int)lane_id();
     const uint32_t lt = (1u << lane) - 1u;
-    const int pb = nearest_bin<NB>(slot, b0, -1), nb = nearest_bin<NB>(slot, b0 + VB, 1);
-    if (pb <= b0 + VB - 1 - NB || nb >= b0 + NB) return false;   // (only this range has samples)
+    const int before = nearest_bin(NB, slot, b0, -1), after = nearest_bin(NB, slot, b0 + VB, 1);
+    if (before <= b0 + VB - 1 - NB || after >= b0 + NB) return false;   // (only this range has samples)
     bool has[VB / 32];
     float2 own[VB / 32];
     int len = 1;
@@ -396,7 +407,7 @@ __device__ __forceinline__ bool make_vertices(VertexSmem &sm, const unsigned lon
         len += __popc(m);
     }
     if (lane < 2) {
-        const int j = lane ? nb : pb;
+        const int j = lane ? after : before;
         const int w = j < 0 ? j + NB : (j >= NB ? j - NB : j);
         const int at = lane ? len : 0;
         sm.p[0][at] = point(~(uint32_t)__ldcg(slot + w));
@@ -444,11 +455,11 @@ __device__ __forceinline__ bool make_vertices(VertexSmem &sm, const unsigned lon
             const float num = lx * ey - ly * ex;
             const float own_den = (v.x - c.x) * ey - (v.y - c.y) * ex;
             if (!ok || num > own_den * (1.0f + 0x1p-18f)) {   // (own_den > 0: the sample is on the chord's side of c)
-                const float2 d = fan_direction<NB>((float)b + 0.5f);
+                const float2 d = fan_direction(nb, (float)b + 0.5f);
                 const float s = num / (d.x * ey - d.y * ex) * (1.0f - 0x1p-20f);
                 const float2 q = make_float2(__fmaf_rn(s, d.x, c.x), __fmaf_rn(s, d.y, c.y));
                 if (fabsf(q.x) <= 3.0e38f && fabsf(q.y) <= 3.0e38f &&
-                    vertex_bin<NB>(__fsub_rn(q.x, c.x), __fsub_rn(q.y, c.y), kFanMargin) == b &&
+                    vertex_bin(nb, __fsub_rn(q.x, c.x), __fsub_rn(q.y, c.y), kFanMargin) == b &&
                     orient(Lp.x, Lp.y, Rp.x, Rp.y, q.x, q.y) > 0 && orient(Lp.x, Lp.y, Rp.x, Rp.y, c.x, c.y) > 0) {
                     v = q;
                     ok = true;
@@ -469,8 +480,8 @@ __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict_
     if (!fan_live(kc, oct, n)) return;
     const int warp = (int)(threadIdx.x >> 5);
     const int b0 = (int)(blockIdx.x * (VT / 32) + warp) * VB;
-    const bool ok = make_vertices<kFanBins>(
-        sm[warp], kc->slot, b0, make_float2(oct->cx, oct->cy),
+    const bool ok = make_vertices(
+        Level1{}, sm[warp], kc->slot, b0, make_float2(oct->cx, oct->cy),
         [&](uint32_t i) { return input_point(pts, (int64_t)i < n ? i : 0u); }, at<Kgon>(ws, L.kgon)->raw);
     if (!ok && lane_id() == 0) kc->bad = 1u;
 }
@@ -493,7 +504,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
         return;
     }
     const float cx = oct->cx, cy = oct->cy;
-    const float2 v = g->raw[src], next = g->raw[next_bin(b)];
+    const float2 v = g->raw[src], next = g->raw[b + 1 == kFanBins ? 0 : b + 1];
     g->v[b] = v;
     // the next bin's vertex: its own point, or this one's again
     const float2 w = next.x == next.x ? next : v;
@@ -523,34 +534,51 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
 // ---------------------------------------------------------------------------
 // the filter pass
 // ---------------------------------------------------------------------------
-// The warp's kept points (mask: this lane's items; get(q): the point and its
-// index) to the end of the survivor list.
-template <class Get>
-__device__ __forceinline__ void append_survivors(uint32_t mask, void *ws, const Layout &L, Get get)
-{
-    const uint32_t lane = lane_id(), c = __popc(mask);
-    if (!__any_sync(0xffffffffu, c != 0u)) return;
-    uint32_t incl = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += u;
+// Where survivors go: sort keys, payloads and their number.
+struct Sink {
+    uint32_t *count, *keys;
+    unsigned long long *pay;
+    __device__ __forceinline__ void put(uint32_t pos, float2 p, uint32_t i) const
+    {
+        keys[pos] = ord_key(p.x);
+        pay[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
     }
+};
+
+// What a filter pass has in shared memory beside its queues and vertices.
+struct FilterSmem {
+    OctSmem so;
+    Sink sink;
+    uint32_t octs;
+    uint32_t item;
+};
+
+// The warp's kept points (mask: this lane's items among N; get(q): the point
+// and its index) to the end of the survivor list, item by item, so that the
+// lanes' writes (and the points they read again) are neighbours.
+template <int N, class Get>
+__device__ __forceinline__ void append_survivors(uint32_t mask, uint32_t total, const Sink &sink, Get get)
+{
+    const uint32_t lt = (1u << lane_id()) - 1u;
     uint32_t pos = 0;
-    if (lane == 31) pos = atomicAdd(&at<Ctrl>(ws, L.ctrl)->surv_count, incl);
-    pos = __shfl_sync(0xffffffffu, pos, 31) + incl - c;
-#pragma unroll 1
-    for (; mask; mask &= mask - 1u, ++pos) {
-        uint32_t i;
-        const float2 p = get(__ffs(mask) - 1, i);
-        at<uint32_t>(ws, L.keys[0])[pos] = ord_key(p.x);
-        at<unsigned long long>(ws, L.pay[0])[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
+    if (lane_id() == 0) pos = atomicAdd(sink.count, total);
+    pos = __shfl_sync(0xffffffffu, pos, 0);
+#pragma unroll N > 4 ? 4 : N
+    for (int q = 0; q < N; ++q) {
+        const bool mine = (mask >> q) & 1u;
+        const uint32_t m = __ballot_sync(0xffffffffu, mine);
+        if (mine) {
+            uint32_t i;
+            const float2 p = get(q, i);
+            sink.put(pos + __popc(m & lt), p, i);
+        }
+        pos += __popc(m);
     }
 }
 
 // The speculative sweep's candidates (extremes.cu; every other point is
 // proven inside the octagon): a warp per slice, the exact test.
-__device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *ws, const Layout &L)
+__device__ __forceinline__ uint32_t filter_candidates(const FilterSmem &fs, void *ws, const Layout &L)
 {
     const SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const uint32_t *cidx = at<uint32_t>(ws, L.keys[1]);
@@ -566,13 +594,15 @@ __device__ __forceinline__ uint32_t filter_candidates(const OctSmem &so, void *w
             bool keep = e0 + lane < c;
             if (keep) {
                 p = cpt[s0 + e0 + lane];
-                keep = keep_point<false>(so, p.x, p.y);
+                keep = keep_point<false>(fs.so, p.x, p.y);
             }
             mine += keep ? 1u : 0u;
-            append_survivors(keep ? 1u : 0u, ws, L, [&](int, uint32_t &i) {
-                i = cidx[s0 + e0 + lane];
-                return p;
-            });
+            const uint32_t total = __popc(__ballot_sync(0xffffffffu, keep));
+            if (total)
+                append_survivors<1>(keep ? 1u : 0u, total, fs.sink, [&](int, uint32_t &i) {
+                    i = cidx[s0 + e0 + lane];
+                    return p;
+                });
         }
     }
     return mine;
@@ -588,10 +618,14 @@ struct PointQueue {
     uint32_t n;   // warp-uniform
 };
 
+template <class Bins>
 struct FanView {
-    bool test;   // candidates
+    bool fan;       // there is one
+    Bins nb;
     SharedFan F;
     float2 c;
+    float rho2t;    // r2 < rho2t proves |p - c| below the disk's radius
+    bool disk;      // try the disk first
 };
 
 // An index with this bit (n < 2^30) is a point the octagon's forms may have
@@ -599,21 +633,24 @@ struct FanView {
 constexpr uint32_t kUnsettled = 0x80000000u;
 
 // Whether point p (i: its index and kUnsettled) survives; octs counts the
-// octagon survivors among the unsettled ones.
-__device__ __forceinline__ bool settle(const OctSmem &so, const FanView &f, bool fan, uint32_t i, float2 p, uint32_t &octs)
+// octagon survivors among the unsettled ones.  test: a candidate.
+template <class Bins>
+__device__ __forceinline__ bool settle(const OctSmem &so, const FanView<Bins> &f, bool test, uint32_t i, float2 p,
+                                       uint32_t &octs)
 {
     bool keep = true;
     if (i & kUnsettled) {
         keep = keep_point<false>(so, p.x, p.y);
         octs += keep ? 1u : 0u;
     }
-    if (f.test || ((i & kUnsettled) && fan)) keep = keep && !fan_inside<kFanBins>(f.F, f.c, sub2(p, f.c), p);
+    if (test || ((i & kUnsettled) && f.fan)) keep = keep && !fan_inside(f.nb, f.F, f.c, sub2(p, f.c), p);
     return keep;
 }
 
 // The last (up to) 32 points of the queue: the survivors to the list.
-__device__ __forceinline__ void queue_drain(PointQueue &q, const OctSmem &so, const FanView &f, bool fan,
-                                            const float *__restrict__ pts, void *ws, const Layout &L, uint32_t &octs)
+template <class Bins>
+__device__ __forceinline__ void queue_drain(PointQueue &q, const FilterSmem &fs, const FanView<Bins> &f, bool test,
+                                            const float *__restrict__ pts, uint32_t &octs)
 {
     const uint32_t lane = lane_id(), m = min(q.n, 32u);
     q.n -= m;
@@ -621,164 +658,184 @@ __device__ __forceinline__ void queue_drain(PointQueue &q, const OctSmem &so, co
     const uint32_t e = q.i[q.n + (keep ? lane : 0u)], i = e & ~kUnsettled;
     const float2 p = input_point(pts, i);
     __syncwarp();   // the slots may be filled again
-    if (keep) keep = settle(so, f, fan, e, p, octs);
+    if (keep) keep = settle(fs.so, f, test, e, p, octs);
     const uint32_t b = __ballot_sync(0xffffffffu, keep);
     if (!b) return;
     uint32_t pos = 0;
-    if (lane == 0) pos = atomicAdd(&at<Ctrl>(ws, L.ctrl)->surv_count, (uint32_t)__popc(b));
+    if (lane == 0) pos = atomicAdd(fs.sink.count, (uint32_t)__popc(b));
     pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(b & ((1u << lane) - 1u));
-    if (keep) {
-        at<uint32_t>(ws, L.keys[0])[pos] = ord_key(p.x);
-        at<unsigned long long>(ws, L.pay[0])[pos] = ((unsigned long long)ord_key(p.y) << 32) | i;
+    if (keep) fs.sink.put(pos, p, i);
+}
+
+// Tiles tile, tile + step, ... below t1 of the set pts (n points), by a group
+// of kFiltThreads threads whose warps have queues of their own: a thread tests
+// its 16 points of a tile eight at a time: the octagon's affine forms, then
+// (fan) the fan test, branch-free -- or, in a warp where the disk holds most
+// points, the disk test, the others going to the queue.  bits: a second
+// polygon has refined the count pass's keep bits, which then stand for the
+// octagon test.  octs counts the octagon survivors.
+template <int G, class Bins>
+__device__ __forceinline__ void filter_tiles(const FilterSmem &fs, const FanView<Bins> &f, uint32_t *queue,
+                                             const float *__restrict__ pts, uint32_t n, uint32_t tile, uint32_t t1,
+                                             uint32_t step, const uint16_t *bits, uint32_t &octs)
+{
+    const uint32_t t = threadIdx.x % kFiltThreads, lt = (1u << lane_id()) - 1u;
+    const bool edges = !bits && fs.so.has_edges;
+    PointQueue q{queue, 0u};
+    bool use_disk = f.fan && f.disk;   // (then the queue holds candidates)
+    for (; tile < t1; tile += step) {
+        const uint32_t base = tile * kFiltTile;
+        if (t == 0 && tile + step < t1) {   // the next tile streams into L2 meanwhile
+            const uint32_t nb = base + step * kFiltTile;
+            const uintptr_t next = reinterpret_cast<uintptr_t>(pts + 2 * (size_t)nb);
+            const uint32_t head = (uint32_t)(next & 8u);   // (a set may start 8 bytes past a 16-byte boundary)
+            const uint32_t bytes = (min((uint32_t)kFiltTile, n - nb) * 8u - head) & ~15u;
+            if (bytes) bulk_prefetch_l2(reinterpret_cast<const void *>(next + head), bytes);
+        }
+        // kept: octagon survivors; drop: those of them inside the disk or the
+        // fan; near: some may be undecided, and all of this lane's are settled
+        // when they leave the queue (rare: next to the octagon)
+        uint32_t kept = 0xffffu, drop = 0;
+        bool near = false;
+        if (bits) kept = bits[tile * kFiltThreads + t];
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            float px[8], py[8];
+            if (base + kFiltTile <= n) load_part<G, 8>(pts, base, t, half, px, py);
+            else kept &= ~(0xffu << (8 * half)) |
+                         load_part_ragged<G, 8>(pts, n, base, t, half, f.c.x, f.c.y, px, py) << (8 * half);
+            if (edges) {
+                uint32_t out8;
+                near |= oct_decide<8>(fs.so, px, py, out8);
+                kept &= ~(0xffu << (8 * half)) | out8 << (8 * half);
+            }
+            if (!f.fan) continue;
+            uint32_t in = 0;
+            if (use_disk) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float dx = __fsub_rn(px[k], f.c.x), dy = __fsub_rn(py[k], f.c.y);
+                    if (__fmaf_rn(dx, dx, __fmul_rn(dy, dy)) < f.rho2t) in |= 1u << k;
+                }
+            } else if (__any_sync(0xffffffffu, ((kept >> (8 * half)) & 0xffu) != 0u)) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (k % 4 == 0) asm volatile("" ::: "memory");   // four points at a time (more would spill)
+                    const float2 p = make_float2(px[k], py[k]);
+                    if (fan_inside(f.nb, f.F, f.c, sub2(p, f.c), p)) in |= 1u << k;
+                }
+            }
+            drop |= in << (8 * half);
+        }
+        uint32_t live = near ? kept : kept & ~drop;
+        if (!near) octs += __popc(kept);
+        const uint32_t total = __reduce_add_sync(0xffffffffu, __popc(live));
+        if (use_disk) {   // a warp that finds under a quarter of a tile's points in the disk stops testing it
+            const uint32_t tried = __reduce_add_sync(0xffffffffu, __popc(kept));
+            if (4u * total > 3u * tried) {
+                while (q.n) queue_drain(q, fs, f, true, pts, octs);
+                if (!near) octs -= __popc(kept);
+                use_disk = false;
+                tile -= step;   // once more, with the fan
+                continue;
+            }
+        }
+        if (total == 0u) continue;
+        if (total <= kMany) {
+            // (a ballot per round: a lane has few points)
+            uint32_t m;
+            while ((m = __ballot_sync(0xffffffffu, live != 0u)) != 0u) {
+                if (live)
+                    q.i[q.n + __popc(m & lt)] = (uint32_t)item_point<G>(base, t, __ffs(live) - 1) | (near ? kUnsettled : 0u);
+                live &= live - 1u;
+                q.n += __popc(m);
+                __syncwarp();
+                if (q.n >= 32u) queue_drain(q, fs, f, use_disk, pts, octs);
+            }
+        } else {   // many at once: the points are read again
+            if (use_disk || near) {
+#pragma unroll 1
+                for (uint32_t m = live; m; m &= m - 1u) {
+                    const uint32_t i = (uint32_t)item_point<G>(base, t, __ffs(m) - 1);
+                    if (!settle(fs.so, f, use_disk, i | (near ? kUnsettled : 0u), input_point(pts, i), octs))
+                        live &= ~(m & (0u - m));
+                }
+            }
+            const uint32_t left = __reduce_add_sync(0xffffffffu, __popc(live));
+            if (left)
+                append_survivors<kFiltItems>(live, left, fs.sink, [&](int k, uint32_t &i) {
+                    i = (uint32_t)item_point<G>(base, t, k);
+                    return input_point(pts, i);
+                });
+        }
+    }
+    while (q.n) queue_drain(q, fs, f, use_disk, pts, octs);
+}
+
+// The vertices in shared memory, with the repeated ends.
+__device__ __forceinline__ void load_fan(float2 *sv, const float2 *V, int nb)
+{
+    // (both 16-byte aligned, nb even; four loads in flight)
+    const float4 *src = reinterpret_cast<const float4 *>(V);
+    float4 *dst = reinterpret_cast<float4 *>(sv);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nb / 2; i += blockDim.x) dst[i] = __ldg(src + i);
+    if (threadIdx.x == 0) {
+        sv[-1] = __ldg(V + nb - 1);
+        sv[nb] = __ldg(V);
+        sv[nb + 1] = __ldg(V + 1);
     }
 }
 
-// The tiles go in contiguous ranges to groups of kFiltThreads threads; a
-// thread tests its 16 points of a tile eight at a time: the octagon's affine
-// forms, then (fan) the fan test, branch-free -- or, in a warp where the disk
-// holds most points, the disk test, the others going to the queue.
-// bits_mode: a second polygon has refined the count pass's keep bits, which
-// then stand for the octagon test.
-// One block of 1024 threads per SM: the vertices and the queues take its
-// shared memory.  Bound by issue and the vertices' bank conflicts on
-// circle-like sets (about 18 instructions for the octagon, 27 for the fan and
-// two vertex reads per point) and by HBM on others.  Testing and writing in
-// one pass replaces a count pass, a fan pass and a scatter that each read the
-// points again: 274 + 455 + 214 us on 10^8 points of the unit circle.
+// (2^-20 covers the rounding of a point's binary32 squared distance)
+__device__ __forceinline__ float disk_limit(float rho2) { return __fmul_rd(rho2, 1.0f - 0x1p-20f); }
+
+// The tiles go in contiguous ranges to groups of kFiltThreads threads.  One
+// block of 768 threads per SM: the vertices and the queues take its shared
+// memory, and what its registers do not hold would go to L2.  Bound by issue
+// and the vertices' bank conflicts on circle-like sets (about 18 instructions
+// for the octagon, 27 for the fan and two vertex reads per point) and by the
+// points' latency on others.  Testing and writing in one pass replaces a
+// count pass, a fan pass and a scatter that each read the points again: 274 +
+// 455 + 214 us on 10^8 points of the unit circle.
 template <int G>
 __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restrict__ pts, uint32_t n, void *ws, Layout L,
                                                             int has_fan, int use_bits, const int32_t *kdev)
 {
     kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ OctSmem so;
-    __shared__ uint32_t s_oct;
+    __shared__ FilterSmem fs;
     const Octagon *oct = at<Octagon>(ws, L.oct);
     if (oct->abort) return;
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
-    fill_octagon(so, oct);
-    if (threadIdx.x == 0) s_oct = 0u;
+    fill_octagon(fs.so, oct);
+    if (threadIdx.x == 0) {
+        fs.octs = 0u;
+        fs.sink = Sink{&at<Ctrl>(ws, L.ctrl)->surv_count, at<uint32_t>(ws, L.keys[0]),
+                       at<unsigned long long>(ws, L.pay[0])};
+    }
     const Kgon *g = at<Kgon>(ws, L.kgon);
     const bool fan = has_fan && !oct->spec && fan_ready(kc, g);
-    float2 *sv = reinterpret_cast<float2 *>(smem_raw + kQueueSmem) + 1;
-    if (fan) {
-        for (int i = threadIdx.x; i < kFanBins; i += CT) sv[i] = __ldg(g->v + i);
-        if (threadIdx.x == 0) {
-            sv[-1] = __ldg(g->v + kFanBins - 1);
-            sv[kFanBins] = __ldg(g->v);
-            sv[kFanBins + 1] = __ldg(g->v + 1);
-        }
-    }
+    float2 *sv = reinterpret_cast<float2 *>(smem_raw + kQueueSmem) + 2;
+    if (fan) load_fan(sv, g->v, kFanBins);
     __syncthreads();
     uint32_t octs = 0;   // octagon survivors of this thread
     if (oct->spec) {
-        octs = filter_candidates(so, ws, L);
+        octs = filter_candidates(fs, ws, L);
     } else {
-        const bool bits_mode = use_bits && (!kdev || *kdev != 8);
-        const float2 c = make_float2(so.cx, so.cy);
-        const SharedFan F(sv);
-        const uint32_t warp = threadIdx.x >> 5, lt = (1u << lane_id()) - 1u;
-        PointQueue q{reinterpret_cast<uint32_t *>(smem_raw) + warp * kQueue, 0u};
-        // r2 < rho2t proves |p - c|^2 < rho^2 (2^-20 covers the rounding of r2)
-        const float rho2t = fan ? __fmul_rd(fan_rho2(kc), 1.0f - 0x1p-20f) : 0.0f;
-        bool use_disk = fan;   // (then the queue holds candidates)
-        const bool edges = !bits_mode && so.has_edges;
+        const FanView<Level1> f{fan, Level1{}, SharedFan(sv), make_float2(fs.so.cx, fs.so.cy),
+                                fan ? disk_limit(fan_rho2(kc)) : 0.0f, true};
         const uint32_t ntiles = (n + kFiltTile - 1) / kFiltTile;   // (n < 2^30)
-        const uint32_t t = threadIdx.x % kFiltThreads, gi = blockIdx.x * CG + threadIdx.x / kFiltThreads;
+        const uint32_t gi = blockIdx.x * CG + threadIdx.x / kFiltThreads;
         const uint32_t per = (ntiles + gridDim.x * CG - 1) / (gridDim.x * CG);
-        const uint32_t t1 = min(ntiles, (gi + 1) * per);
-        for (uint32_t tile = gi * per; tile < t1; ++tile) {
-            const uint32_t base = tile * kFiltTile;
-            if (t == 0 && tile + 1 < t1) {   // the next tile streams into L2 meanwhile
-                const float *next = pts + 2 * (size_t)(base + kFiltTile);
-                if ((reinterpret_cast<uintptr_t>(next) & 15u) == 0)
-                    bulk_prefetch_l2(next, (min((uint32_t)kFiltTile, n - base - kFiltTile) * 8u) & ~15u);
-            }
-            // kept: octagon survivors; drop: those of them inside the disk or
-            // the fan; near: some may be undecided, and all of this lane's are
-            // settled when they leave the queue (rare: next to the octagon)
-            uint32_t kept = 0xffffu, drop = 0;
-            bool near = false;
-            if (bits_mode) kept = at<uint16_t>(ws, L.keep_bits)[tile * kFiltThreads + t];
-#pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-                float px[8], py[8];
-                if (base + kFiltTile <= n) load_part<G, 8>(pts, base, t, half, px, py);
-                else kept &= ~(0xffu << (8 * half)) |
-                             load_part_ragged<G, 8>(pts, n, base, t, half, c.x, c.y, px, py) << (8 * half);
-                if (edges) {
-                    uint32_t out8;
-                    near |= oct_decide<8>(so, px, py, out8);
-                    kept &= ~(0xffu << (8 * half)) | out8 << (8 * half);
-                }
-                if (!fan) continue;
-                uint32_t in = 0;
-                if (use_disk) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const float dx = __fsub_rn(px[k], c.x), dy = __fsub_rn(py[k], c.y);
-                        if (__fmaf_rn(dx, dx, __fmul_rn(dy, dy)) < rho2t) in |= 1u << k;
-                    }
-                } else if (__any_sync(0xffffffffu, ((kept >> (8 * half)) & 0xffu) != 0u)) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        if (k % 4 == 0) asm volatile("" ::: "memory");   // four points at a time (more would spill)
-                        const float2 p = make_float2(px[k], py[k]);
-                        if (fan_inside<kFanBins>(F, c, sub2(p, c), p)) in |= 1u << k;
-                    }
-                }
-                drop |= in << (8 * half);
-            }
-            uint32_t live = near ? kept : kept & ~drop;
-            if (!near) octs += __popc(kept);
-            const uint32_t total = __reduce_add_sync(0xffffffffu, __popc(live));
-            if (use_disk) {   // a warp that finds under a quarter of a tile's points in the disk stops testing it
-                const uint32_t tried = __reduce_add_sync(0xffffffffu, __popc(kept));
-                if (4u * total > 3u * tried) {
-                    while (q.n) queue_drain(q, so, FanView{true, F, c}, fan, pts, ws, L, octs);
-                    if (!near) octs -= __popc(kept);
-                    use_disk = false;
-                    --tile;   // once more, with the fan
-                    continue;
-                }
-            }
-            if (total == 0u) continue;
-            const FanView f{use_disk, F, c};
-            if (q.n + total <= (uint32_t)kQueue) {
-                uint32_t at = q.n;
-                q.n += total;
-                // (a ballot per round: a lane has few points)
-                while (at < q.n) {
-                    const uint32_t m = __ballot_sync(0xffffffffu, live != 0u);
-                    if (live)
-                        q.i[at + __popc(m & lt)] = (uint32_t)item_point<G>(base, t, __ffs(live) - 1) | (near ? kUnsettled : 0u);
-                    live &= live - 1u;
-                    at += __popc(m);
-                }
-                __syncwarp();
-                while (q.n >= 32u) queue_drain(q, so, f, fan, pts, ws, L, octs);
-            } else {   // many at once: each lane its own, the points read again
-                if (f.test || near) {
-#pragma unroll 1
-                    for (uint32_t m = live; m; m &= m - 1u) {
-                        const uint32_t i = (uint32_t)item_point<G>(base, t, __ffs(m) - 1);
-                        if (!settle(so, f, fan, i | (near ? kUnsettled : 0u), input_point(pts, i), octs))
-                            live &= ~(m & (0u - m));
-                    }
-                }
-                append_survivors(live, ws, L, [&](int k, uint32_t &i) {
-                    const int64_t j = item_point<G>(base, t, k);
-                    i = (uint32_t)j;
-                    return input_point(pts, j);
-                });
-            }
-        }
-        while (q.n) queue_drain(q, so, FanView{use_disk, F, c}, fan, pts, ws, L, octs);
+        filter_tiles<G>(fs, f, reinterpret_cast<uint32_t *>(smem_raw) + (threadIdx.x >> 5) * kQueue, pts, n, gi * per,
+                        min(ntiles, (gi + 1) * per), 1u,
+                        use_bits && (!kdev || *kdev != 8) ? at<uint16_t>(ws, L.keep_bits) : nullptr, octs);
     }
     octs = __reduce_add_sync(0xffffffffu, octs);
-    if (lane_id() == 0 && octs) atomicAdd(&s_oct, octs);
+    if (lane_id() == 0 && octs) atomicAdd(&fs.octs, octs);
     __syncthreads();
-    if (threadIdx.x == 0 && s_oct) atomicAdd(&kc->s_oct, s_oct);
+    if (threadIdx.x == 0 && fs.octs) atomicAdd(&kc->s_oct, fs.octs);
 }
 
 // ---------------------------------------------------------------------------
@@ -827,7 +884,7 @@ __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint3
     const float cx = g->cx, cy = g->cy, r2ref = far_ref(*oct);
     for (uint32_t i = blockIdx.x * F2T + threadIdx.x; i < m; i += gridDim.x * F2T) {
         const float2 p = surv_point(keys, pay, i);
-        const int b = vertex_bin<kFan2Bins>(__fsub_rn(p.x, cx), __fsub_rn(p.y, cy), kFan2Margin);
+        const int b = vertex_bin(Level2{}, __fsub_rn(p.x, cx), __fsub_rn(p.y, cy), kFan2Margin);
         if (b < 0) continue;
         const unsigned long long v = ((unsigned long long)far_key(p.x, p.y, cx, cy, r2ref) << 32) | (uint32_t)~i;
         if (v > __ldcg(&slot[b])) atomicMax(&slot[b], v);   // the read only saves atomics
@@ -858,7 +915,7 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
     V[b] = v;
     if (b < 2) V[kFan2Bins + b] = v;
     if (b == kFan2Bins - 1) V[-1] = v;
-    const unsigned long long nextp = slot[next_bin<kFan2Bins>(b)];
+    const unsigned long long nextp = slot[b + 1 == kFan2Bins ? 0 : b + 1];
     const float2 w = nextp != 0ull ? surv_point(keys, pay, ~(uint32_t)nextp) : v;
     const bool edge = v.x != w.x || v.y != w.y;
     // c strictly left of v -> w, proven in binary32 or exactly
@@ -908,7 +965,7 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
 #pragma unroll
             for (int k = 0; k < F2I; ++k) {
                 const float2 p = make_float2(key_float(kv[k]), key_float((uint32_t)(pv[k] >> 32)));
-                if (fan_inside<kFan2Bins>(F, c, sub2(p, c), p)) in |= 1u << k;
+                if (fan_inside(Level2{}, F, c, sub2(p, c), p)) in |= 1u << k;
             }
             keep &= ~in;
         }
@@ -1003,361 +1060,549 @@ cudaError_t launch_hull_filter(const float *pts, int64_t n, void *ws, const Layo
 namespace {
 
 // ---------------------------------------------------------------------------
-// many sets (ch_hull_batched): the same fan for every set with at least
-// kKgonMinS octagon survivors, between the batched count pass and its scan
+// many sets (ch_hull_batched): the same filter per set.  A set's survivors go
+// to its own stretch of the sort arrays (from its first point's position), so
+// no scan over tiles places them.  Sets of at least kBxFanMinN points with
+// enough octagon survivors in a sample get a fan of up to kBxTileBins bins per
+// tile, smoothed as the single set's; one whose fan drops less than an eighth
+// of a sample goes without.
 // ---------------------------------------------------------------------------
-constexpr int kFanSmem = kFanBins * 8;
-constexpr int FT = 512;                  // threads per block of the bins pass
-constexpr int FITEMS = 8;                // points per thread per tile there
-// The signs orient_f32 certifies, as two flags (det > bound, -det > bound;
-// neither when undecided or when the terms may have overflowed): the same
-// arithmetic on the rounded differences a - c and b - c, without turning
-// the flags into an integer.
-struct Sgn {
-    bool pos, neg;
-};
-__device__ __forceinline__ Sgn sgn_ref(float acx, float acy, float bcx, float bcy)
+constexpr int64_t kBxFanMinN = 16384;
+constexpr int64_t kBxTightMinN = 65536;
+constexpr int kBxSample = 256;        // points of a set's estimates
+constexpr int kPlainChunk = 16;       // tiles per work item of the sets without a fan
+static_assert(kFanBins % kBxBinRun == 0 && kBxTileBins % kBxBinRun == 0 && kBxBinRun == VB * VT / 32, "whole runs of bins");
+
+// A fan's bins and sample, by what limits it.  Points of a circle (tight)
+// differ in radius by the rounding of their coordinates: only short chords lie
+// above enough of them, so as many bins as shared memory holds and every or
+// every second tile (fewer than 65536 points: nearly all are vertices, no
+// fan).  Elsewhere the farthest of few samples in a wide sector do: a bin per
+// 16 points, at most 8192, and a sample of about 65536 points.  (With the
+// circle's choice for all sets, 4096 sets' bins, vertices and vertex tables
+// took 1.7 ms more.)
+__device__ __forceinline__ uint32_t bx_bins(uint32_t ntiles, bool tight)
 {
-    const float detleft = __fmul_rn(acx, bcy);
-    const float detright = __fmul_rn(acy, bcx);
-    const float det = __fsub_rn(detleft, detright);
-    const float detsum = __fadd_rn(fabsf(detleft), fabsf(detright));
-    const float eb = __fmaf_ru(detsum, 2.384185791015625e-07f /* 2^-22 */, 7.174648137343064e-43f /* 2^-140 */);
-    const bool ok = detsum <= 3.0e38f;
-    return {ok && det > eb, ok && -det > eb};
+    return tight ? min(ntiles * kBxTileBins, (uint32_t)kFanBins)
+                 : min((ntiles * 256u + kBxBinRun - 1u) / kBxBinRun * kBxBinRun, 8192u);
+}
+__device__ __forceinline__ uint32_t bx_stride(int64_t n, bool tight)
+{
+    return tight ? (n > (1 << 17) ? 2u : 1u) : (uint32_t)max(1ll, min(8ll, (long long)(n >> 16)));
 }
 
-template <int NB = kFanBins>
-__device__ __forceinline__ int fan_signs_f32(const float2 *V, float cx, float cy, float px, float py)
+// One warp per set: whether it gets a fan -- at least 2048 octagon survivors,
+// estimated from kBxSample evenly spaced points.
+__global__ void __launch_bounds__(256) bx_fan_want_kernel(const float *__restrict__ pts, void *ws, BatchLayout BL)
 {
-    const float dx = __fsub_rn(px, cx), dy = __fsub_rn(py, cy);
-    const int b = (int)min(fan_bin<NB>(dx, dy), NB - 1u);
-    const float2 v = V[b];
-    const Sgn o = sgn_ref(__fsub_rn(v.x, cx), __fsub_rn(v.y, cy), dx, dy);                   // (v, p, c)
-    const float2 w = V[o.pos ? next_bin<NB>(b) : prev_bin<NB>(b)];
-    const Sgn e1 = sgn_ref(__fsub_rn(v.x, px), __fsub_rn(v.y, py), __fsub_rn(w.x, px), __fsub_rn(w.y, py));   // (v, w, p)
-    const Sgn e2 = sgn_ref(dx, dy, __fsub_rn(w.x, cx), __fsub_rn(w.y, cy));                   // (p, w, c)
-    // inside: the three signs certified equal (strictly inside the triangle
-    // on o's side); outside: one of the edges certified opposite to o
-    const bool in = (o.pos && e1.pos && e2.pos) || (o.neg && e1.neg && e2.neg);
-    const bool out = (o.pos && (e1.neg || e2.neg)) || (o.neg && (e1.pos || e2.pos));
-    return in ? 1 : (out ? 0 : 2);
+    kernel_entry();
+    const int64_t b = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (b >= BL.num_sets) return;
+    const SetInfo &S = at<SetInfo>(ws, BL.sets)[b];
+    const Octagon &o = at<Octagon>(ws, BL.octs)[b];
+    FanInfo &f = at<FanInfo>(ws, BL.fan)[b];
+    uint32_t out = 0;
+    float lo = __int_as_float(0x7f800000), hi = 0.0f;   // squared distances
+    const bool may = !at<BatchCtrl>(ws, BL.bctrl)->abort && !o.abort && o.has_edges && S.n >= kBxFanMinN;   // warp-uniform
+    if (may) {
+        const float2 *p = reinterpret_cast<const float2 *>(pts) + S.pt_begin;
+        float2 v[kBxSample / 32];
+#pragma unroll
+        for (int r = 0; r < kBxSample / 32; ++r) v[r] = __ldg(p + S.n * (r * 32 + (int)lane_id()) / kBxSample);
+#pragma unroll
+        for (int r = 0; r < kBxSample / 32; ++r) {
+            const float x = __fsub_rn(v[r].x, o.cx), y = __fsub_rn(v[r].y, o.cy);
+            float m = __int_as_float(0x7f800000);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m = min_nan(m, __fmaf_rn(o.tx[k], x, __fmaf_rn(o.ty[k], y, o.tz[k])));
+            out += m > 1.0f ? 0u : 1u;
+            const float r2 = __fmaf_rn(x, x, __fmul_rn(y, y));
+            lo = fminf(lo, r2);
+            hi = fmaxf(hi, r2);
+        }
+        out = __reduce_add_sync(0xffffffffu, out);
+        // (non-negative: their bits order as they do)
+        lo = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(lo)));
+        hi = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(hi)));
+    }
+    if (lane_id() == 0) {
+        const bool tight = hi - lo <= hi * 0x1p-16f;
+        f.tight = tight ? 1u : 0u;
+        f.nb = bx_bins(S.ntiles, tight);
+        f.want = may && (int64_t)out * S.n >= (int64_t)2048 * kBxSample && (!tight || S.n >= kBxTightMinN) ? 1u : 0u;
+    }
 }
 
-template <int NB = kFanBins>
-__device__ __noinline__ bool fan_inside_exact(const float2 *V, float cx, float cy, float px, float py)
+// One block: the lists of the fan sets and of all work items (runs of `chunk`
+// tiles of a fan set, of kPlainChunk tiles of another, of kBxBinRun bins).
+__global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, BatchLayout BL, uint32_t chunk)
 {
-    const int b = (int)min(fan_bin<NB>(px - cx, py - cy), NB - 1u);
-    const float2 v = V[b];
-    const int o = orient(cx, cy, v.x, v.y, px, py);
-    if (o == 0) return false;
-    const float2 w = V[o > 0 ? next_bin<NB>(b) : prev_bin<NB>(b)];
-    return orient(v.x, v.y, w.x, w.y, px, py) == o && orient(w.x, w.y, cx, cy, px, py) == o;
+    kernel_entry();
+    __shared__ uint32_t s_w[4][32];
+    BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
+    if (bc->abort) return;
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    FanInfo *fan = at<FanInfo>(ws, BL.fan);
+    uint2 *fi = at<uint2>(ws, BL.fan_items), *pi = at<uint2>(ws, BL.plain_items), *bi = at<uint2>(ws, BL.bin_items);
+    const int64_t B = BL.num_sets;
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
+    const int64_t per = ceil_div(B, (int64_t)blockDim.x);
+    const int64_t b0 = min((int64_t)threadIdx.x * per, B), b1 = min(b0 + per, B);
+    uint32_t c[4] = {0, 0, 0, 0};   // fan sets, fan items, plain items, bin runs
+    for (int64_t b = b0; b < b1; ++b) {
+        const uint32_t nt = sets[b].ntiles;
+        if (fan[b].want) {
+            c[0] += 1u;
+            c[1] += (nt + chunk - 1) / chunk;
+            c[3] += fan[b].nb / kBxBinRun;
+        } else {
+            c[2] += (nt + kPlainChunk - 1) / kPlainChunk;
+        }
+    }
+    uint32_t run[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t incl = c[q];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += u;
+        }
+        if (lane == 31) s_w[q][warp] = incl;
+        run[q] = incl - c[q];
+    }
+    __syncthreads();
+    uint32_t tot[4] = {0, 0, 0, 0};
+    for (uint32_t w = 0; w < blockDim.x / 32; ++w) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (w < warp) run[q] += s_w[q][w];
+            tot[q] += s_w[q][w];
+        }
+    }
+    for (int64_t b = b0; b < b1; ++b) {
+        const uint32_t nt = sets[b].ntiles;
+        if (fan[b].want) {
+            const uint32_t nb = fan[b].nb;
+            fan[b].bad = fan[b].ready = 0u;
+            at<uint32_t>(ws, BL.fan_set)[run[0]++] = (uint32_t)b;
+            for (uint32_t t = 0; t < nt; t += chunk) fi[run[1]++] = make_uint2((uint32_t)b, t);
+            for (uint32_t k = 0; k < nb; k += kBxBinRun) bi[run[3]++] = make_uint2((uint32_t)b, k);
+        } else {
+            for (uint32_t t = 0; t < nt; t += kPlainChunk) pi[run[2]++] = make_uint2((uint32_t)b, t);
+        }
+    }
+    if (threadIdx.x == 0) {
+        bc->nfan = tot[0];
+        bc->nfan_items = tot[1];
+        bc->nplain_items = tot[2];
+        bc->nbin_items = tot[3];
+    }
 }
 
-constexpr int kBxBinStride = 2;   // built-in: the bins see every 2nd tile of a set (1 and 4 measured slower overall)
+// A set's slots, vertices (in the same place once the slots are read) and
+// vertices before empty bins are filled.
+__device__ __forceinline__ unsigned long long *bx_slots(void *ws, const BatchLayout &BL, const SetInfo &S)
+{
+    return at<unsigned long long>(ws, BL.fan_slot) + (size_t)S.tile_base * kBxTileBins;
+}
+__device__ __forceinline__ float2 *bx_raw(void *ws, const BatchLayout &BL, const SetInfo &S)
+{
+    return at<float2>(ws, BL.fan_raw) + (size_t)S.tile_base * kBxTileBins;
+}
 
-// One block: numbers the sets that get a fan and lays out the refine's
-// work items (runs of up to kBxFanChunk tiles of one such set).
-__global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, Layout L, BatchLayout BL, uint32_t chunk)
+__global__ void __launch_bounds__(256) bx_fan_zero_kernel(void *ws, BatchLayout BL)
+{
+    kernel_entry();
+    const uint2 *bi = at<uint2>(ws, BL.bin_items);
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const uint32_t n = at<BatchCtrl>(ws, BL.bctrl)->nbin_items;
+    for (uint32_t w = blockIdx.x; w < n; w += gridDim.x) {
+        unsigned long long *slot = bx_slots(ws, BL, sets[bi[w].x]) + bi[w].y;
+        for (int k = threadIdx.x; k < kBxBinRun; k += 256) slot[k] = 0ull;
+    }
+}
+
+// Per work item of a fan set, every stride-th tile (counted from the set's
+// first; 0: the built-in choice): the bins' farthest points, as
+// fan_bins_kernel.
+__global__ void __launch_bounds__(kFiltThreads, 5) bx_fan_bins_kernel(const float *__restrict__ pts, void *ws, BatchLayout BL,
+                                                                      uint32_t chunk, uint32_t stride)
+{
+    kernel_entry();
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const Octagon *octs = at<Octagon>(ws, BL.octs);
+    const uint2 *items = at<uint2>(ws, BL.fan_items);
+    const uint32_t nitems = at<BatchCtrl>(ws, BL.bctrl)->nfan_items, t = threadIdx.x;
+    constexpr uint32_t parts = kFiltItems / BI;
+    // (eight tiles of an item at a time: the set's data are looked up once)
+    const uint32_t units = chunk / kBxFanChunkMin;
+    for (uint32_t w = blockIdx.x; w < nitems * units; w += gridDim.x) {
+        const uint2 item = items[w / units];
+        const SetInfo &S = sets[item.x];
+        const FanInfo &info = at<FanInfo>(ws, BL.fan)[item.x];
+        const uint32_t st = stride ? stride : bx_stride(S.n, info.tight);
+        const uint32_t first = (item.y + w % units * kBxFanChunkMin + st - 1) / st * st;
+        const uint32_t end = min(item.y + (w % units + 1) * kBxFanChunkMin, S.ntiles);
+        if (first >= end) continue;   // block-uniform
+        const Octagon &o = octs[item.x];
+        const SetBins nb{info.nb};
+        const float cx = o.cx, cy = o.cy, r2ref = far_ref(o);
+        const float *p2 = pts + 2 * S.pt_begin;
+        unsigned long long *slot = bx_slots(ws, BL, S);
+        const uint32_t n = (uint32_t)S.n, steps = ((end - first + st - 1) / st) * parts;   // parts of every st-th tile
+        float px[BI], py[BI];
+        uint32_t live = 0;
+        const auto fetch = [&](uint32_t u) {
+            const uint32_t base = (first + u / parts * st) * kFiltTile;
+            const int part = (int)(u % parts);
+            if (base + kFiltTile <= n) {
+                load_part<1, BI>(p2, base, t, part, px, py);
+                live = (1u << BI) - 1u;
+            } else {
+                live = load_part_ragged<1, BI>(p2, n, base, t, part, cx, cy, px, py);
+            }
+        };
+        fetch(0);
+        for (uint32_t u = 0; u < steps; ++u) {
+            float qx[BI], qy[BI];
+            const uint32_t mine = live;
+#pragma unroll
+            for (int k = 0; k < BI; ++k) {
+                qx[k] = px[k];
+                qy[k] = py[k];
+            }
+            if (u + 1 < steps) fetch(u + 1);
+            raise_bins(nb, slot, qx, qy, mine, make_float2(cx, cy), r2ref, [&](int k) {
+                return (uint32_t)item_point<1>((first + u / parts * st) * kFiltTile, t, (int)(BI * (u % parts)) + k);
+            });
+        }
+    }
+}
+
+// A block per run of kBxBinRun bins: the vertices (make_vertices).
+__global__ void __launch_bounds__(VT) bx_fan_vertex_kernel(const float *__restrict__ pts, void *ws, BatchLayout BL)
+{
+    kernel_entry();
+    __shared__ VertexSmem sm[VT / 32];
+    const uint2 *bi = at<uint2>(ws, BL.bin_items);
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const Octagon *octs = at<Octagon>(ws, BL.octs);
+    const uint32_t n = at<BatchCtrl>(ws, BL.bctrl)->nbin_items;
+    const int warp = (int)(threadIdx.x >> 5);
+    for (uint32_t w = blockIdx.x; w < n; w += gridDim.x) {
+        const uint2 item = bi[w];
+        const SetInfo &S = sets[item.x];
+        const float2 *p = reinterpret_cast<const float2 *>(pts) + S.pt_begin;
+        const int64_t m = S.n;
+        const FanInfo &info = at<FanInfo>(ws, BL.fan)[item.x];
+        if (info.tight) {   // the farthest samples themselves (a chord's rounded point would lie deeper)
+            const unsigned long long *slot = bx_slots(ws, BL, S);
+            float2 *raw = bx_raw(ws, BL, S);
+            for (int k = (int)item.y + (int)threadIdx.x; k < (int)item.y + kBxBinRun; k += VT) {
+                const unsigned long long v = __ldcg(slot + k);
+                const uint32_t i = ~(uint32_t)v;
+                raw[k] = v != 0ull ? __ldg(p + ((int64_t)i < m ? i : 0u)) : make_float2(__int_as_float(0x7fc00000), 0.0f);
+            }
+            continue;   // block-uniform
+        }
+        const bool ok = make_vertices(
+            SetBins{info.nb}, sm[warp], bx_slots(ws, BL, S), (int)item.y + warp * VB,
+            make_float2(octs[item.x].cx, octs[item.x].cy), [&](uint32_t i) { return __ldg(p + ((int64_t)i < m ? i : 0u)); },
+            bx_raw(ws, BL, S));
+        if (!ok && lane_id() == 0) at<FanInfo>(ws, BL.fan)[item.x].bad = 1u;
+        __syncwarp();
+    }
+}
+
+// A block per fan set: empty bins repeat the vertex before them; the proofs
+// of fan_build_kernel; and whether the fan drops at least an eighth of a
+// sample.
+__global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restrict__ pts, void *ws, BatchLayout BL)
+{
+    kernel_entry();
+    __shared__ int s_w[BT / 32];
+    __shared__ int s_last;
+    __shared__ uint32_t s_inv, s_edges, s_bad, s_in, s_seen;
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const Octagon *octs = at<Octagon>(ws, BL.octs);
+    const uint32_t nfan = at<BatchCtrl>(ws, BL.bctrl)->nfan;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    for (uint32_t k = blockIdx.x; k < nfan; k += gridDim.x) {
+        const uint32_t set = at<uint32_t>(ws, BL.fan_set)[k];
+        const SetInfo &S = sets[set];
+        const Octagon &o = octs[set];
+        FanInfo &info = at<FanInfo>(ws, BL.fan)[set];
+        const float2 *raw = bx_raw(ws, BL, S);
+        float2 *V = reinterpret_cast<float2 *>(bx_slots(ws, BL, S));
+        const SetBins nb{info.nb};
+        const int NB = (int)nb.n;
+        const float cx = o.cx, cy = o.cy;
+        const bool off = info.bad || !(__fadd_rn(__fsub_rn(o.bxh, o.bxl), __fsub_rn(o.byh, o.byl)) < 0x1p62f);
+        __syncthreads();   // the shared words of the previous set have been read
+        if (tid == 0) {
+            s_last = -1;
+            s_inv = s_edges = s_in = s_seen = 0u;
+            s_bad = off ? 1u : 0u;
+        }
+        __syncthreads();
+        if (off) continue;   // block-uniform
+        int last = -1;   // the last bin with a vertex (what the first empty bins repeat)
+        for (int b = (int)tid; b < NB; b += BT)
+            if (raw[b].x == raw[b].x) last = b;
+        last = __reduce_max_sync(0xffffffffu, last);
+        if (lane == 0) atomicMax(&s_last, last);
+        __syncthreads();
+        int carry = s_last;
+        if (carry < 0) continue;   // block-uniform
+        uint32_t inv = 0, edges = 0;
+        bool bad = false;
+        for (int b0 = 0; b0 < NB; b0 += BT) {   // (NB is a multiple of kBxBinRun: the last chunk may be half full)
+            const int b = b0 + (int)tid;
+            const float2 mine = b < NB ? raw[b] : make_float2(__int_as_float(0x7fc00000), 0.0f);
+            int src = mine.x == mine.x ? b : -1;
+#pragma unroll
+            for (int q = 1; q < 32; q <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, src, q);
+                if (lane >= (uint32_t)q) src = max(src, u);
+            }
+            if (lane == 31) s_w[warp] = src;
+            __syncthreads();
+            int all = -1;
+            for (uint32_t w = 0; w < BT / 32; ++w) {
+                if (w < warp) src = max(src, s_w[w]);
+                all = max(all, s_w[w]);
+            }
+            __syncthreads();   // s_w is written again by the next chunk
+            if (src < 0) src = carry;
+            if (all >= 0) carry = all;
+            if (b < NB) {
+                const float2 v = src == b ? mine : raw[src], next = raw[b + 1 == NB ? 0 : b + 1];
+                V[b] = v;
+                const float2 w = next.x == next.x ? next : v;
+                if (v.x != w.x || v.y != w.y) {
+                    const float r = disk_bound(cx, cy, v, w);
+                    bad |= r < 0.0f;
+                    inv = max(inv, ~__float_as_uint(fmaxf(r, 0.0f)));
+                    ++edges;
+                }
+            }
+        }
+        inv = __reduce_max_sync(0xffffffffu, inv);
+        edges = __reduce_add_sync(0xffffffffu, edges);
+        if (lane == 0) {
+            atomicMax(&s_inv, inv);
+            atomicAdd(&s_edges, edges);
+        }
+        if (bad) s_bad = 1u;
+        __syncthreads();
+        const float rho2 = __uint_as_float(~s_inv);
+        if (s_bad || s_edges < 3u || !(rho2 > 0x1p-120f)) continue;   // block-uniform
+        if (tid < (uint32_t)kBxSample) {   // (points of the first and last bins, whose neighbours wrap, are left out)
+            const float2 p = __ldg(reinterpret_cast<const float2 *>(pts) + S.pt_begin + S.n * tid / kBxSample);
+            const float2 c = make_float2(cx, cy), d = sub2(p, c);
+            const uint32_t b = fan_bin_biased(nb, d.x, d.y) - kBinBias;
+            bool in = false;
+            const bool seen = b >= 1u && b + 1u < nb.n;
+            if (seen) {
+                const float2 Q = __ldcg(V + b);
+                float e1, e2;
+                const float side = det_bound(sub2(Q, c), d, e1);
+                const float2 W = __ldcg(V + (side > 0.0f ? b + 1u : b - 1u));
+                const float det = det_bound(sub2(W, Q), sub2(p, Q), e2);
+                in = fabsf(side) > e1 && (side > 0.0f ? det : -det) > e2;
+            }
+            const uint32_t ni = __popc(__ballot_sync(0xffffffffu, in)), ns = __popc(__ballot_sync(0xffffffffu, seen));
+            if (lane == 0) {
+                atomicAdd(&s_in, ni);
+                atomicAdd(&s_seen, ns);
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            info.rho2 = rho2;
+            info.ready = 8u * s_in >= s_seen ? 1u : 0u;
+        }
+    }
+}
+
+// The octagon, the sink and (fan) the vertices of set b into shared memory.
+__device__ __forceinline__ void bx_load_set(FilterSmem &fs, float2 *sv, void *ws, const Layout &L, const BatchLayout &BL,
+                                            uint32_t b)
+{
+    const SetInfo &S = at<SetInfo>(ws, BL.sets)[b];
+    fill_octagon(fs.so, at<Octagon>(ws, BL.octs) + b);
+    if (threadIdx.x == 0)
+        fs.sink = Sink{at<uint32_t>(ws, BL.soct) + b, at<uint32_t>(ws, L.keys[0]) + S.pt_begin,
+                       at<unsigned long long>(ws, L.pay[0]) + S.pt_begin};
+    const FanInfo &info = at<FanInfo>(ws, BL.fan)[b];
+    if (sv && info.ready) load_fan(sv, reinterpret_cast<const float2 *>(bx_slots(ws, BL, S)), (int)info.nb);
+}
+
+// Persistent blocks take the fan sets' work items by ticket; octagon and
+// vertices are read again only when the set changes (a set's items follow one
+// another).
+__global__ void __launch_bounds__(CT, 1) bx_hull_filter_kernel(const float *__restrict__ pts, void *ws, Layout L,
+                                                               BatchLayout BL, uint32_t chunk)
+{
+    kernel_entry();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ FilterSmem fs;
+    float2 *sv = reinterpret_cast<float2 *>(smem_raw + kQueueSmem) + 2;
+    BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const uint2 *items = at<uint2>(ws, BL.fan_items);
+    const uint32_t nitems = bc->nfan_items;
+    uint32_t *queue = reinterpret_cast<uint32_t *>(smem_raw) + (threadIdx.x >> 5) * kQueue;
+    uint32_t cur = 0xffffffffu, octs = 0;
+    for (;;) {
+        __syncthreads();   // the item and the set's data have been read
+        if (threadIdx.x == 0) fs.item = atomicAdd(&bc->fan_ticket, 1u);
+        __syncthreads();
+        const uint32_t w = fs.item;
+        if (w >= nitems) break;
+        const uint2 item = items[w];
+        if (item.x != cur) {
+            cur = item.x;
+            bx_load_set(fs, sv, ws, L, BL, cur);
+            __syncthreads();
+        }
+        const SetInfo &S = sets[cur];
+        const FanInfo &info = at<FanInfo>(ws, BL.fan)[cur];
+        const bool fan = info.ready != 0u;
+        const FanView<SetBins> f{fan, SetBins{info.nb}, SharedFan(sv), make_float2(fs.so.cx, fs.so.cy),
+                                 fan ? disk_limit(info.rho2) : 0.0f, info.tight == 0u};
+        const float *p = pts + 2 * S.pt_begin;
+        const uint32_t first = item.y + threadIdx.x / kFiltThreads, end = min(item.y + chunk, S.ntiles);
+        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0)
+            filter_tiles<2>(fs, f, queue, p, (uint32_t)S.n, first, end, (uint32_t)CG, nullptr, octs);
+        else
+            filter_tiles<1>(fs, f, queue, p, (uint32_t)S.n, first, end, (uint32_t)CG, nullptr, octs);
+    }
+}
+
+// The same for the sets without a fan: many small blocks, no vertices.
+__global__ void __launch_bounds__(kFiltThreads, 3) bx_plain_filter_kernel(const float *__restrict__ pts, void *ws, Layout L,
+                                                                          BatchLayout BL)
+{
+    kernel_entry();
+    __shared__ FilterSmem fs;
+    __shared__ uint32_t s_queue[kFiltThreads / 32 * kQueue];
+    BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
+    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const uint2 *items = at<uint2>(ws, BL.plain_items);
+    const uint32_t nitems = bc->nplain_items;
+    uint32_t cur = 0xffffffffu, octs = 0;
+    for (;;) {
+        __syncthreads();   // the item and the set's data have been read
+        if (threadIdx.x == 0) fs.item = atomicAdd(&bc->plain_ticket, 1u);
+        __syncthreads();
+        const uint32_t w = fs.item;
+        if (w >= nitems) break;
+        const uint2 item = items[w];
+        if (item.x != cur) {
+            cur = item.x;
+            bx_load_set(fs, nullptr, ws, L, BL, cur);
+            __syncthreads();
+        }
+        if (fs.so.abort) continue;   // block-uniform
+        const SetInfo &S = sets[cur];
+        const FanView<SetBins> f{false, SetBins{4u}, SharedFan(nullptr), make_float2(fs.so.cx, fs.so.cy), 0.0f, false};
+        filter_tiles<1>(fs, f, s_queue + (threadIdx.x >> 5) * kQueue, pts + 2 * S.pt_begin, (uint32_t)S.n, item.y,
+                        min(item.y + (uint32_t)kPlainChunk, S.ntiles), 1u, nullptr, octs);
+    }
+}
+
+// One block: each set's survivors and the layout of the later stages: its
+// super-chunks (4096 survivors, also the sort tiles) and merge-tree nodes.
+__global__ void __launch_bounds__(1024) bx_layout_kernel(void *ws, BatchLayout BL)
 {
     kernel_entry();
     __shared__ uint32_t s_w[2][32];
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const Octagon *octs = at<Octagon>(ws, BL.octs);
-    const uint32_t *soct = at<uint32_t>(ws, BL.soct);
-    const uint32_t *nonfin = at<uint32_t>(ws, BL.nonfinite);
-    int32_t *fan_id = at<int32_t>(ws, BL.fan_id);
-    uint32_t *fan_set = at<uint32_t>(ws, BL.fan_set);
-    uint2 *items = at<uint2>(ws, BL.fan_items);
-    const int64_t B = BL.num_sets;
-    const bool off = bc->abort != 0;
+    if (bc->abort) return;
+    SetInfo *sets = at<SetInfo>(ws, BL.sets);
+    const uint32_t *count = at<uint32_t>(ws, BL.soct);
+    uint32_t *sc_set = at<uint32_t>(ws, BL.sc_set);
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
+    const int64_t B = BL.num_sets;
     const int64_t per = ceil_div(B, (int64_t)blockDim.x);
     const int64_t b0 = min((int64_t)threadIdx.x * per, B), b1 = min(b0 + per, B);
-    auto wants = [&](int64_t b) {
-        return !off && soct[b] >= kKgonMinS && !octs[b].abort && octs[b].has_edges && nonfin[b] == 0u;
-    };
-    uint32_t nf = 0, ni = 0;
-    for (int64_t b = b0; b < b1; ++b)
-        if (wants(b)) {
-            ++nf;
-            ni += (uint32_t)ceil_div((int64_t)sets[b].ntiles, (int64_t)chunk);
-        }
-    uint32_t inf = nf, ini = ni;
+    uint32_t sc = 0, nd = 0;
+    for (int64_t b = b0; b < b1; ++b) {
+        const uint32_t nsc = (uint32_t)ceil_div((int64_t)count[b], kChainC);
+        sc += nsc;
+        nd += nsc > 0 ? (uint32_t)tree_nodes(nsc) + 1u : 0u;
+    }
+    uint32_t i1 = sc, i2 = nd;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t a = __shfl_up_sync(0xffffffffu, inf, o), c = __shfl_up_sync(0xffffffffu, ini, o);
+        const uint32_t u1 = __shfl_up_sync(0xffffffffu, i1, o), u2 = __shfl_up_sync(0xffffffffu, i2, o);
         if (lane >= (uint32_t)o) {
-            inf += a;
-            ini += c;
+            i1 += u1;
+            i2 += u2;
         }
     }
     if (lane == 31) {
-        s_w[0][warp] = inf;
-        s_w[1][warp] = ini;
+        s_w[0][warp] = i1;
+        s_w[1][warp] = i2;
     }
     __syncthreads();
-    uint32_t bf = 0, bi = 0, tf = 0, ti = 0;
+    uint32_t rsc = i1 - sc, rnd = i2 - nd, tsc = 0;
     for (uint32_t w = 0; w < blockDim.x / 32; ++w) {
         if (w < warp) {
-            bf += s_w[0][w];
-            bi += s_w[1][w];
+            rsc += s_w[0][w];
+            rnd += s_w[1][w];
         }
-        tf += s_w[0][w];
-        ti += s_w[1][w];
+        tsc += s_w[0][w];
     }
-    uint32_t f = bf + inf - nf, it = bi + ini - ni;
     for (int64_t b = b0; b < b1; ++b) {
-        if (wants(b) && f < (uint32_t)BL.max_fan) {
-            fan_id[b] = (int32_t)f;
-            fan_set[f] = (uint32_t)b;
-            for (uint32_t c = 0; c < sets[b].ntiles; c += chunk) items[it++] = make_uint2(f, sets[b].tile_base + c);
-            ++f;
-        } else {
-            fan_id[b] = -1;
-        }
+        const uint32_t s = count[b], nsc = (uint32_t)ceil_div((int64_t)s, kChainC);
+        SetInfo &S = sets[b];
+        S.surv_base = (uint64_t)S.pt_begin;
+        S.s = s;
+        S.nsc = nsc;
+        S.sc_base = rsc;
+        S.node_base = rnd;
+        for (uint32_t k = 0; k < nsc; ++k) sc_set[rsc + k] = (uint32_t)b;
+        rsc += nsc;
+        rnd += nsc > 0 ? (uint32_t)tree_nodes(nsc) + 1u : 0u;
     }
-    if (threadIdx.x == 0) {
-        bc->nfan = min(tf, (uint32_t)BL.max_fan);
-        bc->nitems = min(ti, (uint32_t)BL.max_items);
-    }
-}
-
-// Per work item, every kBxBinStride-th tile (counted from the set's first):
-// each point's bin around the set's box centre, packed (far_key << 32 |
-// ~index) into the fan's global slots by atomicMax (the read first saves
-// most atomics).
-__global__ void __launch_bounds__(FT) bx_fan_bins_kernel(const float *__restrict__ pts, void *ws, Layout L,
-                                                         BatchLayout BL, uint32_t chunk, uint32_t stride)
-{
-    kernel_entry();
-    const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const Octagon *octs = at<Octagon>(ws, BL.octs);
-    const uint32_t *fan_set = at<uint32_t>(ws, BL.fan_set);
-    const uint2 *items = at<uint2>(ws, BL.fan_items);
-    unsigned long long *slots = at<unsigned long long>(ws, BL.fan_slot);
-    const uint32_t nitems = bc->nitems;
-    for (uint32_t w = blockIdx.x; w < nitems; w += gridDim.x) {
-        const uint2 item = items[w];
-        const uint32_t b = fan_set[item.x];
-        const SetInfo &S = sets[b];
-        const float cx = octs[b].cx, cy = octs[b].cy, r2ref = far_ref(octs[b]);
-        const float2 *p2 = reinterpret_cast<const float2 *>(pts) + S.pt_begin;
-        unsigned long long *sl = slots + (size_t)item.x * kFanBins;
-        const uint32_t tend = min(item.y + chunk, S.tile_base + S.ntiles);
-        for (uint32_t t = item.y; t < tend; ++t) {
-            if ((t - S.tile_base) % stride) continue;
-            const int64_t lo = (int64_t)(t - S.tile_base) * kFiltTile, hi = min(lo + kFiltTile, S.n);
-            float2 p[FITEMS];
-#pragma unroll
-            for (int r = 0; r < FITEMS; ++r) {
-                const int64_t i = lo + r * FT + threadIdx.x;
-                p[r] = i < hi ? __ldg(p2 + i) : make_float2(0.0f, 0.0f);
-            }
-#pragma unroll
-            for (int r = 0; r < FITEMS; ++r) {
-                const int64_t i = lo + r * FT + threadIdx.x;
-                if (i < hi) {
-                    const float dx = p[r].x - cx, dy = p[r].y - cy;
-                    const int bin = (int)min(fan_bin(dx, dy), kFanBins - 1u);
-                    const unsigned long long v =
-                        ((unsigned long long)far_key(p[r].x, p[r].y, cx, cy, r2ref) << 32) | (uint32_t)~(uint32_t)i;
-                    if (v > __ldcg(sl + bin)) atomicMax(sl + bin, v);
-                }
-            }
-        }
-    }
-}
-
-// One block per fan (grid-stride): the exact centre check against the
-// set's octagon, then every bin's vertex (the sampled point of the last
-// non-empty bin at or before it, cyclically), and the slots are left zero
-// for the next call.  Thread t owns the kBinsPerThread consecutive bins
-// from t * kBinsPerThread: a scan in registers, one block scan of the
-// threads' last non-empty bins.
-constexpr int kBinsPerThread = kFanBins / BT;
-static_assert(kFanBins % BT == 0, "bins split evenly over the threads");
-
-__global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restrict__ pts, void *ws, Layout L,
-                                                          BatchLayout BL)
-{
-    kernel_entry();
-    __shared__ int s_w[BT / 32];
-    __shared__ int s_ok;
-    const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const Octagon *octs = at<Octagon>(ws, BL.octs);
-    const uint32_t *fan_set = at<uint32_t>(ws, BL.fan_set);
-    uint32_t *fan_ok = at<uint32_t>(ws, BL.fan_ok);
-    float2 *fan_c = at<float2>(ws, BL.fan_c);
-    unsigned long long *slots = at<unsigned long long>(ws, BL.fan_slot);
-    float2 *verts = at<float2>(ws, BL.fan_v);
-    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    const uint32_t nfan = bc->nfan;
-    for (uint32_t k = blockIdx.x; k < nfan; k += gridDim.x) {
-        const uint32_t b = fan_set[k];
-        const Octagon &oct = octs[b];
-        const float cx = oct.cx, cy = oct.cy;
-        unsigned long long *sl = slots + (size_t)k * kFanBins + (size_t)tid * kBinsPerThread;
-        float2 *V = verts + (size_t)k * kFanBins + (size_t)tid * kBinsPerThread;
-        const float2 *p2 = reinterpret_cast<const float2 *>(pts) + sets[b].pt_begin;
-        const int64_t nb = sets[b].n;
-        __syncthreads();   // shared words of the previous fan have been read
-        if (tid == 0) s_ok = 1;
-        __syncthreads();
-        if (tid < 8 && ((oct.valid >> tid) & 1u) && orient(oct.ax[tid], oct.ay[tid], oct.bx[tid], oct.by[tid], cx, cy) <= 0)
-            s_ok = 0;
-        // this thread's bins: the point index of each non-empty one, ~0u empty
-        uint32_t idx[kBinsPerThread];
-        int mylast = -1;
-#pragma unroll
-        for (int j = 0; j < kBinsPerThread; ++j) {
-            const unsigned long long v = __ldcg(sl + j);
-            idx[j] = v != 0ull ? ~(uint32_t)v : ~0u;
-            if (v != 0ull) mylast = j;
-        }
-        // the last non-empty bin of the threads before this one (exclusive
-        // max-scan over thread order), and the last overall (wrap-around)
-        int incl = mylast >= 0 ? (int)(tid * kBinsPerThread) + mylast : -1;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= (uint32_t)o) incl = max(incl, u);
-        }
-        int excl = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) excl = -1;
-        if (lane == 31) s_w[warp] = incl;
-        __syncthreads();
-        int before = -1, last = -1;
-        for (uint32_t w = 0; w < BT / 32; ++w) {
-            if (w < warp) before = max(before, s_w[w]);
-            last = max(last, s_w[w]);
-        }
-        before = max(before, excl);
-        const bool live = s_ok && last >= 0;
-        if (live) {
-            // the vertex index of a bin with no sample: that of the last
-            // non-empty bin before it (cyclically); it lies in another
-            // thread's range, read from the slots (not zeroed yet)
-            int cur = before >= 0 ? before : last;
-            uint32_t ci = ~(uint32_t)__ldcg(slots + (size_t)k * kFanBins + cur);
-#pragma unroll
-            for (int j = 0; j < kBinsPerThread; ++j) {
-                if (idx[j] != ~0u) ci = idx[j];
-                V[j] = __ldg(p2 + ((int64_t)ci < nb ? ci : 0u));
-            }
-        }
-        __syncthreads();   // every read of the slots is done
-#pragma unroll
-        for (int j = 0; j < kBinsPerThread; ++j) sl[j] = 0ull;
-        if (tid == 0) {
-            fan_ok[k] = live ? 1u : 0u;
-            fan_c[k] = make_float2(cx, cy);
-        }
-    }
-}
-
-// Persistent blocks take work items by ticket; the 27648 vertices of the
-// item's fan are loaded into shared memory when the fan changes (items of
-// one fan are consecutive).  The four groups of kFiltThreads threads share
-// the item's tiles; thread t holds the 16 keep bits of count-pass thread t
-// (point lo + r * 256 + t for bit r).  Kept points strictly inside the fan
-// lose their bit, and the tile's count drops by the number removed.
-__global__ void __launch_bounds__(CT, 1) bx_fan_refine_kernel(const float *__restrict__ pts, void *ws, Layout L,
-                                                              BatchLayout BL, uint32_t chunk)
-{
-    kernel_entry();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *sv = reinterpret_cast<float2 *>(smem_raw);   // kFanBins vertices
-    __shared__ uint32_t s_item;
-    BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    const SetInfo *sets = at<SetInfo>(ws, BL.sets);
-    const uint32_t *fan_set = at<uint32_t>(ws, BL.fan_set);
-    const uint32_t *fan_ok = at<uint32_t>(ws, BL.fan_ok);
-    const float2 *fan_c = at<float2>(ws, BL.fan_c);
-    const float2 *verts = at<float2>(ws, BL.fan_v);
-    const uint2 *items = at<uint2>(ws, BL.fan_items);
-    uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    const uint32_t nitems = bc->nitems;
-    const uint32_t grp = threadIdx.x / kFiltThreads, t = threadIdx.x % kFiltThreads, lane = lane_id();
-    int64_t cur = -1;
-    for (;;) {
-        __syncthreads();   // s_item of the previous item has been read
-        if (threadIdx.x == 0) s_item = atomicAdd(&bc->fan_ticket, 1u);
-        __syncthreads();
-        const uint32_t w = s_item;
-        if (w >= nitems) break;
-        const uint2 item = items[w];
-        if (!fan_ok[item.x]) continue;   // block-uniform
-        if ((int64_t)item.x != cur) {
-            const float4 *src = reinterpret_cast<const float4 *>(verts + (size_t)item.x * kFanBins);
-            float4 *dst = reinterpret_cast<float4 *>(sv);
-            for (int i = threadIdx.x; i < kFanBins / 2; i += CT) dst[i] = __ldg(src + i);
-            __syncthreads();
-            cur = item.x;
-        }
-        const SetInfo &S = sets[fan_set[item.x]];
-        const float2 c = fan_c[item.x];
-        const float2 *p2 = reinterpret_cast<const float2 *>(pts) + S.pt_begin;
-        const uint32_t tend = min(item.y + chunk, S.tile_base + S.ntiles);
-        for (uint32_t tile = item.y + grp; tile < tend; tile += CG) {
-            const int64_t lo = (int64_t)(tile - S.tile_base) * kFiltTile;
-            const uint32_t kb = bits[(size_t)tile * kFiltThreads + t];
-            uint32_t in = 0;
-            if (kb) {
-                float2 p[kFiltItems];
-#pragma unroll
-                for (int r = 0; r < kFiltItems; ++r)
-                    p[r] = ((kb >> r) & 1u) ? __ldcs(p2 + lo + r * kFiltThreads + t) : make_float2(0.0f, 0.0f);
-                uint32_t und = 0;
-#pragma unroll
-                for (int r = 0; r < kFiltItems; ++r) {
-                    const int f = fan_signs_f32(sv, c.x, c.y, p[r].x, p[r].y);
-                    in |= (f == 1 ? 1u : 0u) << r;
-                    und |= (f == 2 ? 1u : 0u) << r;
-                }
-                in &= kb;
-                und &= kb;
-                while (und) {
-                    const int r = __ffs(und) - 1;
-                    und &= und - 1u;
-                    const float2 q = p2[lo + r * kFiltThreads + t];
-                    if (fan_inside_exact(sv, c.x, c.y, q.x, q.y)) in |= 1u << r;
-                }
-                if (in) bits[(size_t)tile * kFiltThreads + t] = (uint16_t)(kb & ~in);
-            }
-            uint32_t removed = __popc(in);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, o);
-            if (lane == 0 && removed) atomicAdd(&status[tile], 0ull - (unsigned long long)removed);
-        }
-    }
+    if (threadIdx.x == 0) bc->nsc = tsc;
 }
 
 }  // namespace
 
-cudaError_t launch_bx_fan(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st)
+cudaError_t launch_bx_filter(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st)
 {
     const int sms = sm_count();
-    static const bool attrs = [] {
-        cudaFuncSetAttribute(bx_fan_refine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFanSmem);
+    static const bool attrs = [] {   // thread-safe one-time initialisation
+        cudaFuncSetAttribute(bx_hull_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kQueueSmem + kFanTable);
         return true;
     }();
     (void)attrs;
     const uint32_t chunk = tune_value(CH_TUNE_BX_FAN_CHUNK) ? (uint32_t)tune_value(CH_TUNE_BX_FAN_CHUNK) : kBxFanChunk;
-    const uint32_t stride = tune_value(CH_TUNE_BX_FAN_STRIDE) ? (uint32_t)tune_value(CH_TUNE_BX_FAN_STRIDE)
-                                                              : kBxBinStride;
+    const uint32_t stride = (uint32_t)tune_value(CH_TUNE_BX_FAN_STRIDE);
+    const int tuned = tune_value(CH_TUNE_BX_FILTER);
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * 5, BL.tiles_max));
     probe_before(CH_K_KGON, st);
-    launch_next(bx_fan_select_kernel, 1, 1024, 0, st, ws, L, BL, chunk);
-    launch_next(bx_fan_bins_kernel, (unsigned)(sms * 4), FT, 0, st, pts, ws, L, BL, chunk, stride);
-    launch_next(bx_fan_build_kernel, (unsigned)(sms * 2), BT, 0, st, pts, ws, L, BL);
-    launch_next(bx_fan_refine_kernel, (unsigned)sms, CT, kFanSmem, st, pts, ws, L, BL, chunk);
-    note_kernels(CH_K_KGON, 4);
+    launch_next(bx_fan_want_kernel, (unsigned)ceil_div(BL.num_sets, 8), 256, 0, st, pts, ws, BL);
+    launch_next(bx_fan_select_kernel, 1, 1024, 0, st, ws, BL, chunk);
+    launch_next(bx_fan_zero_kernel, g, 256, 0, st, ws, BL);
+    launch_next(bx_fan_bins_kernel, g, kFiltThreads, 0, st, pts, ws, BL, chunk, stride);
+    launch_next(bx_fan_vertex_kernel, g, VT, 0, st, pts, ws, BL);
+    launch_next(bx_fan_build_kernel, (unsigned)std::min<int64_t>((int64_t)sms * 2, BL.num_sets), BT, 0, st, pts, ws, BL);
+    note_kernels(CH_K_KGON, 6);
     probe_after(CH_K_KGON, st);
+    probe_before(CH_K_FILTER, st);
+    launch_next(bx_plain_filter_kernel,
+                (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * (tuned ? tuned : 3), BL.tiles_max)),
+                kFiltThreads, 0, st, pts, ws, L, BL);
+    launch_next(bx_hull_filter_kernel, (unsigned)std::min<int64_t>(sms, BL.tiles_max), CT, kQueueSmem + kFanTable, st, pts,
+                ws, L, BL, chunk);
+    launch_next(bx_layout_kernel, 1, 1024, 0, st, ws, BL);
+    note_kernels(CH_K_FILTER, 3);
+    probe_after(CH_K_FILTER, st);
     return cudaGetLastError();
 }
 

@@ -129,9 +129,6 @@ cudaError_t launch_bx_setup(const int64_t *offsets, void *ws, const Layout &L, c
                             int64_t n_cap, cudaStream_t st);
 cudaError_t launch_bx_extremes(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
 cudaError_t launch_bx_filter(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
-// the fan test of the sets with many octagon survivors, on the batched
-// count pass's keep bits and tile counts (kgon.cu)
-cudaError_t launch_bx_fan(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
 cudaError_t launch_bx_sort(void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
 cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st);
 // copies every set's chains to its part of hull_idx (after hull_offsets)
