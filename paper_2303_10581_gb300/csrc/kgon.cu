@@ -1088,7 +1088,7 @@ __device__ __forceinline__ uint32_t bx_bins(uint32_t ntiles, bool tight)
 }
 __device__ __forceinline__ uint32_t bx_stride(int64_t n, bool tight)
 {
-    return tight ? (n > (1 << 17) ? 2u : 1u) : (uint32_t)max(1ll, min(8ll, (long long)(n >> 16)));
+    return tight ? 1u : (uint32_t)max(1ll, min(8ll, (long long)(n >> 16)));
 }
 
 // One warp per set: whether it gets a fan -- at least 2048 octagon survivors,
