@@ -22,9 +22,7 @@ constexpr int kFiltThreads = 256;     // fused test + compaction
 constexpr int kFiltItems = 16;        // points per thread per tile
 constexpr int kFiltTile = kFiltThreads * kFiltItems;   // 4096 points = 32 KB
 constexpr int kFiltMaxBlocks = 4096;                  // grid cap of the two-pass filter
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortTile = kSortThreads * kSortItems;   // 4096 keys
+constexpr int kSortTile = 4096;       // keys per sort tile
 constexpr int kSortPasses = 4;        // 32-bit x keys, 8-bit digits
 constexpr int kLeafC = 16;            // points per leaf chain (one thread)
 constexpr int kChainThreads = 256;    // leaves per super-chunk (one block)

@@ -33,13 +33,21 @@ namespace ch {
 
 namespace {
 
-constexpr int NW = kSortThreads / 32;
+// Threads per block of a pass.  One set has few tiles, and 512 threads finish
+// a tile sooner (10^6 circle points, 3 blocks an SM either way: 234 -> 223 us
+// the whole hull); many sets fill the chip with tiles, and 256 threads share
+// the digits' bookkeeping among fewer warps (4096 sets: 8.14 ms, 8.33 with 512).
+constexpr int kPassThreads = 512;
+constexpr int kBxPassThreads = 256;
+constexpr int kPassBlocks = 3;   // per SM: as many as the shared memory holds
 
+template <int T>
 struct SortSmem {
+    static constexpr int NW = T / 32;
     unsigned long long pay[kSortTile];   // payload, element order
     uint32_t keys[kSortTile];            // keys, digit-sorted order
     uint16_t inv[kSortTile];             // digit-sorted position -> element
-    uint32_t wh[NW][256];                // per-warp digit counts, then per-warp offsets
+    alignas(16) uint16_t wh[NW][256];                // per-warp digit counts, then per-warp offsets
     uint32_t tstart[256];                // start of each digit inside the sorted tile
     uint32_t gbase[256];                 // output position of the tile's digit run, minus tstart
     uint32_t dbase[256];                 // global start of each digit (exclusive scan of the histogram)
@@ -47,8 +55,9 @@ struct SortSmem {
     uint32_t tile;
 };
 
-// exclusive scan of v over the 256 threads of the block; returns the total
-__device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t &excl, uint32_t *warp_tot)
+// exclusive scan of v over the block's threads (two barriers)
+template <int NW>
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t (&warp_tot)[NW])
 {
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
     uint32_t incl = v;
@@ -59,16 +68,11 @@ __device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t &exc
     }
     if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
-    uint32_t before = 0, total = 0;
+    uint32_t before = 0;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        const uint32_t t = warp_tot[w];
-        if (w < (int)warp) before += t;
-        total += t;
-    }
-    excl = before + incl - v;
+    for (int w = 0; w < NW; ++w) before += w < (int)warp ? warp_tot[w] : 0u;
     __syncthreads();
-    return total;
+    return before + incl - v;
 }
 
 __global__ void __launch_bounds__(256) sort_hist_kernel(void *ws, Layout L)
@@ -190,17 +194,19 @@ struct PassIO {
 // out_base + (segment digit start + rank in digit).  `first`: the
 // segment's first tile (its prefix is its own count).  Expects sm.dbase
 // (the segment's digit starts) set and sm.wh cleared, behind a barrier.
-__device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_t tile, int64_t base,
+template <int T>
+__device__ __forceinline__ void pass_tile(SortSmem<T> &sm, const PassIO &io, int64_t tile, int64_t base,
                                           uint32_t tile_n, int64_t out_base, uint32_t out_n, int shift, bool first,
                                           void *ws, const Layout &L, uint32_t site)
 {
+    constexpr int NW = T / 32, kItems = kSortTile / T;
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     const uint32_t lt = (1u << lane) - 1u;
     // keys to registers, payload to shared memory (element order)
-    uint32_t k[kSortItems];
+    uint32_t k[kItems];
 #pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-        const uint32_t e = warp * (32 * kSortItems) + j * 32 + lane;
+    for (int j = 0; j < kItems; ++j) {
+        const uint32_t e = warp * (32 * kItems) + j * 32 + lane;
         if (e < tile_n) {
             k[j] = __ldcs(io.kin + base + e);
             sm.pay[e] = __ldcs(io.pin + base + e);
@@ -209,10 +215,10 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
         }
     }
     // stable rank inside the warp, items in element order (j, lane)
-    uint16_t rank[kSortItems];
+    uint16_t rank[kItems];
 #pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-        const uint32_t e = warp * (32 * kSortItems) + j * 32 + lane;
+    for (int j = 0; j < kItems; ++j) {
+        const uint32_t e = warp * (32 * kItems) + j * 32 + lane;
         const bool ok = e < tile_n;
         const uint32_t d = ok ? (k[j] >> shift) & 255u : 256u;
         const uint32_t peers = __match_any_sync(0xffffffffu, d);
@@ -220,25 +226,27 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
         uint32_t cur = 0;
         if (ok) cur = sm.wh[warp][d];
         __syncwarp();
-        if (ok && before == 0) sm.wh[warp][d] = cur + __popc(peers);
+        if (ok && before == 0) sm.wh[warp][d] = (uint16_t)(cur + __popc(peers));
         __syncwarp();
         rank[j] = (uint16_t)(cur + before);
     }
     __syncthreads();
     // per digit: exclusive offsets across warps and the tile count
+    // (thread tid owns digit tid; the threads past them only join the scan)
     uint32_t cnt = 0;
+    if (tid < 256u) {
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        const uint32_t c = sm.wh[w][tid];
-        sm.wh[w][tid] = cnt;
-        cnt += c;
+        for (int w = 0; w < NW; ++w) {
+            const uint32_t c = sm.wh[w][tid];
+            sm.wh[w][tid] = (uint16_t)cnt;
+            cnt += c;
+        }
     }
-    uint32_t tstart;
-    block_excl_scan256(cnt, tstart, sm.warp_tot);
-    sm.tstart[tid] = tstart;
-    // decoupled look-back per digit (thread tid owns digit tid)
-    {
+    const uint32_t tstart = block_excl_scan(cnt, sm.warp_tot);
+    // decoupled look-back per digit
+    if (tid < 256u) {
         const uint32_t d = tid;
+        sm.tstart[d] = tstart;
         uint32_t *mine = io.status + tile * 256 + d;
         uint32_t excl = 0;
         if (first) {
@@ -253,8 +261,8 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
     __syncthreads();   // every digit's tstart is read below (gbase after the next barrier)
     // digit-sorted keys and the inverse permutation
 #pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-        const uint32_t e = warp * (32 * kSortItems) + j * 32 + lane;
+    for (int j = 0; j < kItems; ++j) {
+        const uint32_t e = warp * (32 * kItems) + j * 32 + lane;
         if (e < tile_n) {
             const uint32_t d = (k[j] >> shift) & 255u;
             const uint32_t pos = sm.tstart[d] + sm.wh[warp][d] + rank[j];
@@ -267,8 +275,8 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
     // matters after a look-back wait gave up
     if (tile_n == kSortTile) {
 #pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            const uint32_t i = j * kSortThreads + tid;
+        for (int j = 0; j < kItems; ++j) {
+            const uint32_t i = j * T + tid;
             const uint32_t key = sm.keys[i];
             const uint32_t pos = sm.gbase[(key >> shift) & 255u] + i;
             if (pos < out_n) {
@@ -277,7 +285,7 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
             }
         }
     } else {
-        for (uint32_t i = tid; i < tile_n; i += kSortThreads) {
+        for (uint32_t i = tid; i < tile_n; i += T) {
             const uint32_t key = sm.keys[i];
             const uint32_t pos = sm.gbase[(key >> shift) & 255u] + i;
             if (pos < out_n) {
@@ -289,11 +297,11 @@ __device__ __forceinline__ void pass_tile(SortSmem &sm, const PassIO &io, int64_
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSortThreads, 3) sort_pass_kernel(void *ws, Layout L, int p)
+__global__ void __launch_bounds__(kPassThreads, kPassBlocks) sort_pass_kernel(void *ws, Layout L, int p)
 {
     kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
+    SortSmem<kPassThreads> &sm = *reinterpret_cast<SortSmem<kPassThreads> *>(smem_raw);
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
@@ -314,9 +322,8 @@ __global__ void __launch_bounds__(kSortThreads, 3) sort_pass_kernel(void *ws, La
     }
     // global digit starts
     {
-        uint32_t ex;
-        block_excl_scan256(ctrl->hist[p][tid], ex, sm.warp_tot);
-        sm.dbase[tid] = ex;
+        const uint32_t ex = block_excl_scan(tid < 256u ? ctrl->hist[p][tid] : 0u, sm.warp_tot);
+        if (tid < 256u) sm.dbase[tid] = ex;
     }
     for (;;) {
         if (tid == 0) {
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) sort_pass_kernel(void *ws, La
                 bulk_prefetch_l2(io.pin + ahead * kSortTile, (nn * 8u) & ~15u);
             }
         }
-        for (int d = lane; d < 256; d += 32) sm.wh[warp][d] = 0u;
+        reinterpret_cast<uint4 *>(sm.wh[warp])[lane] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         const int64_t tile = sm.tile;
         if (tile >= ntiles) break;
@@ -386,11 +393,11 @@ __global__ void __launch_bounds__(256) bx_sort_hist_kernel(void *ws, Layout L, B
     }
 }
 
-__global__ void __launch_bounds__(kSortThreads, 3) bx_sort_pass_kernel(void *ws, Layout L, BatchLayout BL, int p)
+__global__ void __launch_bounds__(kBxPassThreads, kPassBlocks) bx_sort_pass_kernel(void *ws, Layout L, BatchLayout BL, int p)
 {
     kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
+    SortSmem<kBxPassThreads> &sm = *reinterpret_cast<SortSmem<kBxPassThreads> *>(smem_raw);
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -410,7 +417,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) bx_sort_pass_kernel(void *ws,
     }
     for (;;) {
         if (tid == 0) sm.tile = atomicAdd(&bc->sort_ticket[p], 1u);
-        for (int d = lane; d < 256; d += 32) sm.wh[warp][d] = 0u;
+        reinterpret_cast<uint4 *>(sm.wh[warp])[lane] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         const int64_t tile = sm.tile;
         if (tile >= ntiles) break;
@@ -419,9 +426,9 @@ __global__ void __launch_bounds__(kSortThreads, 3) bx_sort_pass_kernel(void *ws,
         const int64_t seg = (int64_t)sets[b].surv_base;
         const uint32_t seg_n = sets[b].s;
         {   // this set's digit starts (the scan's barriers also order sm.wh)
-            uint32_t ex;
-            block_excl_scan256(hist[((size_t)b * kSortPasses + p) * 256 + tid], ex, sm.warp_tot);
-            sm.dbase[tid] = ex;
+            const uint32_t ex = block_excl_scan(
+                tid < 256u ? hist[((size_t)b * kSortPasses + p) * 256 + tid] : 0u, sm.warp_tot);
+            if (tid < 256u) sm.dbase[tid] = ex;
         }
         pass_tile(sm, io, tile, seg + ltile * kSortTile,
                   (uint32_t)min((int64_t)kSortTile, (int64_t)seg_n - ltile * kSortTile), seg, seg_n, 8 * p,
@@ -432,9 +439,9 @@ __global__ void __launch_bounds__(kSortThreads, 3) bx_sort_pass_kernel(void *ws,
 int pass_blocks_per_sm()
 {
     static const int cached = [] {   // thread-safe one-time initialisation
-        cudaFuncSetAttribute(sort_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+        cudaFuncSetAttribute(sort_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem<kPassThreads>));
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, sort_pass_kernel, kSortThreads, sizeof(SortSmem));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, sort_pass_kernel, kPassThreads, sizeof(SortSmem<kPassThreads>));
         return v > 0 ? v : 1;
     }();
     return cached;
@@ -444,9 +451,9 @@ int bx_pass_blocks_per_sm()
 {
     static const int cached = [] {
         cudaFuncSetAttribute(bx_sort_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(SortSmem));
+                             (int)sizeof(SortSmem<kBxPassThreads>));
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, bx_sort_pass_kernel, kSortThreads, sizeof(SortSmem));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, bx_sort_pass_kernel, kBxPassThreads, sizeof(SortSmem<kBxPassThreads>));
         return v > 0 ? v : 1;
     }();
     return cached;
@@ -469,7 +476,7 @@ cudaError_t launch_bx_sort(void *ws, const Layout &L, const BatchLayout &BL, cud
         1, std::min<int64_t>(cap, (int64_t)sm_count() * (tuned ? tuned : bx_pass_blocks_per_sm())));
     for (int p = 0; p < kSortPasses; ++p) {
         probe_before(CH_K_SORT_PASS, st);
-        launch_next(bx_sort_pass_kernel, (unsigned)pb, kSortThreads, sizeof(SortSmem), st, ws, L, BL, p);
+        launch_next(bx_sort_pass_kernel, (unsigned)pb, kBxPassThreads, sizeof(SortSmem<kBxPassThreads>), st, ws, L, BL, p);
         note_kernels(CH_K_SORT_PASS, 1);
         probe_after(CH_K_SORT_PASS, st);
         e = cudaGetLastError();
@@ -495,7 +502,7 @@ cudaError_t launch_sort(void *ws, const Layout &L, cudaStream_t st)
     if (pb < 1) pb = 1;
     for (int p = 0; p < kSortPasses; ++p) {
         probe_before(CH_K_SORT_PASS, st);
-        launch_next(sort_pass_kernel, (unsigned)pb, kSortThreads, sizeof(SortSmem), st, ws, L, p);
+        launch_next(sort_pass_kernel, (unsigned)pb, kPassThreads, sizeof(SortSmem<kPassThreads>), st, ws, L, p);
         note_kernels(CH_K_SORT_PASS, 1);
         probe_after(CH_K_SORT_PASS, st);
         e = cudaGetLastError();
