@@ -22,6 +22,15 @@ constexpr int kFiltThreads = 256;     // fused test + compaction
 constexpr int kFiltItems = 16;        // points per thread per tile
 constexpr int kFiltTile = kFiltThreads * kFiltItems;   // 4096 points = 32 KB
 constexpr int kFiltMaxBlocks = 4096;                  // grid cap of the two-pass filter
+// Tiles [first_tile(T, G, b), first_tile(T, G, b + 1)) are block b's in the
+// two-pass filter and in the passes that follow its count pass (G <= T
+// blocks): shares that differ by one tile at most.  (Equal shares, the last
+// blocks without any, left 119 of 608 blocks idle on 2442 tiles.)
+__host__ __device__ inline int64_t first_tile(int64_t tiles, int64_t blocks, int64_t b) { return b * tiles / blocks; }
+__host__ __device__ inline int64_t tile_block(int64_t tiles, int64_t blocks, int64_t t)
+{
+    return ((t + 1) * blocks - 1) / tiles;
+}
 constexpr int kSortTile = 4096;       // keys per sort tile
 constexpr int kSortPasses = 4;        // 32-bit x keys, 8-bit digits
 constexpr int kLeafC = 16;            // points per leaf chain (one thread)

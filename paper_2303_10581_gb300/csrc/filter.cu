@@ -114,193 +114,96 @@ __device__ __forceinline__ uint32_t load_test(const float *__restrict__ pts, int
     return near ? settle_near<BOX>(so, keep, [&](int q) { return input_point(pts, item_point<G>(base, tid, q)); }) : keep;
 }
 
-// Kept points per (row, warp), turned into exclusive offsets in row-major
-// order (the point order of the tile) in s_off by warp 0.  Returns the tile
-// total to warp 0.  The caller synchronises before and after.
-template <int G>
-__device__ __forceinline__ void row_counts(uint32_t keep, uint32_t (&s_off)[kFiltItems / G][NW])
-{
-    constexpr int ROWS = kFiltItems / G;
-    const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int h = 0; h < G; ++h) c += __popc(__ballot_sync(0xffffffffu, (keep >> (r * G + h)) & 1u));
-        if (lane == 0) s_off[r][warp] = c;
-    }
-}
-
-template <int G>
-__device__ __forceinline__ uint32_t scan_rows_warp0(uint32_t (&s_off)[kFiltItems / G][NW])
-{
-    constexpr int PER = (kFiltItems / G) * NW / 32;
-    const uint32_t lane = lane_id();
-    uint32_t *flat = &s_off[0][0];
-    uint32_t loc[PER];
-    uint32_t sum = 0;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        loc[k] = flat[lane * PER + k];
-        sum += loc[k];
-    }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += t;
-    }
-    uint32_t run = incl - sum;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        flat[lane * PER + k] = run;
-        run += loc[k];
-    }
-    return __shfl_sync(0xffffffffu, incl, 31);
-}
-
-// Writes the kept points of one tile; excl is the tile's output offset.
+// The block writes the kept points of one tile in point order from the
+// threads' keep bits (out_off: the tile's first output position): a row is
+// one load of every thread, kFiltThreads * G consecutive points.  The loads
+// are under way while the warps count their rows; every warp then scans all
+// (row, warp) counts itself, so there is one barrier a tile, and s_cnt
+// alternates between two arrays.
+// Bound by latency and the writes.  (A warp per tile left three of eight
+// warps idle on a block's five tiles: 10^7 displaced points, 9.4 M of them
+// written, 62 us; this 45.)
 template <int G, bool KEYS>
-__device__ __forceinline__ void scatter_tile(uint32_t keep, int64_t base, uint64_t excl,
-                                             const uint32_t (&s_off)[kFiltItems / G][NW], const float *__restrict__ pts,
+__device__ __forceinline__ void scatter_tile(const float *__restrict__ pts, int64_t n, uint32_t kb, int64_t base,
+                                             uint32_t out_off, uint32_t (&s_cnt)[kFiltItems / G][NW],
                                              uint32_t *surv_idx, float2 *surv_pts, uint32_t *out_keys,
                                              unsigned long long *out_pay)
 {
     constexpr int ROWS = kFiltItems / G;
-    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
-    const uint32_t lt = (1u << lane) - 1u;
+    constexpr uint32_t RM = (1u << G) - 1u;   // a row's bits among a thread's 16
+    constexpr int PER = ROWS * NW / 32;
+    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id(), lt = (1u << lane) - 1u;
+    float px[kFiltItems], py[kFiltItems];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-        uint32_t pre = s_off[r][warp];
+        const int64_t i = item_point<G>(base, tid, r * G);
+        if constexpr (G == 2) {
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if ((kb >> (2 * r)) & 3u) {
+                if (i + 1 < n) {
+                    v = __ldcs(reinterpret_cast<const float4 *>(pts) + i / 2);
+                } else {
+                    const float2 a = reinterpret_cast<const float2 *>(pts)[i];
+                    v = make_float4(a.x, a.y, 0.0f, 0.0f);
+                }
+            }
+            px[2 * r] = v.x;
+            py[2 * r] = v.y;
+            px[2 * r + 1] = v.z;
+            py[2 * r + 1] = v.w;
+        } else {
+            float2 v = make_float2(0.0f, 0.0f);
+            if ((kb >> r) & 1u) v = __ldcs(reinterpret_cast<const float2 *>(pts) + i);
+            px[r] = v.x;
+            py[r] = v.y;
+        }
+    }
 #pragma unroll
-        for (int h = 0; h < G; ++h) pre += __popc(__ballot_sync(0xffffffffu, (keep >> (r * G + h)) & 1u) & lt);
+    for (int r = 0; r < ROWS; ++r) {
+        const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(kb & (RM << (r * G))));
+        if (lane == 0) s_cnt[r][warp] = c;
+    }
+    __syncthreads();
+    // lane l holds the counts l * PER .. of the rows' warps, row-major: the point order
+    const uint32_t *flat = &s_cnt[0][0];
+    uint32_t loc[PER], sum = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        loc[k] = sum;
+        sum += flat[lane * PER + k];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += u;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) loc[k] += out_off + incl - sum;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const uint32_t e = (uint32_t)r * NW + warp;   // this warp's place among the counts
+        uint32_t pos = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const uint32_t v = __shfl_sync(0xffffffffu, loc[k], e / PER);
+            if (e % PER == (uint32_t)k) pos = v;
+        }
+#pragma unroll
+        for (int h = 0; h < G; ++h) pos += __popc(__ballot_sync(0xffffffffu, (kb >> (r * G + h)) & 1u) & lt);
 #pragma unroll
         for (int h = 0; h < G; ++h) {
-            if ((keep >> (r * G + h)) & 1u) {
-                const int64_t pos = (int64_t)excl + pre;
-                const int64_t i = item_point<G>(base, tid, r * G + h);
-                const uint32_t idx = (uint32_t)i;
-                const float2 p = input_point(pts, i);
-                if constexpr (KEYS) {
-                    out_keys[pos] = ord_key(p.x);
-                    out_pay[pos] = ((unsigned long long)ord_key(p.y) << 32) | idx;
-                } else {
-                    surv_idx[pos] = idx;
-                    if (surv_pts) surv_pts[pos] = p;
-                }
-                ++pre;
+            const int q = r * G + h;
+            if (!((kb >> q) & 1u)) continue;
+            const uint32_t idx = (uint32_t)item_point<G>(base, tid, q);
+            if constexpr (KEYS) {
+                out_keys[pos] = ord_key(px[q]);
+                out_pay[pos] = ((unsigned long long)ord_key(py[q]) << 32) | idx;
+            } else {
+                surv_idx[pos] = idx;
+                if (surv_pts) surv_pts[pos] = make_float2(px[q], py[q]);
             }
-        }
-    }
-}
-
-// One warp writes the kept points of one tile in point order, from the
-// stored keep bits: the tile's 256 filter threads in eight groups of 32
-// (group k holds threads 32 k + lane), each thread with kFiltItems / G rows
-// of G points (point base + (r * 256 + t) * G + h).  The warp first counts
-// every row's kept points (each row's first output position), asks L2 for
-// all of its lanes' kept points at once, then per group loads the group's
-// kept rows together and writes them (the warps of a block take different
-// tiles and never wait on one another).
-template <int G, bool KEYS>
-__device__ __forceinline__ void scatter_tile_warp(const float *__restrict__ pts, int64_t n,
-                                                  const uint16_t *__restrict__ tbits, int64_t base, uint32_t out_off,
-                                                  uint32_t *surv_idx, float2 *surv_pts, uint32_t *out_keys,
-                                                  unsigned long long *out_pay)
-{
-    constexpr int ROWS = kFiltItems / G;
-    constexpr uint32_t RM = (1u << G) - 1u;   // a row's bits among a thread's 16
-    const uint32_t lane = lane_id(), lt = (1u << lane) - 1u;
-    uint32_t kb[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) kb[k] = tbits[k * 32 + lane];
-    uint32_t racc[ROWS];   // next output position of row r
-    {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = kb[2 * j] | (kb[2 * j + 1] << 16);
-        uint32_t run = out_off;
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            const uint32_t m = (RM << (r * G)) * 0x10001u;
-            uint32_t c = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) c += __popc(w[j] & m);
-            racc[r] = run;
-            run += __reduce_add_sync(0xffffffffu, c);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            if ((kb[k] >> (r * G)) & RM)
-                prefetch_l2(pts + 2 * (base + (int64_t)(r * kFiltThreads + k * 32 + lane) * G));
-        }
-    }
-    const auto put = [&](uint32_t pos, float x, float y, uint32_t idx) {
-        if constexpr (KEYS) {
-            out_keys[pos] = ord_key(x);
-            out_pay[pos] = ((unsigned long long)ord_key(y) << 32) | idx;
-        } else {
-            surv_idx[pos] = idx;
-            if (surv_pts) surv_pts[pos] = make_float2(x, y);
-        }
-    };
-    // (one group at a time: its bits again from L1, so that the compiler
-    // keeps one group's loads in registers, not all eight)
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-        const uint32_t kbk = tbits[k * 32 + lane];
-        if (!__any_sync(0xffffffffu, kbk != 0u)) continue;
-        const uint32_t t = k * 32 + lane;
-        if constexpr (G == 2) {
-            float4 v[ROWS];
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                v[r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if ((kbk >> (2 * r)) & 3u) {
-                    const int64_t i = base + (int64_t)(r * kFiltThreads + t) * 2;
-                    if (i + 1 < n) {
-                        v[r] = __ldcs(reinterpret_cast<const float4 *>(pts) + i / 2);
-                    } else {
-                        const float2 a = reinterpret_cast<const float2 *>(pts)[i];
-                        v[r] = make_float4(a.x, a.y, 0.0f, 0.0f);
-                    }
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const uint32_t m = (kbk >> (2 * r)) & 3u;
-                const uint32_t b0 = __ballot_sync(0xffffffffu, m & 1u), b1 = __ballot_sync(0xffffffffu, m & 2u);
-                if (!(b0 | b1)) continue;
-                uint32_t pos = racc[r] + __popc(b0 & lt) + __popc(b1 & lt);
-                racc[r] += __popc(b0) + __popc(b1);
-                const uint32_t idx = (uint32_t)(base + (int64_t)(r * kFiltThreads + t) * 2);
-                if (m & 1u) put(pos++, v[r].x, v[r].y, idx);
-                if (m & 2u) put(pos, v[r].z, v[r].w, idx + 1u);
-            }
-        } else {   // 16 rows of one point: two halves of 8 loads
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float2 v[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int r = 8 * h + q;
-                    v[q] = make_float2(0.0f, 0.0f);
-                    if ((kbk >> r) & 1u) v[q] = __ldcs(reinterpret_cast<const float2 *>(pts) + base + r * kFiltThreads + t);
-                }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int r = 8 * h + q;
-                    const uint32_t m = (kbk >> r) & 1u;
-                    const uint32_t b0 = __ballot_sync(0xffffffffu, m);
-                    if (!b0) continue;
-                    const uint32_t pos = racc[r] + __popc(b0 & lt);
-                    racc[r] += __popc(b0);
-                    if (m) put(pos, v[q].x, v[q].y, (uint32_t)(base + r * kFiltThreads + t));
-                }
-            }
+            ++pos;
         }
     }
 }
@@ -322,7 +225,8 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
 {
     kernel_entry();
     __shared__ OctSmem so;
-    __shared__ uint32_t s_off[kFiltItems / G][NW];
+    __shared__ uint32_t s_row[kFiltItems / G][NW];
+    __shared__ uint32_t s_w[NW];
     __shared__ uint32_t s_tile;
     __shared__ unsigned long long s_excl;
     __shared__ uint32_t s_total;
@@ -342,10 +246,11 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
         if (tile >= ntiles) break;
         const int64_t base = tile * kFiltTile;
         const uint32_t keep = load_test<G, BOX>(pts, n, base, so);
-        row_counts<G>(keep, s_off);
+        const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(keep));
+        if (lane == 0) s_w[warp] = c;
         __syncthreads();
         if (warp == 0) {
-            const uint32_t total = scan_rows_warp0<G>(s_off);
+            const uint32_t total = __reduce_add_sync(0xffffffffu, lane < (uint32_t)NW ? s_w[lane] : 0u);
             unsigned long long excl = 0;
             if (tile == 0) {
                 if (lane == 0) st_release_u64(status, kFlagP | total);
@@ -362,8 +267,8 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
         }
         __syncthreads();
         if (s_total != 0)
-            scatter_tile<G, KEYS>(keep, base, s_excl, s_off, pts, surv_idx, surv_pts, at<uint32_t>(ws, L.keys[0]),
-                                  at<unsigned long long>(ws, L.pay[0]));
+            scatter_tile<G, KEYS>(pts, n, keep, base, (uint32_t)s_excl, s_row, surv_idx, surv_pts,
+                                  at<uint32_t>(ws, L.keys[0]), at<unsigned long long>(ws, L.pay[0]));
         __syncthreads();
     }
 }
@@ -556,11 +461,10 @@ __global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const flo
     const uint32_t lane = lane_id();
     // a contiguous range of tiles per block, so the scatter pass finds
     // every tile's output offset from the block totals and its own range
-    const int64_t per = ceil_div(ntiles, (int64_t)gridDim.x);
-    const int64_t t1 = min(ntiles, (int64_t)(blockIdx.x + 1) * per);
+    const int64_t t0 = first_tile(ntiles, gridDim.x, blockIdx.x), t1 = first_tile(ntiles, gridDim.x, blockIdx.x + 1);
     uint32_t part = 0;   // this thread's share of the block total
     bool first = true, lockstep = true;
-    for (int64_t w0 = (int64_t)blockIdx.x * per; w0 < t1; w0 += kCountRing) {
+    for (int64_t w0 = t0; w0 < t1; w0 += kCountRing) {
         const int64_t w1 = min(t1, w0 + kCountRing);
         for (int64_t tile = w0; tile < w1; ++tile) {
             if (threadIdx.x == 0 && tile + 1 < t1) {   // the next tile streams into L2 meanwhile
@@ -613,6 +517,7 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
     __shared__ uint32_t s_list[kFiltThreads];    // non-empty tiles of a chunk: offset in chunk
     __shared__ uint32_t s_loff[kFiltThreads];    // and their output offsets
     __shared__ uint32_t s_nlist;
+    __shared__ uint32_t s_row[2][kFiltItems / G][NW];
     __shared__ uint32_t s_spec;
     __shared__ SpecScatterSmem s_sp;
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
@@ -663,8 +568,7 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
     }
     if (blockIdx.x == 0 && tid == 0) write_count(KEYS, ctrl, surv_count, total);
     __syncthreads();   // s_red is reused below
-    const int64_t per = ceil_div(ntiles, (int64_t)gridDim.x);
-    const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(ntiles, r0 + per);
+    const int64_t r0 = first_tile(ntiles, gridDim.x, blockIdx.x), r1 = first_tile(ntiles, gridDim.x, blockIdx.x + 1);
     uint32_t run = before;
     for (int64_t c0 = r0; c0 < r1; c0 += kFiltThreads) {
         // this chunk's tile counts: exclusive scan and the non-empty ones
@@ -700,10 +604,14 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
         if (tid == 0) s_nlist = nlist;
         __syncthreads();
         const uint32_t nl = s_nlist;
-        for (uint32_t li = warp; li < nl; li += NW)
-            scatter_tile_warp<G, KEYS>(pts, n, bits + (c0 + s_list[li]) * kFiltThreads, (c0 + s_list[li]) * kFiltTile,
-                                       s_loff[li], surv_idx, surv_pts, out_keys, out_pay);
-        __syncthreads();   // s_list, s_loff and s_red are rebuilt for the next chunk
+        uint32_t kb = nl ? bits[(c0 + s_list[0]) * kFiltThreads + tid] : 0u;
+        for (uint32_t li = 0; li < nl; ++li) {
+            const uint32_t mine = kb;
+            if (li + 1 < nl) kb = bits[(c0 + s_list[li + 1]) * kFiltThreads + tid];
+            scatter_tile<G, KEYS>(pts, n, mine, (c0 + s_list[li]) * kFiltTile, s_loff[li], s_row[li & 1u], surv_idx,
+                                  surv_pts, out_keys, out_pay);
+        }
+        __syncthreads();   // s_list, s_loff, s_row and s_red are written again for the next chunk
         run += chunk_total;
     }
 }

@@ -314,11 +314,10 @@ __global__ void __launch_bounds__(kFiltThreads) kx_count_kernel(const float *__r
     unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
     uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
     const int64_t ntiles = ceil_div(n, (int64_t)kFiltTile);
-    const int64_t per = ceil_div(ntiles, (int64_t)gridDim.x);
-    const int64_t t1 = std::min<int64_t>(ntiles, (int64_t)(blockIdx.x + 1) * per);
+    const int64_t t1 = first_tile(ntiles, gridDim.x, blockIdx.x + 1);
     const uint32_t t = threadIdx.x, warp = t >> 5, lane = lane_id();
     uint32_t block_total = 0;
-    for (int64_t tile = (int64_t)blockIdx.x * per; tile < t1; ++tile) {
+    for (int64_t tile = first_tile(ntiles, gridDim.x, blockIdx.x); tile < t1; ++tile) {
         const int64_t base = tile * kFiltTile;
         if (t == 0 && tile + 1 < t1) {   // the next tile streams into L2 meanwhile
             const int64_t nb = base + kFiltTile;
@@ -557,7 +556,6 @@ __global__ void __launch_bounds__(ST) kx_sv_refine_kernel(const float *__restric
     uint32_t *bsum = at<uint32_t>(ws, L.filt_bsum);
     const float2 *p2 = reinterpret_cast<const float2 *>(pts);
     const int64_t ntiles = ceil_div(n, (int64_t)kFiltTile);
-    const int64_t per_block = ceil_div(ntiles, (int64_t)bc);
     const uint32_t t = threadIdx.x, lane = lane_id();
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const uint32_t kb = bits[tile * kFiltThreads + t];
@@ -573,7 +571,7 @@ __global__ void __launch_bounds__(ST) kx_sv_refine_kernel(const float *__restric
         for (int o = 16; o > 0; o >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, o);
         if (lane == 0 && removed) {
             atomicAdd(&status[tile], 0ull - (unsigned long long)removed);
-            atomicSub(&bsum[tile / per_block], removed);
+            atomicSub(&bsum[tile_block(ntiles, bc, tile)], removed);
         }
     }
 }
