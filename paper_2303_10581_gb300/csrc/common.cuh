@@ -95,6 +95,7 @@ struct ExtCtrl {
 // them, as many as one block's shared memory holds)
 constexpr int kFanBins = 27648;
 
+constexpr uint32_t kKgonMinS = 1u << 16;   // fewer octagon survivors: not worth a fan
 struct KgonCtrl {                          // zeroed with the control block
     unsigned long long slot[kFanBins];     // packed (far_key << 32 | ~index): farthest sampled input point per bin
     uint32_t sample, inside;               // points sampled for the bins, octagon survivors among them

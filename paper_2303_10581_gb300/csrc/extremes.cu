@@ -17,6 +17,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "fan.cuh"
 #include "launch.h"
 #include "mlp.cuh"
 
@@ -61,6 +62,13 @@ __device__ __forceinline__ void combine(float &k, uint32_t &i, float ok, uint32_
     }
 }
 
+// A power of two g with g v in [1, 2) (v = 0, or out of g's range: near it).
+__device__ __forceinline__ float pow2_inverse(float v)
+{
+    const int e = (int)(__float_as_uint(v) >> 23) - 127;   // v >= 0
+    return __uint_as_float((uint32_t)(127 - max(-126, min(e, 126))) << 23);
+}
+
 }  // namespace
 
 // Builds the filter polygon from the eight vertex indices.  Run by one full
@@ -90,33 +98,40 @@ __device__ __forceinline__ void combine(float &k, uint32_t &i, float ok, uint32_
 // The affine form of edge k (octtest.cuh), with c the box centre, u* = px -
 // cx, v* = py - cy exactly, (ex, ey) = b - a and K = ex (ay - cy) - ey (ax -
 // cx): the orientation is t = -ey u* + ex v* - K.  Let U >= |u*|, V >= |v*|
-// over the box, S = |ey| U + |ex| V + |K| and s = 2^21 / S.  The form has the
-// coefficients fl(-ey s), fl(ex s), fl(-K s) (binary64, rounded once) and
-// takes fl(u*), fl(v*) and two FMAs: each of its three terms gets at most
-// four relative errors of eps = 2^-24 (coefficient, difference, two FMAs),
-// so |T - s t| <= 4 eps s S (1 + 2^-20) < 0.51 < 1 for every point of the
-// box (underflows are below 2^-20: every term is at most 2^21 and the form
-// only decides values beyond 1).  An edge of zero length gets T = 2.  When
-// the box is not finite or a coefficient overflows, all forms are zero: T =
-// 0, undecided.
+// over the box, S >= |ey| U + |ex| V + |K| and s <= 2^21 / S.  The form has
+// the coefficients -fl(fl(ey) s), fl(fl(ex) s), -fl(fl(K) s) and takes fl(u*),
+// fl(v*) and two FMAs: each of its three terms gets at most five relative
+// errors of eps = 2^-24 (two in the coefficient, difference, two FMAs), so
+// |T - s t| <= 5 eps s S (1 + 2^-20) < 0.64 < 1 for every point of the box
+// (underflows are below 2^-20: every term is at most 2^21 and the form only
+// decides values beyond 1).  K, a difference of products, is the sum of two
+// binary32 numbers to 2^-40 of S before it is rounded.  x and y are first
+// scaled by powers of two that bring the box near [1, 2) x [1, 2), so no
+// product overflows or loses bits that count.  An edge of zero length gets T
+// = 2.  When the box is not finite or a coefficient overflows, all forms are
+// zero: T = 0, undecided.  (In binary64, whose instructions take some 70
+// cycles each here, the forms took 4900 cycles of this serial tail.)
 //
 // A closed axis-aligned rectangle whose four corners are, exactly, strictly
 // left of every valid edge lies strictly inside the polygon (the region
 // "strictly left of every edge" is an intersection of open half-planes,
-// hence convex); points in it are discarded with four comparisons.  The
-// largest of a few concentric candidates that passes is kept.
+// hence convex); points in it are discarded with four comparisons.  Among
+// the rectangles similar to the box and concentric with it the largest is
+// found edge by edge (t at a corner is -K minus a multiple of the size),
+// taken a little smaller and proven; one that fails is halved.
 __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_t *ext8, Octagon *out, bool data_extremes)
 {
     const uint32_t lane = lane_id();
     const uint32_t k = lane & 7u;
     const float2 a = pts[ext8[k]];
-    const float2 b = pts[ext8[(k + 1) & 7u]];
+    const auto of = [&](float v, int j) { return __shfl_sync(0xffffffffu, v, j); };
+    const float2 b = make_float2(of(a.x, (k + 1) & 7u), of(a.y, (k + 1) & 7u));
     float xmax, ymax, xmin, ymin;
     if (data_extremes) {   // bounding box from R, T, L, B
-        xmax = pts[ext8[0]].x;
-        ymax = pts[ext8[2]].y;
-        xmin = pts[ext8[4]].x;
-        ymin = pts[ext8[6]].y;
+        xmax = of(a.x, 0);
+        ymax = of(a.y, 2);
+        xmin = of(a.x, 4);
+        ymin = of(a.y, 6);
     } else {               // bounding box of all eight vertices (lanes k, k ^ 1, ... of each group of 8)
         xmax = xmin = a.x;
         ymax = ymin = a.y;
@@ -131,14 +146,12 @@ __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_
     const bool valid = !(a.x == b.x && a.y == b.y);
     const float dx = __fsub_rn(b.x, a.x), dy = __fsub_rn(b.y, a.y);
     const float W = __fsub_rn(xmax, xmin), H = __fsub_rn(ymax, ymin);
+    const bool finite = W <= 3.0e38f && H <= 3.0e38f;
     float bound = __int_as_float(0x7f800000);  // +inf: binary32 test off
-    if (W <= 3.0e38f && H <= 3.0e38f) {
-        double M = __dadd_ru(__dmul_ru(fabs((double)dx), (double)H), __dmul_ru(fabs((double)dy), (double)W));
-        M = __dmul_ru(M, 1.0 + 0x1p-20);
-        if (M <= 0x1p100) {
-            double B = __dadd_ru(__dmul_ru(M, 0x1p-22), 0x1p-140);
-            bound = __double2float_ru(B);
-        }
+    if (finite) {
+        const float M =
+            __fmul_ru(__fadd_ru(__fmul_ru(fabsf(dx), H), __fmul_ru(fabsf(dy), W)), 1.0f + 0x1p-20f);
+        if (M <= 0x1p100f) bound = __fadd_ru(__fmul_ru(M, 0x1p-22f), 0x1p-140f);
     }
     const uint32_t vmask = __ballot_sync(0xffffffffu, valid) & 0xffu;
     if (lane < 8) {
@@ -150,36 +163,51 @@ __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_
         out->dy[k] = dy;
         out->bound[k] = bound;
     }
-    const double cxd = 0.5 * ((double)xmin + (double)xmax);
-    const double cyd = 0.5 * ((double)ymin + (double)ymax);
+    // (halves first: the sum cannot overflow)
+    const float cx = __fadd_rn(0.5f * xmin, 0.5f * xmax), cy = __fadd_rn(0.5f * ymin, 0.5f * ymax);
+    const float gx = pow2_inverse(W), gy = pow2_inverse(H);
+    const float U = __fmul_ru(gx, fmaxf(__fsub_ru(xmax, cx), __fsub_ru(cx, xmin)));
+    const float V = __fmul_ru(gy, fmaxf(__fsub_ru(ymax, cy), __fsub_ru(cy, ymin)));
+    float ex, exl, ey, eyl, px, pxl, py, pyl;   // the edge and its first vertex from c, scaled, as pairs
+    two_diff(b.x, a.x, ex, exl);
+    two_diff(b.y, a.y, ey, eyl);
+    two_diff(a.x, cx, px, pxl);
+    two_diff(a.y, cy, py, pyl);
+    ex *= gx, exl *= gx, px *= gx, pxl *= gx;
+    ey *= gy, eyl *= gy, py *= gy, pyl *= gy;
+    const float q = __fmul_rn(ex, py), w = __fmul_rn(ey, px);
+    const float ql = __fmaf_rn(ex, py, -q) + (ex * pyl + exl * py), wl = __fmaf_rn(ey, px, -w) + (ey * pxl + eyl * px);
+    float Kh, Kl;
+    two_diff(q, w, Kh, Kl);
+    const float K = __fadd_rn(Kh, Kl + (ql - wl));
+    const float S = __fmul_ru(__fadd_ru(__fadd_ru(__fmul_ru(fabsf(ey), U), __fmul_ru(fabsf(ex), V)), fabsf(K)),
+                              1.0f + 0x1p-20f);
     {
-        const double cx = (double)(float)cxd, cy = (double)(float)cyd;
-        const double ex = (double)b.x - a.x, ey = (double)b.y - a.y;
-        const double K = ex * ((double)a.y - cy) - ey * ((double)a.x - cx);
-        const double U = fmax((double)xmax - cx, cx - (double)xmin), V = fmax((double)ymax - cy, cy - (double)ymin);
-        const double sc = 0x1p21 / ((fabs(ey) * U + fabs(ex) * V + fabs(K)) * (1.0 + 0x1p-20));
-        const float tx = (float)(-ey * sc), ty = (float)(ex * sc), tz = (float)(-K * sc);
+        const float sc = fminf(__fdiv_rd(0x1p21f, S), 0x1p126f);
+        const float tx = -(ey * sc) * gx, ty = (ex * sc) * gy, tz = -(K * sc);
         const bool fin = !valid || (fabsf(tx) <= 3.0e38f && fabsf(ty) <= 3.0e38f && fabsf(tz) <= 3.0e38f);
-        const bool on = __all_sync(0xffffffffu, fin && W <= 3.0e38f && H <= 3.0e38f);
+        const bool on = __all_sync(0xffffffffu, fin && finite);
         if (lane < 8) {
             out->tx[k] = on && valid ? tx : 0.0f;
             out->ty[k] = on && valid ? ty : 0.0f;
             out->tz[k] = on ? (valid ? tz : 2.0f) : 0.0f;
         }
     }
-    const double hw = 0.5 * ((double)xmax - (double)xmin);
-    const double hh = 0.5 * ((double)ymax - (double)ymin);
     // quick-discard rectangle: lane = (corner c = lane / 8, edge k)
     float xl = 1.0f, xh = -1.0f, yl = 1.0f, yh = -1.0f;  // empty
     if (vmask != 0) {
-        const double fr[8] = {0.80, 0.74, 0.68, 0.62, 0.55, 0.45, 0.35, 0.25};
-        for (int j = 0; j < 8; ++j) {
-            const float rxl = (float)(cxd - fr[j] * hw), rxh = (float)(cxd + fr[j] * hw);
-            const float ryl = (float)(cyd - fr[j] * hh), ryh = (float)(cyd + fr[j] * hh);
-            const uint32_t c = lane >> 3;
-            const float px = (c == 0 || c == 3) ? rxl : rxh;
-            const float py = (c < 2) ? ryl : ryh;
-            bool ok = !valid || orient(a.x, a.y, b.x, b.y, px, py) > 0;
+        const float hw = 0.5f * W, hh = 0.5f * H;
+        float f = -K / (fabsf(ey) * (gx * hw) + fabsf(ex) * (gy * hh));   // (K < 0: c is inside edge k)
+        f = valid && finite ? (f > 0.0f ? f : 0.0f) : 1.0f;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) f = fminf(f, __shfl_xor_sync(0xffffffffu, f, o));
+        f *= 1.0f - 0x1p-10f;
+        const uint32_t c = lane >> 3;
+        for (int tries = 0; tries < 3 && f > 0.02f; ++tries, f *= 0.5f) {
+            const float rxl = cx - f * hw, rxh = cx + f * hw, ryl = cy - f * hh, ryh = cy + f * hh;
+            const float qx = (c == 0 || c == 3) ? rxl : rxh;
+            const float qy = (c < 2) ? ryl : ryh;
+            bool ok = !valid || orient(a.x, a.y, b.x, b.y, qx, qy) > 0;
             if (!(rxl <= rxh && ryl <= ryh)) ok = false;
             if (__all_sync(0xffffffffu, ok)) {
                 xl = rxl;
@@ -198,8 +226,8 @@ __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_
         out->xh = xh;
         out->yl = yl;
         out->yh = yh;
-        out->cx = (float)cxd;
-        out->cy = (float)cyd;
+        out->cx = cx;
+        out->cy = cy;
         out->bxl = xmin;
         out->bxh = xmax;
         out->byl = ymin;
@@ -334,7 +362,8 @@ template <bool SPEC>
 __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *__restrict__ pts, int64_t n,
                                                                   void *ws, Layout L, uint32_t *ext8_out,
                                                                   int build_polygon, unsigned long long *zero_ptr,
-                                                                  int64_t zero_words, uint32_t cap,
+                                                                  int64_t zero_words, int64_t skip0, int64_t skip1,
+                                                                  uint32_t cap,
                                                                   const __nv_bfloat16 *learn, float *learn_dirs,
                                                                   int32_t *learn_k)
 {
@@ -349,7 +378,8 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
     // clear what the following kernels of this call expect to be zero
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gthreads = (int64_t)nsweep * blockDim.x;
-    for (int64_t w = gtid; w < zero_words; w += gthreads) zero_ptr[w] = 0ull;
+    for (int64_t w = gtid; w < skip0; w += gthreads) zero_ptr[w] = 0ull;
+    for (int64_t w = skip1 + gtid; w < zero_words; w += gthreads) zero_ptr[w] = 0ull;
 
     bool nan_seen = false;
     // full tiles: this thread's largest key per slot and (in shared memory)
@@ -558,61 +588,53 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
         for (int j = 0; j < 8; ++j)
             if (wslot == j) combine(b.k[j], b.i[j], wkey, widx);
     }
-    // warp reduction
+    // warp reduction: the largest key, then the lowest index that has it,
+    // packed so that the larger value is the better one (0: no point)
+    __shared__ unsigned long long s_best[kExtThreads / 32][8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float ok = __shfl_xor_sync(0xffffffffu, b.k[j], o);
-            const uint32_t oi = __shfl_xor_sync(0xffffffffu, b.i[j], o);
-            combine(b.k[j], b.i[j], ok, oi);
-        }
+    for (int j = 0; j < 8; ++j) {
+        const uint32_t key = b.i[j] != 0xffffffffu ? ord_key(b.k[j]) : 0u;
+        const uint32_t m = __reduce_max_sync(0xffffffffu, key);
+        const uint32_t i = __reduce_min_sync(0xffffffffu, key == m ? b.i[j] : 0xffffffffu);
+        if (lane == 0) s_best[warp][j] = i != 0xffffffffu ? ((unsigned long long)m << 32) | (uint32_t)~i : 0ull;
     }
-    __shared__ float sk[kExtThreads / 32][8];
-    __shared__ uint32_t si[kExtThreads / 32][8];
-    __shared__ int s_nonfinite;
     __shared__ bool s_last;
-    if (threadIdx.x == 0) s_nonfinite = 0;
-    __syncthreads();
-    if (nan_seen) s_nonfinite = 1;
-    if (lane == 0) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            sk[warp][j] = b.k[j];
-            si[warp][j] = b.i[j];
-        }
-    }
-    __syncthreads();
+    const bool nans = __syncthreads_or(nan_seen);
+    unsigned long long packed = 0;   // warp 0, lane j < 8: slot j's best over the block
     if (warp == 0) {
-        // lane j < 8 folds slot j over the block's warps
-        if (lane < 8) {
-            float k = sk[0][lane];
-            uint32_t i = si[0][lane];
-            for (int w = 1; w < kExtThreads / 32; ++w) combine(k, i, sk[w][lane], si[w][lane]);
-            if (i != 0xffffffffu) {
-                const unsigned long long packed = ((unsigned long long)ord_key(k) << 32) | (uint32_t)~i;
-                atomicMax(&ctrl->ext_slot[lane], packed);
-            }
-        }
-        if (lane == 0 && s_nonfinite) atomicOr(&ctrl->nonfinite, 1u);
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) s_last = atomicAdd(&ctrl->ext_done, 1u) == nsweep - 1;
+        // lane = (slot, every fourth warp)
+        for (uint32_t w = lane >> 3; w < (uint32_t)kExtThreads / 32; w += 4) packed = max(packed, s_best[w][lane & 7u]);
+        packed = max(packed, __shfl_xor_sync(0xffffffffu, packed, 8));
+        packed = max(packed, __shfl_xor_sync(0xffffffffu, packed, 16));
     }
-    __syncthreads();
-    if (!s_last || warp != 0) return;
+    uint32_t bad = 0;
+    if (nsweep == 1u) {   // this block saw every point
+        if (warp != 0) return;
+        bad = nans ? 1u : 0u;
+    } else {
+        if (warp == 0) {
+            if (lane < 8 && packed) atomicMax(&ctrl->ext_slot[lane], packed);
+            if (lane == 0 && nans) atomicOr(&ctrl->nonfinite, 1u);
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) s_last = atomicAdd(&ctrl->ext_done, 1u) == nsweep - 1;
+        }
+        __syncthreads();
+        if (!s_last || warp != 0) return;
 
-    // last block: decode, reset the slots for the next call, build polygon
-    __threadfence();
+        // last block: take the slots, reset them for the next call
+        __threadfence();
+        if (lane < 8) packed = atomicExch(&ctrl->ext_slot[lane], 0ull);
+        if (lane == 8) bad = atomicExch(&ctrl->nonfinite, 0u);
+        if (lane == 0) ctrl->ext_done = 0;
+    }
+    // decode, build the polygon
     __shared__ uint32_t s_ext[8];
     if (lane < 8) {
-        const unsigned long long packed = atomicExch(&ctrl->ext_slot[lane], 0ull);
         const uint32_t idx = ~(uint32_t)packed;
         s_ext[lane] = idx;
         ext8_out[lane] = idx;
     }
-    uint32_t bad = lane == 0 ? atomicExch(&ctrl->nonfinite, 0u) : 0u;
-    if (lane == 0) ctrl->ext_done = 0;
     __syncwarp();
     // an infinite coordinate makes an infinite R, T, L or B vertex (a slot
     // left without a point means its keys were all NaN, already flagged)
@@ -1026,6 +1048,11 @@ cudaError_t launch_extremes(const float *pts, int64_t n, void *ws, const Layout 
 {
     const __nv_bfloat16 *learn = static_cast<const __nv_bfloat16 *>(learn_params);
     const unsigned extra = learn ? 1u : 0u;
+    // the fan's bins (221 KB) stay as they are when no fan is made: a call on
+    // few points has one block, which took 4 us to clear them
+    const int64_t bins0 = (int64_t)(L.kgon_ctrl - L.ctrl) / 8;
+    const bool no_fan = zero_words > bins0 + kFanBins && n < (int64_t)kKgonMinS;
+    const int64_t skip0 = no_fan ? bins0 : zero_words, skip1 = no_fan ? bins0 + kFanBins : zero_words;
     const int64_t pairs = (n + 1) / 2;
     const int64_t tiles = ceil_div(pairs, (int64_t)kExtPairs);
     // the speculative sweep: large sets only, one candidate segment per
@@ -1040,7 +1067,7 @@ cudaError_t launch_extremes(const float *pts, int64_t n, void *ws, const Layout 
             spec_sample_kernel<<<kSampleBlocks, kSampleThreads, 0, st>>>(pts, n, ws, L, (uint32_t)blocks,
                                                                          (uint32_t)cap);
             launch_next(extremes_kernel<true>, (unsigned)blocks + extra, kExtThreads, 0, st, pts, n, ws, L, ext8, 1, zero_ptr,
-                                                                                   zero_words, (uint32_t)cap, learn,
+                                                                                   zero_words, skip0, skip1, (uint32_t)cap, learn,
                                                                                    learn_dirs, learn_k);
             note_kernels(CH_K_EXTREMES, 2);
             probe_after(CH_K_EXTREMES, st);
@@ -1053,7 +1080,7 @@ cudaError_t launch_extremes(const float *pts, int64_t n, void *ws, const Layout 
     if (blocks < 1) blocks = 1;
     probe_before(CH_K_EXTREMES, st);
     extremes_kernel<false><<<(unsigned)blocks + extra, kExtThreads, 0, st>>>(pts, n, ws, L, ext8, build_polygon ? 1 : 0,
-                                                                             zero_ptr, zero_words, 0u, learn,
+                                                                             zero_ptr, zero_words, skip0, skip1, 0u, learn,
                                                                              learn_dirs, learn_k);
     note_kernels(CH_K_EXTREMES, 1);
     probe_after(CH_K_EXTREMES, st);

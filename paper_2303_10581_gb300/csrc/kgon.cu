@@ -65,7 +65,6 @@ namespace {
 
 constexpr int CT = 768;                  // threads per block of the filter pass: groups
 constexpr int CG = CT / kFiltThreads;    // groups of kFiltThreads, each with its own tiles
-constexpr uint32_t kKgonMinS = 1u << 16; // fewer octagon survivors: not worth a pass
 constexpr int kFanTable = (kFanBins + 4) * 8;  // vertices, the last again before them and the first two after them (and padding)
 constexpr int kQueue = 64;                     // points a warp of the filter pass queues (under 32, and 32 more)
 constexpr uint32_t kMany = 128;                // a warp's survivors of a tile that go straight to the list
