@@ -175,9 +175,7 @@ extern "C" ch_status ch_hull_kgon(const float *pts, int64_t n, const float *dirs
         e = launch_filter_scatter(pts, n, grid, ws, L, nullptr, nullptr, nullptr, true, st);
         probe_after(CH_K_FILTER, st);
     }
-    if (e == cudaSuccess) e = launch_small_hull(ws, L, hull_idx, hull_count, st);
-    if (e == cudaSuccess) e = launch_sort(ws, L, st);
-    if (e == cudaSuccess) e = launch_chain(ws, L, hull_idx, hull_count, st);
+    if (e == cudaSuccess) e = launch_hull_stage(ws, L, hull_idx, hull_count, st);
     return cuda_status(e);
 }
 
@@ -195,9 +193,7 @@ cudaError_t hull_pipeline(const float *pts, int64_t n, uint32_t *hull_idx, uint3
                                     learn_params, learn_dirs, learn_k);
     if (e == cudaSuccess)
         e = variant == 1 ? launch_filter_keys_single(pts, n, ws, L, st) : launch_hull_filter(pts, n, ws, L, kg, st);
-    if (e == cudaSuccess) e = launch_small_hull(ws, L, hull_idx, hull_count, st);
-    if (e == cudaSuccess) e = launch_sort(ws, L, st);
-    if (e == cudaSuccess) e = launch_chain(ws, L, hull_idx, hull_count, st);
+    if (e == cudaSuccess) e = launch_hull_stage(ws, L, hull_idx, hull_count, st);
     return e;
 }
 

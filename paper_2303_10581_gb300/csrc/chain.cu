@@ -62,6 +62,9 @@ constexpr int CS = kChainStride;    // chain slots per super-chunk
 constexpr int NL = SC + 2;          // sequence capacity: SC points + 2 look-ahead slots
 constexpr int NWB = LT / 32;        // warps per block
 constexpr int kLongRun = 32;        // a longer run of equal x is reduced by a warp
+constexpr int kCopyParts = 4;                  // a range is shared by so many warps
+constexpr int kCopyLen = CS / kCopyParts;      // entries per part
+static_assert(CS % kCopyParts == 0, "parts cover a super-chunk's slots");
 constexpr int LWMAX = ((NL + NWB - 1) / NWB + 31) / 32;   // longest leaf (17)
 
 // pop / advance test: lower chains drop a vertex when the turn is not
@@ -177,10 +180,16 @@ __device__ void merge_walk(Acc &A, int side, int fa, int la, int fb, int lb)
 // ---------------------------------------------------------------------------
 struct ChainSmem {
     float2 pts[NL];               // staged points; [SC], [SC+1]: look-ahead lowest / highest
-    uint16_t list[3][NL];         // run starts, sequences and elimination ping-pong
-    uint8_t stk[LWMAX * LT];      // leaf stacks: entry j of leaf t at [j * LT + t]
-    int16_t lb[LT];               // leaf t's first entry in the flat list array
-    int16_t lo[LT], hi[LT], prv[LT], nxt[LT], first[LT], last[LT];
+    union {
+        struct {
+            uint16_t list[3][NL];         // run starts, sequences and elimination ping-pong
+            uint8_t stk[LWMAX * LT];      // leaf stacks: entry j of leaf t at [j * LT + t]
+            int16_t lb[LT];               // leaf t's first entry in the flat list array
+            int16_t lo[LT], hi[LT], prv[LT], nxt[LT], first[LT], last[LT];
+        };
+        unsigned long long tmp[SC];       // local_sort's second buffer (pts is its first)
+    };
+    uint16_t perm[SC];            // unsorted set: staged point -> its place in the input
     uint32_t wsum[LT / 32];
     uint32_t total;
     float red_y[2][LT / 32];      // look-ahead reduction scratch
@@ -463,19 +472,104 @@ __device__ __forceinline__ void block_extreme_y(ChainSmem &s, float ylo, unsigne
     __syncthreads();
 }
 
+// Stages the m <= SC unsorted survivors at `base` in the order of x (equal x
+// in any order): pts and perm.  Each warp sorts 32 keys at a time in registers
+// (a bitonic network), then runs are merged in pairs: every key finds its
+// place from its rank in its own run and a binary search in the other.
+// Bound by latency.  A set that fits one block need not be written back
+// between digits: the histogram and four passes over global memory take 57 us
+// on 4200 survivors, this 27 on 4096.  (Every key by a binary search in the
+// other run instead of the serial merge: 40.)
+__device__ void local_sort(ChainSmem &sm, const ChainPtrs &P, int64_t base, int m)
+{
+    const int t = threadIdx.x, lane = t & 31;
+    const int C = ((m + LT - 1) / LT) | 1;   // outputs per thread and round; odd: no bank conflicts in the stores
+    unsigned long long *src = reinterpret_cast<unsigned long long *>(sm.pts), *dst = sm.tmp;
+    for (int i0 = t - lane; i0 < m; i0 += LT) {
+        const int i = i0 + lane;
+        unsigned long long v = i < m ? ((unsigned long long)__ldg(P.keys + base + i) << 32) | (uint32_t)i : ~0ull;
+#pragma unroll
+        for (int g = 2; g <= 32; g <<= 1) {
+#pragma unroll
+            for (int h = g >> 1; h > 0; h >>= 1) {
+                const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, h);
+                if ((o < v) == (((lane & g) == 0) == ((lane & h) == 0))) v = o;
+            }
+        }
+        if (i < m) src[i] = v;
+    }
+    __syncthreads();
+    for (int w = 32; w < m; w <<= 1) {
+        int o = t * C, pair = o & ~(2 * w - 1);
+        const int end = min(o + C, m);
+        if (o < end) {
+            // places a and b in the pair's two runs before output o
+            int la = min(w, m - pair), lb = min(w, max(0, m - pair - w));
+            int lo = max(0, o - pair - lb), hi = min(o - pair, la);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (src[pair + mid] < src[pair + w + (o - pair) - 1 - mid]) lo = mid + 1;
+                else hi = mid;
+            }
+            int a = lo, b = o - pair - lo;
+            unsigned long long ka = a < la ? src[pair + a] : ~0ull, kb = b < lb ? src[pair + w + b] : ~0ull;
+            for (; o < end; ++o) {
+                if (o == pair + 2 * w) {   // the next pair
+                    pair = o;
+                    la = min(w, m - pair);
+                    lb = min(w, max(0, m - pair - w));
+                    a = b = 0;
+                    ka = src[pair];
+                    kb = lb > 0 ? src[pair + w] : ~0ull;
+                }
+                const bool first = ka < kb;
+                dst[o] = first ? ka : kb;
+                if (first) {
+                    ++a;
+                    ka = a < la ? src[pair + a] : ~0ull;
+                } else {
+                    ++b;
+                    kb = b < lb ? src[pair + w + b] : ~0ull;
+                }
+            }
+        }
+        __syncthreads();
+        unsigned long long *u = src;
+        src = dst;
+        dst = u;
+    }
+    unsigned long long v[SC / LT];
+#pragma unroll
+    for (int k = 0; k < SC / LT; ++k)
+        if (t + k * LT < m) v[k] = src[t + k * LT];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < SC / LT; ++k) {
+        const int i = t + k * LT;
+        if (i >= m) continue;
+        const uint32_t e = (uint32_t)v[k];
+        sm.pts[i] = make_float2(key_float((uint32_t)(v[k] >> 32)), key_float((uint32_t)(__ldg(P.pay + base + e) >> 32)));
+        sm.perm[i] = (uint16_t)e;
+    }
+}
+
 // The chains of one super-chunk: sorted positions [base, base + m) of a set
-// occupying [sbeg, send); results go to chain slot j.  Called by all
-// threads of the block.
+// occupying [sbeg, send); results go to chain slot j.  LOCAL: the super-chunk
+// is a whole set and not sorted yet.  Called by all threads of the block.
+template <bool LOCAL>
 __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t base, int m, int64_t sbeg,
                            int64_t send)
 {
+    const auto place = [&](int e) { return base + (LOCAL ? (int)sm.perm[e] : e); };   // of a staged point
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const float kInf = __int_as_float(0x7f800000);
     const int64_t sc = j;
     {
         // ---- stage the super-chunk (coalesced), decoded to points
-        for (int i = t; i < m; i += LT) sm.pts[i] = sorted_point(P, base + i);
+        if constexpr (LOCAL) local_sort(sm, P, base, m);
+        else
+            for (int i = t; i < m; i += LT) sm.pts[i] = sorted_point(P, base + i);
         if (t == 0) {
             sm.has_prev = base > sbeg;
             sm.prev_x = base > sbeg ? key_float(__ldg(P.keys + base - 1)) : 0.0f;
@@ -546,7 +640,7 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
         // index.  A thread takes a short run, a warp a long one (the extreme
         // x of a circle holds thousands of points: 120 us for one thread).
         const auto index_of = [&](int e) {
-            return e < SC ? (uint32_t)__ldg(P.pay + base + e) : sm.ext_idx[e - SC];
+            return e < SC ? (uint32_t)__ldg(P.pay + place(e)) : sm.ext_idx[e - SC];
         };
         const auto lower = [&](float y, int e, float y0, int e0) {
             return y < y0 || (y == y0 && e != e0 && index_of(e) < index_of(e0));
@@ -720,7 +814,7 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
                     float2 *dpt = P.pt[side] + sc * CS;
                     for (int q = t; q < blen; q += LT) {
                         const int e = flat[bcur * NL + q];
-                        dpos[q] = e < SC ? (uint32_t)(base + e) : sm.ext_pos[e - SC];
+                        dpos[q] = e < SC ? (uint32_t)place(e) : sm.ext_pos[e - SC];
                         dpt[q] = sm.pts[e];
                     }
                     if (t == 0) {
@@ -793,7 +887,7 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
             float2 *dpt = P.pt[side] + sc * CS + off;
             for (int q = 0; q < c; ++q) {
                 const int e = flat[lbase + sm.stk[(l + q) * LT + t]];
-                dpos[q] = e < SC ? (uint32_t)(base + e) : sm.ext_pos[e - SC];
+                dpos[q] = e < SC ? (uint32_t)place(e) : sm.ext_pos[e - SC];
                 dpt[q] = sm.pts[e];
             }
             if (t == 0) {
@@ -805,7 +899,12 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
     }
 }
 
-__global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L)
+__device__ __forceinline__ void copy_chain_part(const ChainPtrs &P, int side, int64_t c, int part, uint32_t off0,
+                                                uint32_t hl, uint32_t hu, uint32_t *out, int64_t limit);
+
+// At most SC survivors (the sort has left them alone): one block sorts them
+// and writes the hull itself, and the later kernels have nothing to do.
+__global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t *hull_idx, uint32_t *hull_count)
 {
     kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -814,6 +913,19 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L)
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
     if (s == 0) return;
+    if (s <= (uint32_t)SC) {
+        if (blockIdx.x != 0) return;
+        const ChainPtrs P = chain_ptrs(ws, L, ctrl->sort_in);
+        superchunk<true>(sm, P, 0, 0, (int)s, 0, s);   // (ends with a barrier)
+        const uint32_t hl = (uint32_t)__ldcg(P.hi[0]) + 1u, hu = (uint32_t)__ldcg(P.hi[1]) + 1u;
+        for (int it = (int)(threadIdx.x >> 5); it < 2 * kCopyParts; it += NWB)
+            copy_chain_part(P, it & 1, 0, it >> 1, 0u, hl, hu, hull_idx, L.n);
+        if (threadIdx.x == 0) {
+            *hull_count = hl + (hu >= 2 ? hu - 2 : 0u);
+            ctrl->small_done = 1u;
+        }
+        return;
+    }
     const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
     const int64_t nsc = ceil_div((int64_t)s, SC);
     for (int64_t sc = blockIdx.x; sc < nsc; sc += gridDim.x) {
@@ -824,7 +936,7 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L)
             bulk_prefetch_l2(P.keys + nxt * SC, (nn * 4u) & ~15u);
             bulk_prefetch_l2(P.pay + nxt * SC, (nn * 8u) & ~15u);
         }
-        superchunk(sm, P, sc, sc * SC, (int)min((int64_t)SC, (int64_t)s - sc * SC), 0, s);
+        superchunk<false>(sm, P, sc, sc * SC, (int)min((int64_t)SC, (int64_t)s - sc * SC), 0, s);
     }
 }
 
@@ -860,7 +972,8 @@ __global__ void __launch_bounds__(LT) bx_chain_kernel(void *ws, Layout L, BatchL
         const uint32_t b = sc_set[j];
         const int64_t sb = (int64_t)sets[b].surv_base, n = sets[b].s;
         const int64_t local = j - sets[b].sc_base;
-        superchunk(sm, P, j, sb + local * SC, (int)min((int64_t)SC, n - local * SC), sb, sb + n);
+        if (n <= (int64_t)kBxLocalMax) superchunk<true>(sm, P, j, sb, (int)n, sb, sb + n);
+        else superchunk<false>(sm, P, j, sb + local * SC, (int)min((int64_t)SC, n - local * SC), sb, sb + n);
     }
 }
 
@@ -967,9 +1080,6 @@ __device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t
 // The warp knows where its range goes, so no position is searched for and
 // the chains are copied once.  limit: positions the hull may fill (only a
 // look-back that gave up could pass it).
-constexpr int kCopyParts = 4;                  // a range is shared by so many warps
-constexpr int kCopyLen = CS / kCopyParts;      // entries per part
-static_assert(CS % kCopyParts == 0, "parts cover a super-chunk's slots");
 
 __device__ __forceinline__ void copy_chain_part(const ChainPtrs &P, int side, int64_t c, int part, uint32_t off0,
                                                 uint32_t hl, uint32_t hu, uint32_t *out, int64_t limit)
@@ -1106,6 +1216,7 @@ __global__ void __launch_bounds__(kSmallHull) small_hull_kernel(void *ws, Layout
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
+    if (s == 0 && threadIdx.x == 0) *hull_count = 0u;   // (no later kernel may follow)
     if (s == 0 || s > (uint32_t)kSmallHull) return;
     const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5, lt = (1u << lane) - 1u;
     unsigned long long k = ~0ull;   // after every point
@@ -1185,7 +1296,7 @@ __global__ void __launch_bounds__(kSmallHull) small_hull_kernel(void *ws, Layout
 
 }  // namespace
 
-cudaError_t launch_small_hull(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
+static cudaError_t launch_small_hull(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
 {
     probe_before(CH_K_CHAIN, st);
     launch_next(small_hull_kernel, 1, kSmallHull, 0, st, ws, L, hull_idx, hull_count);
@@ -1194,7 +1305,7 @@ cudaError_t launch_small_hull(void *ws, const Layout &L, uint32_t *hull_idx, uin
     return cudaGetLastError();
 }
 
-cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
+static cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
 {
     const int sms = sm_count();
     int64_t cb = L.n_chunks;
@@ -1207,7 +1318,12 @@ cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t
     if (cb > (int64_t)sms * per_sm) cb = (int64_t)sms * per_sm;
     if (cb < 1) cb = 1;
     probe_before(CH_K_CHAIN, st);
-    launch_next(chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L);
+    launch_next(chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L, hull_idx, hull_count);
+    if (L.n <= SC) {   // one super-chunk at most: that kernel wrote the hull
+        note_kernels(CH_K_CHAIN, 1);
+        probe_after(CH_K_CHAIN, st);
+        return cudaGetLastError();
+    }
     launch_next(chain_merge_kernel, (unsigned)ceil_div(L.n_chunks, 32), 32, 0, st, ws, L);
     note_kernels(CH_K_CHAIN, 2);
     probe_after(CH_K_CHAIN, st);
@@ -1228,6 +1344,16 @@ cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t
     note_kernels(CH_K_FINISH, 1);
     probe_after(CH_K_FINISH, st);
     return cudaGetLastError();
+}
+
+// The hull of the survivors.  Few points need few of the kernels: each idle
+// launch is more than 1 us (1000 points: 31 us with all of them, 20 without).
+cudaError_t launch_hull_stage(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st)
+{
+    cudaError_t e = launch_small_hull(ws, L, hull_idx, hull_count, st);
+    if (e == cudaSuccess && L.n > SC) e = launch_sort(ws, L, st);
+    if (e == cudaSuccess && L.n > kSmallHull) e = launch_chain(ws, L, hull_idx, hull_count, st);
+    return e;
 }
 
 cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st)

@@ -283,13 +283,18 @@ struct BatchCtrl {
     uint32_t tiles;       // point tiles over all sets
     uint32_t nsc;         // super-chunks over all sets
     uint32_t abort;       // bad offsets: nothing is computed
-    uint32_t filt_ticket, emit_ticket, pad0;
+    uint32_t filt_ticket, emit_ticket;
+    uint32_t nsc_sort;    // the sort's tiles among them (the sets that the chain kernel sorts come after)
     uint32_t sort_ticket[kSortPasses];
     uint32_t h_lower, h_upper;
     uint32_t nfan;        // sets that get a fan (kgon.cu)
     uint32_t nfan_items, nplain_items, nbin_items;   // work items
     uint32_t fan_ticket, plain_ticket;               // next work item of the filter passes
 };
+// The chain kernel sorts a set of so few survivors itself.  (1000 sets of 10^2
+// to 10^4 points: 390 us with none, 364 so, 433 with 4096: the sort's passes
+// run beside one another and wait for the larger sets anyway.)
+constexpr uint32_t kBxLocalMax = 1024;
 constexpr int kBxFanChunk = 32;       // tiles per work item of the fan sets' filter pass (built-in)
 constexpr int kBxFanChunkMin = 8;     // the smallest tunable one (sizes the work-item lists)
 constexpr int kBxTileBins = 1024;     // a set has up to this many bins per tile of 4096 points (kFanBins at most)

@@ -1517,7 +1517,7 @@ __global__ void __launch_bounds__(kFiltThreads, 3) bx_plain_filter_kernel(const 
 __global__ void __launch_bounds__(1024) bx_layout_kernel(void *ws, BatchLayout BL)
 {
     kernel_entry();
-    __shared__ uint32_t s_w[2][32];
+    __shared__ uint32_t s_w[3][32];
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -1527,47 +1527,60 @@ __global__ void __launch_bounds__(1024) bx_layout_kernel(void *ws, BatchLayout B
     const int64_t B = BL.num_sets;
     const int64_t per = ceil_div(B, (int64_t)blockDim.x);
     const int64_t b0 = min((int64_t)threadIdx.x * per, B), b1 = min(b0 + per, B);
-    uint32_t sc = 0, nd = 0;
+    // super-chunks in two classes: the sort's, then those of the few-survivor
+    // sets, which the chain kernel sorts itself
+    uint32_t sc = 0, one = 0, nd = 0;
     for (int64_t b = b0; b < b1; ++b) {
         const uint32_t nsc = (uint32_t)ceil_div((int64_t)count[b], kChainC);
-        sc += nsc;
+        if (count[b] - 1u < kBxLocalMax) ++one;
+        else sc += nsc;
         nd += nsc > 0 ? (uint32_t)tree_nodes(nsc) + 1u : 0u;
     }
-    uint32_t i1 = sc, i2 = nd;
+    uint32_t i0 = one, i1 = sc, i2 = nd;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u1 = __shfl_up_sync(0xffffffffu, i1, o), u2 = __shfl_up_sync(0xffffffffu, i2, o);
+        const uint32_t u0 = __shfl_up_sync(0xffffffffu, i0, o), u1 = __shfl_up_sync(0xffffffffu, i1, o),
+                       u2 = __shfl_up_sync(0xffffffffu, i2, o);
         if (lane >= (uint32_t)o) {
+            i0 += u0;
             i1 += u1;
             i2 += u2;
         }
     }
     if (lane == 31) {
-        s_w[0][warp] = i1;
-        s_w[1][warp] = i2;
+        s_w[0][warp] = i0;
+        s_w[1][warp] = i1;
+        s_w[2][warp] = i2;
     }
     __syncthreads();
-    uint32_t rsc = i1 - sc, rnd = i2 - nd, tsc = 0;
+    uint32_t rone = i0 - one, rsc = i1 - sc, rnd = i2 - nd, tsc = 0, tone = 0;
     for (uint32_t w = 0; w < blockDim.x / 32; ++w) {
         if (w < warp) {
-            rsc += s_w[0][w];
-            rnd += s_w[1][w];
+            rone += s_w[0][w];
+            rsc += s_w[1][w];
+            rnd += s_w[2][w];
         }
-        tsc += s_w[0][w];
+        tone += s_w[0][w];
+        tsc += s_w[1][w];
     }
+    rone += tsc;
     for (int64_t b = b0; b < b1; ++b) {
         const uint32_t s = count[b], nsc = (uint32_t)ceil_div((int64_t)s, kChainC);
         SetInfo &S = sets[b];
         S.surv_base = (uint64_t)S.pt_begin;
         S.s = s;
         S.nsc = nsc;
-        S.sc_base = rsc;
+        uint32_t &at_sc = s - 1u < kBxLocalMax ? rone : rsc;
+        S.sc_base = at_sc;
         S.node_base = rnd;
-        for (uint32_t k = 0; k < nsc; ++k) sc_set[rsc + k] = (uint32_t)b;
-        rsc += nsc;
+        for (uint32_t k = 0; k < nsc; ++k) sc_set[at_sc + k] = (uint32_t)b;
+        at_sc += nsc;
         rnd += nsc > 0 ? (uint32_t)tree_nodes(nsc) + 1u : 0u;
     }
-    if (threadIdx.x == 0) bc->nsc = tsc;
+    if (threadIdx.x == 0) {
+        bc->nsc = tsc + tone;
+        bc->nsc_sort = tsc;
+    }
 }
 
 }  // namespace

@@ -113,15 +113,11 @@ cudaError_t launch_learned_choice(const float *pts, int64_t n, const void *param
 cudaError_t launch_hull_filter(const float *pts, int64_t n, void *ws, const Layout &L, const KgonStage *kg,
                                cudaStream_t st);
 
-// the whole hull in one block when few points survived the filter (the
-// sort and chain kernels then stop at once); otherwise nothing
-cudaError_t launch_small_hull(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st);
-
-// stable LSD radix sort of the survivor (key, index) pairs held in ws
+// stable radix sort of the survivors by x (nothing when one block will sort them)
 cudaError_t launch_sort(void *ws, const Layout &L, cudaStream_t st);
 
-// monotone chain over the sorted survivors; writes the hull
-cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st);
+// sort, monotone chains and assembly of the hull from the survivors
+cudaError_t launch_hull_stage(void *ws, const Layout &L, uint32_t *hull_idx, uint32_t *hull_count, cudaStream_t st);
 
 // ---- many sets (ch_hull_batched); every stage works per set
 // validates offsets (points beyond n_cap: CH_ERR_CAPACITY) and maps tiles to sets

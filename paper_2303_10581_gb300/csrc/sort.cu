@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256) sort_hist_kernel(void *ws, Layout L)
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
+    if (s <= (uint32_t)kChainC) return;   // one block sorts them as it builds the chains
     const int64_t ntiles = ceil_div((int64_t)s, kSortTile);
     // the first executed pass reads the survivors' buffer and its status
     uint32_t *status0 = at<uint32_t>(ws, L.sort_status[ctrl->sort_in]);
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(kPassThreads, kPassBlocks) sort_pass_kernel(vo
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
-    if (s == 0 || ctrl->pass_skip[p]) return;
+    if (s <= (uint32_t)kChainC || ctrl->pass_skip[p]) return;
     const uint32_t src = ctrl->pass_src[p], dst = src ^ 1u;
     const int64_t ntiles = ceil_div((int64_t)s, kSortTile);
     const PassIO io{at<uint32_t>(ws, L.keys[src]), at<unsigned long long>(ws, L.pay[src]),
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(256) bx_sort_hist_kernel(void *ws, Layout L, B
     uint32_t *hist = at<uint32_t>(ws, BL.hist);
     const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
     uint32_t *status0 = at<uint32_t>(ws, L.sort_status[0]);
-    const uint32_t nsc = bc->nsc;
+    const uint32_t nsc = bc->nsc_sort;
     {
         const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
         for (int64_t w = gtid; w < (int64_t)nsc * 256; w += (int64_t)gridDim.x * blockDim.x) status0[w] = 0u;
@@ -399,11 +400,11 @@ __global__ void __launch_bounds__(kBxPassThreads, kPassBlocks) bx_sort_pass_kern
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem<kBxPassThreads> &sm = *reinterpret_cast<SortSmem<kBxPassThreads> *>(smem_raw);
     BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
-    if (bc->abort) return;
+    if (bc->abort || bc->nsc_sort == 0u) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
     const uint32_t *sc_set = at<uint32_t>(ws, BL.sc_set);
     const uint32_t *hist = at<uint32_t>(ws, BL.hist);
-    const int64_t ntiles = bc->nsc;
+    const int64_t ntiles = bc->nsc_sort;
     const uint32_t src = (uint32_t)p & 1u, dst = src ^ 1u;
     const PassIO io{at<uint32_t>(ws, L.keys[src]), at<unsigned long long>(ws, L.pay[src]),
                     at<uint32_t>(ws, L.keys[dst]), at<unsigned long long>(ws, L.pay[dst]),
