@@ -117,7 +117,7 @@ __device__ __forceinline__ int warp_elim_pass(const float2 *pts, const uint16_t 
 }
 
 // ---------------------------------------------------------------------------
-// tangent walk, shared by the in-block and the global merge
+// tangent walk of the in-block merge (the global one: MergeSide)
 // ---------------------------------------------------------------------------
 // Acc provides lo/hi/prv/nxt get+set per chunk and point(side, chunk, k).
 template <class Acc>
@@ -339,85 +339,146 @@ __device__ __forceinline__ float2 sorted_point(const ChainPtrs &P, int64_t q)
     return make_float2(key_float(__ldg(P.keys + q)), key_float((uint32_t)(__ldg(P.pay + q) >> 32)));
 }
 
-// Values written by other blocks are read through L2 (ld.cg): this
-// thread's L1 may hold stale lines.
-struct GlobalAcc {
-    const ChainPtrs &P;
-    __device__ int lo(int side, int c) const { return __ldcg(P.lo[side] + c); }
-    __device__ int hi(int side, int c) const { return __ldcg(P.hi[side] + c); }
-    __device__ int prv(int side, int c) const { return __ldcg(P.prv[side] + c); }
-    __device__ int nxt(int side, int c) const { return __ldcg(P.nxt[side] + c); }
-    __device__ void set_range(int side, int c, int l, int h) const
+// The common tangent of two neighbouring chains, by one warp: the merge_walk of
+// chunks fa..la | fb..lb.  Values written by other blocks are read through L2
+// (ld.cg): this thread's L1 may hold stale lines.
+// The walk's steps are dependent loads, some 0.6 us each, and a merge takes
+// tens of them.  Trees on the way (one thread per node): 10^8 ellipse points
+// 154 us, 39 so; 10^6 circle points 68, 28.
+// Here the lanes test 32 vertices at once, the next 32 in a row first, then 32
+// spread over the rest of the chunk: as seen from a point beside it, the
+// vertices of a strictly convex chain that the walk passes come before those
+// it does not.
+struct MergeSide {
+    const float2 *pt;
+    int32_t *lo, *hi, *prv, *nxt;
+    int side;
+    __device__ float2 point(int c, int k) const { return __ldcg(pt + (int64_t)c * CS + k); }
+
+    // From vertex k of chunk c on (step d = 1: up to e, -1: down to e): the
+    // number of vertices that are passed, 0 .. |e - k|, as seen from `from`;
+    // p, vertex k, becomes the vertex reached.
+    __device__ int passed(int c, int k, int e, int d, const float2 &from, float2 &p) const
     {
-        P.lo[side][c] = l;
-        P.hi[side][c] = h;
+        const int lane = (int)lane_id(), n = d > 0 ? e - k : k - e;
+        int i = 0, stride = 1;
+        while (i < n) {
+            const int l = i + lane * stride;
+            bool pass = false;
+            float2 u = p, v = p;
+            if (l < n) {
+                u = point(c, k + d * l);
+                v = point(c, k + d * (l + 1));
+                pass = d > 0 ? drop(side, from, u, v) : drop(side, v, u, from);
+            }
+            const int f = __ffs(~__ballot_sync(0xffffffffu, pass)) - 1;   // the first that stays (-1: none)
+            if (f == 0) break;
+            // passed for sure: all before and at the last lane that passed
+            const int last = f < 0 ? 31 : f - 1;
+            i += last * stride + 1;
+            p.x = __shfl_sync(0xffffffffu, v.x, last);
+            p.y = __shfl_sync(0xffffffffu, v.y, last);
+            if (f > 0 && stride == 1) break;
+            stride = max(1, (n - i + 31) / 32);
+            if (f > 0) stride = 1;
+        }
+        return i;
     }
-    __device__ void set_lo(int side, int c, int l) const { P.lo[side][c] = l; }
-    __device__ void set_hi(int side, int c, int h) const { P.hi[side][c] = h; }
-    __device__ void link(int side, int a, int b) const
+
+    __device__ void merge(int fa, int la, int fb, int lb) const
     {
-        P.nxt[side][a] = b;
-        P.prv[side][b] = a;
+        const int lane = (int)lane_id();
+        int ca = la, cb = fb;
+        int loa = __ldcg(lo + ca), ka = __ldcg(hi + ca), kb = __ldcg(lo + cb), hib = __ldcg(hi + cb);
+        float2 pa = point(ca, ka), pb = point(cb, kb);
+        for (;;) {
+            bool moved = false;
+            for (;;) {   // advance b
+                const int m = passed(cb, kb, hib, 1, pa, pb);
+                moved |= m > 0;
+                kb += m;
+                if (kb < hib || cb == lb) break;
+                const int nc = __ldcg(nxt + cb), nk = __ldcg(lo + nc);
+                const float2 q = point(nc, nk);
+                if (!drop(side, pa, pb, q)) break;
+                if (lane == 0) lo[cb] = 1, hi[cb] = 0;   // that chunk is gone
+                cb = nc;
+                kb = nk;
+                hib = __ldcg(hi + nc);
+                pb = q;
+                moved = true;
+            }
+            for (;;) {   // retreat a
+                const int m = passed(ca, ka, loa, -1, pb, pa);
+                moved |= m > 0;
+                ka -= m;
+                if (ka > loa || ca == fa) break;
+                const int pc = __ldcg(prv + ca), pk = __ldcg(hi + pc);
+                const float2 q = point(pc, pk);
+                if (!drop(side, q, pa, pb)) break;
+                if (lane == 0) lo[ca] = 1, hi[ca] = 0;
+                ca = pc;
+                ka = pk;
+                loa = __ldcg(lo + pc);
+                pa = q;
+                moved = true;
+            }
+            if (!moved) break;
+        }
+        if (lane == 0) {
+            hi[ca] = ka;
+            lo[cb] = kb;
+            nxt[ca] = cb;
+            prv[cb] = ca;
+        }
     }
-    __device__ float2 point(int side, int c, int k) const { return __ldcg(P.pt[side] + (int64_t)c * CS + k); }
 };
 
-// first / last live super-chunk (absolute index) of tree node (level, j)
-// of a tree whose leaves are super-chunks coff + 0 .. and whose nodes start
-// at node noff; level 0 = super-chunk coff + j
-__device__ __forceinline__ void node_ends(const ChainPtrs &P, int level, int64_t coff, int64_t noff, int64_t nb,
-                                          int64_t j, int side, int32_t &first, int32_t &last)
+// One warp climbs one side of a set's merge tree from its super-chunk c (0 <=
+// c < nsc; leaves at coff, nodes at noff): the second child to arrive at a
+// node merges its two children and continues upward (no warp ever waits).
+__device__ void climb(const ChainPtrs &P, int side, int64_t c, int64_t nsc, int64_t coff, int64_t noff)
 {
-    if (level == 0) {
-        const bool live = __ldcg(P.hi[side] + coff + j) >= __ldcg(P.lo[side] + coff + j);
-        first = last = live ? (int32_t)(coff + j) : -1;
-    } else {
-        first = __ldcg(P.node + (noff + nb + j) * 4 + 2 * side);
-        last = __ldcg(P.node + (noff + nb + j) * 4 + 2 * side + 1);
-    }
-}
-
-// Climb the merge tree of one set from its super-chunk c (0 <= c < nsc;
-// leaves at coff, nodes at noff): the second child to arrive at a node
-// merges its two children and continues upward.
-__device__ void climb(const ChainPtrs &P, int64_t c, int64_t nsc, int64_t coff, int64_t noff)
-{
-    GlobalAcc G{P};
+    const MergeSide M{P.pt[side], P.lo[side], P.hi[side], P.prv[side], P.nxt[side], side};
+    const uint32_t lane = lane_id();
     int64_t node = c, w = nsc, nb_child = 0, nb = 0;   // nb: base of the level above
     int level = 0;
+    // first and last live super-chunk (absolute; -1: none) of child j of this level
+    const auto ends = [&](int64_t j) {
+        if (level == 0) {
+            const int ci = (int)(coff + j);
+            return __ldcg(M.hi + ci) >= __ldcg(M.lo + ci) ? make_int2(ci, ci) : make_int2(-1, -1);
+        }
+        const int32_t *r = P.node + (noff + nb_child + j) * 4 + 2 * side;
+        return make_int2(__ldcg(r), __ldcg(r + 1));
+    };
     while (w > 1) {
         const int64_t parent = node >> 1, pw = (w + 1) / 2;
-        const int64_t sib = node ^ 1;
-        int32_t rec[4];
-        if (sib >= w) {
-#pragma unroll
-            for (int side = 0; side < 2; ++side)
-                node_ends(P, level, coff, noff, nb_child, node, side, rec[2 * side], rec[2 * side + 1]);
+        int2 rec;
+        if ((node ^ 1) >= w) {
+            rec = ends(node);
         } else {
-            __threadfence();
-            if (atomicAdd(P.node_cnt + noff + nb + parent, 1) == 0) return;   // first to arrive: the sibling merges
-            __threadfence();
-            const int64_t a = parent * 2, b = a + 1;
-#pragma unroll
-            for (int side = 0; side < 2; ++side) {
-                int32_t fa, la, fb, lb;
-                node_ends(P, level, coff, noff, nb_child, a, side, fa, la);
-                node_ends(P, level, coff, noff, nb_child, b, side, fb, lb);
-                if (la < 0) {
-                    rec[2 * side] = fb;
-                    rec[2 * side + 1] = lb;
-                } else if (fb < 0) {
-                    rec[2 * side] = fa;
-                    rec[2 * side + 1] = la;
-                } else {
-                    merge_walk(G, side, fa, la, fb, lb);
-                    rec[2 * side] = fa;
-                    rec[2 * side + 1] = lb;
-                }
+            int before = 0;
+            if (lane == 0) {
+                __threadfence();
+                before = atomicAdd(P.node_cnt + noff + nb + parent, side ? 0x10000 : 1) >> (side ? 16 : 0);
+                __threadfence();
+            }
+            if ((__shfl_sync(0xffffffffu, before, 0) & 0xffff) == 0) return;   // first to arrive: the sibling merges
+            const int2 A = ends(parent * 2), B = ends(parent * 2 + 1);
+            if (A.y < 0) rec = B;
+            else if (B.x < 0) rec = A;
+            else {
+                M.merge(A.x, A.y, B.x, B.y);
+                rec = make_int2(A.x, B.y);
             }
         }
-#pragma unroll
-        for (int f = 0; f < 4; ++f) P.node[(noff + nb + parent) * 4 + f] = rec[f];
+        if (lane == 0) {
+            int32_t *r = P.node + (noff + nb + parent) * 4 + 2 * side;
+            r[0] = rec.x;
+            r[1] = rec.y;
+        }
+        __syncwarp();
         node = parent;
         nb_child = nb;
         nb += pw;
@@ -940,9 +1001,10 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t 
     }
 }
 
-// Global merge tree over the super-chunks: one thread per super-chunk
-// climbs; the second child to reach a node merges the pair.
-__global__ void __launch_bounds__(32) chain_merge_kernel(void *ws, Layout L)
+// Global merge tree over the super-chunks: a warp per super-chunk and side.
+constexpr int kMergeThreads = 128;
+
+__global__ void __launch_bounds__(kMergeThreads) chain_merge_kernel(void *ws, Layout L)
 {
     kernel_entry();
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
@@ -950,9 +1012,9 @@ __global__ void __launch_bounds__(32) chain_merge_kernel(void *ws, Layout L)
     const uint32_t s = hull_stage_count(ctrl, oct);
     if (s == 0) return;
     const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
-    const int64_t nsc = ceil_div((int64_t)s, SC);
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < nsc) climb(P, c, nsc, 0, 0);
+    const int64_t nsc = ceil_div((int64_t)s, SC), step = (int64_t)gridDim.x * (kMergeThreads / 32);
+    for (int64_t i = ((int64_t)blockIdx.x * kMergeThreads + threadIdx.x) >> 5; i < 2 * nsc; i += step)
+        climb(P, (int)(i & 1), i >> 1, nsc, 0, 0);
 }
 
 // ---- many sets: super-chunks never span two sets; each set has its own
@@ -977,7 +1039,7 @@ __global__ void __launch_bounds__(LT) bx_chain_kernel(void *ws, Layout L, BatchL
     }
 }
 
-__global__ void __launch_bounds__(32) bx_merge_kernel(void *ws, Layout L, BatchLayout BL)
+__global__ void __launch_bounds__(kMergeThreads) bx_merge_kernel(void *ws, Layout L, BatchLayout BL)
 {
     kernel_entry();
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
@@ -985,10 +1047,18 @@ __global__ void __launch_bounds__(32) bx_merge_kernel(void *ws, Layout L, BatchL
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
     const uint32_t *sc_set = at<uint32_t>(ws, BL.sc_set);
     const ChainPtrs P = chain_ptrs(ws, L, 0);
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= (int64_t)bc->nsc) return;
-    const uint32_t b = sc_set[j];
-    climb(P, j - sets[b].sc_base, sets[b].nsc, sets[b].sc_base, sets[b].node_base);
+    const int64_t nsc = bc->nsc_sort, step = (int64_t)gridDim.x * (kMergeThreads / 32);   // (the others are alone)
+    for (int64_t i = ((int64_t)blockIdx.x * kMergeThreads + threadIdx.x) >> 5; i < 2 * nsc; i += step) {
+        const int64_t j = i >> 1;
+        const SetInfo &S = sets[sc_set[j]];
+        climb(P, (int)(i & 1), j - S.sc_base, S.nsc, S.sc_base, S.node_base);
+    }
+}
+
+// blocks for the merge tree of up to n super-chunks
+unsigned merge_grid(int64_t n)
+{
+    return (unsigned)std::min<int64_t>(ceil_div(2 * n, kMergeThreads / 32), (int64_t)sm_count() * 8);
 }
 
 // Output offsets of the live chain ranges of super-chunks [0, nc), per side:
@@ -1324,7 +1394,7 @@ static cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, u
         probe_after(CH_K_CHAIN, st);
         return cudaGetLastError();
     }
-    launch_next(chain_merge_kernel, (unsigned)ceil_div(L.n_chunks, 32), 32, 0, st, ws, L);
+    launch_next(chain_merge_kernel, merge_grid(L.n_chunks), kMergeThreads, 0, st, ws, L);
     note_kernels(CH_K_CHAIN, 2);
     probe_after(CH_K_CHAIN, st);
     cudaError_t e = cudaGetLastError();
@@ -1370,7 +1440,7 @@ cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cu
     if (cb < 1) cb = 1;
     probe_before(CH_K_CHAIN, st);
     launch_next(bx_chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L, BL);
-    launch_next(bx_merge_kernel, (unsigned)ceil_div(BL.tiles_max, 32), 32, 0, st, ws, L, BL);
+    launch_next(bx_merge_kernel, merge_grid(BL.tiles_max), kMergeThreads, 0, st, ws, L, BL);
     note_kernels(CH_K_CHAIN, 2);
     probe_after(CH_K_CHAIN, st);
     cudaError_t e = cudaGetLastError();
