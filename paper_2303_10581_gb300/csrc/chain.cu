@@ -4,28 +4,29 @@
 // The paper copies the candidates to the host and calls CGAL; its
 // conclusion names a fully device-resident hull as the next step.  Here:
 //
-//  0. runs: the survivors arrive sorted by x (equal x in any order).  In a run of equal x only the lowest point can be a vertex of
-//     the lower chain and only the highest one of the upper chain, because
-//     the others lie strictly above (below) it on the same vertical.  The
-//     exceptions are the first x, whose lowest point starts both chains and
-//     whose highest point follows it on the upper chain, and the last x,
-//     whose highest point ends both chains after its lowest point on the
-//     lower chain.  Each run is reduced to those representatives (first
-//     occurrence on ties, i.e. the lowest index, which also collapses equal
+//  0. runs: the survivors arrive sorted by x (equal x in any order), or are
+//     so few that the block sorts them itself.  In a run of equal x only the
+//     lowest point can be a vertex of the lower chain and only the highest
+//     one of the upper chain, because the others lie strictly above (below)
+//     it on the same vertical.  The exceptions are the first x, whose lowest
+//     point starts both chains and whose highest point follows it on the
+//     upper chain, and the last x, whose highest point ends both chains after
+//     its lowest point on the lower chain.  Each run is reduced to those
+//     representatives (on ties the lowest index, which also collapses equal
 //     points).  A block owns the runs starting in its 4096-point
 //     super-chunk and looks ahead (block-parallel) when its last run
 //     continues past the super-chunk.
-//  1. elimination: per side, parallel passes over the representatives drop
-//     every point whose turn with its current neighbours is not strict (for
-//     the lower chain: on or above the segment joining them).  Such a point
-//     lies on or above a segment between two points of the set, so it is
-//     not a strict vertex of the lower hull and the sequential chain would
-//     pop it too; a sequence where every turn is strict is its own monotone
-//     chain.  Each warp first runs passes over its share of the sequence
-//     (its two ends stay); then the warps' survivors are concatenated and
-//     the passes continue over the whole super-chunk sequence (block-wide
-//     while long, one warp once short) until nothing changes.  The
-//     converged sequence is written out as the super-chunk's chain.
+//  1. elimination: of the points between a side's two ends only those
+//     strictly beyond the segment joining the ends stay, and then parallel
+//     passes drop every point whose turn with its current neighbours is not
+//     strict (for the lower chain: on or above the segment joining them).
+//     Such a point lies on or above a segment between two points of the set,
+//     so it is not a strict vertex of the lower hull and the sequential
+//     chain would pop it too; a sequence where every turn is strict is its
+//     own monotone chain.  Half of the block's warps take each side: a pass
+//     over the whole sequence, passes inside each warp's share, and again
+//     until a whole pass drops nothing.  The sequence is written out as the
+//     super-chunk's chain.
 //  2. fallback, when the passes do not converge within their cap: what is
 //     left is cut into leaves; one thread runs the sequential monotone
 //     chain on each, and the leaf chains are merged pairwise up a binary
@@ -61,7 +62,8 @@ constexpr int SC = kChainC;         // points per super-chunk
 constexpr int CS = kChainStride;    // chain slots per super-chunk
 constexpr int NL = SC + 2;          // sequence capacity: SC points + 2 look-ahead slots
 constexpr int NWB = LT / 32;        // warps per block
-constexpr int kLongRun = 32;        // a longer run of equal x is reduced by a warp
+constexpr int NWS = NWB / 2;        // warps per side
+constexpr int SY = NL + 6;
 constexpr int kCopyParts = 4;                  // a range is shared by so many warps
 constexpr int kCopyLen = CS / kCopyParts;      // entries per part
 static_assert(CS % kCopyParts == 0, "parts cover a super-chunk's slots");
@@ -76,12 +78,14 @@ __device__ __forceinline__ bool drop(int side, const float2 &a, const float2 &b,
 }
 
 // One strict-turn elimination pass of a warp over the sequence
-// src[0 .. len) of point indices (its two ends always stay): the kept
-// entries go to dst in order; returns how many.  len >= 3.  Two 32-entry
-// chunks per step, binary32 tier of both tests first, so their latencies
-// overlap.
+// src[0 .. len) of point indices: the kept entries go to dst in order;
+// returns how many.  Its two ends stay unless there is a neighbour before
+// (left) or after (right) them.  Two 32-entry chunks per step, binary32 tier
+// of both tests first, so their latencies overlap.  (Inlined once a kernel, and the block's loops are not unrolled: a
+// block runs most of this code a few times, and fetching it counts.  A call
+// would lose the address space of its arguments.)
 __device__ __forceinline__ int warp_elim_pass(const float2 *pts, const uint16_t *src, uint16_t *dst, int len,
-                                              int side, int lane, uint32_t lt)
+                                              int side, int lane, uint32_t lt, bool left = false, bool right = false)
 {
     int kept = 0;
     for (int c0 = 0; c0 < len; c0 += 64) {
@@ -92,11 +96,11 @@ __device__ __forceinline__ int warp_elim_pass(const float2 *pts, const uint16_t 
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             j[u] = c0 + 32 * u + lane;
-            test[u] = j[u] > 0 && j[u] < len - 1;
-            const int jj = test[u] ? j[u] : 1;
-            a[u] = pts[src[jj - 1]];
+            test[u] = (j[u] > 0 || left) && (j[u] < len - 1 || (right && j[u] < len));
+            const int jj = min(j[u], len - 1);   // (no test: any readable neighbours)
             b[u] = pts[src[jj]];
-            c[u] = pts[src[jj + 1]];
+            a[u] = test[u] ? pts[src[jj - 1]] : b[u];
+            c[u] = test[u] ? pts[src[jj + 1]] : b[u];
             o[u] = orient_f32(a[u].x, a[u].y, b[u].x, b[u].y, c[u].x, c[u].y);
         }
 #pragma unroll
@@ -178,11 +182,21 @@ __device__ void merge_walk(Acc &A, int side, int fa, int la, int fb, int lb)
 // ---------------------------------------------------------------------------
 // in-block state; one side (lower or upper) is processed at a time
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void side_barrier(int side)   // of the warps that work on one side
+{
+    __syncwarp();   // (whole warps arrive)
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + side), "n"(NWS * 32) : "memory");
+}
+
 struct ChainSmem {
     float2 pts[NL];               // staged points; [SC], [SC+1]: look-ahead lowest / highest
     union {
         struct {
-            uint16_t list[3][NL];         // run starts, sequences and elimination ping-pong
+            // from 0: the two sides' sequences one after the other (a point
+            // between the ends is on one side at most: up to SC + 4 entries);
+            // from SY: lowest / highest point of the run that ends at a point,
+            // then the passes' other buffer
+            uint16_t seq[SY + 2 * NL];
             uint8_t stk[LWMAX * LT];      // leaf stacks: entry j of leaf t at [j * LT + t]
             int16_t lb[LT];               // leaf t's first entry in the flat list array
             int16_t lo[LT], hi[LT], prv[LT], nxt[LT], first[LT], last[LT];
@@ -198,10 +212,9 @@ struct ChainSmem {
     uint32_t ext_idx[2];          // and their point indices
     float prev_x;
     int has_prev;
-    int seq_len;
-    int wcur, wdone;              // single-warp passes: buffer and convergence
-    int nlong;                    // runs longer than kLongRun, and which
-    uint16_t lrun[SC / (kLongRun + 1) + 1];
+    int seq_len[2];               // per side: its length, and whether every turn is strict
+    int strict[2];
+    int run[4];                   // lowest, highest point of the set's first run, of its last
 };
 
 // leaf c's entries start at flat[lb[c]]; its stack holds offsets from there
@@ -250,51 +263,6 @@ __device__ __forceinline__ uint32_t block_scan(ChainSmem &s, uint32_t v)
     if (t == 0) s.total = total;
     __syncthreads();
     return before + incl - v;
-}
-
-// Stable compaction of positions [0, count).  Warp w owns the segment
-// [w*S, w*S + S) and walks it 32 consecutive positions at a time, so lanes
-// touch consecutive entries (no bank conflicts); keep(j) decides, out
-// receives src(j) for the kept j.  Returns the number kept (all threads).
-template <class Keep, class Src>
-__device__ __forceinline__ int block_compact(ChainSmem &s, int count, Keep keep, Src src, uint16_t *out)
-{
-    constexpr int NWARP = LT / 32;
-    constexpr int MAXC = (NL + NWARP * 32 - 1) / (NWARP * 32) + 1;   // 32-position chunks per warp
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int S = (((count + NWARP - 1) / NWARP) + 31) & ~31;   // segment, a multiple of 32
-    const int j0 = warp * S;
-    const uint32_t lt = (1u << lane) - 1u;
-    uint32_t masks[MAXC];
-    int n = 0;
-#pragma unroll
-    for (int c = 0; c < MAXC; ++c) {
-        uint32_t m = 0;
-        if (c * 32 < S) {
-            const int j = j0 + c * 32 + lane;
-            m = __ballot_sync(0xffffffffu, j < count && keep(j));
-        }
-        masks[c] = m;
-        n += __popc(m);
-    }
-    if (lane == 0) s.wsum[warp] = (uint32_t)n;
-    __syncthreads();
-    uint32_t before = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < NWARP; ++w) {
-        const uint32_t u = s.wsum[w];
-        if (w < warp) before += u;
-        total += u;
-    }
-    uint32_t o = before;
-#pragma unroll
-    for (int c = 0; c < MAXC; ++c) {
-        const uint32_t m = masks[c];
-        if ((m >> lane) & 1u) out[o + __popc(m & lt)] = src(j0 + c * 32 + lane);
-        o += __popc(m);
-    }
-    __syncthreads();
-    return (int)total;
 }
 
 // ---------------------------------------------------------------------------
@@ -574,24 +542,25 @@ __device__ void local_sort(ChainSmem &sm, const ChainPtrs &P, int64_t base, int 
             }
             int a = lo, b = o - pair - lo;
             unsigned long long ka = a < la ? src[pair + a] : ~0ull, kb = b < lb ? src[pair + w + b] : ~0ull;
-            for (; o < end; ++o) {
-                if (o == pair + 2 * w) {   // the next pair
-                    pair = o;
-                    la = min(w, m - pair);
-                    lb = min(w, max(0, m - pair - w));
-                    a = b = 0;
-                    ka = src[pair];
-                    kb = lb > 0 ? src[pair + w] : ~0ull;
+            for (;;) {
+                const int stop = min(end, pair + 2 * w);
+                for (; o < stop; ++o) {
+                    const bool first = ka < kb;
+                    dst[o] = first ? ka : kb;
+                    a += first ? 1 : 0;
+                    b += first ? 0 : 1;
+                    const bool more = first ? a < la : b < lb;
+                    const unsigned long long next = more ? src[pair + (first ? a : w + b)] : ~0ull;
+                    ka = first ? next : ka;
+                    kb = first ? kb : next;
                 }
-                const bool first = ka < kb;
-                dst[o] = first ? ka : kb;
-                if (first) {
-                    ++a;
-                    ka = a < la ? src[pair + a] : ~0ull;
-                } else {
-                    ++b;
-                    kb = b < lb ? src[pair + w + b] : ~0ull;
-                }
+                if (o == end) break;
+                pair = o;   // the next pair
+                la = min(w, m - pair);
+                lb = min(w, max(0, m - pair - w));
+                a = b = 0;
+                ka = src[pair];
+                kb = lb > 0 ? src[pair + w] : ~0ull;
             }
         }
         __syncthreads();
@@ -615,20 +584,19 @@ __device__ void local_sort(ChainSmem &sm, const ChainPtrs &P, int64_t base, int 
 }
 
 // The chains of one super-chunk: sorted positions [base, base + m) of a set
-// occupying [sbeg, send); results go to chain slot j.  LOCAL: the super-chunk
+// occupying [sbeg, send); results go to chain slot j.  local: the super-chunk
 // is a whole set and not sorted yet.  Called by all threads of the block.
-template <bool LOCAL>
-__device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t base, int m, int64_t sbeg,
-                           int64_t send)
+__device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t base, int m,
+                                           int64_t sbeg, int64_t send, bool local)
 {
-    const auto place = [&](int e) { return base + (LOCAL ? (int)sm.perm[e] : e); };   // of a staged point
+    const auto place = [&](int e) { return base + (local ? (int)sm.perm[e] : e); };   // of a staged point
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const float kInf = __int_as_float(0x7f800000);
     const int64_t sc = j;
     {
         // ---- stage the super-chunk (coalesced), decoded to points
-        if constexpr (LOCAL) local_sort(sm, P, base, m);
+        if (local) local_sort(sm, P, base, m);
         else
             for (int i = t; i < m; i += LT) sm.pts[i] = sorted_point(P, base + i);
         if (t == 0) {
@@ -637,14 +605,9 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
         }
         __syncthreads();
 
-        // ---- runs of equal x that start in this super-chunk
-        const int R = block_compact(
-            sm, m,
-            [&](int i) {
-                return i == 0 ? !(sm.has_prev && sm.pts[0].x == sm.prev_x) : sm.pts[i].x != sm.pts[i - 1].x;
-            },
-            [](int i) { return (uint16_t)i; }, sm.list[2]);
-        if (R == 0) {   // the whole super-chunk continues an earlier run
+        const float xr = sm.pts[m - 1].x;
+        const bool cont = sm.has_prev && sm.pts[0].x == sm.prev_x;   // it starts inside a run
+        if (cont && xr == sm.prev_x) {   // the whole super-chunk continues an earlier run
             if (t == 0)
                 for (int side = 0; side < 2; ++side) {
                     P.lo[side][sc] = 0;
@@ -654,7 +617,6 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
             return;
         }
         // ---- look ahead when the last run continues past the super-chunk
-        const float xr = sm.pts[m - 1].x;
         const bool ext = base + m < send && key_float(__ldg(P.keys + base + m)) == xr;
         int64_t run_end = base + m;
         if (ext) {
@@ -696,10 +658,6 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
         }
         const bool holds_last = run_end == send;
         __syncthreads();
-        // ---- representatives: lowest (list[0]) and highest (list[1]) point of
-        // each run; equal points (the sort does not order a run): the lowest
-        // index.  A thread takes a short run, a warp a long one (the extreme
-        // x of a circle holds thousands of points: 120 us for one thread).
         const auto index_of = [&](int e) {
             return e < SC ? (uint32_t)__ldg(P.pay + place(e)) : sm.ext_idx[e - SC];
         };
@@ -709,191 +667,272 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
         const auto higher = [&](float y, int e, float y0, int e0) {
             return y > y0 || (y == y0 && e != e0 && index_of(e) < index_of(e0));
         };
-        const auto put = [&](int k, int lo, float ylo, int hi, float yhi) {
-            if (k == R - 1 && ext) {
-                if (lower(sm.pts[SC].y, SC, ylo, lo)) lo = SC;
-                if (higher(sm.pts[SC + 1].y, SC + 1, yhi, hi)) hi = SC + 1;
-            }
-            sm.list[0][k] = (uint16_t)lo;
-            sm.list[1][k] = (uint16_t)hi;
-        };
-        if (t == 0) sm.nlong = 0;
-        __syncthreads();
-        for (int k = t; k < R; k += LT) {
-            const int r0 = sm.list[2][k];
-            const int r1 = k + 1 < R ? sm.list[2][k + 1] : m;
-            if (r1 - r0 > kLongRun) {
-                sm.lrun[atomicAdd(&sm.nlong, 1)] = (uint16_t)k;
-                continue;
-            }
-            int lo = r0, hi = r0;
-            float ylo = sm.pts[r0].y, yhi = ylo;
-            for (int i = r0 + 1; i < r1; ++i) {
-                const float y = sm.pts[i].y;
-                if (lower(y, i, ylo, lo)) {
-                    ylo = y;
-                    lo = i;
+        // ---- runs, their lowest and highest points, and the sides' sequences
+        // in one sweep.  A warp takes a segment of the points and the runs that
+        // start in it, 32 points at a time (a scan over the lanes of a run;
+        // equal points: the lowest index).  Lower: the lowest of every run, then
+        // the highest of the very last run; upper: the lowest of the very first
+        // run, then the highest of every run.  Of the points beside the first
+        // and last x only those strictly below (above) the segment joining two
+        // points there can be vertices (a ring's chunk holds both arcs by
+        // turns).  Bound by latency, like all of this kernel on few chunks:
+        // runs, representatives and sequences in steps of their own (a thread
+        // per run) took 24000 to 48000 cycles on a ring's chunk, this %SW%.
+        uint16_t *const low = sm.seq + SY, *const high = low + NL;
+        int n0, n1;
+        {
+            const float2 A = sm.pts[0], B = sm.pts[m - 1];
+            const int S = (((m + NWB - 1) / NWB) + 31) & ~31, j0 = min(warp * S, m), j1 = min(j0 + S, m);
+            const bool starts = j0 == 0 ? !cont : j0 < m && sm.pts[j0].x != sm.pts[j0 - 1].x;   // with a run of its own
+            const bool crosses = j1 < m && j1 > j0 && sm.pts[j1].x == sm.pts[j1 - 1].x;         // its last run goes on
+            uint32_t masks0 = 0, masks1 = 0, c01 = 0;   // lane c: the kept ones of the c-th 32 points; both counts
+            bool owned = starts;                        // the run open at the 32 points' start, and its state
+            float cylo = 0.0f, cyhi = 0.0f;
+            int clo = 0, chi = 0;
+#pragma unroll 1
+            for (int c = 0; j0 + c * 32 < j1; ++c) {
+                const int i = min(j0 + c * 32 + lane, j1 - 1);
+                const bool in = j0 + c * 32 + lane < j1;
+                const float2 p = sm.pts[i];
+                const bool head = in && (i == j0 ? starts : sm.pts[i - 1].x != p.x);
+                const bool tail = in && (i == j1 - 1 || sm.pts[i + 1].x != p.x);
+                const uint32_t hm = __ballot_sync(0xffffffffu, head), vm = __ballot_sync(0xffffffffu, in);
+                int lo = i, hi = i;
+                float ylo = p.y, yhi = p.y;
+                bool mine = true;
+                if (hm != vm) {
+                    const uint32_t upto = hm & (lt | (1u << lane));
+                    const int start = upto ? 31 - __clz(upto) : 0;
+#pragma unroll 1
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const float y1 = __shfl_up_sync(0xffffffffu, ylo, o), y2 = __shfl_up_sync(0xffffffffu, yhi, o);
+                        const int e1 = __shfl_up_sync(0xffffffffu, lo, o), e2 = __shfl_up_sync(0xffffffffu, hi, o);
+                        if (lane - o >= start) {
+                            if (lower(y1, e1, ylo, lo)) {
+                                ylo = y1;
+                                lo = e1;
+                            }
+                            if (higher(y2, e2, yhi, hi)) {
+                                yhi = y2;
+                                hi = e2;
+                            }
+                        }
+                    }
+                    if (upto == 0u) {
+                        mine = owned;
+                        if (c > 0) {
+                            if (lower(cylo, clo, ylo, lo)) {
+                                ylo = cylo;
+                                lo = clo;
+                            }
+                            if (higher(cyhi, chi, yhi, hi)) {
+                                yhi = cyhi;
+                                hi = chi;
+                            }
+                        }
+                    }
                 }
-                if (higher(y, i, yhi, hi)) {
-                    yhi = y;
-                    hi = i;
+                int end_of_run = i + 1;
+                if (crosses && j0 + c * 32 + 32 >= j1) {   // the run of the segment's last point goes on
+                    const int last = j1 - 1 - (j0 + c * 32);
+                    float ay = __int_as_float(0x7f800000), by = -ay;
+                    int ae = -1, be = -1, q = j1 + lane;
+                    for (; q < m && sm.pts[q].x == sm.pts[j1 - 1].x; q += 32) {
+                        const float y = sm.pts[q].y;
+                        if (ae < 0 || lower(y, q, ay, ae)) {
+                            ay = y;
+                            ae = q;
+                        }
+                        if (be < 0 || higher(y, q, by, be)) {
+                            by = y;
+                            be = q;
+                        }
+                    }
+                    __syncwarp();
+                    const int stop = (int)__reduce_min_sync(0xffffffffu, (uint32_t)min(q, m));   // the first past the run
+#pragma unroll 1
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const float y1 = __shfl_xor_sync(0xffffffffu, ay, o), y2 = __shfl_xor_sync(0xffffffffu, by, o);
+                        const int e1 = __shfl_xor_sync(0xffffffffu, ae, o), e2 = __shfl_xor_sync(0xffffffffu, be, o);
+                        if (e1 >= 0 && (ae < 0 || lower(y1, e1, ay, ae))) {
+                            ay = y1;
+                            ae = e1;
+                        }
+                        if (e2 >= 0 && (be < 0 || higher(y2, e2, by, be))) {
+                            by = y2;
+                            be = e2;
+                        }
+                    }
+                    if (lane == last) {
+                        if (lower(ay, ae, ylo, lo)) {
+                            ylo = ay;
+                            lo = ae;
+                        }
+                        if (higher(by, be, yhi, hi)) {
+                            yhi = by;
+                            hi = be;
+                        }
+                        end_of_run = stop;
+                    }
                 }
+                const bool rep = tail && mine;
+                int o0 = 0, o1 = 0;
+                const bool end = p.x == A.x || p.x == B.x;
+                if (rep) {
+                    if (ext && end_of_run == m) {   // and past the super-chunk
+                        if (lower(sm.pts[SC].y, SC, ylo, lo)) lo = SC;
+                        if (higher(sm.pts[SC + 1].y, SC + 1, yhi, hi)) hi = SC + 1;
+                    }
+                    low[i] = (uint16_t)lo;
+                    high[i] = (uint16_t)hi;
+                    if (p.x == A.x) {
+                        sm.run[0] = lo;
+                        sm.run[1] = hi;
+                    }
+                    if (p.x == B.x) {
+                        sm.run[2] = lo;
+                        sm.run[3] = hi;
+                    }
+                    if (!end) {
+                        const float2 u = sm.pts[lo];
+                        o0 = o1 = orient(A.x, A.y, u.x, u.y, B.x, B.y);
+                        if (hi != lo) {
+                            const float2 v = sm.pts[hi];
+                            o1 = orient(A.x, A.y, v.x, v.y, B.x, B.y);
+                        }
+                    }
+                }
+                const uint32_t m0 = __ballot_sync(0xffffffffu, rep && (end || o0 > 0));
+                const uint32_t m1 = __ballot_sync(0xffffffffu, rep && (end || o1 < 0));
+                if (lane == c) {
+                    masks0 = m0;
+                    masks1 = m1;
+                }
+                c01 += __popc(m0) + (__popc(m1) << 16);
+                cylo = __shfl_sync(0xffffffffu, ylo, 31);
+                cyhi = __shfl_sync(0xffffffffu, yhi, 31);
+                clo = __shfl_sync(0xffffffffu, lo, 31);
+                chi = __shfl_sync(0xffffffffu, hi, 31);
+                owned = __shfl_sync(0xffffffffu, mine ? 1 : 0, 31) != 0;
             }
-            put(k, lo, ylo, hi, yhi);
-        }
-        __syncthreads();
-        for (int q = warp; q < sm.nlong; q += NWB) {
-            const int k = sm.lrun[q];
-            const int r0 = sm.list[2][k];
-            const int r1 = k + 1 < R ? sm.list[2][k + 1] : m;
-            int lo = r0 + lane, hi = lo;   // (a long run has a point for every lane)
-            float ylo = sm.pts[lo].y, yhi = ylo;
-            for (int i = lo + 32; i < r1; i += 32) {
-                const float y = sm.pts[i].y;
-                if (lower(y, i, ylo, lo)) {
-                    ylo = y;
-                    lo = i;
-                }
-                if (higher(y, i, yhi, hi)) {
-                    yhi = y;
-                    hi = i;
-                }
-            }
+            if (lane == 0) sm.wsum[warp] = c01;
+            __syncthreads();
+            const bool last_two = holds_last && sm.pts[sm.run[3]].y > sm.pts[sm.run[2]].y;
+            const bool first_two = base == sbeg && sm.pts[sm.run[1]].y > sm.pts[sm.run[0]].y;
+            uint32_t before = 0, total = 0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float y1 = __shfl_xor_sync(0xffffffffu, ylo, o), y2 = __shfl_xor_sync(0xffffffffu, yhi, o);
-                const int e1 = __shfl_xor_sync(0xffffffffu, lo, o), e2 = __shfl_xor_sync(0xffffffffu, hi, o);
-                if (lower(y1, e1, ylo, lo)) {
-                    ylo = y1;
-                    lo = e1;
-                }
-                if (higher(y2, e2, yhi, hi)) {
-                    yhi = y2;
-                    hi = e2;
-                }
+            for (int w = 0; w < NWB; ++w) {
+                const uint32_t u = sm.wsum[w];
+                if (w < warp) before += u;
+                total += u;
             }
-            if (lane == 0) put(k, lo, ylo, hi, yhi);
+            n0 = (int)(total & 0xffffu) + (last_two ? 1 : 0);
+            n1 = (int)(total >> 16) + (first_two ? 1 : 0);
+            int at0 = (int)(before & 0xffffu), at1 = n0 + (int)(before >> 16) + (first_two ? 1 : 0);
+#pragma unroll 2
+            for (int c = 0; j0 + c * 32 < j1; ++c) {
+                const int j = j0 + c * 32 + lane;
+                const uint32_t m0 = __shfl_sync(0xffffffffu, masks0, c), m1 = __shfl_sync(0xffffffffu, masks1, c);
+                if ((m0 >> lane) & 1u) sm.seq[at0 + __popc(m0 & lt)] = low[j];
+                if ((m1 >> lane) & 1u) sm.seq[at1 + __popc(m1 & lt)] = high[j];
+                at0 += __popc(m0);
+                at1 += __popc(m1);
+            }
+            if (t == 0) {
+                if (last_two) sm.seq[n0 - 1] = (uint16_t)sm.run[3];
+                if (first_two) sm.seq[n0] = (uint16_t)sm.run[0];
+            }
+            __syncthreads();
+        }
+
+        // ---- elimination, half of the block per side: rounds of one pass over
+        // the whole sequence, each warp its share, then passes inside the
+        // shares (their ends stay), then the shares closed up again; done when
+        // the first pass of a round drops nothing
+        {
+            const int side = warp / NWS, gw = warp % NWS;
+            uint16_t *const X = sm.seq + (side ? n0 : 0), *const Y = X + SY;
+            int len = side ? n1 : n0, w0 = 0, wl = 0, pass = 0, round = 0;
+            bool strict = len <= 2, whole = true, in_y = false;
+#pragma unroll 1
+            while (!strict) {
+                if (whole) {
+                    const int S = (len + NWS - 1) / NWS;
+                    w0 = min(gw * S, len);
+                    wl = min(S, len - w0);
+                    in_y = false;
+                }
+                const int kept = warp_elim_pass(sm.pts, (in_y ? Y : X) + w0, (in_y ? X : Y) + w0, wl, side, lane, lt,
+                                                whole && w0 > 0, whole && w0 + wl < len);
+                in_y = !in_y;
+                bool closed = kept <= 2;
+                if (whole) {
+                    if (lane == 0) sm.wsum[warp] = (uint32_t)kept;
+                    side_barrier(side);
+                    int total = 0;
+#pragma unroll
+                    for (int w = 0; w < NWS; ++w) total += (int)sm.wsum[side * NWS + w];
+                    if (total == len) {
+                        strict = true;
+                        break;
+                    }
+                    whole = false;
+                    pass = 0;
+                } else {
+                    closed |= kept == wl || ++pass == kElimPasses;
+                }
+                wl = kept;
+                if (!closed) continue;
+                if (!in_y) {
+                    for (int i = lane; i < wl; i += 32) Y[w0 + i] = X[w0 + i];
+                }
+                side_barrier(side);   // wsum has been read
+                if (lane == 0) sm.wsum[warp] = (uint32_t)wl;
+                side_barrier(side);
+                int at = 0;
+                len = 0;
+#pragma unroll
+                for (int w = 0; w < NWS; ++w) {
+                    const int u = (int)sm.wsum[side * NWS + w];
+                    if (w < gw) at += u;
+                    len += u;
+                }
+                for (int i = lane; i < wl; i += 32) X[at + i] = Y[w0 + i];
+                side_barrier(side);
+                strict = len <= 2;
+                if (++round == kElimRounds) break;
+                whole = true;
+            }
+            if (gw == 0 && lane == 0) {
+                sm.seq_len[side] = len;
+                sm.strict[side] = strict ? 1 : 0;
+            }
         }
         __syncthreads();
-        const uint16_t first_lo = sm.list[0][0];
-        const bool first_two = base == sbeg && sm.pts[sm.list[1][0]].y > sm.pts[first_lo].y;
 
         for (int side = 0; side < 2; ++side) {
-            // ---- this side's sequence in list[0]
-            if (side == 0) {
-                // lowest of every run, then the highest of the very last run
+            const int o = side ? n0 : 0, blen = sm.seq_len[side];
+            const uint16_t *flat = sm.seq + o;
+            if (sm.strict[side]) {   // its own chain
+                uint32_t *dpos = P.pos[side] + sc * CS;
+                float2 *dpt = P.pt[side] + sc * CS;
+                for (int q = t; q < blen; q += LT) {
+                    const int e = flat[q];
+                    dpos[q] = e < SC ? (uint32_t)place(e) : sm.ext_pos[e - SC];
+                    dpt[q] = sm.pts[e];
+                }
                 if (t == 0) {
-                    int len = R;
-                    if (holds_last && sm.pts[sm.list[1][R - 1]].y > sm.pts[sm.list[0][R - 1]].y)
-                        sm.list[0][len++] = sm.list[1][R - 1];
-                    sm.seq_len = len;
+                    P.lo[side][sc] = 0;
+                    P.hi[side][sc] = blen - 1;
                 }
-            } else {
-                // the lowest of the very first run, then the highest of every run
-                const int off = first_two ? 1 : 0;
-                for (int k = t; k < R; k += LT) sm.list[0][k + off] = sm.list[1][k];
-                if (t == 0) {
-                    if (first_two) sm.list[0][0] = first_lo;
-                    sm.seq_len = R + off;
-                }
+                continue;
             }
-            __syncthreads();
-            const int len = sm.seq_len;
-            // ---- per warp: its share of the sequence, [warp * S, warp * S + S)
-            const int S = (len + NWB - 1) / NWB;
-            int w0 = warp * S;
-            int wl = max(0, min(S, len - w0));   // this warp's live length
-            uint16_t *flat = &sm.list[0][0];
-            int cur = 0;                          // 0: list[0], 2: list[2]
-            // elimination passes over the warp's segment; its two ends stay
-            for (int pass = 0; pass < kElimPasses && wl > 2; ++pass) {
-                const int kept = warp_elim_pass(sm.pts, flat + cur * NL + w0, flat + (2 - cur) * NL + w0, wl, side,
-                                                lane, lt);
-                cur = 2 - cur;
-                const bool done = kept == wl;
-                wl = kept;
-                if (done) break;
-            }
-            // ---- block level: the warps' survivors concatenated in list[2],
-            // then passes over the whole sequence.  A sequence whose every
-            // turn is strict is its own chain: no leaves, no merges.
-            if (cur == 2)
-                for (int i = lane; i < wl; i += 32) flat[w0 + i] = flat[2 * NL + w0 + i];
-            if (lane == 0) sm.wsum[warp] = (uint32_t)wl;
-            __syncthreads();
-            {
-                int off = 0, tot = 0;
-#pragma unroll
-                for (int w = 0; w < NWB; ++w) {
-                    const int u = (int)sm.wsum[w];
-                    if (w < warp) off += u;
-                    tot += u;
-                }
-                for (int i = lane; i < wl; i += 32) flat[2 * NL + off + i] = flat[w0 + i];
-                __syncthreads();
-                int blen = tot, bcur = 2;
-                bool chain_done = blen <= 2;
-                // long: all threads, block-wide compaction
-                for (int bp = 0; bp < kBlockElimPasses && !chain_done && blen > kWarpSeqMax; ++bp) {
-                    const uint16_t *src = flat + bcur * NL;
-                    const int bl = blen;
-                    const int kept = block_compact(
-                        sm, bl,
-                        [&](int j) {
-                            return j == 0 || j == bl - 1 ||
-                                   !drop(side, sm.pts[src[j - 1]], sm.pts[src[j]], sm.pts[src[j + 1]]);
-                        },
-                        [&](int j) { return src[j]; }, flat + (2 - bcur) * NL);
-                    bcur = 2 - bcur;
-                    chain_done = kept == bl || kept <= 2;
-                    blen = kept;
-                }
-                if (!chain_done && blen <= kWarpSeqMax) {
-                    // short: one warp runs the passes, no block barriers
-                    if (warp == 0) {
-                        int bl = blen, wc = bcur, done = 0;
-                        for (int bp = 0; bp < kBlockElimPasses && !done; ++bp) {
-                            const int kept =
-                                warp_elim_pass(sm.pts, flat + wc * NL, flat + (2 - wc) * NL, bl, side, lane, lt);
-                            wc = 2 - wc;
-                            done = kept == bl || kept <= 2;
-                            bl = kept;
-                        }
-                        if (lane == 0) {
-                            sm.seq_len = bl;
-                            sm.wcur = wc;
-                            sm.wdone = done;
-                        }
-                    }
-                    __syncthreads();
-                    blen = sm.seq_len;
-                    bcur = sm.wcur;
-                    chain_done = sm.wdone != 0;
-                }
-                if (chain_done) {   // write the chain and go to the other side
-                    uint32_t *dpos = P.pos[side] + sc * CS;
-                    float2 *dpt = P.pt[side] + sc * CS;
-                    for (int q = t; q < blen; q += LT) {
-                        const int e = flat[bcur * NL + q];
-                        dpos[q] = e < SC ? (uint32_t)place(e) : sm.ext_pos[e - SC];
-                        dpt[q] = sm.pts[e];
-                    }
-                    if (t == 0) {
-                        P.lo[side][sc] = 0;
-                        P.hi[side][sc] = blen - 1;
-                    }
-                    __syncthreads();
-                    continue;
-                }
-                // not yet a chain: leaves and merges over the block's sequence
-                const int S2 = (blen + NWB - 1) / NWB;
-                w0 = warp * S2;
-                wl = max(0, min(S2, blen - w0));
-                cur = bcur;
-            }
+            // not yet a chain: leaves and merges over the block's sequence
+            const int S2 = (blen + NWB - 1) / NWB, w0 = warp * S2;
+            const int wl = max(0, min(S2, blen - w0));
             // ---- leaf chains: lane l takes [l * LW, l * LW + LW) of the warp's list
             const int LW = (wl + 31) / 32;
-            const int lbase = cur * NL + w0 + lane * LW;
+            const int lbase = w0 + lane * LW;
             const int cnt = max(0, min(LW, wl - lane * LW));
             sm.lb[t] = (int16_t)lbase;
             int h = 0;
@@ -915,7 +954,7 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
             sm.first[t] = sm.last[t] = (int16_t)(h > 0 ? t : -1);
             __syncwarp();
             // ---- merge tree: five levels inside the warp, then three across warps
-            SmemAcc A{sm, flat};
+            const SmemAcc A{sm, flat};
             for (int w = 1; w < 32; w *= 2) {
                 if (lane < 32 / (2 * w)) {
                     const int a0 = warp * 32 + 2 * lane * w, b0 = a0 + w;
@@ -957,6 +996,7 @@ __device__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t
             }
             __syncthreads();
         }
+        __syncthreads();   // sm is staged again
     }
 }
 
@@ -974,20 +1014,8 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t 
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
     if (s == 0) return;
-    if (s <= (uint32_t)SC) {
-        if (blockIdx.x != 0) return;
-        const ChainPtrs P = chain_ptrs(ws, L, ctrl->sort_in);
-        superchunk<true>(sm, P, 0, 0, (int)s, 0, s);   // (ends with a barrier)
-        const uint32_t hl = (uint32_t)__ldcg(P.hi[0]) + 1u, hu = (uint32_t)__ldcg(P.hi[1]) + 1u;
-        for (int it = (int)(threadIdx.x >> 5); it < 2 * kCopyParts; it += NWB)
-            copy_chain_part(P, it & 1, 0, it >> 1, 0u, hl, hu, hull_idx, L.n);
-        if (threadIdx.x == 0) {
-            *hull_count = hl + (hu >= 2 ? hu - 2 : 0u);
-            ctrl->small_done = 1u;
-        }
-        return;
-    }
-    const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
+    const bool local = s <= (uint32_t)SC;   // not sorted yet
+    const ChainPtrs P = chain_ptrs(ws, L, local ? ctrl->sort_in : ctrl->final_buf);
     const int64_t nsc = ceil_div((int64_t)s, SC);
     for (int64_t sc = blockIdx.x; sc < nsc; sc += gridDim.x) {
         // the block's next super-chunk streams into L2 meanwhile
@@ -997,7 +1025,15 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t 
             bulk_prefetch_l2(P.keys + nxt * SC, (nn * 4u) & ~15u);
             bulk_prefetch_l2(P.pay + nxt * SC, (nn * 8u) & ~15u);
         }
-        superchunk<false>(sm, P, sc, sc * SC, (int)min((int64_t)SC, (int64_t)s - sc * SC), 0, s);
+        superchunk(sm, P, sc, sc * SC, (int)min((int64_t)SC, (int64_t)s - sc * SC), 0, s, local);
+    }
+    if (!local || blockIdx.x != 0) return;
+    const uint32_t hl = (uint32_t)__ldcg(P.hi[0]) + 1u, hu = (uint32_t)__ldcg(P.hi[1]) + 1u;   // (behind a barrier)
+    for (int it = (int)(threadIdx.x >> 5); it < 2 * kCopyParts; it += NWB)
+        copy_chain_part(P, it & 1, 0, it >> 1, 0u, hl, hu, hull_idx, L.n);
+    if (threadIdx.x == 0) {
+        *hull_count = hl + (hu >= 2 ? hu - 2 : 0u);
+        ctrl->small_done = 1u;
     }
 }
 
@@ -1034,8 +1070,8 @@ __global__ void __launch_bounds__(LT) bx_chain_kernel(void *ws, Layout L, BatchL
         const uint32_t b = sc_set[j];
         const int64_t sb = (int64_t)sets[b].surv_base, n = sets[b].s;
         const int64_t local = j - sets[b].sc_base;
-        if (n <= (int64_t)kBxLocalMax) superchunk<true>(sm, P, j, sb, (int)n, sb, sb + n);
-        else superchunk<false>(sm, P, j, sb + local * SC, (int)min((int64_t)SC, n - local * SC), sb, sb + n);
+        superchunk(sm, P, j, sb + local * SC, (int)min((int64_t)SC, n - local * SC), sb, sb + n,
+                   n <= (int64_t)kBxLocalMax);
     }
 }
 

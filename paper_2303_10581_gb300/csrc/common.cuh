@@ -38,8 +38,7 @@ constexpr int kChainThreads = 256;    // leaves per super-chunk (one block)
 constexpr int kChainC = kLeafC * kChainThreads;   // 4096 points per super-chunk
 constexpr int kChainStride = kChainC + 8;          // chain slots per super-chunk (up to kChainC + 1 used)
 constexpr int kElimPasses = 12;       // cap on the per-warp elimination passes
-constexpr int kBlockElimPasses = 24;  // cap on the passes over a super-chunk's whole sequence
-constexpr int kWarpSeqMax = 256;      // whole-sequence passes run in one warp up to this length
+constexpr int kElimRounds = 24;       // cap on the rounds over a side's whole sequence
 constexpr int kEmitThreads = 256;     // chunks per emit tile (one per thread)
 constexpr int64_t kMaxHullN = (int64_t)1 << 30;
 constexpr int64_t kMaxN = ((int64_t)1 << 32) - 1;
@@ -476,6 +475,21 @@ __device__ __forceinline__ float2 key_point(unsigned long long k)
     return make_float2(key_float((uint32_t)(k >> 32)), key_float((uint32_t)k));
 }
 
+// a - b = s + e and a + b = s + e exactly (Knuth's two-sum, binary32
+// round to nearest; the intrinsics are never contracted into an FMA)
+__device__ __forceinline__ void two_diff(float a, float b, float &s, float &e)
+{
+    s = __fsub_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
+}
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
 // ---------------------------------------------------------------------------
 // exact orientation: sign of (b - a) x (c - a) for binary32 inputs
 // ---------------------------------------------------------------------------
@@ -587,7 +601,7 @@ __device__ __forceinline__ int orient_near(float ax, float ay, float bx, float b
 // eps = 2^-24 when nothing under- or overflows; 4 eps * detsum leaves room
 // for the rounding of the bound itself, and 2^-140 absorbs the absolute
 // error of products that fall into the subnormal range.  Undecided cases
-// try tier 1b, then tier 2.
+// go on to tier 2.
 // The binary32 tier alone, branch-free: the sign when the bound proves it,
 // 2 otherwise.
 __device__ __forceinline__ int orient_f32(float ax, float ay, float bx, float by, float cx, float cy)
@@ -601,25 +615,47 @@ __device__ __forceinline__ int orient_f32(float ax, float ay, float bx, float by
     return detsum <= 3.0e38f ? o : 2;
 }
 
-// orient_f32 of (a, b, c) given the rounded differences a - c = (acx, acy)
-// and b - c = (bcx, bcy): the same arithmetic after the subtractions.
-__device__ __forceinline__ int orient_f32_ref(float acx, float acy, float bcx, float bcy)
+// Tier 2: the differences as exact pairs (two-diff), the products and their
+// rounding errors (FMA), everything of second order added up in binary32: the
+// sign when the bound proves it, 2 otherwise.  With eps = 2^-24 the second-
+// order terms are below 6 eps detsum in sum, so their ten roundings and the
+// omitted product of two low parts cost less than 64 eps^2 detsum = 2^-42
+// detsum, and 2^-138 absorbs products in the subnormal range.  It settles
+// nearly every near-collinear triple of a ring's neighbours.  In binary64 (at
+// a 64th of the rate here, some 70 cycles an instruction) one such lane held
+// its warp for a thousand cycles: %OP%.
+__device__ __forceinline__ int orient_pair(float ax, float ay, float bx, float by, float cx, float cy)
 {
-    float detleft = __fmul_rn(acx, bcy);
-    float detright = __fmul_rn(acy, bcx);
-    float det = __fsub_rn(detleft, detright);
-    float detsum = __fadd_rn(fabsf(detleft), fabsf(detright));
-    float eb = __fmaf_ru(detsum, 2.384185791015625e-07f /* 2^-22 */, 7.174648137343064e-43f /* 2^-140 */);
+    float u, ul, v, vl, w, wl, z, zl;
+    two_diff(ax, cx, u, ul);
+    two_diff(by, cy, v, vl);
+    two_diff(ay, cy, w, wl);
+    two_diff(bx, cx, z, zl);
+    const float p = __fmul_rn(u, v), q = __fmul_rn(w, z);
+    const float pe = __fmaf_rn(u, v, -p), qe = __fmaf_rn(w, z, -q);
+    const float pl = __fmaf_rn(u, vl, __fmul_rn(ul, v)), ql = __fmaf_rn(w, zl, __fmul_rn(wl, z));
+    float s, sl;
+    two_diff(p, q, s, sl);
+    const float t = __fadd_rn(__fadd_rn(__fsub_rn(pe, qe), __fsub_rn(pl, ql)), sl);
+    const float det = __fadd_rn(s, t), detsum = __fadd_rn(fabsf(p), fabsf(q));
+    const float eb = __fmaf_ru(detsum, 0x1p-42f, 0x1p-138f);
     const int o = det > eb ? 1 : (-det > eb ? -1 : 2);
     return detsum <= 3.0e38f ? o : 2;
 }
 
-// The tiers after binary32: exact differences, binary64, expansions.
+// The tiers after that: equal points, exact differences, binary64, expansions
+// (whose 200 binary64 steps are some 15000 cycles).
+static __device__ __noinline__ int orient_last(float ax, float ay, float bx, float by, float cx, float cy)
+{
+    if ((ax == cx && ay == cy) || (bx == cx && by == cy) || (ax == bx && ay == by)) return 0;
+    const int o = orient_near(ax, ay, bx, by, cx, cy);
+    return o != 2 ? o : orient_d(ax, ay, bx, by, cx, cy);
+}
+
 __device__ __forceinline__ int orient_rest(float ax, float ay, float bx, float by, float cx, float cy)
 {
-    const int o = orient_near(ax, ay, bx, by, cx, cy);
-    if (o != 2) return o;
-    return orient_d(ax, ay, bx, by, cx, cy);
+    const int o = orient_pair(ax, ay, bx, by, cx, cy);
+    return o != 2 ? o : orient_last(ax, ay, bx, by, cx, cy);
 }
 
 __device__ __forceinline__ int orient(float ax, float ay, float bx, float by, float cx, float cy)

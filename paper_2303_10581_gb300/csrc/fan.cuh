@@ -70,21 +70,6 @@ __device__ __forceinline__ float2 fan_direction(Bins nb, float a)
     return make_float2(q < 2.0f ? 1.0f - fabsf(t) : fabsf(t) - 1.0f, t);
 }
 
-// a - b = s + e and a + b = s + e exactly (Knuth's two-sum, binary32
-// round to nearest; the intrinsics are never contracted into an FMA)
-__device__ __forceinline__ void two_diff(float a, float b, float &s, float &e)
-{
-    s = __fsub_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
-}
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // Order key for the farthest-point choice of a bin: |p - c|^2 - r2ref,
 // from the differences p - c and their squares as exact pairs (two-sum,
 // two-product by FMA), rounded once at the end.  The binary32 square

@@ -49,7 +49,7 @@ __device__ __noinline__ bool keep_point(const Octagon &o, float x, float y)
         const float bnd = o.bound[e];
         if (t > bnd) continue;
         if (t < -bnd) return true;
-        if (orient_d(o.ax[e], o.ay[e], o.bx[e], o.by[e], x, y) <= 0) return true;
+        if (orient_rest(o.ax[e], o.ay[e], o.bx[e], o.by[e], x, y) <= 0) return true;
     }
     return false;
 }
