@@ -103,9 +103,20 @@ __device__ __forceinline__ int warp_elim_pass(const float2 *pts, const uint16_t 
             c[u] = test[u] ? pts[src[jj + 1]] : b[u];
             o[u] = orient_f32(a[u].x, a[u].y, b[u].x, b[u].y, c[u].x, c[u].y);
         }
+        if (__any_sync(0xffffffffu, (test[0] && o[0] == 2) || (test[1] && o[1] == 2))) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
-            if (test[u] && o[u] == 2) o[u] = orient_rest(a[u].x, a[u].y, b[u].x, b[u].y, c[u].x, c[u].y);
+            for (int u = 0; u < 2; ++u)
+                if (o[u] == 2) o[u] = orient_pair(a[u].x, a[u].y, b[u].x, b[u].y, c[u].x, c[u].y);
+#pragma unroll 1
+            for (int u = 0; u < 2; ++u) {
+                const float2 A = u ? a[1] : a[0], B = u ? b[1] : b[0], C = u ? c[1] : c[0];
+                if ((u ? test[1] && o[1] == 2 : test[0] && o[0] == 2)) {
+                    const int r = orient_last(A.x, A.y, B.x, B.y, C.x, C.y);
+                    o[0] = u ? o[0] : r;
+                    o[1] = u ? r : o[1];
+                }
+            }
+        }
         uint32_t m[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -271,35 +282,29 @@ __device__ __forceinline__ uint32_t block_scan(ChainSmem &s, uint32_t v)
 struct ChainPtrs {
     const uint32_t *keys;             // sorted ord(x)
     const unsigned long long *pay;    // sorted ord(y) << 32 | index
-    uint32_t *pos[2];                 // chain vertices: sorted positions, super-chunk c at [c * CS, ...)
-    float2 *pt[2];                    // chain vertices: coordinates
-    int32_t *lo[2], *hi[2], *prv[2], *nxt[2];
+    uint32_t *pos0, *pos1;            // chain vertices: sorted positions, super-chunk c at [c * CS, ...)
+    float2 *pt0, *pt1;                // chain vertices: coordinates
+    int32_t *chunk;                   // per side lo, hi (the surviving range), then per side prv, nxt, n_chunks each
+    int64_t n_chunks;
     int32_t *node;                    // 4 ints per tree node: firstL lastL firstU lastU
-    int32_t *node_cnt;                // arrivals per node (zeroed at the start of each call)
+    int32_t *node_cnt;                // arrivals per node and side (zeroed at the start of each call)
+
+    // (no arrays: an index known only at run time would put them in local memory)
+    __device__ uint32_t *pos(int side) const { return side ? pos1 : pos0; }
+    __device__ float2 *pt(int side) const { return side ? pt1 : pt0; }
+    __device__ int32_t *lo(int side) const { return chunk + 2 * side * n_chunks; }
+    __device__ int32_t *hi(int side) const { return chunk + (2 * side + 1) * n_chunks; }
+    __device__ int32_t *prv(int side) const { return chunk + (4 + 2 * side) * n_chunks; }
+    __device__ int32_t *nxt(int side) const { return chunk + (5 + 2 * side) * n_chunks; }
 };
 
 __device__ __forceinline__ ChainPtrs chain_ptrs(void *ws, const Layout &L, uint32_t buf)
 {
-    ChainPtrs P;
-    P.keys = at<uint32_t>(ws, L.keys[buf]);
-    P.pay = at<unsigned long long>(ws, L.pay[buf]);
-    for (int side = 0; side < 2; ++side) {
-        P.pos[side] = at<uint32_t>(ws, L.chain_pos[side]);
-        P.pt[side] = at<float2>(ws, L.chain_pt[side]);
-    }
-    int32_t *ck = at<int32_t>(ws, L.chunk);
-    const int64_t nc = L.n_chunks;
-    P.lo[0] = ck + 0 * nc;
-    P.hi[0] = ck + 1 * nc;
-    P.lo[1] = ck + 2 * nc;
-    P.hi[1] = ck + 3 * nc;
-    P.prv[0] = ck + 4 * nc;
-    P.nxt[0] = ck + 5 * nc;
-    P.prv[1] = ck + 6 * nc;
-    P.nxt[1] = ck + 7 * nc;
-    P.node = at<int32_t>(ws, L.node);
-    P.node_cnt = at<int32_t>(ws, L.node_cnt);
-    return P;
+    return {buf ? at<uint32_t>(ws, L.keys[1]) : at<uint32_t>(ws, L.keys[0]),
+            buf ? at<unsigned long long>(ws, L.pay[1]) : at<unsigned long long>(ws, L.pay[0]),
+            at<uint32_t>(ws, L.chain_pos[0]), at<uint32_t>(ws, L.chain_pos[1]),
+            at<float2>(ws, L.chain_pt[0]), at<float2>(ws, L.chain_pt[1]),
+            at<int32_t>(ws, L.chunk), L.n_chunks, at<int32_t>(ws, L.node), at<int32_t>(ws, L.node_cnt)};
 }
 
 __device__ __forceinline__ float2 sorted_point(const ChainPtrs &P, int64_t q)
@@ -407,7 +412,7 @@ struct MergeSide {
 // node merges its two children and continues upward (no warp ever waits).
 __device__ void climb(const ChainPtrs &P, int side, int64_t c, int64_t nsc, int64_t coff, int64_t noff)
 {
-    const MergeSide M{P.pt[side], P.lo[side], P.hi[side], P.prv[side], P.nxt[side], side};
+    const MergeSide M{P.pt(side), P.lo(side), P.hi(side), P.prv(side), P.nxt(side), side};
     const uint32_t lane = lane_id();
     int64_t node = c, w = nsc, nb_child = 0, nb = 0;   // nb: base of the level above
     int level = 0;
@@ -610,8 +615,8 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
         if (cont && xr == sm.prev_x) {   // the whole super-chunk continues an earlier run
             if (t == 0)
                 for (int side = 0; side < 2; ++side) {
-                    P.lo[side][sc] = 0;
-                    P.hi[side][sc] = -1;
+                    P.lo(side)[sc] = 0;
+                    P.hi(side)[sc] = -1;
                 }
             __syncthreads();
             return;
@@ -677,7 +682,7 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
         // points there can be vertices (a ring's chunk holds both arcs by
         // turns).  Bound by latency, like all of this kernel on few chunks:
         // runs, representatives and sequences in steps of their own (a thread
-        // per run) took 24000 to 48000 cycles on a ring's chunk, this %SW%.
+        // per run) took 24000 to 48000 cycles on a ring's chunk, this 16000 to 36000.
         uint16_t *const low = sm.seq + SY, *const high = low + NL;
         int n0, n1;
         {
@@ -701,35 +706,33 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
                 float ylo = p.y, yhi = p.y;
                 bool mine = true;
                 if (hm != vm) {
+                    uint32_t ilo = (uint32_t)__ldg(P.pay + place(i)), ihi = ilo;   // equal points: by index
+                    const auto take = [&](float y1, uint32_t i1, int e1, float y2, uint32_t i2, int e2) {
+                        if (y1 < ylo || (y1 == ylo && i1 < ilo)) {
+                            ylo = y1;
+                            ilo = i1;
+                            lo = e1;
+                        }
+                        if (y2 > yhi || (y2 == yhi && i2 < ihi)) {
+                            yhi = y2;
+                            ihi = i2;
+                            hi = e2;
+                        }
+                    };
                     const uint32_t upto = hm & (lt | (1u << lane));
                     const int start = upto ? 31 - __clz(upto) : 0;
 #pragma unroll 1
                     for (int o = 1; o < 32; o <<= 1) {
                         const float y1 = __shfl_up_sync(0xffffffffu, ylo, o), y2 = __shfl_up_sync(0xffffffffu, yhi, o);
+                        const uint32_t i1 = __shfl_up_sync(0xffffffffu, ilo, o), i2 = __shfl_up_sync(0xffffffffu, ihi, o);
                         const int e1 = __shfl_up_sync(0xffffffffu, lo, o), e2 = __shfl_up_sync(0xffffffffu, hi, o);
-                        if (lane - o >= start) {
-                            if (lower(y1, e1, ylo, lo)) {
-                                ylo = y1;
-                                lo = e1;
-                            }
-                            if (higher(y2, e2, yhi, hi)) {
-                                yhi = y2;
-                                hi = e2;
-                            }
-                        }
+                        if (lane - o >= start) take(y1, i1, e1, y2, i2, e2);
                     }
                     if (upto == 0u) {
                         mine = owned;
-                        if (c > 0) {
-                            if (lower(cylo, clo, ylo, lo)) {
-                                ylo = cylo;
-                                lo = clo;
-                            }
-                            if (higher(cyhi, chi, yhi, hi)) {
-                                yhi = cyhi;
-                                hi = chi;
-                            }
-                        }
+                        if (c > 0)   // the run open before these points
+                            take(cylo, (uint32_t)__ldg(P.pay + place(clo)), clo, cyhi,
+                                 (uint32_t)__ldg(P.pay + place(chi)), chi);
                     }
                 }
                 int end_of_run = i + 1;
@@ -914,16 +917,16 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
             const int o = side ? n0 : 0, blen = sm.seq_len[side];
             const uint16_t *flat = sm.seq + o;
             if (sm.strict[side]) {   // its own chain
-                uint32_t *dpos = P.pos[side] + sc * CS;
-                float2 *dpt = P.pt[side] + sc * CS;
+                uint32_t *dpos = P.pos(side) + sc * CS;
+                float2 *dpt = P.pt(side) + sc * CS;
                 for (int q = t; q < blen; q += LT) {
                     const int e = flat[q];
                     dpos[q] = e < SC ? (uint32_t)place(e) : sm.ext_pos[e - SC];
                     dpt[q] = sm.pts[e];
                 }
                 if (t == 0) {
-                    P.lo[side][sc] = 0;
-                    P.hi[side][sc] = blen - 1;
+                    P.lo(side)[sc] = 0;
+                    P.hi(side)[sc] = blen - 1;
                 }
                 continue;
             }
@@ -983,16 +986,16 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
             const int l = sm.lo[t], hh = sm.hi[t];
             const int c = hh >= l ? hh - l + 1 : 0;
             const int off = (int)block_scan(sm, (uint32_t)c);
-            uint32_t *dpos = P.pos[side] + sc * CS + off;
-            float2 *dpt = P.pt[side] + sc * CS + off;
+            uint32_t *dpos = P.pos(side) + sc * CS + off;
+            float2 *dpt = P.pt(side) + sc * CS + off;
             for (int q = 0; q < c; ++q) {
                 const int e = flat[lbase + sm.stk[(l + q) * LT + t]];
                 dpos[q] = e < SC ? (uint32_t)place(e) : sm.ext_pos[e - SC];
                 dpt[q] = sm.pts[e];
             }
             if (t == 0) {
-                P.lo[side][sc] = 0;
-                P.hi[side][sc] = (int)sm.total - 1;
+                P.lo(side)[sc] = 0;
+                P.hi(side)[sc] = (int)sm.total - 1;
             }
             __syncthreads();
         }
@@ -1028,7 +1031,7 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t 
         superchunk(sm, P, sc, sc * SC, (int)min((int64_t)SC, (int64_t)s - sc * SC), 0, s, local);
     }
     if (!local || blockIdx.x != 0) return;
-    const uint32_t hl = (uint32_t)__ldcg(P.hi[0]) + 1u, hu = (uint32_t)__ldcg(P.hi[1]) + 1u;   // (behind a barrier)
+    const uint32_t hl = (uint32_t)__ldcg(P.hi(0)) + 1u, hu = (uint32_t)__ldcg(P.hi(1)) + 1u;   // (behind a barrier)
     for (int it = (int)(threadIdx.x >> 5); it < 2 * kCopyParts; it += NWB)
         copy_chain_part(P, it & 1, 0, it >> 1, 0u, hl, hu, hull_idx, L.n);
     if (threadIdx.x == 0) {
@@ -1127,7 +1130,7 @@ __device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t
         if (c < nc) {
 #pragma unroll
             for (int side = 0; side < 2; ++side) {
-                const int32_t lo = __ldcg(P.lo[side] + c), hi = __ldcg(P.hi[side] + c);
+                const int32_t lo = __ldcg(P.lo(side) + c), hi = __ldcg(P.hi(side) + c);
                 cnt[side] = hi >= lo ? hi - lo + 1 : 0;
             }
         }
@@ -1190,9 +1193,9 @@ __device__ void emit_body(void *ws, const Layout &L, const ChainPtrs &P, int64_t
 __device__ __forceinline__ void copy_chain_part(const ChainPtrs &P, int side, int64_t c, int part, uint32_t off0,
                                                 uint32_t hl, uint32_t hu, uint32_t *out, int64_t limit)
 {
-    const int32_t lo = __ldcg(P.lo[side] + c), cnt = __ldcg(P.hi[side] + c) - lo + 1;
+    const int32_t lo = __ldcg(P.lo(side) + c), cnt = __ldcg(P.hi(side) + c) - lo + 1;
     const int32_t k1 = min(cnt, (part + 1) * kCopyLen);
-    const uint32_t *chain = P.pos[side] + c * CS + lo;
+    const uint32_t *chain = P.pos(side) + c * CS + lo;
     constexpr int U = 4;   // entries per lane in flight
     for (int32_t k0 = part * kCopyLen + (int32_t)lane_id(); k0 < k1; k0 += 32 * U) {
         uint32_t sp[U], ix[U];

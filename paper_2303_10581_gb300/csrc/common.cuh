@@ -623,7 +623,7 @@ __device__ __forceinline__ int orient_f32(float ax, float ay, float bx, float by
 // detsum, and 2^-138 absorbs products in the subnormal range.  It settles
 // nearly every near-collinear triple of a ring's neighbours.  In binary64 (at
 // a 64th of the rate here, some 70 cycles an instruction) one such lane held
-// its warp for a thousand cycles: %OP%.
+// its warp for a thousand cycles.
 __device__ __forceinline__ int orient_pair(float ax, float ay, float bx, float by, float cx, float cy)
 {
     float u, ul, v, vl, w, wl, z, zl;
