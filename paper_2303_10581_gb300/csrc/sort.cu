@@ -14,8 +14,7 @@
 // Structure (one-sweep style, Adinets & Merrill 2022): one histogram kernel
 // computes all four digit histograms in a single read and marks passes
 // whose digit is constant (skipped); each remaining pass is one persistent
-// kernel that ranks a 4096-key tile in shared memory (warp match_any
-// ranking, stable), finds the tile's per-digit global offsets by a
+// kernel that ranks a 4096-key tile in shared memory (per warp, stable), finds the tile's per-digit global offsets by a
 // decoupled look-back over 256 digit counters, and writes the tile out
 // digit-sorted, so stores are runs of consecutive addresses.  The payload
 // is staged in shared memory in element order and gathered through the
@@ -54,6 +53,17 @@ struct SortSmem {
     uint32_t warp_tot[NW];
     uint32_t tile;
 };
+
+// Each warp its digit counts and ranking words, before a tile.
+template <int T>
+__device__ __forceinline__ void clear_counts(SortSmem<T> &sm)
+{
+    const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<uint4 *>(sm.wh[warp])[lane] = zero;
+    reinterpret_cast<uint4 *>(sm.keys + warp * 256)[lane] = zero;
+    reinterpret_cast<uint4 *>(sm.keys + warp * 256)[32 + lane] = zero;
+}
 
 // exclusive scan of v over the block's threads (two barriers)
 template <int NW>
@@ -215,19 +225,34 @@ __device__ __forceinline__ void pass_tile(SortSmem<T> &sm, const PassIO &io, int
             k[j] = 0u;
         }
     }
-    // stable rank inside the warp, items in element order (j, lane)
+    // stable rank inside the warp, items in element order (j, lane).  The lanes
+    // of a digit find each other through a word per digit in shared memory:
+    // match.any takes a step per distinct digit, and with 28 of them among 32
+    // keys ranking was half of a tile's time (7500 of 17000 cycles, 2200 so).
+    // It stays for the top digit, the sign and most of the exponent: few
+    // values, whose lanes would meet at one word.
+    const bool top = shift == 24;
+    uint32_t *const mask = sm.keys + warp * 256;   // (cleared; the sorted keys come later)
     uint16_t rank[kItems];
 #pragma unroll
     for (int j = 0; j < kItems; ++j) {
         const uint32_t e = warp * (32 * kItems) + j * 32 + lane;
         const bool ok = e < tile_n;
-        const uint32_t d = ok ? (k[j] >> shift) & 255u : 256u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t before = __popc(peers & lt);
-        uint32_t cur = 0;
-        if (ok) cur = sm.wh[warp][d];
+        const uint32_t d = (k[j] >> shift) & 255u;
+        uint32_t peers;
+        if (top) {
+            peers = __match_any_sync(0xffffffffu, ok ? d : 256u);
+        } else {
+            if (ok) atomicOr(mask + d, 1u << lane);
+            __syncwarp();
+            peers = ok ? mask[d] : 0u;
+        }
+        const uint32_t cur = ok ? sm.wh[warp][d] : 0u, before = __popc(peers & lt);
         __syncwarp();
-        if (ok && before == 0) sm.wh[warp][d] = (uint16_t)(cur + __popc(peers));
+        if (ok && before == 0) {
+            sm.wh[warp][d] = (uint16_t)(cur + __popc(peers));
+            if (!top) mask[d] = 0u;
+        }
         __syncwarp();
         rank[j] = (uint16_t)(cur + before);
     }
@@ -340,7 +365,7 @@ __global__ void __launch_bounds__(kPassThreads, kPassBlocks) sort_pass_kernel(vo
                 bulk_prefetch_l2(io.pin + ahead * kSortTile, (nn * 8u) & ~15u);
             }
         }
-        reinterpret_cast<uint4 *>(sm.wh[warp])[lane] = make_uint4(0u, 0u, 0u, 0u);
+        clear_counts(sm);
         __syncthreads();
         const int64_t tile = sm.tile;
         if (tile >= ntiles) break;
@@ -418,7 +443,7 @@ __global__ void __launch_bounds__(kBxPassThreads, kPassBlocks) bx_sort_pass_kern
     }
     for (;;) {
         if (tid == 0) sm.tile = atomicAdd(&bc->sort_ticket[p], 1u);
-        reinterpret_cast<uint4 *>(sm.wh[warp])[lane] = make_uint4(0u, 0u, 0u, 0u);
+        clear_counts(sm);
         __syncthreads();
         const int64_t tile = sm.tile;
         if (tile >= ntiles) break;
