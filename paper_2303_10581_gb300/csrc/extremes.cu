@@ -860,50 +860,96 @@ __global__ void octagon_kernel(const float *__restrict__ pts, int64_t n, const u
 // Each block takes a contiguous range of tiles; the running extremes are
 // folded into the set's slots whenever the range moves on to another set
 // (sets are contiguous in tile order, so a block flushes once per set it
-// touches).
-template <int NWARP>
-__device__ __forceinline__ void bx_flush(Best &best, float &nf, int64_t b, unsigned long long *slots,
-                                         uint32_t *nonfin, float (&sk)[NWARP][8], uint32_t (&si)[NWARP][8], int &s_bad)
+// touches).  As in the sweep of one set, a thread keeps each slot's largest
+// key and the first tile that had it; the point is found at the flush, by
+// reading the winners' points again.  (An index per point and slot made it
+// bound by issue: 4096 sets of 445 M points 984 us; so, and with one
+// wave of blocks, about 700.)
+constexpr int kBxWinners = 32;       // of a slot at once; more look for themselves
+constexpr int kBxExtThreads = 1024;   // per SM
+
+struct BxFlush {
+    uint32_t key[8], cnt[8], idx[8];
+    uint2 win[8][kBxWinners];    // thread, tile
+};
+
+__device__ __forceinline__ uint32_t slot_key(int j, float2 p)
 {
-    const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+    float k[8];
+    slot_keys(p.x, p.y, k);
+    float v = k[0];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float ok = __shfl_xor_sync(0xffffffffu, best.k[j], o);
-            const uint32_t oi = __shfl_xor_sync(0xffffffffu, best.i[j], o);
-            combine(best.k[j], best.i[j], ok, oi);
-        }
+    for (int q = 1; q < 8; ++q) v = j == q ? k[q] : v;
+    return ord_key(v);
+}
+
+template <int T>
+__device__ __forceinline__ void bx_flush(BxFlush &f, float (&bk)[8], int32_t (&bt)[8], bool &nan_seen, int64_t b,
+                                         const SetInfo &S, const float2 *__restrict__ p2, unsigned long long *slots,
+                                         uint32_t *nonfin)
+{
+    constexpr int R = kFiltTile / T;   // points per thread per tile
+    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
+    const auto point = [&](uint32_t th, int32_t tile, int r) {
+        return ((int64_t)tile - (int64_t)S.tile_base) * kFiltTile + r * T + th;
+    };
+    if (tid < 8) {
+        f.key[tid] = f.cnt[tid] = 0u;
+        f.idx[tid] = 0xffffffffu;
     }
-    __syncthreads();   // sk, si and s_bad of the previous flush have been read
-    if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
-    if (nf != nf) s_bad = 1;
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            sk[warp][j] = best.k[j];
-            si[warp][j] = best.i[j];
-        }
-    __syncthreads();
-    if (warp == 0 && lane < 8) {
-        float k = sk[0][lane];
-        uint32_t i = si[0][lane];
-        for (int w = 1; w < NWARP; ++w) combine(k, i, sk[w][lane], si[w][lane]);
-        if (i != 0xffffffffu)
-            atomicMax(&slots[(size_t)b * 8 + lane], ((unsigned long long)ord_key(k) << 32) | (uint32_t)~i);
-        if (lane == 0 && s_bad) atomicOr(&nonfin[b], 1u);
-    }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        best.k[j] = __int_as_float(0x7fc00000);
-        best.i[j] = 0xffffffffu;
+        const uint32_t m = __reduce_max_sync(0xffffffffu, bt[j] >= 0 ? ord_key(bk[j]) : 0u);
+        if (lane == 0) atomicMax(&f.key[j], m);
     }
-    nf = 0.0f;
+    bool bad = __syncthreads_or(nan_seen);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (bt[j] < 0 || ord_key(bk[j]) != f.key[j]) continue;
+        const uint32_t k = atomicAdd(&f.cnt[j], 1u);
+        if (k < (uint32_t)kBxWinners) {
+            f.win[j][k] = make_uint2(tid, (uint32_t)bt[j]);
+            continue;
+        }
+        for (int r = 0; r < R; ++r) {
+            const int64_t i = point(tid, bt[j], r);
+            if (i < S.n && slot_key(j, p2[i]) == f.key[j]) {
+                atomicMin(&f.idx[j], (uint32_t)i);
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    if (warp < 8) {   // a warp per slot
+        uint32_t best = 0xffffffffu;
+        for (uint32_t k = 0; k < min(f.cnt[warp], (uint32_t)kBxWinners); ++k) {
+            const uint2 w = f.win[warp][k];
+            const int64_t i = point(w.x, (int32_t)w.y, (int)lane);
+            if (lane < (uint32_t)R && i < S.n && slot_key((int)warp, p2[i]) == f.key[warp]) best = min(best, (uint32_t)i);
+        }
+        best = __reduce_min_sync(0xffffffffu, best);
+        if (lane == 0) atomicMin(&f.idx[warp], best);
+    }
+    __syncthreads();
+    if (tid < 8) {
+        // an infinite coordinate is an extreme of x or y
+        if ((tid & 1u) == 0u && !(fabsf(key_float(f.key[tid])) <= 3.402823466e38f)) bad = true;
+        if (f.idx[tid] != 0xffffffffu)
+            atomicMax(&slots[b * 8 + tid], ((unsigned long long)f.key[tid] << 32) | (uint32_t)~f.idx[tid]);
+        if (bad) nonfin[b] = 1u;
+    }
+    __syncthreads();   // f is set up again
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        bk[j] = __int_as_float(0x7fc00000);
+        bt[j] = -1;
+    }
+    nan_seen = false;
 }
 
 template <int T>   // threads per block: each holds kFiltTile / T points of a tile
-__global__ void __launch_bounds__(T) bx_extremes_kernel(const float *__restrict__ pts, void *ws, Layout L,
+__global__ void __launch_bounds__(T, kBxExtThreads / T) bx_extremes_kernel(const float *__restrict__ pts, void *ws, Layout L,
                                                         BatchLayout BL)
 {
     kernel_entry();
@@ -913,25 +959,25 @@ __global__ void __launch_bounds__(T) bx_extremes_kernel(const float *__restrict_
     const uint32_t *tile_set = at<uint32_t>(ws, BL.tile_set);
     unsigned long long *slots = at<unsigned long long>(ws, BL.ext_slot);
     uint32_t *nonfin = at<uint32_t>(ws, BL.nonfinite);
-    __shared__ float sk[T / 32][8];
-    __shared__ uint32_t si_[T / 32][8];
-    __shared__ int s_bad;
+    __shared__ BxFlush f;
     const int64_t NT = bc->tiles;
-    const int64_t per = ceil_div(NT, (int64_t)gridDim.x);
-    const int64_t t0 = (int64_t)blockIdx.x * per, t1 = min(NT, t0 + per);
+    const int64_t t0 = (int64_t)blockIdx.x * NT / gridDim.x, t1 = ((int64_t)blockIdx.x + 1) * NT / gridDim.x;
     constexpr int R = kFiltTile / T;   // points per thread per tile
-    Best best;
+    float bk[8];
+    int32_t bt[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        best.k[j] = __int_as_float(0x7fc00000);
-        best.i[j] = 0xffffffffu;
+        bk[j] = __int_as_float(0x7fc00000);   // NaN: none yet
+        bt[j] = -1;
     }
-    float nf = 0.0f;
+    bool nan_seen = false;
     int64_t cur = -1;
     for (int64_t t = t0; t < t1; ++t) {
         const int64_t b = tile_set[t];   // block-uniform
         if (b != cur) {
-            if (cur >= 0) bx_flush(best, nf, cur, slots, nonfin, sk, si_, s_bad);
+            if (cur >= 0)
+                bx_flush<T>(f, bk, bt, nan_seen, cur, sets[cur],
+                            reinterpret_cast<const float2 *>(pts) + sets[cur].pt_begin, slots, nonfin);
             cur = b;
         }
         const int64_t lo = (t - sets[b].tile_base) * (int64_t)kFiltTile;
@@ -950,18 +996,31 @@ __global__ void __launch_bounds__(T) bx_extremes_kernel(const float *__restrict_
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int64_t i = lo + r * T + threadIdx.x;
-            v[r] = i < hi ? __ldcs(p2 + i) : make_float2(0.0f, 0.0f);
+            v[r] = __ldcs(p2 + (i < hi ? i : lo));   // (past the end: the tile's first point once more)
         }
+        float tb[8];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int64_t i = lo + r * T + threadIdx.x;
-            if (i < hi) {
-                nf = __fmaf_rn(v[r].x, 0.0f, __fmaf_rn(v[r].y, 0.0f, nf));
-                consider(best, v[r].x, v[r].y, (uint32_t)i);
+            float k[8];
+            slot_keys(v[r].x, v[r].y, k);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (r == 0) tb[j] = k[j];
+                else tb[j] = j == 0 || j == 2 ? max_nan(tb[j], k[j]) : fmaxf(tb[j], k[j]);
+            }
+        }
+        nan_seen |= (tb[0] != tb[0]) | (tb[2] != tb[2]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (!(tb[j] <= bk[j])) {
+                bk[j] = tb[j];
+                bt[j] = (int32_t)t;
             }
         }
     }
-    if (cur >= 0) bx_flush(best, nf, cur, slots, nonfin, sk, si_, s_bad);
+    if (cur >= 0)
+        bx_flush<T>(f, bk, bt, nan_seen, cur, sets[cur], reinterpret_cast<const float2 *>(pts) + sets[cur].pt_begin,
+                    slots, nonfin);
 }
 
 __global__ void __launch_bounds__(256) bx_octagon_kernel(const float *__restrict__ pts, void *ws, Layout L,
@@ -996,8 +1055,10 @@ __global__ void __launch_bounds__(256) bx_octagon_kernel(const float *__restrict
 
 cudaError_t launch_bx_extremes(const float *pts, void *ws, const Layout &L, const BatchLayout &BL, cudaStream_t st)
 {
-    const int per_sm = tune_value(CH_TUNE_BX_EXTREMES) ? tune_value(CH_TUNE_BX_EXTREMES) : 8;
     const int items = tune_value(CH_TUNE_BX_EXT_ITEMS) ? tune_value(CH_TUNE_BX_EXT_ITEMS) : 16;
+    // one wave: every block a share of the tiles
+    const int per_sm = tune_value(CH_TUNE_BX_EXTREMES) ? tune_value(CH_TUNE_BX_EXTREMES)
+                                                       : kBxExtThreads / (kFiltTile / items);
     int64_t blocks = std::min<int64_t>(BL.tiles_max, (int64_t)sm_count() * per_sm);
     const unsigned g = (unsigned)std::max<int64_t>(blocks, 1);
     probe_before(CH_K_EXTREMES, st);
