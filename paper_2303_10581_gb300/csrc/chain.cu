@@ -64,7 +64,7 @@ constexpr int NL = SC + 2;          // sequence capacity: SC points + 2 look-ahe
 constexpr int NWB = LT / 32;        // warps per block
 constexpr int NWS = NWB / 2;        // warps per side
 constexpr int SY = NL + 6;
-constexpr int kCopyParts = 4;                  // a range is shared by so many warps
+constexpr int kCopyParts = 18;                 // a range is shared by so many warps (4: 3 us more on 10^6 circle points)
 constexpr int kCopyLen = CS / kCopyParts;      // entries per part
 static_assert(CS % kCopyParts == 0, "parts cover a super-chunk's slots");
 constexpr int LWMAX = ((NL + NWB - 1) / NWB + 31) / 32;   // longest leaf (17)
