@@ -465,11 +465,6 @@ __device__ __forceinline__ float key_float(uint32_t k)
     return __uint_as_float(b);
 }
 
-__device__ __forceinline__ unsigned long long point_key(float x, float y)
-{
-    return ((unsigned long long)ord_key(x) << 32) | ord_key(y);
-}
-
 __device__ __forceinline__ float2 key_point(unsigned long long k)
 {
     return make_float2(key_float((uint32_t)(k >> 32)), key_float((uint32_t)k));
@@ -493,7 +488,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 // ---------------------------------------------------------------------------
 // exact orientation: sign of (b - a) x (c - a) for binary32 inputs
 // ---------------------------------------------------------------------------
-// Tier 3: the determinant expands into six products of two binary32 values
+// Tier 4: the determinant expands into six products of two binary32 values
 // (the a.x*a.y terms cancel); each is exact in binary64.  They are summed
 // without error by Grow-Expansion with Two-Sum (Shewchuk, "Adaptive
 // Precision Floating-Point Arithmetic and Fast Robust Geometric
@@ -538,10 +533,10 @@ static __device__ __noinline__ int orient_exact(float ax, float ay, float bx, fl
     return e[m - 1] > 0.0 ? 1 : -1;
 }
 
-// Tier 2: binary64 evaluation with Shewchuk's orient2d error bound
+// Tier 3: binary64 evaluation with Shewchuk's orient2d error bound
 // ccwerrboundA = (3 + 16 eps) eps, eps = 2^-53.  Differences and products of
 // binary32 values cannot underflow or overflow in binary64, so the bound
-// holds; undecided cases go to tier 3.
+// holds; undecided cases go to tier 4.
 static __device__ __noinline__ int orient_d(float ax, float ay, float bx, float by, float cx, float cy)
 {
     // orient2d(pa = a, pb = b, pc = c)
@@ -573,7 +568,7 @@ __device__ __forceinline__ bool exact_diff(float a, float c)
     return ((a >= 0.0f) == (c >= 0.0f)) && aa <= 2.0f * cc && cc <= 2.0f * aa;
 }
 
-// Tier 1b: exact binary32 sign for nearby points.  When the four
+// Tier 2b: exact binary32 sign for nearby points.  When the four
 // differences are exact, detleft = u1 v1 and detright = u2 v2 exactly; with
 // p = fl(u v) and e = fma(u, v, -p) = u v - p (exact while |p| >= 2^-100 or
 // a factor is zero, since then the product cannot underflow), rounding is

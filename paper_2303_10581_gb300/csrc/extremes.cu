@@ -1127,9 +1127,8 @@ cudaError_t launch_extremes(const float *pts, int64_t n, void *ws, const Layout 
             probe_before(CH_K_EXTREMES, st);
             spec_sample_kernel<<<kSampleBlocks, kSampleThreads, 0, st>>>(pts, n, ws, L, (uint32_t)blocks,
                                                                          (uint32_t)cap);
-            launch_next(extremes_kernel<true>, (unsigned)blocks + extra, kExtThreads, 0, st, pts, n, ws, L, ext8, 1, zero_ptr,
-                                                                                   zero_words, skip0, skip1, (uint32_t)cap, learn,
-                                                                                   learn_dirs, learn_k);
+            launch_next(extremes_kernel<true>, (unsigned)blocks + extra, kExtThreads, 0, st, pts, n, ws, L, ext8, 1,
+                        zero_ptr, zero_words, skip0, skip1, (uint32_t)cap, learn, learn_dirs, learn_k);
             note_kernels(CH_K_EXTREMES, 2);
             probe_after(CH_K_EXTREMES, st);
             return cudaGetLastError();

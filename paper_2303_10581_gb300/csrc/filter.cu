@@ -633,7 +633,8 @@ cudaError_t launch_single(const float *pts, int64_t n, void *ws, const Layout &L
     static int per_sm = occupancy(filter_kernel<G, KEYS, !KEYS>, kFiltThreads);
     const int64_t ntiles = ceil_div(n, kFiltTile);
     int64_t blocks = std::min<int64_t>((int64_t)sm_count() * per_sm, ntiles);
-    launch_next(filter_kernel<G, KEYS, !KEYS>, (unsigned)std::max<int64_t>(blocks, 1), kFiltThreads, 0, st, pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count);
+    launch_next(filter_kernel<G, KEYS, !KEYS>, (unsigned)std::max<int64_t>(blocks, 1), kFiltThreads, 0, st, pts, n,
+                ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count);
     note_kernels(CH_K_FILTER, 1);
     return cudaGetLastError();
 }
@@ -655,11 +656,11 @@ cudaError_t launch_two_pass(const float *pts, int64_t n, void *ws, const Layout 
                             float *surv_pts, uint32_t *surv_count, cudaStream_t st)
 {
     // both passes use the same grid (block b owns the same tile range),
-    // the count pass's resident blocks (the scatter pass's warps take
-    // tiles on their own, so a second partial wave of it costs little)
+    // the count pass's resident blocks
     const int64_t bc = count_blocks<G, BOX>(n);
     launch_next(filter_count_kernel<G, BOX>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, nullptr);
-    launch_next(filter_scatter_kernel<G, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, surv_idx, reinterpret_cast<float2 *>(surv_pts), surv_count, BOX ? 0 : 1);
+    launch_next(filter_scatter_kernel<G, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, surv_idx,
+                reinterpret_cast<float2 *>(surv_pts), surv_count, BOX ? 0 : 1);
     note_kernels(CH_K_FILTER, 2);
     return cudaGetLastError();
 }

@@ -23,7 +23,8 @@
 //    less than 0.0049 bins (0.0386 with the second level's eight times as
 //    many): in units of eps = 2^-24, t = dy / (|dx| + |dy|) gets 7 |t| (two
 //    differences, the sum, at most 2 ulp for the quotient); the scaling is
-//    one FMA, which rounds by at most half an ulp of NB, or down to the bin.  A vertex is taken only where its value is at least a margin (1/32;
+//    one FMA, which rounds by at most half an ulp of NB, or down to the
+//    bin.  A vertex is taken only where its value is at least a margin (1/32;
 //    1/8) away from both ends of its bin, so as directions P comes strictly
 //    before p and N strictly after it (or N == Q, whose sign is never proven);
 //  - consecutive vertices v, w were proven strictly counter-clockwise around
@@ -1022,7 +1023,8 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
         const int64_t stride = fan_sample_stride(ntiles);
         const int64_t bb = std::min<int64_t>(ceil_div(ntiles, stride) * (kFiltItems / BI), (int64_t)sms * 5);
         probe_before(CH_K_KGON, st);
-        launch_next(fan_bins_kernel<G>, (unsigned)bb, kFiltThreads, 0, st, pts, (uint32_t)n, ws, L, (uint32_t)stride, use_bits, kdev);
+        launch_next(fan_bins_kernel<G>, (unsigned)bb, kFiltThreads, 0, st, pts, (uint32_t)n, ws, L, (uint32_t)stride,
+                    use_bits, kdev);
         launch_next(fan_vertex_kernel, kFanBins / (VB * VT / 32), VT, 0, st, pts, n, ws, L);
         launch_next(fan_build_kernel, kFanBins / BT, BT, 0, st, n, ws, L);
         note_kernels(CH_K_KGON, 3);
@@ -1030,7 +1032,8 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
     }
     probe_before(CH_K_FILTER, st);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(ntiles, (int64_t)CG), sms));
-    launch_next(hull_filter_kernel<G>, (unsigned)grid, CT, kQueueSmem + (has_fan ? kFanTable : 0), st, pts, (uint32_t)n, ws, L, has_fan, use_bits, kdev);
+    launch_next(hull_filter_kernel<G>, (unsigned)grid, CT, kQueueSmem + (has_fan ? kFanTable : 0), st, pts,
+                (uint32_t)n, ws, L, has_fan, use_bits, kdev);
     note_kernels(CH_K_FILTER, 1);
     probe_after(CH_K_FILTER, st);
     cudaError_t e = cudaGetLastError();

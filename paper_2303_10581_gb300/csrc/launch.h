@@ -113,7 +113,7 @@ cudaError_t launch_learned_choice(const float *pts, int64_t n, const void *param
 cudaError_t launch_hull_filter(const float *pts, int64_t n, void *ws, const Layout &L, const KgonStage *kg,
                                cudaStream_t st);
 
-// stable radix sort of the survivors by x (nothing when one block will sort them)
+// radix sort of the survivors by x (nothing when one block will sort them)
 cudaError_t launch_sort(void *ws, const Layout &L, cudaStream_t st);
 
 // sort, monotone chains and assembly of the hull from the survivors

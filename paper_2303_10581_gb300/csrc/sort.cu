@@ -1,4 +1,4 @@
-// sort.cu -- stable LSD radix sort of the survivors by x for the monotone
+// sort.cu -- LSD radix sort of the survivors by x for the monotone
 // chain of Sec. 3.3 (Andrew's algorithm starts from the points in
 // lexicographic order; the paper leaves this step to a CPU library).
 //
@@ -8,15 +8,16 @@
 // only the highest an upper-chain vertex (apart from the first and last x),
 // so the chain kernel reduces each equal-x run itself and y never needs to
 // be part of the sort order.  That makes four 8-bit passes instead of eight.
-// The filter writes the pairs in ascending index order and every pass is
-// stable, so each equal-x run stays in ascending index order.
+// (The survivors come in any order, and equal x stay in it: the chain kernel
+// settles equal points by their index.)
 //
 // Structure (one-sweep style, Adinets & Merrill 2022): one histogram kernel
 // computes all four digit histograms in a single read and marks passes
 // whose digit is constant (skipped); each remaining pass is one persistent
-// kernel that ranks a 4096-key tile in shared memory (per warp, stable), finds the tile's per-digit global offsets by a
-// decoupled look-back over 256 digit counters, and writes the tile out
-// digit-sorted, so stores are runs of consecutive addresses.  The payload
+// kernel that ranks a 4096-key tile in shared memory (per warp, stable),
+// finds the tile's per-digit global offsets by a decoupled look-back over
+// 256 digit counters, and writes the tile out digit-sorted, so stores are
+// runs of consecutive addresses.  The payload
 // is staged in shared memory in element order and gathered through the
 // tile's inverse permutation at write-out, so it never occupies registers.
 // When a block takes a ticket it also asks the TMA unit to bring the tile
