@@ -1220,7 +1220,7 @@ __global__ void __launch_bounds__(kEmitThreads) emit_kernel(void *ws, Layout L)
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
-    if (s == 0) return;
+    if (s <= (uint32_t)(kEmitThreads * SC)) return;   // hull_copy_kernel adds so few ranges up itself
     const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
     EmitArgs E{{at<uint32_t>(ws, L.emit_off[0]), at<uint32_t>(ws, L.emit_off[1])},
                &ctrl->emit_ticket[0],
@@ -1230,25 +1230,67 @@ __global__ void __launch_bounds__(kEmitThreads) emit_kernel(void *ws, Layout L)
 
 // The hull and its vertex count: the chains' surviving ranges (original
 // indices, the low half of the payload) straight to their positions, a warp
-// per part of a super-chunk's range.
+// per part of a super-chunk's range.  Up to kEmitThreads super-chunks each
+// block adds their lengths up itself, which costs it less than a launch in
+// between.
 __global__ void __launch_bounds__(kEmitThreads) hull_copy_kernel(void *ws, Layout L, uint32_t *hull_idx,
                                                                  uint32_t *hull_count)
 {
     kernel_entry();
+    __shared__ uint32_t s_off[2][kEmitThreads], s_w[2][kEmitThreads / 32];
     const Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     if (ctrl->small_done) return;
-    const uint32_t hl = ctrl->h_lower, hu = ctrl->h_upper;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *hull_count = hl == 0 ? 0u : hl + (hu >= 2 ? hu - 2 : 0u);
     const uint32_t s = hull_stage_count(ctrl, at<Octagon>(ws, L.oct));
-    if (s == 0) return;
+    if (s == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *hull_count = 0u;
+        return;
+    }
     const ChainPtrs P = chain_ptrs(ws, L, ctrl->final_buf);
-    const int64_t items = ceil_div((int64_t)s, SC) * 2 * kCopyParts;
-    const int64_t warps = (int64_t)gridDim.x * (kEmitThreads / 32);
+    const int64_t nsc = ceil_div((int64_t)s, SC);
+    const bool few = nsc <= kEmitThreads;
+    uint32_t hl = ctrl->h_lower, hu = ctrl->h_upper;
+    if (few) {
+        const int c = (int)threadIdx.x, lane = c & 31;
+        uint32_t n[2] = {0u, 0u}, incl[2];
+        if (c < nsc) {
+#pragma unroll
+            for (int side = 0; side < 2; ++side)
+                n[side] = (uint32_t)max(0, __ldcg(P.hi(side) + c) - __ldcg(P.lo(side) + c) + 1);
+        }
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            incl[side] = n[side];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, incl[side], o);
+                if (lane >= o) incl[side] += u;
+            }
+            if (lane == 31) s_w[side][c >> 5] = incl[side];
+        }
+        __syncthreads();
+        uint32_t total[2];
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            uint32_t before = 0;
+            total[side] = 0u;
+#pragma unroll
+            for (int w = 0; w < kEmitThreads / 32; ++w) {
+                if (w < c >> 5) before += s_w[side][w];
+                total[side] += s_w[side][w];
+            }
+            s_off[side][c] = before + incl[side] - n[side];
+        }
+        hl = total[0];
+        hu = total[1];
+        __syncthreads();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *hull_count = hl == 0 ? 0u : hl + (hu >= 2 ? hu - 2 : 0u);
+    const int64_t items = nsc * 2 * kCopyParts, warps = (int64_t)gridDim.x * (kEmitThreads / 32);
     for (int64_t it = ((int64_t)blockIdx.x * kEmitThreads + threadIdx.x) >> 5; it < items; it += warps) {
         const int64_t c = it / (2 * kCopyParts);
         const int side = (int)(it / kCopyParts) & 1;
-        copy_chain_part(P, side, c, (int)(it % kCopyParts), __ldg(at<uint32_t>(ws, L.emit_off[side]) + c), hl, hu,
-                        hull_idx, L.n);
+        const uint32_t off = few ? s_off[side][c] : __ldg(at<uint32_t>(ws, side ? L.emit_off[1] : L.emit_off[0]) + c);
+        copy_chain_part(P, side, c, (int)(it % kCopyParts), off, hl, hu, hull_idx, L.n);
     }
 }
 
@@ -1438,15 +1480,15 @@ static cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, u
     probe_after(CH_K_CHAIN, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    int64_t eb = L.emit_tiles;
-    if (eb > (int64_t)sms * 4) eb = (int64_t)sms * 4;
-    if (eb < 1) eb = 1;
-    probe_before(CH_K_EMIT, st);
-    launch_next(emit_kernel, (unsigned)eb, kEmitThreads, 0, st, ws, L);
-    note_kernels(CH_K_EMIT, 1);
-    probe_after(CH_K_EMIT, st);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (L.n_chunks > kEmitThreads) {
+        const int64_t eb = std::min<int64_t>(L.emit_tiles, (int64_t)sms * 4);
+        probe_before(CH_K_EMIT, st);
+        launch_next(emit_kernel, (unsigned)eb, kEmitThreads, 0, st, ws, L);
+        note_kernels(CH_K_EMIT, 1);
+        probe_after(CH_K_EMIT, st);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     const int64_t fb = std::min<int64_t>(ceil_div(L.n_chunks * 2 * kCopyParts, kEmitThreads / 32), (int64_t)sms * 4);
     probe_before(CH_K_FINISH, st);
     launch_next(hull_copy_kernel, (unsigned)fb, kEmitThreads, 0, st, ws, L, hull_idx, hull_count);

@@ -1037,10 +1037,15 @@ cudaError_t launch_hull_filter_g(const float *pts, int64_t n, void *ws, const La
     note_kernels(CH_K_FILTER, 1);
     probe_after(CH_K_FILTER, st);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || L.fan2_bins == 0) return e;   // (a set too small for the second level)
-    probe_before(CH_K_KGON, st);
+    // a set too small for the second level, or of fewer than four times as
+    // many points as it asks for: a first level that leaves a quarter of them
+    // is looking at vertices, and three idle launches are 6 % of a call on 2^20
+    // points
     const int lg = tune_value(CH_TUNE_FAN2_MIN_LOG2);
-    launch_next(fan2_max_kernel, sms * 8, F2T, 0, st, ws, L, lg ? (uint32_t)(1ull << lg) : kFan2MinS);
+    const uint32_t min_s = lg ? (uint32_t)(1ull << lg) : kFan2MinS;
+    if (e != cudaSuccess || L.fan2_bins == 0 || n < 4 * (int64_t)min_s) return e;
+    probe_before(CH_K_KGON, st);
+    launch_next(fan2_max_kernel, sms * 8, F2T, 0, st, ws, L, min_s);
     launch_next(fan2_build_kernel, kFan2Bins / BT, BT, 0, st, ws, L);
     const int64_t tb = std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, (int64_t)F2T * F2I), (int64_t)sms * 8));
     launch_next(fan2_test_kernel, (unsigned)tb, F2T, 0, st, ws, L);
