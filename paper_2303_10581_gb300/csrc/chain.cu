@@ -57,17 +57,19 @@ namespace ch {
 
 namespace {
 
-constexpr int LT = kChainThreads;   // leaves per super-chunk
+// Threads per block, and leaves per super-chunk: one set has few super-chunks,
+// and 512 threads finish one sooner (10^6 circle points: 163 us the hull with
+// 256, 154 so); many sets fill the chip, and 256 wait less for one another (4096
+// sets: 1.8 % less than with 512).
+constexpr int kOneThreads = 512;
+constexpr int kBxThreads = kChainThreads;
 constexpr int SC = kChainC;         // points per super-chunk
 constexpr int CS = kChainStride;    // chain slots per super-chunk
 constexpr int NL = SC + 2;          // sequence capacity: SC points + 2 look-ahead slots
-constexpr int NWB = LT / 32;        // warps per block
-constexpr int NWS = NWB / 2;        // warps per side
 constexpr int SY = NL + 6;
 constexpr int kCopyParts = 18;                 // a range is shared by so many warps (4: 3 us more on 10^6 circle points)
 constexpr int kCopyLen = CS / kCopyParts;      // entries per part
 static_assert(CS % kCopyParts == 0, "parts cover a super-chunk's slots");
-constexpr int LWMAX = ((NL + NWB - 1) / NWB + 31) / 32;   // longest leaf (17)
 
 // pop / advance test: lower chains drop a vertex when the turn is not
 // strictly counter-clockwise, upper chains when it is not strictly clockwise
@@ -193,13 +195,17 @@ __device__ void merge_walk(Acc &A, int side, int fa, int la, int fb, int lb)
 // ---------------------------------------------------------------------------
 // in-block state; one side (lower or upper) is processed at a time
 // ---------------------------------------------------------------------------
+template <int LT>
 __device__ __forceinline__ void side_barrier(int side)   // of the warps that work on one side
 {
     __syncwarp();   // (whole warps arrive)
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + side), "n"(NWS * 32) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + side), "n"(LT / 2) : "memory");
 }
 
+template <int LT>
 struct ChainSmem {
+    static constexpr int NWB = LT / 32;                              // warps per block
+    static constexpr int LWMAX = ((NL + NWB - 1) / NWB + 31) / 32;   // longest leaf
     float2 pts[NL];               // staged points; [SC], [SC+1]: look-ahead lowest / highest
     union {
         struct {
@@ -229,8 +235,9 @@ struct ChainSmem {
 };
 
 // leaf c's entries start at flat[lb[c]]; its stack holds offsets from there
+template <int LT>
 struct SmemAcc {
-    ChainSmem &s;
+    ChainSmem<LT> &s;
     const uint16_t *flat;
     __device__ int lo(int, int c) const { return s.lo[c]; }
     __device__ int hi(int, int c) const { return s.hi[c]; }
@@ -253,7 +260,8 @@ struct SmemAcc {
 
 // Exclusive scan of one count per thread over the block; the total goes to
 // s.total.  Contains two barriers.
-__device__ __forceinline__ uint32_t block_scan(ChainSmem &s, uint32_t v)
+template <int LT>
+__device__ __forceinline__ uint32_t block_scan(ChainSmem<LT> &s, uint32_t v)
 {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     uint32_t incl = v;
@@ -462,7 +470,8 @@ __device__ void climb(const ChainPtrs &P, int side, int64_t c, int64_t nsc, int6
 
 // Block reduction of (y, index << 32 | position) pairs: the lowest (highest)
 // y, ties to the lowest index.  Contains two barriers.
-__device__ __forceinline__ void block_extreme_y(ChainSmem &s, float ylo, unsigned long long qlo, float yhi,
+template <int LT>
+__device__ __forceinline__ void block_extreme_y(ChainSmem<LT> &s, float ylo, unsigned long long qlo, float yhi,
                                                 unsigned long long qhi, float &out_ylo, unsigned long long &out_qlo,
                                                 float &out_yhi, unsigned long long &out_qhi)
 {
@@ -514,7 +523,8 @@ __device__ __forceinline__ void block_extreme_y(ChainSmem &s, float ylo, unsigne
 // between digits: the histogram and four passes over global memory take 57 us
 // on 4200 survivors, this 27 on 4096.  (Every key by a binary search in the
 // other run instead of the serial merge: 40.)
-__device__ void local_sort(ChainSmem &sm, const ChainPtrs &P, int64_t base, int m)
+template <int LT>
+__device__ void local_sort(ChainSmem<LT> &sm, const ChainPtrs &P, int64_t base, int m)
 {
     const int t = threadIdx.x, lane = t & 31;
     const int C = ((m + LT - 1) / LT) | 1;   // outputs per thread and round; odd: no bank conflicts in the stores
@@ -591,9 +601,11 @@ __device__ void local_sort(ChainSmem &sm, const ChainPtrs &P, int64_t base, int 
 // The chains of one super-chunk: sorted positions [base, base + m) of a set
 // occupying [sbeg, send); results go to chain slot j.  local: the super-chunk
 // is a whole set and not sorted yet.  Called by all threads of the block.
-__device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, int64_t j, int64_t base, int m,
+template <int LT>
+__device__ __forceinline__ void superchunk(ChainSmem<LT> &sm, const ChainPtrs &P, int64_t j, int64_t base, int m,
                                            int64_t sbeg, int64_t send, bool local)
 {
+    constexpr int NWB = LT / 32, NWS = NWB / 2;   // warps per block, per side
     const auto place = [&](int e) { return base + (local ? (int)sm.perm[e] : e); };   // of a staged point
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
@@ -871,7 +883,7 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
                 bool closed = kept <= 2;
                 if (whole) {
                     if (lane == 0) sm.wsum[warp] = (uint32_t)kept;
-                    side_barrier(side);
+                    side_barrier<LT>(side);
                     int total = 0;
 #pragma unroll
                     for (int w = 0; w < NWS; ++w) total += (int)sm.wsum[side * NWS + w];
@@ -889,9 +901,9 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
                 if (!in_y) {
                     for (int i = lane; i < wl; i += 32) Y[w0 + i] = X[w0 + i];
                 }
-                side_barrier(side);   // wsum has been read
+                side_barrier<LT>(side);   // wsum has been read
                 if (lane == 0) sm.wsum[warp] = (uint32_t)wl;
-                side_barrier(side);
+                side_barrier<LT>(side);
                 int at = 0;
                 len = 0;
 #pragma unroll
@@ -901,7 +913,7 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
                     len += u;
                 }
                 for (int i = lane; i < wl; i += 32) X[at + i] = Y[w0 + i];
-                side_barrier(side);
+                side_barrier<LT>(side);
                 strict = len <= 2;
                 if (++round == kElimRounds) break;
                 whole = true;
@@ -957,7 +969,7 @@ __device__ __forceinline__ void superchunk(ChainSmem &sm, const ChainPtrs &P, in
             sm.first[t] = sm.last[t] = (int16_t)(h > 0 ? t : -1);
             __syncwarp();
             // ---- merge tree: five levels inside the warp, then three across warps
-            const SmemAcc A{sm, flat};
+            const SmemAcc<LT> A{sm, flat};
             for (int w = 1; w < 32; w *= 2) {
                 if (lane < 32 / (2 * w)) {
                     const int a0 = warp * 32 + 2 * lane * w, b0 = a0 + w;
@@ -1008,11 +1020,11 @@ __device__ __forceinline__ void copy_chain_part(const ChainPtrs &P, int side, in
 
 // At most SC survivors (the sort has left them alone): one block sorts them
 // and writes the hull itself, and the later kernels have nothing to do.
-__global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t *hull_idx, uint32_t *hull_count)
+__global__ void __launch_bounds__(kOneThreads) chain_kernel(void *ws, Layout L, uint32_t *hull_idx, uint32_t *hull_count)
 {
     kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ChainSmem &sm = *reinterpret_cast<ChainSmem *>(smem_raw);
+    ChainSmem<kOneThreads> &sm = *reinterpret_cast<ChainSmem<kOneThreads> *>(smem_raw);
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     const Octagon *oct = at<Octagon>(ws, L.oct);
     const uint32_t s = hull_stage_count(ctrl, oct);
@@ -1032,7 +1044,7 @@ __global__ void __launch_bounds__(LT) chain_kernel(void *ws, Layout L, uint32_t 
     }
     if (!local || blockIdx.x != 0) return;
     const uint32_t hl = (uint32_t)__ldcg(P.hi(0)) + 1u, hu = (uint32_t)__ldcg(P.hi(1)) + 1u;   // (behind a barrier)
-    for (int it = (int)(threadIdx.x >> 5); it < 2 * kCopyParts; it += NWB)
+    for (int it = (int)(threadIdx.x >> 5); it < 2 * kCopyParts; it += kOneThreads / 32)
         copy_chain_part(P, it & 1, 0, it >> 1, 0u, hl, hu, hull_idx, L.n);
     if (threadIdx.x == 0) {
         *hull_count = hl + (hu >= 2 ? hu - 2 : 0u);
@@ -1058,11 +1070,11 @@ __global__ void __launch_bounds__(kMergeThreads) chain_merge_kernel(void *ws, La
 
 // ---- many sets: super-chunks never span two sets; each set has its own
 // merge tree; the sorted arrays end up in buffer 0 (four passes)
-__global__ void __launch_bounds__(LT) bx_chain_kernel(void *ws, Layout L, BatchLayout BL)
+__global__ void __launch_bounds__(kBxThreads) bx_chain_kernel(void *ws, Layout L, BatchLayout BL)
 {
     kernel_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ChainSmem &sm = *reinterpret_cast<ChainSmem *>(smem_raw);
+    ChainSmem<kBxThreads> &sm = *reinterpret_cast<ChainSmem<kBxThreads> *>(smem_raw);
     const BatchCtrl *bc = at<BatchCtrl>(ws, BL.bctrl);
     if (bc->abort) return;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
@@ -1461,15 +1473,15 @@ static cudaError_t launch_chain(void *ws, const Layout &L, uint32_t *hull_idx, u
     const int sms = sm_count();
     int64_t cb = L.n_chunks;
     static const int per_sm = [] {   // thread-safe one-time initialisation
-        cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChainSmem));
+        cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChainSmem<kOneThreads>));
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, chain_kernel, LT, sizeof(ChainSmem));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, chain_kernel, kOneThreads, sizeof(ChainSmem<kOneThreads>));
         return v > 0 ? v : 1;
     }();
     if (cb > (int64_t)sms * per_sm) cb = (int64_t)sms * per_sm;
     if (cb < 1) cb = 1;
     probe_before(CH_K_CHAIN, st);
-    launch_next(chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L, hull_idx, hull_count);
+    launch_next(chain_kernel, (unsigned)cb, kOneThreads, sizeof(ChainSmem<kOneThreads>), st, ws, L, hull_idx, hull_count);
     if (L.n <= SC) {   // one super-chunk at most: that kernel wrote the hull
         note_kernels(CH_K_CHAIN, 1);
         probe_after(CH_K_CHAIN, st);
@@ -1511,16 +1523,16 @@ cudaError_t launch_bx_chain(void *ws, const Layout &L, const BatchLayout &BL, cu
 {
     const int sms = sm_count();
     static const int per_sm = [] {   // thread-safe one-time initialisation
-        cudaFuncSetAttribute(bx_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChainSmem));
+        cudaFuncSetAttribute(bx_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChainSmem<kBxThreads>));
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, bx_chain_kernel, LT, sizeof(ChainSmem));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, bx_chain_kernel, kBxThreads, sizeof(ChainSmem<kBxThreads>));
         return v > 0 ? v : 1;
     }();
     int64_t cb = BL.tiles_max;
     if (cb > (int64_t)sms * per_sm) cb = (int64_t)sms * per_sm;
     if (cb < 1) cb = 1;
     probe_before(CH_K_CHAIN, st);
-    launch_next(bx_chain_kernel, (unsigned)cb, LT, sizeof(ChainSmem), st, ws, L, BL);
+    launch_next(bx_chain_kernel, (unsigned)cb, kBxThreads, sizeof(ChainSmem<kBxThreads>), st, ws, L, BL);
     launch_next(bx_merge_kernel, merge_grid(BL.tiles_max), kMergeThreads, 0, st, ws, L, BL);
     note_kernels(CH_K_CHAIN, 2);
     probe_after(CH_K_CHAIN, st);
