@@ -168,7 +168,8 @@ class ClockSampler:
 
 # --------------------------------------------------------------------------- roofline bookkeeping
 
-SMALL_HULL = 512   # at most this many points to sort: one block sorts and chains them (no sort passes)
+SMALL_HULL = 512    # at most this many points to sort: one block sorts and chains them (no chain kernels)
+SMALL_SORT = 4096   # at most this many: the chain kernel's block sorts them (no sort passes)
 
 
 def algorithmic_bytes(kernel, n, s_list, t_list, f_list=None, spec_list=None):
@@ -180,7 +181,7 @@ def algorithmic_bytes(kernel, n, s_list, t_list, f_list=None, spec_list=None):
     level), spec_list 1 for the sets the speculative sweep served (their
     points were read by the extremes sweep: the filter only writes its
     survivors; the candidates it re-reads are not counted).  Sets with at
-    most SMALL_HULL points to sort run no sort and chain kernels."""
+    most SMALL_SORT (SMALL_HULL) points to sort run no sort (chain) kernels."""
     f_list = t_list if f_list is None else f_list
     spec_list = [0] * len(s_list) if spec_list is None else spec_list
     if kernel == "extremes":
@@ -189,13 +190,14 @@ def algorithmic_bytes(kernel, n, s_list, t_list, f_list=None, spec_list=None):
         # read points (unless the sweep served), write key + payload per point kept
         return sum((0 if sp else 8 * n) + 12 * f for f, sp in zip(f_list, spec_list))
     if kernel == "kgon":
-        # the fan test of the octagon survivors when it ran (read their
-        # coordinates); otherwise only samples.  The second level reads the
+        # the fan over the octagon survivors when it ran (their coordinates;
+        # hulls test them in the filter's pass, and this group then only
+        # makes the vertices: an upper bound); otherwise only samples.  The second level reads the
         # first level's survivors twice (sub-bin maxima, test: key +
         # payload) and copies the points it keeps
         return sum((8 * s if f < s else 0) + (24 * f + 24 * t if t < f else 0)
                    for s, t, f in zip(s_list, t_list, f_list))
-    big = [t for t in t_list if t > SMALL_HULL]
+    big = [t for t in t_list if t > SMALL_SORT]
     if kernel == "sort_hist":
         return sum(4 * t for t in big)                      # read the 32-bit keys
     if kernel == "sort_pass":
@@ -203,7 +205,7 @@ def algorithmic_bytes(kernel, n, s_list, t_list, f_list=None, spec_list=None):
         # + payload (8 B): 24 B per point
         return sum(4 * 24 * t for t in big)
     if kernel == "chain":
-        return sum(12 * t for t in big)                     # read the sorted keys and payloads once
+        return sum(12 * t for t in t_list if t > SMALL_HULL)   # read the sorted keys and payloads once
     return None
 
 

@@ -126,7 +126,7 @@ ch_status ch_extremes_filter(const float *pts, int64_t n, uint32_t *ext8, uint32
  * throws survivors away again (not in the paper; the hull is the same): a
  * fan of triangles around the bounding-box centre whose vertices are the
  * farthest sampled survivors of angular bins, and, when that leaves at least
- * 2^19 points (CH_TUNE_FAN2_MIN_LOG2), a second fan over those with eight
+ * 2^19 points (CH_TUNE_FAN2_MIN_LOG2) of at least four times as many, a second fan over those with eight
  * times as many bins; a survivor strictly inside a triangle (exact signs) is
  * no hull vertex. */
 ch_status ch_hull(const float *pts, int64_t n, uint32_t *hull_idx, uint32_t *hull_count,
@@ -227,7 +227,8 @@ typedef enum {
                                    4, 8 or 16, i.e. blocks of 1024, 512 or 256 threads (default 16) */
     CH_TUNE_FAN2_MIN_LOG2 = 7,  /* single-set hull step: the fan's second level runs when the first
                                    leaves at least 2^value points, 10..31 (default 19); sets of
-                                   fewer than 2^19 points have no second level */
+                                   fewer than 2^19 points, or fewer than four times
+                                   that many, have no second level */
     CH_TUNE_COUNT = 8
 } ch_tune_knob;
 ch_status ch_tune_set(int32_t knob, int32_t value);
@@ -323,8 +324,10 @@ typedef enum {
  * two-pass schedule (count, scatter), one with the single pass and in
  * ch_hull (octagon and fan test in one pass); two for CHAIN (chains, tree
  * merge); for KGON three (the fan's bins, vertices, proofs; before FILTER)
- * and three for its second level (sub-bin maxima, vertices, test).  Kernel-launch
- * counting for all ids restarts at zero.  Host-only bookkeeping; creates
+ * and three for its second level (sub-bin maxima, vertices, test).  ch_hull
+ * launches a group only for sets that can need it: CHAIN's second part from
+ * 513 points, the sort, the tree merge and FINISH from 4097, KGON from 2^16,
+ * EMIT from more than 2^20.  Kernel-launch counting for all ids restarts at zero.  Host-only bookkeeping; creates
  * the events.  Process-wide: one probe at a time, driven from one host
  * thread (see "Host threads" above). */
 ch_status ch_probe_start(uint32_t kernel_mask, int32_t max_launches);
