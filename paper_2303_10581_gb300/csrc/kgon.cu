@@ -1383,11 +1383,10 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
             }
             if (lane == 31) s_w[warp] = src;
             __syncthreads();
-            int all = -1;
-            for (uint32_t w = 0; w < BT / 32; ++w) {
-                if (w < warp) src = max(src, s_w[w]);
-                all = max(all, s_w[w]);
-            }
+            static_assert(BT / 32 == 32, "a lane per warp");
+            const int ends = s_w[lane];
+            const int all = __reduce_max_sync(0xffffffffu, ends);
+            src = max(src, __reduce_max_sync(0xffffffffu, lane < warp ? ends : -1));
             __syncthreads();   // s_w is written again by the next chunk
             if (src < 0) src = carry;
             if (all >= 0) carry = all;
