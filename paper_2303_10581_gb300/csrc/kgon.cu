@@ -270,14 +270,11 @@ static_assert(kFanBins % BT == 0, "bins split evenly over the blocks");
 
 __device__ __forceinline__ int block_max(int v, int *s_w)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    v = __reduce_max_sync(0xffffffffu, v);
     __syncthreads();   // s_w may still be read from an earlier call
     if (lane_id() == 0) s_w[threadIdx.x >> 5] = v;
     __syncthreads();
-    int m = -1;
-    for (int w = 0; w < BT / 32; ++w) m = max(m, s_w[w]);
-    return m;
+    return __reduce_max_sync(0xffffffffu, s_w[lane_id()]);   // (32 warps)
 }
 
 // The last bin with a vertex of its own at or before bin blockIdx.x * BT +
@@ -296,7 +293,7 @@ __device__ __forceinline__ int vertex_source(Has has, int *s_w, int *s_scan)
     }
     if (lane == 31) s_scan[warp] = incl;
     __syncthreads();
-    for (int w = 0; w < (int)warp; ++w) incl = max(incl, s_scan[w]);
+    incl = max(incl, __reduce_max_sync(0xffffffffu, lane < warp ? s_scan[lane] : -1));   // (32 warps)
     if (!__syncthreads_or(incl < 0)) return incl;
     int prev = -1;
     for (uint32_t k = 1; k <= gridDim.x && prev < 0; ++k) {   // prev is block-uniform
