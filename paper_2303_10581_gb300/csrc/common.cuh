@@ -81,11 +81,15 @@ struct Octagon {
     float tx[8], ty[8], tz[8];   // edge k's affine form (octtest.cuh)
 };
 
-// extremes reduction state: left zeroed by the last block of every sweep
+// extremes reduction state: left zeroed by the last block of every sweep.
+// (No call zeroes it, so it lies at the same place in the workspace for every
+// n: calls on other sizes must find it as it was left.)
 struct ExtCtrl {
     unsigned long long ext_slot[8];   // packed (key, index) per extreme
     uint32_t ext_done;                // extremes blocks finished
     uint32_t nonfinite;               // a non-finite coordinate was seen
+    uint32_t sample_kmax[8];          // ord_key of the speculative sample's largest slot keys
+    uint32_t sample_done;             // its blocks finished
 };
 
 // second throw-away step of the hull step (kgon.cu): a fan of triangles
@@ -187,9 +191,7 @@ constexpr int kSpecWarps = kExtThreads / 32;   // slices per segment
 constexpr int kSpecCapDiv = 32;           // all slices together hold n / 32 candidates
 constexpr int kSpecKeptSmem = 2048;       // survivors per segment ranked in shared memory
 constexpr int64_t kSpecMinN = 1 << 22;    // smaller sets: the plain two passes
-struct SpecCtrl {
-    uint32_t kmax[8];                     // ord_key of the sample's largest slot keys (self-resetting)
-    uint32_t sample_done;                 // sample blocks finished
+struct SpecCtrl {                         // written anew by every call that speculates
     uint32_t fail;                        // a slice overflowed: fall back (zeroed by the sample kernel)
     uint32_t nseg;                        // segments (sweep blocks) of this call
     uint32_t cap;                         // candidate slots per slice

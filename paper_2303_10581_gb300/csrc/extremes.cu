@@ -750,6 +750,7 @@ __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float
                                                                      Layout L, uint32_t nseg, uint32_t cap)
 {
     kernel_entry();
+    ExtCtrl *ctrl = at<ExtCtrl>(ws, L.extctrl);
     SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const float2 *p2 = reinterpret_cast<const float2 *>(pts);
     const int64_t start = (n - kSampleRun) * (int64_t)blockIdx.x / (gridDim.x - 1);
@@ -782,20 +783,20 @@ __global__ void __launch_bounds__(kSampleThreads) spec_sample_kernel(const float
     if (lane < 8) {
         float m = s_km[0][lane];
         for (int w = 1; w < kSampleThreads / 32; ++w) m = fmaxf(m, s_km[w][lane]);
-        atomicMax(&sc->kmax[lane], ord_key(m));
+        atomicMax(&ctrl->sample_kmax[lane], ord_key(m));
     }
     __threadfence();
     __syncwarp();
-    if (lane == 0) s_last = atomicAdd(&sc->sample_done, 1u) == gridDim.x - 1;
+    if (lane == 0) s_last = atomicAdd(&ctrl->sample_done, 1u) == gridDim.x - 1;
     __syncwarp();
     if (!s_last) return;
     __threadfence();
     __shared__ SpecBox s_box;
     float kmax = 0.0f;
-    if (lane < 8) kmax = key_float(atomicExch(&sc->kmax[lane], 0u));
+    if (lane < 8) kmax = key_float(atomicExch(&ctrl->sample_kmax[lane], 0u));
     kmax = __shfl_sync(0xffffffffu, kmax, (int)(lane & 7u));
     if (lane == 0) {
-        sc->sample_done = 0u;
+        ctrl->sample_done = 0u;
         sc->fail = 0u;
         sc->nseg = nseg;
         sc->cap = cap;
