@@ -103,12 +103,12 @@ struct KgonCtrl {                          // zeroed with the control block
     unsigned long long slot[kFanBins];     // packed (far_key << 32 | ~index): farthest sampled input point per bin
     uint32_t sample, inside;               // points sampled for the bins, octagon survivors among them
     uint32_t s_oct;                        // octagon survivors
-    uint32_t bad;                          // bit 0: samples in one place only; bit 1: consecutive vertices not
-                                           // proven counter-clockwise around c
+    uint32_t bad;                          // samples in one place only
     uint32_t rho_inv;                      // ~bits of a lower bound (binary32) on the squared distance from
                                            // c to the fan's boundary, the largest so far
     uint32_t edges;                        // consecutive vertex pairs with v != w
-    uint32_t pad[2];
+    uint32_t gaps;                         // 1: some of them not proven counter-clockwise around c
+    uint32_t pad;
 };
 
 // second fan level (kgon.cu): over the first level's survivors, kFan2Sub
@@ -131,8 +131,8 @@ struct Fan2Ctrl {                          // zeroed with the control block
 struct Kgon {
     float cx, cy;                          // fan centre
     uint32_t ok;                           // 0: no fan this call
-    uint32_t pad;
-    float2 v[kFanBins];                    // vertex of every bin
+    uint32_t centre;                       // 1: c lies clearly inside the octagon
+    float2 v[kFanBins];                    // vertex of every bin (x = NaN: none, and the wedges beside it keep their points)
     float2 raw[kFanBins];                  // the same before empty bins are filled (x = NaN: none)
 };
 
@@ -308,7 +308,7 @@ struct FanInfo {
     uint32_t nb;          // bins
     uint32_t bad;         // no usable vertices
     uint32_t ready;       // the fan's proofs hold and it drops enough points
-    float rho2;           // lower bound on the squared distance from the centre to the fan's boundary
+    float rho2;           // lower bound on the squared distance from the centre to the fan's boundary (0: none)
     uint32_t pad[2];
 };
 

@@ -30,8 +30,16 @@
 //  - consecutive vertices v, w were proven strictly counter-clockwise around
 //    c (v != w), less than half a turn apart, so p is in the wedge of (Q, N)
 //    or of (P, Q), where strictly left of the edge is the triangle (c, Q, N)
-//    or (c, P, Q).  The triangles wind around c once, so c and the
-//    triangles' interiors are in the interior of a polygon of hull points;
+//    or (c, P, Q).  When all of them were, the triangles wind around c once,
+//    so c and the triangles' interiors are in the interior of a polygon of
+//    hull points.  Where a pair is not proven (a gap of half a turn, seen from
+//    c: a cloud with far outliers that no sample met), its first vertex is
+//    taken out (NaN, with which nothing is proven), so that only the points of
+//    that wedge are kept; then c itself must lie clearly inside the octagon,
+//    whose vertices are input points, for the other triangles to lie in the
+//    hull, and there is no disk.  (One gap switching the fan off: 10^8 points
+//    of a displaced circle and one at ten radii, 49 M of them sorted, 5146 us;
+//    131 thousand and 2140 us when each wedge stood alone.);
 //  - the quotient needs |dx| + |dy| within [2^-126, 2^126]: the set's box is
 //    checked for the upper end, and a point closer to c than 2^-126 is
 //    inside the disk around c that is proven inside the fan (the fan is off
@@ -141,11 +149,30 @@ __device__ __forceinline__ int vertex_bin(Bins nb, float dx, float dy, float mar
     return fabsf(mid) <= 0.5f - margin ? (int)(__float_as_uint(f) - kBinBias) : -1;
 }
 
+// c clearly inside the octagon: every edge's affine form at c (its constant)
+// is at least 2 where 1 proves it (octtest.cuh), so that the points next to c
+// are inside too.
+__device__ __forceinline__ bool centre_inside(const Octagon &o)
+{
+    bool in = true;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) in &= o.tz[k] >= 2.0f;
+    return in;
+}
+
+// Whether a fan's proofs hold: its consecutive vertex pairs v != w that are
+// proven (edges), whether some are not (gaps), a lower bound on its radius (no gaps) or c
+// inside the octagon.
+__device__ __forceinline__ bool fan_holds(uint32_t edges, bool gaps, float rho2, bool centre)
+{
+    return gaps ? edges >= 1u && centre : edges >= 3u && rho2 > 0x1p-120f;
+}
+
 // Whether this call has a fan whose proofs hold (after fan_build_kernel).
 __device__ __forceinline__ float fan_rho2(const KgonCtrl *kc) { return __uint_as_float(~kc->rho_inv); }
 __device__ __forceinline__ bool fan_ready(const KgonCtrl *kc, const Kgon *g)
 {
-    return g->ok && !kc->bad && kc->edges >= 3u && fan_rho2(kc) > 0x1p-120f;
+    return g->ok && fan_holds(kc->edges, kc->gaps != 0u, fan_rho2(kc), g->centre != 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -179,6 +206,23 @@ __device__ __forceinline__ void raise_bins(Bins nb, unsigned long long *slot, co
             if (key >= top[k]) atomicMax(slot + b[k], ((unsigned long long)key << 32) | (uint32_t)~index(k));
         }
     }
+}
+
+// The octagon's vertices raise the bins as well (a warp calls; index(k):
+// vertex k's): far points in tiles that are not sampled are among them.
+template <class Bins, class Index>
+__device__ __forceinline__ void raise_octagon(Bins nb, unsigned long long *slot, const Octagon &o, Index index)
+{
+    const int first = (int)(lane_id() & 1u) * BI;
+    static_assert(2 * BI == 8, "two lanes hold the eight vertices");
+    float qx[BI], qy[BI];
+#pragma unroll
+    for (int k = 0; k < BI; ++k) {
+        qx[k] = o.ax[first + k];
+        qy[k] = o.ay[first + k];
+    }
+    raise_bins(nb, slot, qx, qy, lane_id() < 2u ? (1u << BI) - 1u : 0u, make_float2(o.cx, o.cy), far_ref(o),
+               [&](int k) { return index(first + k); });
 }
 
 // Every stride-th tile, in quarters (1024 points, four a thread) over a
@@ -222,6 +266,10 @@ __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *
         }
     };
     if (blockIdx.x < steps) fetch(blockIdx.x);
+    if (blockIdx.x == gridDim.x - 1 && t < 32u) {
+        const uint32_t *ext8 = at<uint32_t>(ws, L.ext8);
+        raise_octagon(Level1{}, kc->slot, so, [&](int k) { return ext8[k]; });
+    }
     for (uint32_t w = blockIdx.x; w < steps; w += gridDim.x) {
         const uint32_t tile = w / parts * stride, part = w % parts;
         float qx[BI], qy[BI];
@@ -500,7 +548,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     Kgon *g = at<Kgon>(ws, L.kgon);
     const uint32_t tid = threadIdx.x;
-    const bool live = fan_live(kc, oct, n) && !(kc->bad & 1u);   // (bit 1 is set below)
+    const bool live = fan_live(kc, oct, n) && !kc->bad;
     const int b = (int)(blockIdx.x * BT + tid);
     int src = -1;
     if (live) src = vertex_source([&](int j) { return g->raw[j].x == g->raw[j].x; }, s_w, s_scan);   // block-uniform
@@ -509,30 +557,33 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
         return;
     }
     const float cx = oct->cx, cy = oct->cy;
-    const float2 v = g->raw[src], next = g->raw[b + 1 == kFanBins ? 0 : b + 1];
-    g->v[b] = v;
+    float2 v = g->raw[src];
+    const float2 next = g->raw[b + 1 == kFanBins ? 0 : b + 1];
     // the next bin's vertex: its own point, or this one's again
     const float2 w = next.x == next.x ? next : v;
     float r = __int_as_float(0x7f800000);
     const bool edge = v.x != w.x || v.y != w.y;
-    bool bad = false;
+    bool gap = false;
     if (edge) {
         r = disk_bound(cx, cy, v, w);
-        bad = r < 0.0f;
+        gap = r < 0.0f;
+        if (gap) v.x = __int_as_float(0x7fc00000);
     }
+    g->v[b] = v;
     uint32_t inv = ~__float_as_uint(fmaxf(r, 0.0f));
     inv = __reduce_max_sync(0xffffffffu, inv);
-    const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge));
-    bad = __any_sync(0xffffffffu, bad);
+    const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge && !gap));
+    gap = __any_sync(0xffffffffu, gap);
     if (lane_id() == 0) {
         atomicMax(&kc->rho_inv, inv);
         if (edges) atomicAdd(&kc->edges, edges);
-        if (bad) atomicOr(&kc->bad, 2u);
+        if (gap) kc->gaps = 1u;
     }
     if (blockIdx.x == 0 && tid == 0) {
         g->cx = cx;
         g->cy = cy;
         g->ok = 1u;
+        g->centre = centre_inside(*oct) ? 1u : 0u;
     }
 }
 
@@ -829,7 +880,7 @@ __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restr
         octs = filter_candidates(fs, ws, L);
     } else {
         const FanView<Level1> f{fan, Level1{}, SharedFan(sv), make_float2(fs.so.cx, fs.so.cy),
-                                fan ? disk_limit(fan_rho2(kc)) : 0.0f, true};
+                                fan ? disk_limit(fan_rho2(kc)) : 0.0f, kc->gaps == 0u};
         const uint32_t ntiles = (n + kFiltTile - 1) / kFiltTile;   // (n < 2^30)
         const uint32_t gi = blockIdx.x * CG + threadIdx.x / kFiltThreads;
         const uint32_t per = (ntiles + gridDim.x * CG - 1) / (gridDim.x * CG);
@@ -856,8 +907,9 @@ __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restr
 //                       at least kFan2MinS points, or the tuned minimum,
 //                       survived); per sub-bin the farthest survivor
 //  fan2_build_kernel    the vertex of every sub-bin (the previous non-empty
-//                       one for an empty sub-bin, cyclically); the proof
-//                       that consecutive ones are counter-clockwise
+//                       one for an empty sub-bin, cyclically); where the next
+//                       one is not proven counter-clockwise from it: none
+//                       (the first level's proofs put c inside the hull)
 //  fan2_test_kernel     the test of every survivor; the kept ones go to the
 //                       sort's second buffers, which the sort then reads
 // ---------------------------------------------------------------------------
@@ -916,18 +968,18 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
         if (threadIdx.x == 0) f2->bad = 1u;
         return;
     }
-    const float2 v = surv_point(keys, pay, ~(uint32_t)slot[src]);
-    V[b] = v;
-    if (b < 2) V[kFan2Bins + b] = v;
-    if (b == kFan2Bins - 1) V[-1] = v;
+    float2 v = surv_point(keys, pay, ~(uint32_t)slot[src]);
     const unsigned long long nextp = slot[b + 1 == kFan2Bins ? 0 : b + 1];
     const float2 w = nextp != 0ull ? surv_point(keys, pay, ~(uint32_t)nextp) : v;
     const bool edge = v.x != w.x || v.y != w.y;
     // c strictly left of v -> w, proven in binary32 or exactly
-    const bool bad = edge && orient(v.x, v.y, w.x, w.y, g->cx, g->cy) <= 0;
-    const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge));
+    const bool gap = edge && orient(v.x, v.y, w.x, w.y, g->cx, g->cy) <= 0;
+    if (gap) v.x = __int_as_float(0x7fc00000);
+    V[b] = v;
+    if (b < 2) V[kFan2Bins + b] = v;
+    if (b == kFan2Bins - 1) V[-1] = v;
+    const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge && !gap));
     if (lane_id() == 0 && edges) atomicAdd(&f2->edges, edges);
-    if (bad) f2->bad = 1u;
 }
 
 // Bound by the latency of the 1.8 MB table in L2: eight survivors per thread
@@ -941,7 +993,7 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
     Fan2Ctrl *f2 = at<Fan2Ctrl>(ws, L.fan2);
     if (!f2->on) return;
     const uint32_t m = f2->count_in;
-    const bool test = !f2->bad && f2->edges >= 3u;
+    const bool test = !f2->bad && f2->edges != 0u;
     const Kgon *g = at<Kgon>(ws, L.kgon);
     const float2 c = make_float2(g->cx, g->cy);
     const GlobalFan F{at<float2>(ws, L.fan2_v) + 1};
@@ -1276,6 +1328,10 @@ __global__ void __launch_bounds__(kFiltThreads, 5) bx_fan_bins_kernel(const floa
             }
         };
         fetch(0);
+        if (first == 0u && t < 32u) {
+            const unsigned long long *ext = at<unsigned long long>(ws, BL.ext_slot) + (size_t)item.x * 8;
+            raise_octagon(nb, slot, o, [&](int k) { return ~(uint32_t)ext[k]; });
+        }
         for (uint32_t u = 0; u < steps; ++u) {
             float qx[BI], qy[BI];
             const uint32_t mine = live;
@@ -1335,7 +1391,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
     kernel_entry();
     __shared__ int s_w[BT / 32];
     __shared__ int s_last;
-    __shared__ uint32_t s_inv, s_edges, s_bad, s_in, s_seen;
+    __shared__ uint32_t s_inv, s_edges, s_gaps, s_in, s_seen;
     const SetInfo *sets = at<SetInfo>(ws, BL.sets);
     const Octagon *octs = at<Octagon>(ws, BL.octs);
     const uint32_t nfan = at<BatchCtrl>(ws, BL.bctrl)->nfan;
@@ -1354,8 +1410,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
         __syncthreads();   // the shared words of the previous set have been read
         if (tid == 0) {
             s_last = -1;
-            s_inv = s_edges = s_in = s_seen = 0u;
-            s_bad = off ? 1u : 0u;
+            s_inv = s_edges = s_gaps = s_in = s_seen = 0u;
         }
         __syncthreads();
         if (off) continue;   // block-uniform
@@ -1368,7 +1423,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
         int carry = s_last;
         if (carry < 0) continue;   // block-uniform
         uint32_t inv = 0, edges = 0;
-        bool bad = false;
+        bool gaps = false;
         for (int b0 = 0; b0 < NB; b0 += BT) {   // (NB is a multiple of kBxBinRun: the last chunk may be half full)
             const int b = b0 + (int)tid;
             const float2 mine = b < NB ? raw[b] : make_float2(__int_as_float(0x7fc00000), 0.0f);
@@ -1388,15 +1443,20 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
             if (src < 0) src = carry;
             if (all >= 0) carry = all;
             if (b < NB) {
-                const float2 v = src == b ? mine : raw[src], next = raw[b + 1 == NB ? 0 : b + 1];
-                V[b] = v;
+                float2 v = src == b ? mine : raw[src];
+                const float2 next = raw[b + 1 == NB ? 0 : b + 1];
                 const float2 w = next.x == next.x ? next : v;
                 if (v.x != w.x || v.y != w.y) {
                     const float r = disk_bound(cx, cy, v, w);
-                    bad |= r < 0.0f;
                     inv = max(inv, ~__float_as_uint(fmaxf(r, 0.0f)));
-                    ++edges;
+                    if (r < 0.0f) {
+                        gaps = true;
+                        v.x = __int_as_float(0x7fc00000);
+                    } else {
+                        ++edges;
+                    }
                 }
+                V[b] = v;
             }
         }
         inv = __reduce_max_sync(0xffffffffu, inv);
@@ -1405,10 +1465,11 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
             atomicMax(&s_inv, inv);
             atomicAdd(&s_edges, edges);
         }
-        if (bad) s_bad = 1u;
+        if (gaps) s_gaps = 1u;
         __syncthreads();
         const float rho2 = __uint_as_float(~s_inv);
-        if (s_bad || s_edges < 3u || !(rho2 > 0x1p-120f)) continue;   // block-uniform
+        const bool gap = s_gaps != 0u;
+        if (!fan_holds(s_edges, gap, rho2, gap && centre_inside(o))) continue;   // block-uniform
         if (tid < (uint32_t)kBxSample) {   // (points of the first and last bins, whose neighbours wrap, are left out)
             const float2 p = __ldg(reinterpret_cast<const float2 *>(pts) + S.pt_begin + S.n * tid / kBxSample);
             const float2 c = make_float2(cx, cy), d = sub2(p, c);
@@ -1431,7 +1492,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
         }
         __syncthreads();
         if (tid == 0) {
-            info.rho2 = rho2;
+            info.rho2 = gap ? 0.0f : rho2;
             info.ready = 8u * s_in >= s_seen ? 1u : 0u;
         }
     }
@@ -1482,7 +1543,7 @@ __global__ void __launch_bounds__(CT, 1) bx_hull_filter_kernel(const float *__re
         const FanInfo &info = at<FanInfo>(ws, BL.fan)[cur];
         const bool fan = info.ready != 0u;
         const FanView<SetBins> f{fan, SetBins{info.nb}, SharedFan(sv), make_float2(fs.so.cx, fs.so.cy),
-                                 fan ? disk_limit(info.rho2) : 0.0f, info.tight == 0u};
+                                 fan ? disk_limit(info.rho2) : 0.0f, info.tight == 0u && info.rho2 > 0.0f};
         const float *p = pts + 2 * S.pt_begin;
         const uint32_t first = item.y + threadIdx.x / kFiltThreads, end = min(item.y + chunk, S.ntiles);
         if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0)
