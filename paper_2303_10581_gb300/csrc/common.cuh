@@ -103,12 +103,11 @@ struct KgonCtrl {                          // zeroed with the control block
     unsigned long long slot[kFanBins];     // packed (far_key << 32 | ~index): farthest sampled input point per bin
     uint32_t sample, inside;               // points sampled for the bins, octagon survivors among them
     uint32_t s_oct;                        // octagon survivors
-    uint32_t bad;                          // samples in one place only
     uint32_t rho_inv;                      // ~bits of a lower bound (binary32) on the squared distance from
                                            // c to the fan's boundary, the largest so far
     uint32_t edges;                        // consecutive vertex pairs with v != w
     uint32_t gaps;                         // 1: some of them not proven counter-clockwise around c
-    uint32_t pad;
+    uint32_t pad[2];
 };
 
 // second fan level (kgon.cu): over the first level's survivors, kFan2Sub
@@ -306,10 +305,9 @@ struct FanInfo {
     uint32_t want;        // enough octagon survivors (an estimate) for a fan
     uint32_t tight;       // the points' distances from the centre differ by rounding only (a circle)
     uint32_t nb;          // bins
-    uint32_t bad;         // no usable vertices
     uint32_t ready;       // the fan's proofs hold and it drops enough points
     float rho2;           // lower bound on the squared distance from the centre to the fan's boundary (0: none)
-    uint32_t pad[2];
+    uint32_t pad[3];
 };
 
 // Extra workspace of ch_hull_batched, after the single-set regions.

@@ -63,6 +63,7 @@
 //                     payloads, in no particular order (the chain breaks
 //                     ties by the index in the payload)
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "fan.cuh"
@@ -419,34 +420,55 @@ struct VertexSmem {
 };
 
 // The nearest non-empty bin before `from` (dir = -1) or from `from` on (dir =
-// 1), unwrapped; from -+ NB when there is none.
-__device__ __forceinline__ int nearest_bin(int NB, const unsigned long long *slot, int from, int dir)
+// 1), unwrapped, among `reach` of them (a multiple of 32); kNoBin when there is
+// none.  The first 32 nearly always hold one; of the others four times 32 are
+// read at once.
+constexpr int kNoBin = INT_MIN;
+
+__device__ __forceinline__ int nearest_bin(int NB, const unsigned long long *slot, int from, int dir, int reach)
 {
     const int lane = (int)lane_id();
-    for (int k = 0; k < NB; k += 32) {
+    const auto filled = [&](int k) {   // of the 32 bins after the first k
         const int j = dir > 0 ? from + k + lane : from - 1 - k - lane;
         const int w = j < 0 ? j + NB : (j >= NB ? j - NB : j);
-        const uint32_t m = __ballot_sync(0xffffffffu, __ldcg(slot + w) != 0ull);
-        if (m) return dir > 0 ? from + k + __ffs(m) - 1 : from - k - __ffs(m);
+        return k < reach && __ldcg(slot + w) != 0ull;
+    };
+    const auto place = [&](int k, uint32_t m) { return dir > 0 ? from + k + __ffs(m) - 1 : from - k - __ffs(m); };
+    const uint32_t m0 = __ballot_sync(0xffffffffu, filled(0));
+    if (m0) return place(0, m0);
+    for (int k = 32; k < reach; k += 128) {
+        bool f[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) f[u] = filled(k + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t m = __ballot_sync(0xffffffffu, f[u]);
+            if (m) return place(k + 32 * u, m);
+        }
     }
-    return dir > 0 ? from + NB : from - NB;
+    return kNoBin;
 }
 
 // Bins [b0, b0 + VB) of a fan; point(i) reads input point i
-// (clamped to the input); V receives the vertices, x = NaN for none.  False
-// when there are no samples outside the range (no fan).
+// (clamped to the input); V receives the vertices, x = NaN for none.  The
+// neighbours of the range are looked for within an eighth of the turn and 288
+// bins: a chord over more empty bins adds nothing that the wedge over them
+// does not have, and walking the empty bins of a set that is seen from its
+// centre in a small angle (an arc, far outliers, a line) 32 at a time took
+// 117 to 362 us.
 template <class Bins, class Point>
-__device__ __forceinline__ bool make_vertices(Bins nb, VertexSmem &sm, const unsigned long long *slot, int b0, float2 c,
+__device__ __forceinline__ void make_vertices(Bins nb, VertexSmem &sm, const unsigned long long *slot, int b0, float2 c,
                                               Point point, float2 *V)
 {
     const int NB = (int)nb.count();
     const int lane = (int)lane_id();
     const uint32_t lt = (1u << lane) - 1u;
-    const int before = nearest_bin(NB, slot, b0, -1), after = nearest_bin(NB, slot, b0 + VB, 1);
-    if (before <= b0 + VB - 1 - NB || after >= b0 + NB) return false;   // (only this range has samples)
+    const int reach = min(288, NB / 8 & ~31);
+    const int before = nearest_bin(NB, slot, b0, -1, reach), after = nearest_bin(NB, slot, b0 + VB, 1, reach);
+    const int head = before != kNoBin ? 1 : 0;
     bool has[VB / 32];
     float2 own[VB / 32];
-    int len = 1;
+    int len = head;
 #pragma unroll
     for (int h = 0; h < VB / 32; ++h) {
         const unsigned long long v = __ldcg(slot + b0 + 32 * h + lane);
@@ -461,12 +483,14 @@ __device__ __forceinline__ bool make_vertices(Bins nb, VertexSmem &sm, const uns
     }
     if (lane < 2) {
         const int j = lane ? after : before;
-        const int w = j < 0 ? j + NB : (j >= NB ? j - NB : j);
-        const int at = lane ? len : 0;
-        sm.p[0][at] = point(~(uint32_t)__ldcg(slot + w));
-        sm.bin[0][at] = j;
+        if (j != kNoBin) {
+            const int w = j < 0 ? j + NB : (j >= NB ? j - NB : j);
+            const int at = lane ? len : 0;
+            sm.p[0][at] = point(~(uint32_t)__ldcg(slot + w));
+            sm.bin[0][at] = j;
+        }
     }
-    ++len;
+    len += after != kNoBin ? 1 : 0;
     __syncwarp();
     int cur = 0;
     for (int pass = 0; pass < kVertexPasses; ++pass) {
@@ -494,16 +518,16 @@ __device__ __forceinline__ bool make_vertices(Bins nb, VertexSmem &sm, const uns
 #pragma unroll
     for (int h = 0; h < VB / 32; ++h) {
         const int b = b0 + 32 * h + lane;
-        int lo = 0, hi = len - 1;   // last entry at or before bin b (entry 0 is before the range, the last after it)
+        int lo = -1, hi = len;   // the last entry at or before bin b (-1: none), the first after it (len: none)
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (sm.bin[cur][mid] <= b) lo = mid;
             else hi = mid;
         }
-        const float2 Lp = sm.p[cur][lo], Rp = sm.p[cur][lo + 1];
         float2 v = own[h];
         bool ok = has[h];
-        if (sm.bin[cur][lo] != b) {
+        if (lo >= 0 && hi < len && sm.bin[cur][lo] != b) {
+            const float2 Lp = sm.p[cur][lo], Rp = sm.p[cur][hi];
             const float lx = Lp.x - c.x, ly = Lp.y - c.y, ex = Rp.x - Lp.x, ey = Rp.y - Lp.y;
             const float num = lx * ey - ly * ex;
             const float own_den = (v.x - c.x) * ey - (v.y - c.y) * ex;
@@ -521,7 +545,6 @@ __device__ __forceinline__ bool make_vertices(Bins nb, VertexSmem &sm, const uns
         }
         V[b] = ok ? v : make_float2(__int_as_float(0x7fc00000), 0.0f);
     }
-    return true;
 }
 
 __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict__ pts, int64_t n, void *ws, Layout L)
@@ -533,10 +556,9 @@ __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict_
     if (!fan_live(kc, oct, n)) return;
     const int warp = (int)(threadIdx.x >> 5);
     const int b0 = (int)(blockIdx.x * (VT / 32) + warp) * VB;
-    const bool ok = make_vertices(
+    make_vertices(
         Level1{}, sm[warp], kc->slot, b0, make_float2(oct->cx, oct->cy),
         [&](uint32_t i) { return input_point(pts, (int64_t)i < n ? i : 0u); }, at<Kgon>(ws, L.kgon)->raw);
-    if (!ok && lane_id() == 0) kc->bad = 1u;
 }
 
 __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layout L)
@@ -548,7 +570,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     Kgon *g = at<Kgon>(ws, L.kgon);
     const uint32_t tid = threadIdx.x;
-    const bool live = fan_live(kc, oct, n) && !kc->bad;
+    const bool live = fan_live(kc, oct, n);
     const int b = (int)(blockIdx.x * BT + tid);
     int src = -1;
     if (live) src = vertex_source([&](int j) { return g->raw[j].x == g->raw[j].x; }, s_w, s_scan);   // block-uniform
@@ -1248,7 +1270,7 @@ __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, BatchLayo
         const uint32_t nt = sets[b].ntiles;
         if (fan[b].want) {
             const uint32_t nb = fan[b].nb;
-            fan[b].bad = fan[b].ready = 0u;
+            fan[b].ready = 0u;
             at<uint32_t>(ws, BL.fan_set)[run[0]++] = (uint32_t)b;
             for (uint32_t t = 0; t < nt; t += chunk) fi[run[1]++] = make_uint2((uint32_t)b, t);
             for (uint32_t k = 0; k < nb; k += kBxBinRun) bi[run[3]++] = make_uint2((uint32_t)b, k);
@@ -1374,11 +1396,10 @@ __global__ void __launch_bounds__(VT) bx_fan_vertex_kernel(const float *__restri
             }
             continue;   // block-uniform
         }
-        const bool ok = make_vertices(
+        make_vertices(
             SetBins{info.nb}, sm[warp], bx_slots(ws, BL, S), (int)item.y + warp * VB,
             make_float2(octs[item.x].cx, octs[item.x].cy), [&](uint32_t i) { return __ldg(p + ((int64_t)i < m ? i : 0u)); },
             bx_raw(ws, BL, S));
-        if (!ok && lane_id() == 0) at<FanInfo>(ws, BL.fan)[item.x].bad = 1u;
         __syncwarp();
     }
 }
@@ -1406,7 +1427,7 @@ __global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restric
         const SetBins nb{info.nb};
         const int NB = (int)nb.n;
         const float cx = o.cx, cy = o.cy;
-        const bool off = info.bad || !(__fadd_rn(__fsub_rn(o.bxh, o.bxl), __fsub_rn(o.byh, o.byl)) < 0x1p62f);
+        const bool off = !(__fadd_rn(__fsub_rn(o.bxh, o.bxl), __fsub_rn(o.byh, o.byl)) < 0x1p62f);
         __syncthreads();   // the shared words of the previous set have been read
         if (tid == 0) {
             s_last = -1;

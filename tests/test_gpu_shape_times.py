@@ -1,0 +1,58 @@
+"""Inputs whose shape once cost a stage far more than its points: the call's
+time against that of the same call on as many points of a circle.  A case's
+factor is the ratio of the time that the call took before the stage was made
+for other shapes, and a quarter more; what it guards took 1.3 to 3 times the
+factor."""
+import math
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2303_10581_gb300 as ch  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def points(shape, n):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(7)
+    u = torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
+    th = 2 * math.pi * u
+    if shape == "circle":
+        x, y = torch.cos(th), torch.sin(th)
+    elif shape == "horizontal":
+        x, y = u, torch.full_like(u, 0.3)
+    return torch.stack([x, y], 1).float().contiguous()
+
+
+def call_us(call, p):
+    n = len(p)
+    ws = ch.Workspace(n)
+    idx = torch.zeros(n, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    if call == "hull":
+        def run():
+            ch.ch_hull(p, idx, cnt, ws.buf)
+    for _ in range(3):
+        run()
+    best = math.inf
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            run()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 100)
+    ws.check()
+    return best
+
+
+@pytest.mark.parametrize("call,shape,n,factor", [
+    # all bins but two are empty: their neighbours are not searched for through the whole table
+    ("hull", "horizontal", 300_007, 2.5),
+])
+def test_time(call, shape, n, factor):
+    base, us = call_us(call, points("circle", n)), call_us(call, points(shape, n))
+    assert us <= factor * base, (us, base)
