@@ -1407,7 +1407,7 @@ __global__ void __launch_bounds__(VT) bx_fan_vertex_kernel(const float *__restri
 // A block per fan set: empty bins repeat the vertex before them; the proofs
 // of fan_build_kernel; and whether the fan drops at least an eighth of a
 // sample.
-__global__ void __launch_bounds__(BT) bx_fan_build_kernel(const float *__restrict__ pts, void *ws, BatchLayout BL)
+__global__ void __launch_bounds__(BT, 2) bx_fan_build_kernel(const float *__restrict__ pts, void *ws, BatchLayout BL)
 {
     kernel_entry();
     __shared__ int s_w[BT / 32];
