@@ -67,8 +67,6 @@ struct Octagon {
     // order R, TR, T, TL, L, BL, B, BR
     float ax[8], ay[8];     // edge start
     float bx[8], by[8];     // edge end
-    float dx[8], dy[8];     // fl(b - a)
-    float bound[8];         // static error bound of the binary32 test (+inf: off)
     uint32_t valid;         // bit k: edge k has non-zero length
     uint32_t has_edges;     // at least one valid edge
     uint32_t abort;         // non-finite input: later stages do nothing
@@ -560,36 +558,6 @@ static __device__ __noinline__ int orient_d(float ax, float ay, float bx, float 
     return orient_exact(ax, ay, bx, by, cx, cy);
 }
 
-// Sterbenz: a - c is exact in binary32 when a and c have the same sign and
-// are within a factor of two of each other.
-__device__ __forceinline__ bool exact_diff(float a, float c)
-{
-    const float aa = fabsf(a), cc = fabsf(c);
-    return ((a >= 0.0f) == (c >= 0.0f)) && aa <= 2.0f * cc && cc <= 2.0f * aa;
-}
-
-// Tier 2b: exact binary32 sign for nearby points.  When the four
-// differences are exact, detleft = u1 v1 and detright = u2 v2 exactly; with
-// p = fl(u v) and e = fma(u, v, -p) = u v - p (exact while |p| >= 2^-100 or
-// a factor is zero, since then the product cannot underflow), rounding is
-// monotone, so p1 > p2 implies u1 v1 > u2 v2, and when p1 == p2 the
-// determinant is e1 - e2, whose sign survives the one rounding of
-// fl(e1 - e2).  Returns 2 when the preconditions do not hold.
-__device__ __forceinline__ int orient_near(float ax, float ay, float bx, float by, float cx, float cy)
-{
-    if (!(exact_diff(ax, cx) && exact_diff(by, cy) && exact_diff(ay, cy) && exact_diff(bx, cx))) return 2;
-    const float u1 = __fsub_rn(ax, cx), v1 = __fsub_rn(by, cy);
-    const float u2 = __fsub_rn(ay, cy), v2 = __fsub_rn(bx, cx);
-    const float p1 = __fmul_rn(u1, v1), p2 = __fmul_rn(u2, v2);
-    const bool ok1 = (u1 == 0.0f || v1 == 0.0f) || (fabsf(p1) >= 7.888609052210118e-31f /* 2^-100 */ &&
-                                                    fabsf(p1) <= 3.0e38f);
-    const bool ok2 = (u2 == 0.0f || v2 == 0.0f) || (fabsf(p2) >= 7.888609052210118e-31f && fabsf(p2) <= 3.0e38f);
-    if (!(ok1 && ok2)) return 2;
-    if (p1 != p2) return p1 > p2 ? 1 : -1;
-    const float d = __fsub_rn(__fmaf_rn(u1, v1, -p1), __fmaf_rn(u2, v2, -p2));
-    return d > 0.0f ? 1 : (d < 0.0f ? -1 : 0);
-}
-
 // Tier 1: binary32 evaluation with a dynamic bound.  The expression has
 // Shewchuk's orient2d shape (four differences, two products, one
 // subtraction), whose rounding error is below (3 + 16 eps) eps * detsum with
@@ -638,13 +606,53 @@ __device__ __forceinline__ int orient_pair(float ax, float ay, float bx, float b
     return detsum <= 3.0e38f ? o : 2;
 }
 
-// The tiers after that: equal points, exact differences, binary64, expansions
+// A product r = fl(a b) whose rounding error fma(a, b, -r) is exact, as it
+// cannot underflow (or r is an exact zero).
+__device__ __forceinline__ bool exact_product(float a, float b, float r)
+{
+    return a == 0.0f || b == 0.0f || (fabsf(r) >= 0x1p-100f && fabsf(r) <= 3.0e38f);
+}
+// Whether a b == c d, proven.
+__device__ __forceinline__ bool same_product(float a, float b, float c, float d)
+{
+    const float r = __fmul_rn(a, b), s = __fmul_rn(c, d);
+    return exact_product(a, b, r) && exact_product(c, d, s) && r == s && __fmaf_rn(a, b, -r) == __fmaf_rn(c, d, -s);
+}
+
+// The tiers after that: the exactly collinear triples of points on a side of
+// the box, of grids and of lines y = 2^k x, then binary64, then expansions
 // (whose 200 binary64 steps are some 15000 cycles).
+//  - A difference that is zero is exact, so a product with one is zero
+//    whatever its other factor (equal points, points on an axis-parallel
+//    edge).
+//  - Where the four differences are exact (points near one another or of a
+//    grid) the products p + pe, q + qe are too; rounding is monotone, so p > q
+//    implies p + pe > q + qe, and for p == q the sign is that of pe - qe, which
+//    survives its rounding.
+//  - The determinant is zero when its expanded products cancel in pairs.
+// In binary64 they took most of the time of such sets: 60 sets of 150001
+// points on a square's sides 3345 us (1102 so), of a diagonal 4856 (931).
 static __device__ __noinline__ int orient_last(float ax, float ay, float bx, float by, float cx, float cy)
 {
-    if ((ax == cx && ay == cy) || (bx == cx && by == cy) || (ax == bx && ay == by)) return 0;
-    const int o = orient_near(ax, ay, bx, by, cx, cy);
-    return o != 2 ? o : orient_d(ax, ay, bx, by, cx, cy);
+    if (ax == bx && ay == by) return 0;
+    float u, ul, v, vl, w, wl, z, zl;
+    two_diff(ax, cx, u, ul);
+    two_diff(by, cy, v, vl);
+    two_diff(ay, cy, w, wl);
+    two_diff(bx, cx, z, zl);
+    if ((u == 0.0f || v == 0.0f) && (w == 0.0f || z == 0.0f)) return 0;
+    const uint32_t low = (__float_as_uint(ul) | __float_as_uint(vl) | __float_as_uint(wl) | __float_as_uint(zl)) << 1;
+    const float p = __fmul_rn(u, v), q = __fmul_rn(w, z);
+    if (low == 0u && exact_product(u, v, p) && exact_product(w, z, q)) {
+        if (p != q) return p > q ? 1 : -1;
+        const float d = __fsub_rn(__fmaf_rn(u, v, -p), __fmaf_rn(w, z, -q));
+        return d > 0.0f ? 1 : (d < 0.0f ? -1 : 0);
+    }
+    if (same_product(u, v, w, z) && same_product(ul, vl, wl, zl) &&
+        ((same_product(u, vl, w, zl) && same_product(ul, v, wl, z)) ||
+         (same_product(u, vl, wl, z) && same_product(ul, v, w, zl))))
+        return 0;
+    return orient_d(ax, ay, bx, by, cx, cy);
 }
 
 __device__ __forceinline__ int orient_rest(float ax, float ay, float bx, float by, float cx, float cy)

@@ -73,17 +73,7 @@ __device__ __forceinline__ float pow2_inverse(float v)
 
 // Builds the filter polygon from the eight vertex indices.  Run by one full
 // warp.  Edge k joins vertex k to vertex k+1 (mod 8); edges of zero length
-// are disabled.  For each edge the binary32 test
-//   t = fl(fl(dx * fl(py - ay)) - fl(dy * fl(px - ax)))
-// is Shewchuk's orient2d expression for (b, p, a) with the edge differences
-// precomputed; its rounding error is below (3 + 16 eps) eps * (|fl(dx*v)| +
-// |fl(dy*u)|), eps = 2^-24.  Because |px - ax| <= W = xmax - xmin and
-// |py - ay| <= H and rounding is monotone, that sum never exceeds
-// M = (|dx| fl(H) + |dy| fl(W))(1 + 2^-20), so bound = 4 eps M + 2^-140
-// (the last term covers products that underflow) is a static bound valid
-// for every point: t > bound proves "strictly left", t < -bound proves
-// "not left", anything else is decided exactly.  The edge test is disabled
-// (bound = +inf) when the box extents overflow or M > 2^100.
+// are disabled.
 //
 // The box W x H is the closed bounding box of the eight vertices.  When
 // they are the data's extremes (data_extremes: R, T, L, B really are the
@@ -92,8 +82,8 @@ __device__ __forceinline__ float pow2_inverse(float v)
 // the point test to keep every point outside the box first (box_check): a
 // point strictly left of every edge has winding number >= 1 around the
 // vertex sequence, so it lies in the vertices' convex hull and hence in
-// their box; a point outside the box is never strictly inside.  The static
-// bound then holds for every point that reaches the edge test.
+// their box; a point outside the box is never strictly inside.  The bound
+// below then holds for every point that reaches the edge test.
 //
 // The affine form of edge k (octtest.cuh), with c the box centre, u* = px -
 // cx, v* = py - cy exactly, (ex, ey) = b - a and K = ex (ay - cy) - ey (ax -
@@ -144,24 +134,14 @@ __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_
         }
     }
     const bool valid = !(a.x == b.x && a.y == b.y);
-    const float dx = __fsub_rn(b.x, a.x), dy = __fsub_rn(b.y, a.y);
     const float W = __fsub_rn(xmax, xmin), H = __fsub_rn(ymax, ymin);
     const bool finite = W <= 3.0e38f && H <= 3.0e38f;
-    float bound = __int_as_float(0x7f800000);  // +inf: binary32 test off
-    if (finite) {
-        const float M =
-            __fmul_ru(__fadd_ru(__fmul_ru(fabsf(dx), H), __fmul_ru(fabsf(dy), W)), 1.0f + 0x1p-20f);
-        if (M <= 0x1p100f) bound = __fadd_ru(__fmul_ru(M, 0x1p-22f), 0x1p-140f);
-    }
     const uint32_t vmask = __ballot_sync(0xffffffffu, valid) & 0xffu;
     if (lane < 8) {
         out->ax[k] = a.x;
         out->ay[k] = a.y;
         out->bx[k] = b.x;
         out->by[k] = b.y;
-        out->dx[k] = dx;
-        out->dy[k] = dy;
-        out->bound[k] = bound;
     }
     // (halves first: the sum cannot overflow)
     const float cx = __fadd_rn(0.5f * xmin, 0.5f * xmax), cy = __fadd_rn(0.5f * ymin, 0.5f * ymax);

@@ -831,12 +831,17 @@ __device__ __forceinline__ void filter_tiles(const FilterSmem &fs, const FanView
                 if (q.n >= 32u) queue_drain(q, fs, f, use_disk, pts, octs);
             }
         } else {   // many at once: the points are read again
-            if (use_disk || near) {
+            if ((use_disk || near) && live) {   // (the next point is on its way meanwhile)
+                uint32_t m = live, i = (uint32_t)item_point<G>(base, t, __ffs(m) - 1);
+                float2 p = input_point(pts, i);
 #pragma unroll 1
-                for (uint32_t m = live; m; m &= m - 1u) {
-                    const uint32_t i = (uint32_t)item_point<G>(base, t, __ffs(m) - 1);
-                    if (!settle(fs.so, f, use_disk, i | (near ? kUnsettled : 0u), input_point(pts, i), octs))
-                        live &= ~(m & (0u - m));
+                while (m) {
+                    const uint32_t bit = m & (0u - m), mine = i;
+                    m ^= bit;
+                    float2 next = p;
+                    if (m) next = input_point(pts, i = (uint32_t)item_point<G>(base, t, __ffs(m) - 1));
+                    if (!settle(fs.so, f, use_disk, mine | (near ? kUnsettled : 0u), p, octs)) live ^= bit;
+                    p = next;
                 }
             }
             const uint32_t left = __reduce_add_sync(0xffffffffu, __popc(live));

@@ -32,23 +32,31 @@ __device__ __forceinline__ bool outside_box(const Octagon &o, float x, float y)
     return false;
 }
 
-// keep(p) <=> NOT (p strictly left of every valid edge); see
-// build_octagon_warp for the error bound of the binary32 test, which holds
-// for points inside the vertices' bounding box.
+// keep(p) <=> NOT (p strictly left of every valid edge): the forms first,
+// all at once, then exact signs at the edges they leave undecided (the forms
+// hold for points inside the vertices' bounding box; when they are off, all
+// edges are undecided).
+// Bound by latency: few points come here, unless the input lies on the
+// polygon's edges (a rectangle's sides, a coarse grid), and then all.  One edge
+// after the other, each by a static bound first, 300007 points on a square's
+// sides took the filter 74 us and on a 16 x 16 grid 56; so 25 and 20.
 template <bool BOX>
 __device__ __noinline__ bool keep_point(const Octagon &o, float x, float y)
 {
-    if (x >= o.xl && x <= o.xh && y >= o.yl && y <= o.yh) return false;
     if (!o.has_edges || outside_box<BOX>(o, x, y)) return true;
+    const float u = __fsub_rn(x, o.cx), v = __fsub_rn(y, o.cy);
+    uint32_t open = 0;
+    bool out = false;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float t = __fmaf_rn(o.tx[k], u, __fmaf_rn(o.ty[k], v, o.tz[k]));
+        out |= t < -1.0f;
+        open |= t > 1.0f ? 0u : 1u << k;
+    }
+    if (out) return true;
 #pragma unroll 1
-    for (int e = 0; e < 8; ++e) {
-        if (!((o.valid >> e) & 1u)) continue;
-        const float u = __fsub_rn(x, o.ax[e]);
-        const float v = __fsub_rn(y, o.ay[e]);
-        const float t = __fsub_rn(__fmul_rn(o.dx[e], v), __fmul_rn(o.dy[e], u));
-        const float bnd = o.bound[e];
-        if (t > bnd) continue;
-        if (t < -bnd) return true;
+    for (open &= o.valid; open; open &= open - 1u) {
+        const int e = __ffs(open) - 1;
         if (orient_rest(o.ax[e], o.ay[e], o.bx[e], o.by[e], x, y) <= 0) return true;
     }
     return false;
@@ -77,8 +85,8 @@ __device__ __forceinline__ void fill_octagon(OctSmem &so, const Octagon *g)
 
 // N points at once: bit q of `keep` unless point q is proven strictly inside
 // the polygon; the result says whether any of them is undecided
-// (oct_undecided then tells which; the NaN-propagating minima leave a point
-// undecided whose difference overflowed).  The edges are the outer loop, so
+// (keep_point settles it; the NaN-propagating minima leave a point undecided
+// whose difference overflowed).  The edges are the outer loop, so
 // their forms are read once for the N points, and two points share an FMA
 // instruction.
 template <int N>
@@ -115,16 +123,6 @@ __device__ __forceinline__ bool oct_decide(const OctSmem &o, const float (&px)[N
         near = min_nan(near, fabsf(m[q]));
     }
     return !(near > 1.0f);
-}
-
-// Whether point (x, y) is undecided by the same forms.
-static __device__ __noinline__ bool oct_undecided(const OctSmem &o, float x, float y)
-{
-    const float u = __fsub_rn(x, o.cx), v = __fsub_rn(y, o.cy);
-    float m = 2.0f;
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) m = min_nan(m, __fmaf_rn(o.txy[k].x, u, __fmaf_rn(o.txy[k].z, v, o.tzz[k].x)));
-    return !(fabsf(m) > 1.0f);
 }
 
 // Point of item q of the 16 that thread t (of kFiltThreads) has in the

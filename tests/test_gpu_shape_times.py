@@ -23,6 +23,14 @@ def points(shape, n):
         x, y = torch.cos(th), torch.sin(th)
     elif shape == "horizontal":
         x, y = u, torch.full_like(u, 0.3)
+    elif shape == "diagonal":
+        x = y = u
+    elif shape == "grid":
+        x = torch.floor(16 * u)
+        y = torch.floor(16 * torch.rand(n, generator=g, device="cuda", dtype=torch.float64))
+    elif shape == "sides":
+        k, t = torch.floor(4 * u), torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
+        x, y = torch.where(k < 2, t, k - 2), torch.where(k < 2, k, t)
     return torch.stack([x, y], 1).float().contiguous()
 
 
@@ -34,6 +42,19 @@ def call_us(call, p):
     if call == "hull":
         def run():
             ch.ch_hull(p, idx, cnt, ws.buf)
+    elif call == "filter":
+        ext, sp = ch.extremes(p, ws), torch.zeros((n, 2), device="cuda")
+
+        def run():
+            ch.ch_filter(p, ext, idx, sp, cnt, ws.buf)
+    else:   # a batch: sets of that many points
+        m = int(call[5:])
+        sets = -(-n // m)
+        off = torch.clamp(torch.arange(sets + 1, device="cuda") * m, max=n)
+        ws, ho = ch.Workspace(n, sets), torch.zeros(sets + 1, dtype=torch.int64, device="cuda")
+
+        def run():
+            ch.ch_hull_batched(p, off, idx, ho, ws.buf)
     for _ in range(3):
         run()
     best = math.inf
@@ -52,6 +73,12 @@ def call_us(call, p):
 @pytest.mark.parametrize("call,shape,n,factor", [
     # all bins but two are empty: their neighbours are not searched for through the whole table
     ("hull", "horizontal", 300_007, 2.5),
+    # points on the polygon's edges: exact signs without binary64
+    ("filter", "sides", 300_007, 2.9),
+    ("hull", "diagonal", 300_007, 4.0),
+    ("batch60001", "sides", 12_000_200, 2.1),
+    ("batch150001", "grid", 9_000_060, 1.4),
+    ("batch150001", "diagonal", 9_000_060, 6.2),
 ])
 def test_time(call, shape, n, factor):
     base, us = call_us(call, points("circle", n)), call_us(call, points(shape, n))
