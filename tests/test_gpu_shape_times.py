@@ -23,6 +23,9 @@ def points(shape, n):
         x, y = torch.cos(th), torch.sin(th)
     elif shape == "horizontal":
         x, y = u, torch.full_like(u, 0.3)
+    elif shape == "cauchy":   # a heavy-tailed cloud: its box's centre is far from nearly all points
+        z = torch.randn((4, n), generator=g, device="cuda", dtype=torch.float64)
+        x, y = z[0] / z[1], z[2] / z[3]
     elif shape == "diagonal":
         x = y = u
     elif shape == "grid":
@@ -73,6 +76,8 @@ def call_us(call, p):
 @pytest.mark.parametrize("call,shape,n,factor", [
     # all bins but two are empty: their neighbours are not searched for through the whole table
     ("hull", "horizontal", 300_007, 2.5),
+    # nearly all points in a few bins: those inside the octagon are not binned
+    ("hull", "cauchy", 3_000_001, 0.9),
     # points on the polygon's edges: exact signs without binary64
     ("filter", "sides", 300_007, 2.9),
     ("hull", "diagonal", 300_007, 4.0),
