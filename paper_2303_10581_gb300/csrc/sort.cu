@@ -40,6 +40,11 @@ namespace {
 constexpr int kPassThreads = 512;
 constexpr int kBxPassThreads = 256;
 constexpr int kPassBlocks = 3;   // per SM: as many as the shared memory holds
+// A digit with at most so many values among a segment's keys, or the top one
+// (the sign and most of the exponent: most keys have one of a few values),
+// takes match.any.  (Equal keys, 60 sets of 150001: 76 us a pass by words in
+// shared memory, 64 by match.any; with 16 values and more the words win.)
+constexpr int kFewDigits = 8;
 
 template <int T>
 struct SortSmem {
@@ -204,11 +209,12 @@ struct PassIO {
 // One tile of a pass: tile_n <= 4096 (key, payload) pairs from element
 // `base`, ranked stably by digit (key >> shift) & 255 and written to
 // out_base + (segment digit start + rank in digit).  `first`: the
-// segment's first tile (its prefix is its own count).  Expects sm.dbase
+// segment's first tile (its prefix is its own count); `few`: the digit has few
+// values (kFewDigits).  Expects sm.dbase
 // (the segment's digit starts) set and sm.wh cleared, behind a barrier.
 template <int T>
 __device__ __forceinline__ void pass_tile(SortSmem<T> &sm, const PassIO &io, int64_t tile, int64_t base,
-                                          uint32_t tile_n, int64_t out_base, uint32_t out_n, int shift, bool first,
+                                          uint32_t tile_n, int64_t out_base, uint32_t out_n, int shift, bool few, bool first,
                                           void *ws, const Layout &L, uint32_t site)
 {
     constexpr int NW = T / 32, kItems = kSortTile / T;
@@ -230,9 +236,8 @@ __device__ __forceinline__ void pass_tile(SortSmem<T> &sm, const PassIO &io, int
     // of a digit find each other through a word per digit in shared memory:
     // match.any takes a step per distinct digit, and with 28 of them among 32
     // keys ranking was half of a tile's time (7500 of 17000 cycles, 2200 so).
-    // It stays for the top digit, the sign and most of the exponent: few
-    // values, whose lanes would meet at one word.
-    const bool top = shift == 24;
+    // It stays where the digit has few values (FEW), whose lanes would meet at
+    // one word.
     uint32_t *const mask = sm.keys + warp * 256;   // (cleared; the sorted keys come later)
     uint16_t rank[kItems];
 #pragma unroll
@@ -241,7 +246,7 @@ __device__ __forceinline__ void pass_tile(SortSmem<T> &sm, const PassIO &io, int
         const bool ok = e < tile_n;
         const uint32_t d = (k[j] >> shift) & 255u;
         uint32_t peers;
-        if (top) {
+        if (few) {
             peers = __match_any_sync(0xffffffffu, ok ? d : 256u);
         } else {
             if (ok) atomicOr(mask + d, 1u << lane);
@@ -252,7 +257,7 @@ __device__ __forceinline__ void pass_tile(SortSmem<T> &sm, const PassIO &io, int
         __syncwarp();
         if (ok && before == 0) {
             sm.wh[warp][d] = (uint16_t)(cur + __popc(peers));
-            if (!top) mask[d] = 0u;
+            if (!few) mask[d] = 0u;
         }
         __syncwarp();
         rank[j] = (uint16_t)(cur + before);
@@ -348,8 +353,10 @@ __global__ void __launch_bounds__(kPassThreads, kPassBlocks) sort_pass_kernel(vo
         for (int64_t w = gtid; w < ntiles * 256; w += gthreads) status_next[w] = 0u;
     }
     // global digit starts
+    const uint32_t h = tid < 256u ? ctrl->hist[p][tid] : 0u;
+    const bool few = __syncthreads_count(h != 0u) <= kFewDigits || p == kSortPasses - 1;
     {
-        const uint32_t ex = block_excl_scan(tid < 256u ? ctrl->hist[p][tid] : 0u, sm.warp_tot);
+        const uint32_t ex = block_excl_scan(h, sm.warp_tot);
         if (tid < 256u) sm.dbase[tid] = ex;
     }
     for (;;) {
@@ -371,7 +378,7 @@ __global__ void __launch_bounds__(kPassThreads, kPassBlocks) sort_pass_kernel(vo
         const int64_t tile = sm.tile;
         if (tile >= ntiles) break;
         const int64_t base = tile * kSortTile;
-        pass_tile(sm, io, tile, base, (uint32_t)min((int64_t)kSortTile, (int64_t)s - base), 0, s, 8 * p, tile == 0,
+        pass_tile(sm, io, tile, base, (uint32_t)min((int64_t)kSortTile, (int64_t)s - base), 0, s, 8 * p, few, tile == 0,
                   ws, L, 20 + p);
     }
 }
@@ -452,13 +459,15 @@ __global__ void __launch_bounds__(kBxPassThreads, kPassBlocks) bx_sort_pass_kern
         const int64_t ltile = tile - sets[b].sc_base;
         const int64_t seg = (int64_t)sets[b].surv_base;
         const uint32_t seg_n = sets[b].s;
-        {   // this set's digit starts (the scan's barriers also order sm.wh)
-            const uint32_t ex = block_excl_scan(
-                tid < 256u ? hist[((size_t)b * kSortPasses + p) * 256 + tid] : 0u, sm.warp_tot);
+        // this set's digit starts (the scan's barriers also order sm.wh)
+        const uint32_t h = tid < 256u ? hist[((size_t)b * kSortPasses + p) * 256 + tid] : 0u;
+        const bool few = __syncthreads_count(h != 0u) <= kFewDigits || p == kSortPasses - 1;
+        {
+            const uint32_t ex = block_excl_scan(h, sm.warp_tot);
             if (tid < 256u) sm.dbase[tid] = ex;
         }
         pass_tile(sm, io, tile, seg + ltile * kSortTile,
-                  (uint32_t)min((int64_t)kSortTile, (int64_t)seg_n - ltile * kSortTile), seg, seg_n, 8 * p,
+                  (uint32_t)min((int64_t)kSortTile, (int64_t)seg_n - ltile * kSortTile), seg, seg_n, 8 * p, few,
                   ltile == 0, ws, L, 40 + p);
     }
 }
