@@ -75,7 +75,7 @@ struct Octagon {
     float cx, cy;           // bounding-box centre, for the edge order
     float bxl, bxh, byl, byh;   // closed bounding box of the eight vertices
     uint32_t box_check;     // 1: points may lie outside that box (caller-supplied vertices)
-    uint32_t pad2;
+    float scale;            // power of two: the fan works on points times this (1 for boxes of ordinary sizes)
     float tx[8], ty[8], tz[8];   // edge k's affine form (octtest.cuh)
 };
 
@@ -126,7 +126,7 @@ struct Fan2Ctrl {                          // zeroed with the control block
 };
 
 struct Kgon {
-    float cx, cy;                          // fan centre
+    float cx, cy;                          // fan centre (it and the vertices times Octagon::scale)
     uint32_t ok;                           // 0: no fan this call
     uint32_t centre;                       // 1: c lies clearly inside the octagon
     float2 v[kFanBins];                    // vertex of every bin (x = NaN: none, and the wedges beside it keep their points)
@@ -304,7 +304,7 @@ struct FanInfo {
     uint32_t tight;       // the points' distances from the centre differ by rounding only (a circle)
     uint32_t nb;          // bins
     uint32_t ready;       // the fan's proofs hold and it drops enough points
-    float rho2;           // lower bound on the squared distance from the centre to the fan's boundary (0: none)
+    float rho2;           // lower bound on the squared (scaled) distance from the centre to the fan's boundary (0: none)
     uint32_t pad[3];
 };
 

@@ -145,6 +145,7 @@ __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_
     }
     // (halves first: the sum cannot overflow)
     const float cx = __fadd_rn(0.5f * xmin, 0.5f * xmax), cy = __fadd_rn(0.5f * ymin, 0.5f * ymax);
+    const float half = fmaxf(fmaxf(__fsub_rn(xmax, cx), __fsub_rn(cx, xmin)), fmaxf(__fsub_rn(ymax, cy), __fsub_rn(cy, ymin)));
     const float gx = pow2_inverse(W), gy = pow2_inverse(H);
     const float U = __fmul_ru(gx, fmaxf(__fsub_ru(xmax, cx), __fsub_ru(cx, xmin)));
     const float V = __fmul_ru(gy, fmaxf(__fsub_ru(ymax, cy), __fsub_ru(cy, ymin)));
@@ -214,6 +215,7 @@ __device__ void build_octagon_warp(const float2 *__restrict__ pts, const uint32_
         out->byh = ymax;
         out->box_check = data_extremes ? 0u : 1u;
         out->spec = 0u;
+        out->scale = half >= 0x1p-20f && half <= 0x1p20f ? 1.0f : pow2_inverse(half);
     }
 }
 

@@ -94,11 +94,21 @@ __device__ __forceinline__ uint32_t far_key(float px, float py, float cx, float 
     return ord_key(__fadd_rn(__fsub_rn(sh, r2ref), lo));
 }
 
+// A point (the centre) as the fan's arithmetic sees it: times the set's power
+// of two.  Squares and products of differences neither overflow nor vanish
+// then, whatever the set's size; a coordinate that becomes subnormal moves by
+// 2^-150 at most, of a box of size 1 to 4.
+__device__ __forceinline__ float2 fan_space(float2 p, float scale)
+{
+    return make_float2(__fmul_rn(p.x, scale), __fmul_rn(p.y, scale));
+}
+__device__ __forceinline__ float2 fan_centre(const Octagon &o) { return fan_space(make_float2(o.cx, o.cy), o.scale); }
+
 // r2ref of far_key for a polygon's set: the squared distance from its
 // centre to its first vertex (binary32).
 __device__ __forceinline__ float far_ref(const Octagon &o)
 {
-    const float ux = __fsub_rn(o.ax[0], o.cx), uy = __fsub_rn(o.ay[0], o.cy);
+    const float ux = __fmul_rn(__fsub_rn(o.ax[0], o.cx), o.scale), uy = __fmul_rn(__fsub_rn(o.ay[0], o.cy), o.scale);
     return __fmaf_rn(ux, ux, __fmul_rn(uy, uy));
 }
 

@@ -40,14 +40,16 @@
 //    hull, and there is no disk.  (One gap switching the fan off: 10^8 points
 //    of a displaced circle and one at ten radii, 49 M of them sorted, 5146 us;
 //    131 thousand and 2140 us when each wedge stood alone.);
-//  - the quotient needs |dx| + |dy| within [2^-126, 2^126]: the set's box is
-//    checked for the upper end, and a point closer to c than 2^-126 is
-//    inside the disk around c that is proven inside the fan (the fan is off
-//    unless its radius exceeds 2^-60).
+//  - all of this is done on points times a power of two that brings the set's
+//    box near size 1 where it is far from it (fan_space, Octagon::scale), so
+//    that nothing overflows; a coordinate moves by 2^-150 at most, which the
+//    2^-140 in the signs' bounds covers (points, vertices and c within 2^-148
+//    of where they are, in a box of size at most 2^22);
+//  - the quotient needs |dx| + |dy| of at least 2^-126: a point closer to c is
+//    inside the disk around c that is proven inside the fan (without gaps the
+//    fan is off unless its radius exceeds 2^-60) or inside the octagon.
 // Nothing else is exact: a sign that is not proven keeps the point, and what
-// is kept only costs the sort time.  (Sets so small that the products of the
-// signs underflow, below 10^-15, or with a box above 2^62 keep all their
-// points.)
+// is kept only costs the sort time.
 //
 // The disk around c proven inside the fan (a lower bound on the distance
 // from c to every fan edge) lets most points of a displaced circle pass
@@ -90,7 +92,7 @@ static_assert(kQueueSmem % 16 == 0 && kFanTable + kQueueSmem <= 227 * 1024 - 102
 // beyond it in magnitude has the exact sign.  Shewchuk's orient2d error
 // (orient_f32) is below 2^-22 (|l| + |r|) with l, r the products; |r| <= |l| +
 // |det|, so |det| > 2^-20 |l| implies |det| > 2^-22 (|l| + |r|) (2^-140 for
-// products that underflow; the fan's box rules out overflow).
+// products that underflow; fan_space rules out overflow).
 __device__ __forceinline__ float det_bound(float2 ac, float2 bc, float &bound)
 {
     const float l = __fmul_rn(ac.x, bc.y), r = __fmul_rn(ac.y, bc.x);
@@ -209,6 +211,16 @@ __device__ __forceinline__ void raise_bins(Bins nb, unsigned long long *slot, co
     }
 }
 
+__device__ __forceinline__ void to_fan_space(float (&qx)[BI], float (&qy)[BI], float scale)
+{
+    if (scale == 1.0f) return;   // uniform
+#pragma unroll
+    for (int k = 0; k < BI; ++k) {
+        qx[k] = __fmul_rn(qx[k], scale);
+        qy[k] = __fmul_rn(qy[k], scale);
+    }
+}
+
 // The octagon's vertices raise the bins as well (a warp calls; index(k):
 // vertex k's): far points in tiles that are not sampled are among them.
 template <class Bins, class Index>
@@ -219,10 +231,11 @@ __device__ __forceinline__ void raise_octagon(Bins nb, unsigned long long *slot,
     float qx[BI], qy[BI];
 #pragma unroll
     for (int k = 0; k < BI; ++k) {
-        qx[k] = o.ax[first + k];
-        qy[k] = o.ay[first + k];
+        const float2 v = fan_space(make_float2(o.ax[first + k], o.ay[first + k]), o.scale);
+        qx[k] = v.x;
+        qy[k] = v.y;
     }
-    raise_bins(nb, slot, qx, qy, lane_id() < 2u ? (1u << BI) - 1u : 0u, make_float2(o.cx, o.cy), far_ref(o),
+    raise_bins(nb, slot, qx, qy, lane_id() < 2u ? (1u << BI) - 1u : 0u, fan_centre(o), far_ref(o),
                [&](int k) { return index(first + k); });
 }
 
@@ -251,7 +264,8 @@ __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *
     __syncthreads();
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     const bool bits_mode = use_bits && (!kdev || *kdev != 8);
-    const float cx = so.cx, cy = so.cy, r2ref = far_ref(so);
+    const float r2ref = far_ref(so);
+    const float2 c = fan_centre(so);
     const uint32_t t = threadIdx.x;
     constexpr uint32_t parts = kFiltItems / BI;
     const uint32_t ntiles = (n + kFiltTile - 1) / kFiltTile, steps = (ntiles + stride - 1) / stride * parts;
@@ -265,7 +279,7 @@ __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *
             load_part<G, BI>(pts, base, t, part, px, py);
             live = (1u << BI) - 1u;
         } else {
-            live = load_part_ragged<G, BI>(pts, n, base, t, part, cx, cy, px, py);
+            live = load_part_ragged<G, BI>(pts, n, base, t, part, so.cx, so.cy, px, py);
         }
     };
     if (blockIdx.x < steps) fetch(blockIdx.x);
@@ -298,7 +312,8 @@ __global__ void __launch_bounds__(kFiltThreads, 5) fan_bins_kernel(const float *
         }
         if (counts) kept += __popc(mine);
         if (!__any_sync(0xffffffffu, mine != 0u)) continue;
-        raise_bins(Level1{}, kc->slot, qx, qy, mine, make_float2(cx, cy), r2ref, [&](int k) {
+        to_fan_space(qx, qy, so.scale);
+        raise_bins(Level1{}, kc->slot, qx, qy, mine, c, r2ref, [&](int k) {
             return (uint32_t)item_point<G>(tile * kFiltTile, t, (int)(BI * part) + k);
         });
     }
@@ -390,13 +405,12 @@ __device__ __forceinline__ float disk_bound(float cx, float cy, float2 v, float2
     return d < 0.0 ? -1.0f : (d <= 3.0e38 ? __double2float_rd(d) : 3.0e38f);
 }
 
-__device__ __forceinline__ bool fan_live(const KgonCtrl *kc, const Octagon *oct, int64_t n)
+__device__ __forceinline__ bool fan_live(const KgonCtrl *kc, int64_t n)
 {
     // (an aborted call, the speculative sweep's candidates, a polygon without
     // edges: the bins pass left no sample)
     const uint32_t sample = kc->sample;
-    const float box = __fadd_rn(__fsub_rn(oct->bxh, oct->bxl), __fsub_rn(oct->byh, oct->byl));
-    return sample != 0u && (double)kc->inside / sample * (double)n >= (double)kKgonMinS && box < 0x1p62f;
+    return sample != 0u && (double)kc->inside / sample * (double)n >= (double)kKgonMinS;
 }
 
 // The vertices of 64 consecutive bins, a warp: the samples of the bins and of
@@ -553,12 +567,13 @@ __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict_
     __shared__ VertexSmem sm[VT / 32];
     const Octagon *oct = at<Octagon>(ws, L.oct);
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
-    if (!fan_live(kc, oct, n)) return;
+    if (!fan_live(kc, n)) return;
     const int warp = (int)(threadIdx.x >> 5);
     const int b0 = (int)(blockIdx.x * (VT / 32) + warp) * VB;
     make_vertices(
-        Level1{}, sm[warp], kc->slot, b0, make_float2(oct->cx, oct->cy),
-        [&](uint32_t i) { return input_point(pts, (int64_t)i < n ? i : 0u); }, at<Kgon>(ws, L.kgon)->raw);
+        Level1{}, sm[warp], kc->slot, b0, fan_centre(*oct),
+        [&](uint32_t i) { return fan_space(input_point(pts, (int64_t)i < n ? i : 0u), oct->scale); },
+        at<Kgon>(ws, L.kgon)->raw);
 }
 
 __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layout L)
@@ -570,7 +585,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     Kgon *g = at<Kgon>(ws, L.kgon);
     const uint32_t tid = threadIdx.x;
-    const bool live = fan_live(kc, oct, n);
+    const bool live = fan_live(kc, n);
     const int b = (int)(blockIdx.x * BT + tid);
     int src = -1;
     if (live) src = vertex_source([&](int j) { return g->raw[j].x == g->raw[j].x; }, s_w, s_scan);   // block-uniform
@@ -578,7 +593,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
         if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
         return;
     }
-    const float cx = oct->cx, cy = oct->cy;
+    const float2 c = fan_centre(*oct);
     float2 v = g->raw[src];
     const float2 next = g->raw[b + 1 == kFanBins ? 0 : b + 1];
     // the next bin's vertex: its own point, or this one's again
@@ -587,7 +602,7 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
     const bool edge = v.x != w.x || v.y != w.y;
     bool gap = false;
     if (edge) {
-        r = disk_bound(cx, cy, v, w);
+        r = disk_bound(c.x, c.y, v, w);
         gap = r < 0.0f;
         if (gap) v.x = __int_as_float(0x7fc00000);
     }
@@ -602,8 +617,8 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
         if (gap) kc->gaps = 1u;
     }
     if (blockIdx.x == 0 && tid == 0) {
-        g->cx = cx;
-        g->cy = cy;
+        g->cx = c.x;
+        g->cy = c.y;
         g->ok = 1u;
         g->centre = centre_inside(*oct) ? 1u : 0u;
     }
@@ -696,14 +711,23 @@ struct PointQueue {
     uint32_t n;   // warp-uniform
 };
 
-template <class Bins>
+// SCALED: the set's scale is not 1.  (A variant of its own: the loop is bound
+// by issue.)
+template <class Bins_, bool SCALED>
 struct FanView {
+    using Bins = Bins_;
     bool fan;       // there is one
     Bins nb;
     SharedFan F;
-    float2 c;
+    float2 c;       // scaled
     float rho2t;    // r2 < rho2t proves |p - c| below the disk's radius
     bool disk;      // try the disk first
+    float scale;
+    __device__ __forceinline__ float2 space(float x, float y) const
+    {
+        if constexpr (SCALED) return fan_space(make_float2(x, y), scale);
+        return make_float2(x, y);
+    }
 };
 
 // An index with this bit (n < 2^30) is a point the octagon's forms may have
@@ -712,8 +736,8 @@ constexpr uint32_t kUnsettled = 0x80000000u;
 
 // Whether point p (i: its index and kUnsettled) survives; octs counts the
 // octagon survivors among the unsettled ones.  test: a candidate.
-template <class Bins>
-__device__ __forceinline__ bool settle(const OctSmem &so, const FanView<Bins> &f, bool test, uint32_t i, float2 p,
+template <class View>
+__device__ __forceinline__ bool settle(const OctSmem &so, const View &f, bool test, uint32_t i, float2 p,
                                        uint32_t &octs)
 {
     bool keep = true;
@@ -721,13 +745,16 @@ __device__ __forceinline__ bool settle(const OctSmem &so, const FanView<Bins> &f
         keep = keep_point<false>(so, p.x, p.y);
         octs += keep ? 1u : 0u;
     }
-    if (test || ((i & kUnsettled) && f.fan)) keep = keep && !fan_inside(f.nb, f.F, f.c, sub2(p, f.c), p);
+    if (test || ((i & kUnsettled) && f.fan)) {
+        const float2 q = f.space(p.x, p.y);
+        keep = keep && !fan_inside(f.nb, f.F, f.c, sub2(q, f.c), q);
+    }
     return keep;
 }
 
 // The last (up to) 32 points of the queue: the survivors to the list.
-template <class Bins>
-__device__ __forceinline__ void queue_drain(PointQueue &q, const FilterSmem &fs, const FanView<Bins> &f, bool test,
+template <class View>
+__device__ __forceinline__ void queue_drain(PointQueue &q, const FilterSmem &fs, const View &f, bool test,
                                             const float *__restrict__ pts, uint32_t &octs)
 {
     const uint32_t lane = lane_id(), m = min(q.n, 32u);
@@ -752,8 +779,8 @@ __device__ __forceinline__ void queue_drain(PointQueue &q, const FilterSmem &fs,
 // points, the disk test, the others going to the queue.  bits: a second
 // polygon has refined the count pass's keep bits, which then stand for the
 // octagon test.  octs counts the octagon survivors.
-template <int G, class Bins>
-__device__ __forceinline__ void filter_tiles(const FilterSmem &fs, const FanView<Bins> &f, uint32_t *queue,
+template <int G, class View>
+__device__ __forceinline__ void filter_tiles(const FilterSmem &fs, const View &f, uint32_t *queue,
                                              const float *__restrict__ pts, uint32_t n, uint32_t tile, uint32_t t1,
                                              uint32_t step, const uint16_t *bits, uint32_t &octs)
 {
@@ -781,7 +808,7 @@ __device__ __forceinline__ void filter_tiles(const FilterSmem &fs, const FanView
             float px[8], py[8];
             if (base + kFiltTile <= n) load_part<G, 8>(pts, base, t, half, px, py);
             else kept &= ~(0xffu << (8 * half)) |
-                         load_part_ragged<G, 8>(pts, n, base, t, half, f.c.x, f.c.y, px, py) << (8 * half);
+                         load_part_ragged<G, 8>(pts, n, base, t, half, fs.so.cx, fs.so.cy, px, py) << (8 * half);
             if (edges) {
                 uint32_t out8;
                 near |= oct_decide<8>(fs.so, px, py, out8);
@@ -792,14 +819,15 @@ __device__ __forceinline__ void filter_tiles(const FilterSmem &fs, const FanView
             if (use_disk) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const float dx = __fsub_rn(px[k], f.c.x), dy = __fsub_rn(py[k], f.c.y);
+                    const float2 p = f.space(px[k], py[k]);
+                    const float dx = __fsub_rn(p.x, f.c.x), dy = __fsub_rn(p.y, f.c.y);
                     if (__fmaf_rn(dx, dx, __fmul_rn(dy, dy)) < f.rho2t) in |= 1u << k;
                 }
             } else if (__any_sync(0xffffffffu, ((kept >> (8 * half)) & 0xffu) != 0u)) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     if (k % 4 == 0) asm volatile("" ::: "memory");   // four points at a time (more would spill)
-                    const float2 p = make_float2(px[k], py[k]);
+                    const float2 p = f.space(px[k], py[k]);
                     if (fan_inside(f.nb, f.F, f.c, sub2(p, f.c), p)) in |= 1u << k;
                 }
             }
@@ -906,14 +934,21 @@ __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restr
     if (oct->spec) {
         octs = filter_candidates(fs, ws, L);
     } else {
-        const FanView<Level1> f{fan, Level1{}, SharedFan(sv), make_float2(fs.so.cx, fs.so.cy),
-                                fan ? disk_limit(fan_rho2(kc)) : 0.0f, kc->gaps == 0u};
         const uint32_t ntiles = (n + kFiltTile - 1) / kFiltTile;   // (n < 2^30)
         const uint32_t gi = blockIdx.x * CG + threadIdx.x / kFiltThreads;
         const uint32_t per = (ntiles + gridDim.x * CG - 1) / (gridDim.x * CG);
-        filter_tiles<G>(fs, f, reinterpret_cast<uint32_t *>(smem_raw) + (threadIdx.x >> 5) * kQueue, pts, n, gi * per,
-                        min(ntiles, (gi + 1) * per), 1u,
-                        use_bits && (!kdev || *kdev != 8) ? at<uint16_t>(ws, L.keep_bits) : nullptr, octs);
+        uint32_t *const queue = reinterpret_cast<uint32_t *>(smem_raw) + (threadIdx.x >> 5) * kQueue;
+        const uint16_t *const bits = use_bits && (!kdev || *kdev != 8) ? at<uint16_t>(ws, L.keep_bits) : nullptr;
+        const float scale = fs.so.scale, rho2t = fan ? disk_limit(fan_rho2(kc)) : 0.0f;
+        const float2 c = fan_centre(fs.so);
+        const bool disk = kc->gaps == 0u;
+        const uint32_t t0 = gi * per, t1 = min(ntiles, (gi + 1) * per);
+        if (fan && scale != 1.0f)
+            filter_tiles<G>(fs, FanView<Level1, true>{fan, Level1{}, SharedFan(sv), c, rho2t, disk, scale}, queue, pts, n,
+                            t0, t1, 1u, bits, octs);
+        else
+            filter_tiles<G>(fs, FanView<Level1, false>{fan, Level1{}, SharedFan(sv), c, rho2t, disk, 1.0f}, queue, pts, n,
+                            t0, t1, 1u, bits, octs);
     }
     octs = __reduce_add_sync(0xffffffffu, octs);
     if (lane_id() == 0 && octs) atomicAdd(&fs.octs, octs);
@@ -944,9 +979,9 @@ constexpr int F2T = 256;
 constexpr int F2I = 8;   // survivors per thread and step of the test
 static_assert(kFan2Bins % BT == 0, "sub-bins split evenly over the build blocks");
 
-__device__ __forceinline__ float2 surv_point(const uint32_t *keys, const unsigned long long *pay, uint32_t i)
+__device__ __forceinline__ float2 surv_point(const uint32_t *keys, const unsigned long long *pay, uint32_t i, float scale)
 {
-    return make_float2(key_float(keys[i]), key_float((uint32_t)(pay[i] >> 32)));
+    return fan_space(make_float2(key_float(keys[i]), key_float((uint32_t)(pay[i] >> 32))), scale);
 }
 
 __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint32_t min_s)
@@ -965,9 +1000,9 @@ __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint3
     const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
     const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
     unsigned long long *slot = at<unsigned long long>(ws, L.fan2_slot);
-    const float cx = g->cx, cy = g->cy, r2ref = far_ref(*oct);
+    const float cx = g->cx, cy = g->cy, r2ref = far_ref(*oct), scale = oct->scale;
     for (uint32_t i = blockIdx.x * F2T + threadIdx.x; i < m; i += gridDim.x * F2T) {
-        const float2 p = surv_point(keys, pay, i);
+        const float2 p = surv_point(keys, pay, i, scale);
         const int b = vertex_bin(Level2{}, __fsub_rn(p.x, cx), __fsub_rn(p.y, cy), kFan2Margin);
         if (b < 0) continue;
         const unsigned long long v = ((unsigned long long)far_key(p.x, p.y, cx, cy, r2ref) << 32) | (uint32_t)~i;
@@ -995,9 +1030,10 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
         if (threadIdx.x == 0) f2->bad = 1u;
         return;
     }
-    float2 v = surv_point(keys, pay, ~(uint32_t)slot[src]);
+    const float scale = at<Octagon>(ws, L.oct)->scale;
+    float2 v = surv_point(keys, pay, ~(uint32_t)slot[src], scale);
     const unsigned long long nextp = slot[b + 1 == kFan2Bins ? 0 : b + 1];
-    const float2 w = nextp != 0ull ? surv_point(keys, pay, ~(uint32_t)nextp) : v;
+    const float2 w = nextp != 0ull ? surv_point(keys, pay, ~(uint32_t)nextp, scale) : v;
     const bool edge = v.x != w.x || v.y != w.y;
     // c strictly left of v -> w, proven in binary32 or exactly
     const bool gap = edge && orient(v.x, v.y, w.x, w.y, g->cx, g->cy) <= 0;
@@ -1023,6 +1059,7 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
     const bool test = !f2->bad && f2->edges != 0u;
     const Kgon *g = at<Kgon>(ws, L.kgon);
     const float2 c = make_float2(g->cx, g->cy);
+    const float scale = at<Octagon>(ws, L.oct)->scale;
     const GlobalFan F{at<float2>(ws, L.fan2_v) + 1};
     const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
     const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
@@ -1048,7 +1085,7 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
             uint32_t in = 0;
 #pragma unroll
             for (int k = 0; k < F2I; ++k) {
-                const float2 p = make_float2(key_float(kv[k]), key_float((uint32_t)(pv[k] >> 32)));
+                const float2 p = fan_space(make_float2(key_float(kv[k]), key_float((uint32_t)(pv[k] >> 32))), scale);
                 if (fan_inside(Level2{}, F, c, sub2(p, c), p)) in |= 1u << k;
             }
             keep &= ~in;
@@ -1203,11 +1240,12 @@ __global__ void __launch_bounds__(256) bx_fan_want_kernel(const float *__restric
 #pragma unroll
         for (int r = 0; r < kBxSample / 32; ++r) {
             const float x = __fsub_rn(v[r].x, o.cx), y = __fsub_rn(v[r].y, o.cy);
+            const float2 d = fan_space(make_float2(x, y), o.scale);
             float m = __int_as_float(0x7f800000);
 #pragma unroll
             for (int k = 0; k < 8; ++k) m = min_nan(m, __fmaf_rn(o.tx[k], x, __fmaf_rn(o.ty[k], y, o.tz[k])));
             out += m > 1.0f ? 0u : 1u;
-            const float r2 = __fmaf_rn(x, x, __fmul_rn(y, y));
+            const float r2 = __fmaf_rn(d.x, d.x, __fmul_rn(d.y, d.y));
             lo = fminf(lo, r2);
             hi = fmaxf(hi, r2);
         }
@@ -1338,7 +1376,8 @@ __global__ void __launch_bounds__(kFiltThreads, 5) bx_fan_bins_kernel(const floa
         if (first >= end) continue;   // block-uniform
         const Octagon &o = octs[item.x];
         const SetBins nb{info.nb};
-        const float cx = o.cx, cy = o.cy, r2ref = far_ref(o);
+        const float r2ref = far_ref(o), scale = o.scale;
+        const float2 c = fan_centre(o);
         const float *p2 = pts + 2 * S.pt_begin;
         unsigned long long *slot = bx_slots(ws, BL, S);
         const uint32_t n = (uint32_t)S.n, steps = ((end - first + st - 1) / st) * parts;   // parts of every st-th tile
@@ -1351,7 +1390,7 @@ __global__ void __launch_bounds__(kFiltThreads, 5) bx_fan_bins_kernel(const floa
                 load_part<1, BI>(p2, base, t, part, px, py);
                 live = (1u << BI) - 1u;
             } else {
-                live = load_part_ragged<1, BI>(p2, n, base, t, part, cx, cy, px, py);
+                live = load_part_ragged<1, BI>(p2, n, base, t, part, o.cx, o.cy, px, py);
             }
         };
         fetch(0);
@@ -1368,7 +1407,8 @@ __global__ void __launch_bounds__(kFiltThreads, 5) bx_fan_bins_kernel(const floa
                 qy[k] = py[k];
             }
             if (u + 1 < steps) fetch(u + 1);
-            raise_bins(nb, slot, qx, qy, mine, make_float2(cx, cy), r2ref, [&](int k) {
+            to_fan_space(qx, qy, scale);
+            raise_bins(nb, slot, qx, qy, mine, c, r2ref, [&](int k) {
                 return (uint32_t)item_point<1>((first + u / parts * st) * kFiltTile, t, (int)(BI * (u % parts)) + k);
             });
         }
@@ -1397,13 +1437,15 @@ __global__ void __launch_bounds__(VT) bx_fan_vertex_kernel(const float *__restri
             for (int k = (int)item.y + (int)threadIdx.x; k < (int)item.y + kBxBinRun; k += VT) {
                 const unsigned long long v = __ldcg(slot + k);
                 const uint32_t i = ~(uint32_t)v;
-                raw[k] = v != 0ull ? __ldg(p + ((int64_t)i < m ? i : 0u)) : make_float2(__int_as_float(0x7fc00000), 0.0f);
+                raw[k] = v != 0ull ? fan_space(__ldg(p + ((int64_t)i < m ? i : 0u)), octs[item.x].scale)
+                                   : make_float2(__int_as_float(0x7fc00000), 0.0f);
             }
             continue;   // block-uniform
         }
         make_vertices(
             SetBins{info.nb}, sm[warp], bx_slots(ws, BL, S), (int)item.y + warp * VB,
-            make_float2(octs[item.x].cx, octs[item.x].cy), [&](uint32_t i) { return __ldg(p + ((int64_t)i < m ? i : 0u)); },
+            fan_centre(octs[item.x]),
+            [&](uint32_t i) { return fan_space(__ldg(p + ((int64_t)i < m ? i : 0u)), octs[item.x].scale); },
             bx_raw(ws, BL, S));
         __syncwarp();
     }
@@ -1431,15 +1473,13 @@ __global__ void __launch_bounds__(BT, 2) bx_fan_build_kernel(const float *__rest
         float2 *V = reinterpret_cast<float2 *>(bx_slots(ws, BL, S));
         const SetBins nb{info.nb};
         const int NB = (int)nb.n;
-        const float cx = o.cx, cy = o.cy;
-        const bool off = !(__fadd_rn(__fsub_rn(o.bxh, o.bxl), __fsub_rn(o.byh, o.byl)) < 0x1p62f);
+        const float2 c = fan_centre(o);
         __syncthreads();   // the shared words of the previous set have been read
         if (tid == 0) {
             s_last = -1;
             s_inv = s_edges = s_gaps = s_in = s_seen = 0u;
         }
         __syncthreads();
-        if (off) continue;   // block-uniform
         int last = -1;   // the last bin with a vertex (what the first empty bins repeat)
         for (int b = (int)tid; b < NB; b += BT)
             if (raw[b].x == raw[b].x) last = b;
@@ -1473,7 +1513,7 @@ __global__ void __launch_bounds__(BT, 2) bx_fan_build_kernel(const float *__rest
                 const float2 next = raw[b + 1 == NB ? 0 : b + 1];
                 const float2 w = next.x == next.x ? next : v;
                 if (v.x != w.x || v.y != w.y) {
-                    const float r = disk_bound(cx, cy, v, w);
+                    const float r = disk_bound(c.x, c.y, v, w);
                     inv = max(inv, ~__float_as_uint(fmaxf(r, 0.0f)));
                     if (r < 0.0f) {
                         gaps = true;
@@ -1497,8 +1537,8 @@ __global__ void __launch_bounds__(BT, 2) bx_fan_build_kernel(const float *__rest
         const bool gap = s_gaps != 0u;
         if (!fan_holds(s_edges, gap, rho2, gap && centre_inside(o))) continue;   // block-uniform
         if (tid < (uint32_t)kBxSample) {   // (points of the first and last bins, whose neighbours wrap, are left out)
-            const float2 p = __ldg(reinterpret_cast<const float2 *>(pts) + S.pt_begin + S.n * tid / kBxSample);
-            const float2 c = make_float2(cx, cy), d = sub2(p, c);
+            const float2 p = fan_space(__ldg(reinterpret_cast<const float2 *>(pts) + S.pt_begin + S.n * tid / kBxSample), o.scale);
+            const float2 d = sub2(p, c);
             const uint32_t b = fan_bin_biased(nb, d.x, d.y) - kBinBias;
             bool in = false;
             const bool seen = b >= 1u && b + 1u < nb.n;
@@ -1568,11 +1608,16 @@ __global__ void __launch_bounds__(CT, 1) bx_hull_filter_kernel(const float *__re
         const SetInfo &S = sets[cur];
         const FanInfo &info = at<FanInfo>(ws, BL.fan)[cur];
         const bool fan = info.ready != 0u;
-        const FanView<SetBins> f{fan, SetBins{info.nb}, SharedFan(sv), make_float2(fs.so.cx, fs.so.cy),
-                                 fan ? disk_limit(info.rho2) : 0.0f, info.tight == 0u && info.rho2 > 0.0f};
+        const float scale = fs.so.scale, rho2t = fan ? disk_limit(info.rho2) : 0.0f;
+        const float2 c = fan_centre(fs.so);
+        const bool disk = info.tight == 0u && info.rho2 > 0.0f;
         const float *p = pts + 2 * S.pt_begin;
         const uint32_t first = item.y + threadIdx.x / kFiltThreads, end = min(item.y + chunk, S.ntiles);
-        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0)
+        const FanView<SetBins, false> f{fan, SetBins{info.nb}, SharedFan(sv), c, rho2t, disk, 1.0f};
+        if (fan && scale != 1.0f)
+            filter_tiles<1>(fs, FanView<SetBins, true>{fan, SetBins{info.nb}, SharedFan(sv), c, rho2t, disk, scale}, queue,
+                            p, (uint32_t)S.n, first, end, (uint32_t)CG, nullptr, octs);
+        else if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0)
             filter_tiles<2>(fs, f, queue, p, (uint32_t)S.n, first, end, (uint32_t)CG, nullptr, octs);
         else
             filter_tiles<1>(fs, f, queue, p, (uint32_t)S.n, first, end, (uint32_t)CG, nullptr, octs);
@@ -1605,7 +1650,7 @@ __global__ void __launch_bounds__(kFiltThreads, 3) bx_plain_filter_kernel(const 
         }
         if (fs.so.abort) continue;   // block-uniform
         const SetInfo &S = sets[cur];
-        const FanView<SetBins> f{false, SetBins{4u}, SharedFan(nullptr), make_float2(fs.so.cx, fs.so.cy), 0.0f, false};
+        const FanView<SetBins, false> f{false, SetBins{4u}, SharedFan(nullptr), make_float2(0.0f, 0.0f), 0.0f, false, 1.0f};
         filter_tiles<1>(fs, f, s_queue + (threadIdx.x >> 5) * kQueue, pts + 2 * S.pt_begin, (uint32_t)S.n, item.y,
                         min(item.y + (uint32_t)kPlainChunk, S.ntiles), 1u, nullptr, octs);
     }

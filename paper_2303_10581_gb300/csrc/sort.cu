@@ -43,7 +43,7 @@ constexpr int kPassBlocks = 3;   // per SM: as many as the shared memory holds
 // A digit with at most so many values among a segment's keys, or the top one
 // (the sign and most of the exponent: most keys have one of a few values),
 // takes match.any.  (Equal keys, 60 sets of 150001: 76 us a pass by words in
-// shared memory, 64 by match.any; with 16 values and more the words win.)
+// shared memory, 64 by match.any.)
 constexpr int kFewDigits = 8;
 
 template <int T>
