@@ -125,12 +125,15 @@ struct Fan2Ctrl {                          // zeroed with the control block
     uint32_t pad[2];
 };
 
+// (The vertices before empty bins are filled, x = NaN for none, lie in pay[1],
+// free until the second level or the sort: a set with a fan has kKgonMinS
+// points.)
+static_assert(kFanBins <= (int)kKgonMinS, "a set's second payload buffer holds a vertex per bin");
 struct Kgon {
     float cx, cy;                          // fan centre (it and the vertices times Octagon::scale)
     uint32_t ok;                           // 0: no fan this call
     uint32_t centre;                       // 1: c lies clearly inside the octagon
     float2 v[kFanBins];                    // vertex of every bin (x = NaN: none, and the wedges beside it keep their points)
-    float2 raw[kFanBins];                  // the same before empty bins are filled (x = NaN: none)
 };
 
 // K-direction filter polygon (kfilter.cu; the learned proposal's filter)
@@ -297,6 +300,10 @@ constexpr int kBxFanChunk = 32;       // tiles per work item of the fan sets' fi
 constexpr int kBxFanChunkMin = 8;     // the smallest tunable one (sizes the work-item lists)
 constexpr int kBxTileBins = 1024;     // a set has up to this many bins per tile of 4096 points (kFanBins at most)
 constexpr int kBxBinRun = 512;        // bins per block of the vertex kernel
+constexpr int64_t kBxFanMinN = 16384; // smaller sets get no fan
+constexpr int kBxPlainChunk = 16;     // tiles per work item of the sets without a fan
+static_assert(2 * ((kBxFanMinN + kFiltTile - 1) / kFiltTile * kBxTileBins) + 1 <= kBxFanMinN && 2 * kBxTileBins < kFiltTile,
+              "a set's stretch of the sort's payloads holds its fan tables");
 
 // The fan of a set of ch_hull_batched.
 struct FanInfo {
@@ -305,7 +312,6 @@ struct FanInfo {
     uint32_t nb;          // bins
     uint32_t ready;       // the fan's proofs hold and it drops enough points
     float rho2;           // lower bound on the squared (scaled) distance from the centre to the fan's boundary (0: none)
-    uint32_t pad[3];
 };
 
 // Extra workspace of ch_hull_batched, after the single-set regions.
@@ -325,15 +331,16 @@ struct BatchLayout {
     // the fan of the hull step, per set with many octagon survivors (kgon.cu)
     size_t soct;          // u32[B]: survivors per set (in the zeroed range)
     size_t fan;           // FanInfo[B]
-    size_t fan_set;       // u32[B]: the sets with a fan
-    size_t fan_slot;      // u64[tiles_max * kBxTileBins]: farthest sampled point per bin, a set's bins from its
-                          // first tile's; later its vertices
-    size_t fan_raw;       // float2[tiles_max * kBxTileBins]: the vertices before empty bins are filled
+    size_t fan_set;       // u32[max_fan]: the sets with a fan
+    size_t fan_tab;       // the sets' fan tables: pay[1], free until the sort.  In a set's own stretch (from the
+                          // first even point position): u64[nb], the farthest sampled point per bin, later the
+                          // vertices, then float2[nb], the vertices before empty bins are filled.  (A set with
+                          // a fan has at least kBxFanMinN points, and 2 nb + 1 <= n then.)
     size_t fan_items;     // uint2[max_items]: (set, first tile in the set) of each work item of the fan sets
-    size_t plain_items;   // uint2[max_items]: the same of the other sets
+    size_t plain_items;   // uint2[max_plain_items]: the same of the other sets
     size_t bin_items;     // uint2[max_bin_items]: (set, first bin) of each run of kBxBinRun bins
     size_t total;
-    int64_t num_sets, tiles_max, max_items, max_bin_items;
+    int64_t num_sets, tiles_max, max_fan, max_items, max_plain_items, max_bin_items;
 };
 
 __host__ __device__ inline Layout make_layout(int64_t n, int64_t sets = 0)
@@ -426,14 +433,19 @@ __host__ __device__ inline BatchLayout make_batch_layout(const Layout &L, int64_
     B.sc_off[0] = take((size_t)(B.tiles_max + 1) * 4);
     B.sc_off[1] = take((size_t)(B.tiles_max + 1) * 4);
     B.lower = L.keys[1];
-    B.max_items = B.tiles_max / kBxFanChunkMin + sets + 1;
-    B.max_bin_items = B.tiles_max * (kBxTileBins / kBxBinRun) + 1;
+    // sets with a fan, their tiles (n / kFiltTile and a ragged one each), the
+    // others' and the runs of bins
+    B.max_fan = sets < L.n / kBxFanMinN ? sets : L.n / kBxFanMinN;
+    const int64_t fan_tiles = L.n / kFiltTile + B.max_fan, runs = kBxTileBins / kBxBinRun;
+    B.max_items = fan_tiles / kBxFanChunkMin + B.max_fan + 1;
+    B.max_plain_items = B.tiles_max / kBxPlainChunk + sets + 1;
+    B.max_bin_items = (fan_tiles * runs < B.max_fan * (kFanBins / kBxBinRun) ? fan_tiles * runs
+                                                                            : B.max_fan * (kFanBins / kBxBinRun)) + 1;
     B.fan = take((size_t)sets * sizeof(FanInfo));
-    B.fan_set = take((size_t)sets * 4);
-    B.fan_slot = take((size_t)B.tiles_max * kBxTileBins * 8);
-    B.fan_raw = take((size_t)B.tiles_max * kBxTileBins * 8);
+    B.fan_set = take((size_t)B.max_fan * 4);
+    B.fan_tab = L.pay[1];
     B.fan_items = take((size_t)B.max_items * 8);
-    B.plain_items = take((size_t)B.max_items * 8);
+    B.plain_items = take((size_t)B.max_plain_items * 8);
     B.bin_items = take((size_t)B.max_bin_items * 8);
     B.total = o;
     return B;

@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(VT) fan_vertex_kernel(const float *__restrict_
     make_vertices(
         Level1{}, sm[warp], kc->slot, b0, fan_centre(*oct),
         [&](uint32_t i) { return fan_space(input_point(pts, (int64_t)i < n ? i : 0u), oct->scale); },
-        at<Kgon>(ws, L.kgon)->raw);
+        at<float2>(ws, L.pay[1]));
 }
 
 __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layout L)
@@ -584,18 +584,19 @@ __global__ void __launch_bounds__(BT) fan_build_kernel(int64_t n, void *ws, Layo
     const Octagon *oct = at<Octagon>(ws, L.oct);
     KgonCtrl *kc = at<KgonCtrl>(ws, L.kgon_ctrl);
     Kgon *g = at<Kgon>(ws, L.kgon);
+    const float2 *raw = at<float2>(ws, L.pay[1]);
     const uint32_t tid = threadIdx.x;
     const bool live = fan_live(kc, n);
     const int b = (int)(blockIdx.x * BT + tid);
     int src = -1;
-    if (live) src = vertex_source([&](int j) { return g->raw[j].x == g->raw[j].x; }, s_w, s_scan);   // block-uniform
+    if (live) src = vertex_source([&](int j) { return raw[j].x == raw[j].x; }, s_w, s_scan);   // block-uniform
     if (src < 0) {
         if (blockIdx.x == 0 && tid == 0) g->ok = 0u;
         return;
     }
     const float2 c = fan_centre(*oct);
-    float2 v = g->raw[src];
-    const float2 next = g->raw[b + 1 == kFanBins ? 0 : b + 1];
+    float2 v = raw[src];
+    const float2 next = raw[b + 1 == kFanBins ? 0 : b + 1];
     // the next bin's vertex: its own point, or this one's again
     const float2 w = next.x == next.x ? next : v;
     float r = __int_as_float(0x7f800000);
@@ -1195,10 +1196,8 @@ namespace {
 // tile, smoothed as the single set's; one whose fan drops less than an eighth
 // of a sample goes without.
 // ---------------------------------------------------------------------------
-constexpr int64_t kBxFanMinN = 16384;
 constexpr int64_t kBxTightMinN = 65536;
 constexpr int kBxSample = 256;        // points of a set's estimates
-constexpr int kPlainChunk = 16;       // tiles per work item of the sets without a fan
 static_assert(kFanBins % kBxBinRun == 0 && kBxTileBins % kBxBinRun == 0 && kBxBinRun == VB * VT / 32, "whole runs of bins");
 
 // A fan's bins and sample, by what limits it.  Points of a circle (tight)
@@ -1263,7 +1262,7 @@ __global__ void __launch_bounds__(256) bx_fan_want_kernel(const float *__restric
 }
 
 // One block: the lists of the fan sets and of all work items (runs of `chunk`
-// tiles of a fan set, of kPlainChunk tiles of another, of kBxBinRun bins).
+// tiles of a fan set, of kBxPlainChunk tiles of another, of kBxBinRun bins).
 __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, BatchLayout BL, uint32_t chunk)
 {
     kernel_entry();
@@ -1285,7 +1284,7 @@ __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, BatchLayo
             c[1] += (nt + chunk - 1) / chunk;
             c[3] += fan[b].nb / kBxBinRun;
         } else {
-            c[2] += (nt + kPlainChunk - 1) / kPlainChunk;
+            c[2] += (nt + kBxPlainChunk - 1) / kBxPlainChunk;
         }
     }
     uint32_t run[4];
@@ -1318,7 +1317,7 @@ __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, BatchLayo
             for (uint32_t t = 0; t < nt; t += chunk) fi[run[1]++] = make_uint2((uint32_t)b, t);
             for (uint32_t k = 0; k < nb; k += kBxBinRun) bi[run[3]++] = make_uint2((uint32_t)b, k);
         } else {
-            for (uint32_t t = 0; t < nt; t += kPlainChunk) pi[run[2]++] = make_uint2((uint32_t)b, t);
+            for (uint32_t t = 0; t < nt; t += kBxPlainChunk) pi[run[2]++] = make_uint2((uint32_t)b, t);
         }
     }
     if (threadIdx.x == 0) {
@@ -1330,14 +1329,15 @@ __global__ void __launch_bounds__(1024) bx_fan_select_kernel(void *ws, BatchLayo
 }
 
 // A set's slots, vertices (in the same place once the slots are read) and
-// vertices before empty bins are filled.
+// vertices before empty bins are filled (BatchLayout::fan_tab; 16-byte
+// aligned, nb is even).
 __device__ __forceinline__ unsigned long long *bx_slots(void *ws, const BatchLayout &BL, const SetInfo &S)
 {
-    return at<unsigned long long>(ws, BL.fan_slot) + (size_t)S.tile_base * kBxTileBins;
+    return at<unsigned long long>(ws, BL.fan_tab) + ((S.pt_begin + 1) & ~(int64_t)1);
 }
-__device__ __forceinline__ float2 *bx_raw(void *ws, const BatchLayout &BL, const SetInfo &S)
+__device__ __forceinline__ float2 *bx_raw(void *ws, const BatchLayout &BL, const SetInfo &S, uint32_t nb)
 {
-    return at<float2>(ws, BL.fan_raw) + (size_t)S.tile_base * kBxTileBins;
+    return reinterpret_cast<float2 *>(bx_slots(ws, BL, S) + nb);
 }
 
 __global__ void __launch_bounds__(256) bx_fan_zero_kernel(void *ws, BatchLayout BL)
@@ -1433,7 +1433,7 @@ __global__ void __launch_bounds__(VT) bx_fan_vertex_kernel(const float *__restri
         const FanInfo &info = at<FanInfo>(ws, BL.fan)[item.x];
         if (info.tight) {   // the farthest samples themselves (a chord's rounded point would lie deeper)
             const unsigned long long *slot = bx_slots(ws, BL, S);
-            float2 *raw = bx_raw(ws, BL, S);
+            float2 *raw = bx_raw(ws, BL, S, info.nb);
             for (int k = (int)item.y + (int)threadIdx.x; k < (int)item.y + kBxBinRun; k += VT) {
                 const unsigned long long v = __ldcg(slot + k);
                 const uint32_t i = ~(uint32_t)v;
@@ -1446,7 +1446,7 @@ __global__ void __launch_bounds__(VT) bx_fan_vertex_kernel(const float *__restri
             SetBins{info.nb}, sm[warp], bx_slots(ws, BL, S), (int)item.y + warp * VB,
             fan_centre(octs[item.x]),
             [&](uint32_t i) { return fan_space(__ldg(p + ((int64_t)i < m ? i : 0u)), octs[item.x].scale); },
-            bx_raw(ws, BL, S));
+            bx_raw(ws, BL, S, info.nb));
         __syncwarp();
     }
 }
@@ -1469,7 +1469,7 @@ __global__ void __launch_bounds__(BT, 2) bx_fan_build_kernel(const float *__rest
         const SetInfo &S = sets[set];
         const Octagon &o = octs[set];
         FanInfo &info = at<FanInfo>(ws, BL.fan)[set];
-        const float2 *raw = bx_raw(ws, BL, S);
+        const float2 *raw = bx_raw(ws, BL, S, info.nb);
         float2 *V = reinterpret_cast<float2 *>(bx_slots(ws, BL, S));
         const SetBins nb{info.nb};
         const int NB = (int)nb.n;
@@ -1652,7 +1652,7 @@ __global__ void __launch_bounds__(kFiltThreads, 3) bx_plain_filter_kernel(const 
         const SetInfo &S = sets[cur];
         const FanView<SetBins, false> f{false, SetBins{4u}, SharedFan(nullptr), make_float2(0.0f, 0.0f), 0.0f, false, 1.0f};
         filter_tiles<1>(fs, f, s_queue + (threadIdx.x >> 5) * kQueue, pts + 2 * S.pt_begin, (uint32_t)S.n, item.y,
-                        min(item.y + (uint32_t)kPlainChunk, S.ntiles), 1u, nullptr, octs);
+                        min(item.y + (uint32_t)kBxPlainChunk, S.ntiles), 1u, nullptr, octs);
     }
 }
 
