@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
     kernel_entry();
     __shared__ float s_h1[kHid], s_h2[kHid], s_o[kOut], s_d[kOut], s_dh2[kHid], s_part[MT / kHid][kHid];
     const int b = blockIdx.x, t = (int)threadIdx.x, lane = t & 31, warp = t >> 5;
-    const float *x = X + (int64_t)b * kIn;
+    const float *x = X + row(b, kIn);
     constexpr int PW = kHid / (MT / 32);   // layer-1 outputs per warp
     constexpr int C = kIn / 256;           // 8 inputs per lane and chunk of 256
     float xv[C][8];
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
         const float h = fmaxf(lanes_sum<32>(acc[u]) + wf(P, oB1 + warp * PW + u), 0.0f);
         if (lane == u) {
             s_h1[warp * PW + u] = h;
-            H1[b * kHid + warp * PW + u] = h;
+            H1[row(b, kHid) + warp * PW + u] = h;
         }
     }
     __syncthreads();
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
         const float h = fmaxf(lanes_sum<8>(a) + wf(P, oB2 + o8), 0.0f);
         if (l8 == 0) {
             s_h2[o8] = h;
-            H2[b * kHid + o8] = h;
+            H2[row(b, kHid) + o8] = h;
         }
     }
     __syncthreads();
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
     }
     __syncthreads();
     if constexpr (!TRAIN) {
-        if (t < kOut) OUT[b * kOut + t] = s_o[t];
+        if (t < kOut) OUT[row(b, kOut) + t] = s_o[t];
     } else {
         const float invB = 1.0f / (float)B, w = A.lam * A.mask[b];
         if (warp == 0) {   // loss, and the gradient of the logits
@@ -246,17 +246,17 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
             for (int k = 0; k < 4; ++k) {
                 if (lane == k) {
                     s_d[k] = (e[k] / z - (k == y ? 1.0f : 0.0f)) * invB;
-                    A.dOUT[b * kOut + k] = s_d[k];
+                    A.dOUT[row(b, kOut) + k] = s_d[k];
                 }
             }
-            const float d0 = s_o[4 + lane] - A.off[b * 64 + lane], d1 = s_o[36 + lane] - A.off[b * 64 + 32 + lane];
+            const float d0 = s_o[4 + lane] - A.off[row(b, 64) + lane], d1 = s_o[36 + lane] - A.off[row(b, 64) + 32 + lane];
             const float l = lanes_sum<32>(w * d0 * d0 / 64.0f + w * d1 * d1 / 64.0f);
             if (lane == 0) A.loss[b] = logf(z) + mx - s_o[y] + l;
         } else if (warp < 3) {   // the gradient of the offsets
             const int j = t - 32;
-            const float d = w * 2.0f * (s_o[4 + j] - A.off[b * 64 + j]) / 64.0f * invB;
+            const float d = w * 2.0f * (s_o[4 + j] - A.off[row(b, 64) + j]) / 64.0f * invB;
             s_d[4 + j] = d;
-            A.dOUT[b * kOut + 4 + j] = d;
+            A.dOUT[row(b, kOut) + 4 + j] = d;
         }
         __syncthreads();
         constexpr int NP = MT / kHid;        // rows of a column's sum per thread: every NP-th
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
             for (int q = 0; q < NP; ++q) a += s_part[q][t];
             const float g = s_h2[t] > 0.0f ? a : 0.0f;
             s_dh2[t] = g;
-            A.dH2[b * kHid + t] = g;
+            A.dH2[row(b, kHid) + t] = g;
         }
         __syncthreads();
         a = 0.0f;
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(MT) sample_kernel(const float *__restrict__ X,
             a = 0.0f;
 #pragma unroll
             for (int q = 0; q < NP; ++q) a += s_part[q][t];
-            A.dH1[b * kHid + t] = s_h1[t] > 0.0f ? a : 0.0f;
+            A.dH1[row(b, kHid) + t] = s_h1[t] > 0.0f ? a : 0.0f;
         }
     }
 }
@@ -416,8 +416,8 @@ extern "C" ch_status ch_mlp_train_step(const float *X, int32_t B, const int32_t 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     __nv_bfloat16 *P = static_cast<__nv_bfloat16 *>(params);
     // scratch: H1, H2 (B x 64 each), dOUT (B x 68), dH1, dH2 (B x 64 each)
-    float *H1 = scratch, *H2 = H1 + (int64_t)B * kHid, *dOUT = H2 + (int64_t)B * kHid;
-    float *dH1 = dOUT + (int64_t)B * kOut, *dH2 = dH1 + (int64_t)B * kHid;
+    float *H1 = scratch, *H2 = H1 + row(B, kHid), *dOUT = H2 + row(B, kHid);
+    float *dH1 = dOUT + row(B, kOut), *dH2 = dH1 + row(B, kHid);
     const LossArgs A{label, off, mask, lam, dOUT, dH1, dH2, loss};
     if (vec16(X, params)) sample_kernel<true, true><<<B, MT, 0, st>>>(X, B, P, H1, H2, nullptr, A);
     else sample_kernel<false, true><<<B, MT, 0, st>>>(X, B, P, H1, H2, nullptr, A);

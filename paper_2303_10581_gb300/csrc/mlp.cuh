@@ -25,6 +25,10 @@ constexpr int oW3 = oB2 + kHid;
 constexpr int oB3 = oW3 + kOut * kHid;
 constexpr int kParams = oB3 + kOut;
 
+// Where row b of a [B][w] array starts (a batch's outputs pass 2^31 elements at
+// 31.6 million samples).
+__host__ __device__ inline int64_t row(int64_t b, int w) { return b * w; }
+
 __device__ __forceinline__ float wf(const __nv_bfloat16 *P, int i) { return __bfloat162float(P[i]); }
 
 // The learned proposal for one point set in one block (ch_hull_learned):
