@@ -190,11 +190,11 @@ def algorithmic_bytes(kernel, n, s_list, t_list, f_list=None, spec_list=None):
         # read points (unless the sweep served), write key + payload per point kept
         return sum((0 if sp else 8 * n) + 12 * f for f, sp in zip(f_list, spec_list))
     if kernel == "kgon":
-        # the fan over the octagon survivors when it ran (their coordinates;
-        # hulls test them in the filter's pass, and this group then only
-        # makes the vertices: an upper bound); otherwise only samples.  The second level reads the
-        # first level's survivors twice (sub-bin maxima, test: key +
-        # payload) and copies the points it keeps
+        # kernels that test the octagon survivors against the fan themselves
+        # (their coordinates) when it ran; otherwise only samples.  A second
+        # level reads the first level's survivors twice (sub-bin maxima, test:
+        # key + payload) and copies the points it keeps.  ch_hull tests them in
+        # the filter's pass: fan_group_bytes
         return sum((8 * s if f < s else 0) + (24 * f + 24 * t if t < f else 0)
                    for s, t, f in zip(s_list, t_list, f_list))
     big = [t for t in t_list if t > SMALL_SORT]
@@ -207,6 +207,23 @@ def algorithmic_bytes(kernel, n, s_list, t_list, f_list=None, spec_list=None):
     if kernel == "chain":
         return sum(12 * t for t in t_list if t > SMALL_HULL)   # read the sorted keys and payloads once
     return None
+
+
+FAN_BIN_TILES, TILE = 1536, 4096   # the fan's sample: about so many tiles of so many points
+
+
+def fan_group_bytes(n, t_list, f_list, spec_list):
+    """Bytes that ch_hull's fan group (vertices and second level; the test of
+    every point is the filter's) must move in one step: the sampled tiles'
+    points, and in the second level the first one's survivors twice (key +
+    payload: sub-bin maxima, test) and the kept ones' copies.  Sets that the
+    speculative sweep served, and those of fewer than 2^16 points, have no
+    fan."""
+    tiles = -(-n // TILE)
+    stride = max(1, min(16, tiles // FAN_BIN_TILES))
+    sample = 8 * min(n, -(-tiles // stride) * TILE) if n >= 1 << 16 else 0
+    return sum((0 if sp else sample) + (24 * f + 12 * t if t < f else 0)
+               for t, f, sp in zip(t_list, f_list, spec_list))
 
 
 def load_traffic(kernel):
@@ -252,8 +269,9 @@ def traffic_per_launch(kernel, tr, n, s_list, t_list, f_list, spec_list, dists, 
 
 
 def alu_roofline(dom_ms, dom_launches, steps, n, s_list, t_list, clk, dev, dists=None, f_list=None):
-    """Roofline of the fan kernels, which are bound by instruction issue,
-    not by HBM: warp instructions issued per second against the SMs' issue
+    """Roofline of fan kernels that test the octagon survivors themselves
+    (records with warp_inst_per_survivor; ch_hull's fan group does not, and
+    run_ours takes fan_group_bytes): bound by instruction issue, not by HBM: warp instructions issued per second against the SMs' issue
     rate (4 warp schedulers per SM, one warp instruction each per clock, at
     the highest SM clock seen).  The instructions per octagon survivor come
     from ncu captures (profiles/traffic.json, per distribution of the
@@ -457,17 +475,16 @@ def run_ours(args):
     dom_ms, dom_launches = probe[dominant]
     peak, peak_kind = peaks()
     roof = None
-    if dom_launches and dominant == "kgon":
-        roof = alu_roofline(dom_ms, dom_launches, args.steps, n, surv, sorted_pts, clk, dev, list(DISTS), fan1)
-    if dom_launches and roof is None:
-        per_step_bytes = algorithmic_bytes(dominant, n, surv, sorted_pts, fan1, spec)
+    if dom_launches:
+        per_step_bytes = (fan_group_bytes(n, sorted_pts, fan1, spec) if dominant == "kgon"
+                          else algorithmic_bytes(dominant, n, surv, sorted_pts, fan1, spec))
         if per_step_bytes is not None:
             # algorithmic bytes of all timed launches over their summed event
             # time (= per-launch bytes over the average launch duration)
             per_launch_bytes = per_step_bytes * args.steps / dom_launches
             avg_ms = dom_ms / dom_launches
             achieved = per_step_bytes * args.steps / (dom_ms * 1e-3) / 1e9
-            tr = load_traffic(dominant)
+            tr = load_traffic(dominant) if dominant != "kgon" else None
             roof = {"kernel": dominant, "bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
                     "unit": "GB/s", "frac": round(achieved / peak, 4), "peak_source": peak_kind,
                     "traffic": traffic_per_launch(dominant, tr, n, surv, sorted_pts, fan1, spec, list(DISTS),
