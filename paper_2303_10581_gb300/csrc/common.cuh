@@ -27,10 +27,6 @@ constexpr int kFiltMaxBlocks = 4096;                  // grid cap of the two-pas
 // blocks): shares that differ by one tile at most.  (Equal shares, the last
 // blocks without any, left 119 of 608 blocks idle on 2442 tiles.)
 __host__ __device__ inline int64_t first_tile(int64_t tiles, int64_t blocks, int64_t b) { return b * tiles / blocks; }
-__host__ __device__ inline int64_t tile_block(int64_t tiles, int64_t blocks, int64_t t)
-{
-    return ((t + 1) * blocks - 1) / tiles;
-}
 constexpr int kSortTile = 4096;       // keys per sort tile
 constexpr int kSortPasses = 4;        // 32-bit x keys, 8-bit digits
 constexpr int kLeafC = 16;            // points per leaf chain (one thread)
@@ -203,7 +199,6 @@ struct SpecCtrl {                         // written anew by every call that spe
 // polygon it picks (K and the directions)
 struct LearnScratch {
     float feat[1024];
-    float h1[64], h2[64];
     float out[68];
     float dirs[2 * kMaxDirs];
     int32_t K;

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kFiltThreads) filter_kernel(const float *__res
 // Count pass: the exact test of every candidate; the slots of a segment's
 // survivors go to utmp (unordered), their number to skept, and each count
 // block's total to the block totals the fan reads.
-__device__ void spec_count(const Octagon &so, void *ws, const Layout &L, uint32_t (&s_w)[NW])
+__device__ void spec_count(const Octagon &so, void *ws, const Layout &L)
 {
     SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const float2 *cpt = at<float2>(ws, L.pay[1]);
@@ -333,7 +333,6 @@ __device__ void spec_count(const Octagon &so, void *ws, const Layout &L, uint32_
             block_total += s_k;
         }
     }
-    (void)s_w;
     if (threadIdx.x == 0) at<uint32_t>(ws, L.filt_bsum)[blockIdx.x] = block_total;
 }
 
@@ -346,9 +345,8 @@ struct SpecScatterSmem {
 // offset (the survivors of the segments before it); block 0 writes the
 // count.  A segment with more survivors than shared memory holds is ranked
 // from global memory (slower, same result).
-template <bool KEYS>
 __device__ void spec_scatter(SpecScatterSmem &sm, void *ws, const Layout &L, uint32_t *surv_idx, float2 *surv_pts,
-                             uint32_t *surv_count, uint32_t *out_keys, unsigned long long *out_pay)
+                             uint32_t *surv_count)
 {
     const SpecCtrl *sc = at<SpecCtrl>(ws, L.spec);
     const uint32_t *cidx = at<uint32_t>(ws, L.keys[1]);
@@ -366,7 +364,7 @@ __device__ void spec_scatter(SpecScatterSmem &sm, void *ws, const Layout &L, uin
             uint32_t total = 0;
 #pragma unroll
             for (int w = 0; w < NW; ++w) total += sm.red[w];
-            write_count(KEYS, at<Ctrl>(ws, L.ctrl), surv_count, total);
+            *surv_count = total;
         }
     }
     for (uint32_t j = blockIdx.x; j < nseg; j += gridDim.x) {
@@ -397,13 +395,8 @@ __device__ void spec_scatter(SpecScatterSmem &sm, void *ws, const Layout &L, uin
                 for (uint32_t q = 0; q < k; ++q) r += cidx[seg0 + kept_slot[seg0 + q]] < mine ? 1u : 0u;
             const float2 p = cpt[seg0 + slot];
             const size_t pos = (size_t)off + r;
-            if constexpr (KEYS) {
-                out_keys[pos] = ord_key(p.x);
-                out_pay[pos] = ((unsigned long long)ord_key(p.y) << 32) | mine;
-            } else {
-                surv_idx[pos] = mine;
-                if (surv_pts) surv_pts[pos] = p;
-            }
+            surv_idx[pos] = mine;
+            if (surv_pts) surv_pts[pos] = p;
         }
     }
 }
@@ -457,7 +450,7 @@ __global__ void __launch_bounds__(kFiltThreads, 4) filter_count_kernel(const flo
     if (!load_octagon(so, ws, L)) return;   // (its barrier also covers s_cnt)
     if constexpr (!BOX) {
         if (so.spec) {   // the speculative sweep proved all but its candidates inside
-            spec_count(so, ws, L, s_w);
+            spec_count(so, ws, L);
             return;
         }
     }
@@ -525,7 +518,6 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
     __shared__ uint32_t s_nlist;
     __shared__ uint32_t s_row[2][kFiltItems / G][NW];
     __shared__ uint32_t s_spec;
-    __shared__ SpecScatterSmem s_sp;
     Ctrl *ctrl = at<Ctrl>(ws, L.ctrl);
     if (threadIdx.x == 0) {
         const Octagon *oct = at<Octagon>(ws, L.oct);
@@ -537,10 +529,12 @@ __global__ void __launch_bounds__(kFiltThreads, 3) filter_scatter_kernel(const f
         if (blockIdx.x == 0 && threadIdx.x == 0) write_count(KEYS, ctrl, surv_count, 0);
         return;
     }
-    if (s_spec) {   // only the speculative sweep's candidates can survive
-        spec_scatter<KEYS>(s_sp, ws, L, surv_idx, surv_pts, surv_count, at<uint32_t>(ws, L.keys[0]),
-                           at<unsigned long long>(ws, L.pay[0]));
-        return;
+    if constexpr (!KEYS) {   // (the hull step takes the candidates itself)
+        __shared__ SpecScatterSmem s_sp;
+        if (s_spec) {   // only the speculative sweep's candidates can survive
+            spec_scatter(s_sp, ws, L, surv_idx, surv_pts, surv_count);
+            return;
+        }
     }
     const unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
     const uint32_t *bsum = at<uint32_t>(ws, L.filt_bsum);
@@ -712,11 +706,10 @@ cudaError_t launch_filter_keys_single(const float *pts, int64_t n, void *ws, con
 }
 
 cudaError_t launch_filter_count(const float *pts, int64_t n, const int32_t *kdev, void *ws, const Layout &L,
-                                int64_t *grid, cudaStream_t st)
+                                cudaStream_t st)
 {
     const bool vec = (reinterpret_cast<uintptr_t>(pts) & 15u) == 0;
     const int64_t bc = vec ? count_blocks<2, false>(n) : count_blocks<1, false>(n);
-    *grid = bc;
     probe_before(CH_K_FILTER, st);
     if (vec) launch_next(filter_count_kernel<2, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, kdev);
     else launch_next(filter_count_kernel<1, false>, (unsigned)bc, kFiltThreads, 0, st, pts, n, ws, L, kdev);

@@ -534,11 +534,10 @@ __global__ void __launch_bounds__(ST) kx_sv_extremes_kernel(const float *__restr
 }
 
 // The survivors' exact test against the K-gon: bits of kept points strictly
-// inside it are cleared, and the tile's count and its count block's total
-// drop by the number removed (bc: the count pass's grid).
+// inside it are cleared (only the bits are read after this).
 template <int G>
 __global__ void __launch_bounds__(ST) kx_sv_refine_kernel(const float *__restrict__ pts, int64_t n,
-                                                          const int32_t *kdev, int K, void *ws, Layout L, int32_t bc)
+                                                          const int32_t *kdev, int K, void *ws, Layout L)
 {
     kernel_entry();
     __shared__ KPoly sp;
@@ -552,11 +551,9 @@ __global__ void __launch_bounds__(ST) kx_sv_refine_kernel(const float *__restric
     }
     __syncthreads();
     uint16_t *bits = at<uint16_t>(ws, L.keep_bits);
-    unsigned long long *status = at<unsigned long long>(ws, L.filt_status);
-    uint32_t *bsum = at<uint32_t>(ws, L.filt_bsum);
     const float2 *p2 = reinterpret_cast<const float2 *>(pts);
     const int64_t ntiles = ceil_div(n, (int64_t)kFiltTile);
-    const uint32_t t = threadIdx.x, lane = lane_id();
+    const uint32_t t = threadIdx.x;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const uint32_t kb = bits[tile * kFiltThreads + t];
         uint32_t gone = 0;
@@ -566,19 +563,12 @@ __global__ void __launch_bounds__(ST) kx_sv_refine_kernel(const float *__restric
             if (!kx_keep(sp, v.x, v.y)) gone |= 1u << q;
         }
         if (gone) bits[tile * kFiltThreads + t] = (uint16_t)(kb & ~gone);
-        uint32_t removed = __popc(gone);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, o);
-        if (lane == 0 && removed) {
-            atomicAdd(&status[tile], 0ull - (unsigned long long)removed);
-            atomicSub(&bsum[tile_block(ntiles, bc, tile)], removed);
-        }
     }
 }
 
 template <int G>
 cudaError_t launch_kx_sv_stage(const float *pts, int64_t n, const float *dirs, const int32_t *kdev, int K,
-                               uint32_t *ext_out, void *ws, const Layout &L, int64_t bc, cudaStream_t st)
+                               uint32_t *ext_out, void *ws, const Layout &L, cudaStream_t st)
 {
     const int64_t ntiles = ceil_div(n, (int64_t)kFiltTile);
     // the device's choice is mostly "no second polygon": a grid of one block
@@ -590,7 +580,7 @@ cudaError_t launch_kx_sv_stage(const float *pts, int64_t n, const float *dirs, c
     else if (K == 16) launch_next(kx_sv_extremes_kernel<16, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
     else if (K == 32) launch_next(kx_sv_extremes_kernel<32, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
     else launch_next(kx_sv_extremes_kernel<64, G>, g, ST, 0, st, pts, n, dirs, kdev, ext_out, ws, L);
-    launch_next(kx_sv_refine_kernel<G>, g, ST, 0, st, pts, n, kdev, K, ws, L, (int32_t)bc);
+    launch_next(kx_sv_refine_kernel<G>, g, ST, 0, st, pts, n, kdev, K, ws, L);
     note_kernels(CH_K_KGON, 2);
     probe_after(CH_K_KGON, st);
     return cudaGetLastError();
@@ -654,11 +644,11 @@ cudaError_t launch_kx_count(const float *pts, int64_t n, int K, void *ws, const 
 }
 
 cudaError_t launch_kx_sv(const float *pts, int64_t n, const float *dirs, const int32_t *kdev, int K, uint32_t *ext_out,
-                        void *ws, const Layout &L, int64_t bc, cudaStream_t st)
+                        void *ws, const Layout &L, cudaStream_t st)
 {
     const bool vec = (reinterpret_cast<uintptr_t>(pts) & 15u) == 0;
-    return vec ? launch_kx_sv_stage<2>(pts, n, dirs, kdev, K, ext_out, ws, L, bc, st)
-               : launch_kx_sv_stage<1>(pts, n, dirs, kdev, K, ext_out, ws, L, bc, st);
+    return vec ? launch_kx_sv_stage<2>(pts, n, dirs, kdev, K, ext_out, ws, L, st)
+               : launch_kx_sv_stage<1>(pts, n, dirs, kdev, K, ext_out, ws, L, st);
 }
 
 

@@ -1175,9 +1175,8 @@ cudaError_t launch_hull_filter(const float *pts, int64_t n, void *ws, const Layo
 {
     const bool bits = kg && (kg->kdev || kg->K != 8);   // the second polygon's keep bits
     if (bits) {
-        int64_t bc = 0;
-        cudaError_t e = launch_filter_count(pts, n, kg->kdev, ws, L, &bc, st);
-        if (e == cudaSuccess) e = launch_kx_sv(pts, n, kg->dirs, kg->kdev, kg->K, kg->ext_out, ws, L, bc, st);
+        cudaError_t e = launch_filter_count(pts, n, kg->kdev, ws, L, st);
+        if (e == cudaSuccess) e = launch_kx_sv(pts, n, kg->dirs, kg->kdev, kg->K, kg->ext_out, ws, L, st);
         if (e != cudaSuccess) return e;
     }
     const int32_t *kdev = bits ? kg->kdev : nullptr;

@@ -63,10 +63,10 @@ cudaError_t launch_filter(const float *pts, int64_t n, void *ws, const Layout &L
 // the hull step's survivors (sort keys and payloads in buffer 0) with the
 // single-pass schedule
 cudaError_t launch_filter_keys_single(const float *pts, int64_t n, void *ws, const Layout &L, cudaStream_t st);
-// the count pass alone (the data's own extremes), its grid in *grid; kdev:
-// the device's choice of K, 8: the pass returns at once
+// the count pass alone (the data's own extremes), for its keep bits; kdev: the
+// device's choice of K, 8: the pass returns at once
 cudaError_t launch_filter_count(const float *pts, int64_t n, const int32_t *kdev, void *ws, const Layout &L,
-                                int64_t *grid, cudaStream_t st);
+                                cudaStream_t st);
 
 // A second polygon of ch_hull (two passes only): the K-direction polygon
 // over the octagon's survivors (launch_kx_sv).
@@ -98,15 +98,10 @@ cudaError_t launch_kx_count(const float *pts, int64_t n, int K, void *ws, const 
                             cudaStream_t st);
 
 // a K-direction polygon over the octagon's survivors, refining the count
-// pass's keep bits (bc blocks); K is the host's (16, 32, 64; 8: nothing)
+// pass's keep bits; K is the host's (16, 32, 64; 8: nothing)
 // or, with kdev, the device's choice.  ext_out (nullable): its vertices.
 cudaError_t launch_kx_sv(const float *pts, int64_t n, const float *dirs, const int32_t *kdev, int K, uint32_t *ext_out,
-                        void *ws, const Layout &L, int64_t bc, cudaStream_t st);
-// the learned proposal in one block (mlp.cu): features, the MLP, the choice
-// of K and the directions, into the workspace's LearnScratch
-cudaError_t launch_learned_choice(const float *pts, int64_t n, const void *params, void *ws, const Layout &L,
-                                  cudaStream_t st);
-
+                        void *ws, const Layout &L, cudaStream_t st);
 // hull step: the survivors of the octagon (or of the second polygon kg),
 // less the points inside a fan of triangles around the centre where that
 // pays, as sort keys and payloads; their number in Ctrl::surv_count

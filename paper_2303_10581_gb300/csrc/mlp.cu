@@ -29,8 +29,6 @@ namespace {
 
 using namespace mlp;
 
-
-
 // One block of 1024 threads per point set.
 __global__ void __launch_bounds__(1024) features_kernel(const float *__restrict__ pts, int64_t n, float *__restrict__ feat)
 {
@@ -359,28 +357,6 @@ inline bool vec16(const float *X, const void *P)
 
 }  // namespace
 
-namespace {
-
-// ch_hull_learned's proposal in one block (mlp.cuh)
-__global__ void __launch_bounds__(mlp::LT) learned_choice_kernel(const float *__restrict__ pts, int64_t n,
-                                                                 const __nv_bfloat16 *__restrict__ P, LearnScratch *ls)
-{
-    mlp::learned_choice_block(pts, n, P, ls);
-}
-
-}  // namespace
-
-cudaError_t launch_learned_choice(const float *pts, int64_t n, const void *params, void *ws, const Layout &L,
-                                  cudaStream_t st)
-{
-    probe_before(CH_K_KGON, st);
-    learned_choice_kernel<<<1, mlp::LT, 0, st>>>(pts, n, static_cast<const __nv_bfloat16 *>(params),
-                                                at<LearnScratch>(ws, L.learn));
-    note_kernels(CH_K_KGON, 1);
-    probe_after(CH_K_KGON, st);
-    return cudaGetLastError();
-}
-
 }  // namespace ch
 
 using namespace ch;
@@ -428,7 +404,9 @@ extern "C" ch_status ch_mlp_train_step(const float *X, int32_t B, const int32_t 
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ERR_CUDA;
 }
 
-// Floats of scratch that ch_mlp_train_step needs for a batch of B.
+// Floats of scratch for ch_mlp_train_step with a batch of B.  (It uses B (4
+// kHid + kOut) of them; the number is the one that callers have always been
+// given, with room for the outputs and the gradients.)
 extern "C" int64_t ch_mlp_scratch_floats(int32_t B)
 {
     return (int64_t)B * (4 * kHid + 2 * kOut) + kParams;

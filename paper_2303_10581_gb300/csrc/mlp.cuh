@@ -32,7 +32,7 @@ __host__ __device__ inline int64_t row(int64_t b, int w) { return b * w; }
 __device__ __forceinline__ float wf(const __nv_bfloat16 *P, int i) { return __bfloat162float(P[i]); }
 
 // The learned proposal for one point set in one block (ch_hull_learned):
-// the features of features_kernel, the MLP of forward_kernel with each
+// the features of features_kernel, the MLP of sample_kernel with each
 // output's dot product spread over a warp (lanes take every 32nd input,
 // then a shuffle sum), and the choice: K from the arg-max of the four
 // K-logits (lowest on ties; a NaN logit never wins), the offsets (units of
