@@ -81,20 +81,14 @@ __device__ __forceinline__ bool test8(const OctSmem &so, const float (&px)[8], c
 }
 
 // Exact decisions for the kept ones (load(q) reads point q), some of which
-// the affine forms left undecided; the next point is on its way meanwhile.
+// the affine forms left undecided.
 template <bool BOX, class Load>
 __device__ __forceinline__ uint32_t settle_near(const OctSmem &so, uint32_t keep, Load load)
 {
-    uint32_t m = keep;
-    if (!m) return 0u;
-    float2 p = load(__ffs(m) - 1);
 #pragma unroll 1
-    while (m) {
-        const uint32_t bit = m & (0u - m);
-        m ^= bit;
-        const float2 next = m ? load(__ffs(m) - 1) : p;
-        if (!keep_point<BOX>(so, p.x, p.y)) keep ^= bit;
-        p = next;
+    for (uint32_t m = keep; m; m &= m - 1u) {
+        const float2 p = load(__ffs(m) - 1);
+        if (!keep_point<BOX>(so, p.x, p.y)) keep &= ~(m & (0u - m));
     }
     return keep;
 }
