@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(CT, 1) hull_filter_kernel(const float *__restr
         const uint16_t *const bits = use_bits && (!kdev || *kdev != 8) ? at<uint16_t>(ws, L.keep_bits) : nullptr;
         const float scale = fs.so.scale, rho2t = fan ? disk_limit(fan_rho2(kc)) : 0.0f;
         const float2 c = fan_centre(fs.so);
-        const bool disk = kc->gaps == 0u;
+        const bool disk = fan && kc->gaps == 0u;
         const uint32_t t0 = gi * per, t1 = min(ntiles, (gi + 1) * per);
         if (fan && scale != 1.0f)
             filter_tiles<G>(fs, FanView<Level1, true>{fan, Level1{}, SharedFan(sv), c, rho2t, disk, scale}, queue, pts, n,
