@@ -733,8 +733,10 @@ __device__ __forceinline__ void superchunk(ChainSmem<LT> &sm, const ChainPtrs &P
                     };
                     const uint32_t upto = hm & (lt | (1u << lane));
                     const int start = upto ? 31 - __clz(upto) : 0;
+                    // (runs are short: 1053 -> 1020 us on those points)
+                    const int reach = (int)__reduce_max_sync(0xffffffffu, in ? (uint32_t)(lane - start) : 0u);
 #pragma unroll 1
-                    for (int o = 1; o < 32; o <<= 1) {
+                    for (int o = 1; o <= reach; o <<= 1) {
                         const float y1 = __shfl_up_sync(0xffffffffu, ylo, o), y2 = __shfl_up_sync(0xffffffffu, yhi, o);
                         const uint32_t i1 = __shfl_up_sync(0xffffffffu, ilo, o), i2 = __shfl_up_sync(0xffffffffu, ihi, o);
                         const int e1 = __shfl_up_sync(0xffffffffu, lo, o), e2 = __shfl_up_sync(0xffffffffu, hi, o);
@@ -863,7 +865,10 @@ __device__ __forceinline__ void superchunk(ChainSmem<LT> &sm, const ChainPtrs &P
         // ---- elimination, half of the block per side: rounds of one pass over
         // the whole sequence, each warp its share, then passes inside the
         // shares (their ends stay), then the shares closed up again; done when
-        // the first pass of a round drops nothing
+        // the first pass of a round drops nothing.  Many super-chunks are bound
+        // by issue, so a share is whole steps of a pass, and of a short sequence
+        // fewer warps have one (3 10^7 unfiltered circle points, this kernel:
+        // 1242 us with even shares, 1053 so)
         {
             const int side = warp / NWS, gw = warp % NWS;
             uint16_t *const X = sm.seq + (side ? n0 : 0), *const Y = X + SY;
@@ -872,7 +877,7 @@ __device__ __forceinline__ void superchunk(ChainSmem<LT> &sm, const ChainPtrs &P
 #pragma unroll 1
             while (!strict) {
                 if (whole) {
-                    const int S = (len + NWS - 1) / NWS;
+                    const int S = ((len + NWS - 1) / NWS + 63) & ~63;
                     w0 = min(gw * S, len);
                     wl = min(S, len - w0);
                     in_y = false;
