@@ -585,12 +585,25 @@ __device__ __forceinline__ int orient_f32(float ax, float ay, float bx, float by
     return detsum <= 3.0e38f ? o : 2;
 }
 
+// A product r = fl(a b) whose rounding error fma(a, b, -r) is exact, as it
+// cannot underflow (or r is an exact zero).
+__device__ __forceinline__ bool exact_product(float a, float b, float r)
+{
+    return a == 0.0f || b == 0.0f || (fabsf(r) >= 0x1p-100f && fabsf(r) <= 3.0e38f);
+}
+
 // Tier 2: the differences as exact pairs (two-diff), the products and their
 // rounding errors (FMA), everything of second order added up in binary32: the
 // sign when the bound proves it, 2 otherwise.  With eps = 2^-24 the second-
 // order terms are below 6 eps detsum in sum, so their ten roundings and the
 // omitted product of two low parts cost less than 64 eps^2 detsum = 2^-42
-// detsum, and 2^-138 absorbs products in the subnormal range.  It settles
+// detsum, and 2^-138 absorbs products in the subnormal range.  Where the four
+// differences are exact (points near one another or of a grid) the products
+// p + pe, q + qe are too: rounding is monotone, so p > q implies p + pe > q +
+// qe, and for p == q the sign is that of pe - qe, which survives its rounding;
+// so points that are exactly collinear are settled as well, a third of the
+// neighbours' turns where a ring is dense (3 10^7 points, the chain kernel 1020
+// us with these left to the next tier, 864 so).  It settles
 // nearly every near-collinear triple of a ring's neighbours.  In binary64 (at
 // a 64th of the rate here, some 70 cycles an instruction) one such lane held
 // its warp for a thousand cycles.
@@ -607,18 +620,17 @@ __device__ __forceinline__ int orient_pair(float ax, float ay, float bx, float b
     float s, sl;
     two_diff(p, q, s, sl);
     const float t = __fadd_rn(__fadd_rn(__fsub_rn(pe, qe), __fsub_rn(pl, ql)), sl);
+    const uint32_t low = (__float_as_uint(ul) | __float_as_uint(vl) | __float_as_uint(wl) | __float_as_uint(zl)) << 1;
+    if (low == 0u && exact_product(u, v, p) && exact_product(w, z, q)) {
+        const float d = p != q ? __fsub_rn(p, q) : __fsub_rn(pe, qe);
+        return d > 0.0f ? 1 : (d < 0.0f ? -1 : 0);
+    }
     const float det = __fadd_rn(s, t), detsum = __fadd_rn(fabsf(p), fabsf(q));
     const float eb = __fmaf_ru(detsum, 0x1p-42f, 0x1p-138f);
     const int o = det > eb ? 1 : (-det > eb ? -1 : 2);
     return detsum <= 3.0e38f ? o : 2;
 }
 
-// A product r = fl(a b) whose rounding error fma(a, b, -r) is exact, as it
-// cannot underflow (or r is an exact zero).
-__device__ __forceinline__ bool exact_product(float a, float b, float r)
-{
-    return a == 0.0f || b == 0.0f || (fabsf(r) >= 0x1p-100f && fabsf(r) <= 3.0e38f);
-}
 // Whether a b == c d, proven.
 __device__ __forceinline__ bool same_product(float a, float b, float c, float d)
 {
@@ -632,10 +644,6 @@ __device__ __forceinline__ bool same_product(float a, float b, float c, float d)
 //  - A difference that is zero is exact, so a product with one is zero
 //    whatever its other factor (equal points, points on an axis-parallel
 //    edge).
-//  - Where the four differences are exact (points near one another or of a
-//    grid) the products p + pe, q + qe are too; rounding is monotone, so p > q
-//    implies p + pe > q + qe, and for p == q the sign is that of pe - qe, which
-//    survives its rounding.
 //  - The determinant is zero when its expanded products cancel in pairs.
 // In binary64 they took most of the time of such sets: 60 sets of 150001
 // points on a square's sides 3345 us (1102 so), of a diagonal 4856 (931).
@@ -648,13 +656,6 @@ static __device__ __noinline__ int orient_last(float ax, float ay, float bx, flo
     two_diff(ay, cy, w, wl);
     two_diff(bx, cx, z, zl);
     if ((u == 0.0f || v == 0.0f) && (w == 0.0f || z == 0.0f)) return 0;
-    const uint32_t low = (__float_as_uint(ul) | __float_as_uint(vl) | __float_as_uint(wl) | __float_as_uint(zl)) << 1;
-    const float p = __fmul_rn(u, v), q = __fmul_rn(w, z);
-    if (low == 0u && exact_product(u, v, p) && exact_product(w, z, q)) {
-        if (p != q) return p > q ? 1 : -1;
-        const float d = __fsub_rn(__fmaf_rn(u, v, -p), __fmaf_rn(w, z, -q));
-        return d > 0.0f ? 1 : (d < 0.0f ? -1 : 0);
-    }
     if (same_product(u, v, w, z) && same_product(ul, vl, wl, zl) &&
         ((same_product(u, vl, w, zl) && same_product(ul, v, wl, z)) ||
          (same_product(u, vl, wl, z) && same_product(ul, v, w, zl))))
