@@ -471,11 +471,23 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
             }
         }
     }
-    Best b;   // the ragged tile and the unpaired points, point by point
+    Best b;   // the unpaired points and the ragged tile, point by point, in the order of their indices
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         b.k[j] = __int_as_float(0x7fc00000);  // NaN: no candidate yet
         b.i[j] = 0xffffffffu;
+    }
+    // the point before the aligned body (warp 0 of block 0, whose segment comes
+    // first): before this thread's other points, as the first of a key stays
+    if (blockIdx.x == 0 && warp == 0 && head) {
+        const bool mine = lane == 0;
+        const float x = pts[0], y = pts[1];
+        if (mine) {
+            nan_seen |= (x != x) | (y != y);
+            consider(b, x, y, 0);
+        }
+        if constexpr (SPEC)
+            if (spec_live) spec_warp_point(box, mine, 0, x, y, wcnt, cap, sc, cidx, cpt, slice0);
     }
     if ((int64_t)blockIdx.x * per <= nfull && nfull < t1) {   // this block holds the ragged last tile
         const int64_t q0 = nfull * kExtPairs;
@@ -497,19 +509,8 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
             }
         }
     }
-    // the point before the aligned body (warp 0 of block 0, whose segment
-    // comes first) and the odd point after it (warp 0 of the last block,
-    // whose segment comes last)
-    if (blockIdx.x == 0 && warp == 0 && head) {
-        const bool mine = lane == 0;
-        const float x = pts[0], y = pts[1];
-        if (mine) {
-            nan_seen |= (x != x) | (y != y);
-            consider(b, x, y, 0);
-        }
-        if constexpr (SPEC)
-            if (spec_live) spec_warp_point(box, mine, 0, x, y, wcnt, cap, sc, cidx, cpt, slice0);
-    }
+    // the odd point after the aligned body (warp 0 of the last block, whose
+    // segment comes last)
     if (blockIdx.x == nsweep - 1 && warp == 0 && (n - head) % 2 == 1) {
         const bool mine = lane == 0;
         const int64_t i = n - 1;
