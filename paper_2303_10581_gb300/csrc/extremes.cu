@@ -322,6 +322,23 @@ __device__ __forceinline__ void spec_warp_point(const SpecBox &b, bool valid, ui
     }
 }
 
+// Of the lanes of a warp that hold a slot's largest key (lane 4 j's holders:
+// slot j's), those whose tile is the first of theirs.  (Out of line: only ties
+// come here.)
+static __device__ __noinline__ uint32_t first_holders(uint32_t holders, const int32_t (*btile)[kExtThreads])
+{
+    const uint32_t lane = lane_id();
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+        const bool holds = (__shfl_sync(0xffffffffu, holders, 4 * j) >> lane) & 1u;
+        const uint32_t bt = (uint32_t)btile[j][threadIdx.x];
+        const uint32_t first = __reduce_min_sync(0xffffffffu, holds ? bt : 0xffffffffu);
+        const uint32_t w = __ballot_sync(0xffffffffu, holds && bt == first);
+        if ((int)(lane >> 2) == j) holders = w;
+    }
+    return holders;
+}
+
 // One sweep: eight running extremes per thread (per tile, the maxima of the
 // thread's points and the first tile reaching a larger key; the point in
 // it is found at the end), warp + block reduction, grid finish by packed
@@ -526,11 +543,15 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
         if (lane == 0) sc->scnt[blockIdx.x * kSpecWarps + warp] = min(wcnt, cap);
 
     // the full tiles' winners: per slot, the lanes holding the warp's largest
-    // key; their tiles are read again for the first point with that key, four
-    // lanes per slot (one per pair of points a thread has in a tile), so that
-    // all slots' reads are one latency (one slot after the other took 8 us)
+    // key in the first tile that has it; that tile is read again for the first
+    // point with the key, four lanes per slot (one per pair of points a thread
+    // has in a tile), so that all slots' reads are one latency (one slot after
+    // the other took 8 us), until a lane's first pair has the key: the lanes
+    // after it and the pairs behind it come later in the tile.  (Where many
+    // points share an extreme, a set on a box's sides, reading every holder's
+    // pairs took 9 us: 3 10^6 such points 22 us the call, 15 so)
     static_assert(U == 4, "four lanes re-read a thread's pairs of a tile");
-    uint32_t wmask = 0;   // of this lane's slot: the lanes holding the largest key
+    uint32_t wmask = 0;   // of this lane's slot: those lanes
     float wkey = 0.0f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -544,26 +565,30 @@ __global__ void __launch_bounds__(kExtThreads, 2) extremes_kernel(const float *_
         }
     }
     __syncwarp();   // the other lanes' tiles
+    if (__any_sync(0xffffffffu, (wmask & (wmask - 1u)) != 0u)) wmask = first_holders(wmask, s_btile);
     const int wslot = (int)(lane >> 2);
     uint32_t widx = 0xffffffffu;
-    for (uint32_t m = wmask; m; m &= m - 1u) {   // ties: every holder
-        const uint32_t th = (warp << 5) + (uint32_t)(__ffs(m) - 1);
-        const int64_t q = (int64_t)s_btile[wslot][th] * kExtPairs + (lane & 3u) * kExtThreads + th;
-        const float4 v = p4[q];
-        float ka[8], kb[8];
-        slot_keys(v.x, v.y, ka);
-        slot_keys(v.z, v.w, kb);
-        float a = ka[0], d = kb[0];
+    for (uint32_t m = wmask; __any_sync(0xffffffffu, m != 0u);) {   // (the slots step together)
+        if (m) {
+            const uint32_t th = (warp << 5) + (uint32_t)(__ffs(m) - 1);
+            const int64_t q = (int64_t)s_btile[wslot][th] * kExtPairs + (lane & 3u) * kExtThreads + th;
+            const float4 v = p4[q];
+            float ka[8], kb[8];
+            slot_keys(v.x, v.y, ka);
+            slot_keys(v.z, v.w, kb);
+            float a = ka[0], d = kb[0];
 #pragma unroll
-        for (int j = 1; j < 8; ++j) {
-            a = wslot == j ? ka[j] : a;
-            d = wslot == j ? kb[j] : d;
+            for (int j = 1; j < 8; ++j) {
+                a = wslot == j ? ka[j] : a;
+                d = wslot == j ? kb[j] : d;
+            }
+            const uint32_t i0 = (uint32_t)(head + 2 * q);
+            if (d == wkey) widx = min(widx, i0 + 1u);
+            if (a == wkey) widx = min(widx, i0);
+            m &= m - 1u;
         }
-        const uint32_t i0 = (uint32_t)(head + 2 * q);
-        if (d == wkey) widx = min(widx, i0 + 1u);
-        if (a == wkey) widx = min(widx, i0);
+        if (__shfl_sync(0xffffffffu, widx, (int)(lane & ~3u)) != 0xffffffffu) m = 0u;
     }
-    __syncwarp();
     widx = min(widx, __shfl_xor_sync(0xffffffffu, widx, 1));
     widx = min(widx, __shfl_xor_sync(0xffffffffu, widx, 2));
     if ((lane & 3u) == 0u) {   // lane 4 j: slot j's candidate joins its own of the ragged ends
