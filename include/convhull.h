@@ -216,7 +216,8 @@ ch_status ch_hull_learned(const float *pts, int64_t n, const void *params, float
  * knob's range.  The Python package's autotuner sweeps these on a
  * workload and caches the best in JSON. */
 typedef enum {
-    CH_TUNE_BX_EXTREMES = 0,    /* extremes sweep, blocks per SM 1..64 (default 8)          */
+    CH_TUNE_BX_EXTREMES = 0,    /* extremes sweep, blocks per SM 1..64 (default: one wave of 1024 threads an
+                                   SM, i.e. 4, 2 or 1 blocks for 16, 8 or 4 points per thread) */
     CH_TUNE_BX_FILTER = 1,      /* filter of the sets without a fan, blocks per SM (default 3) */
     CH_TUNE_BX_SORT_PASS = 2,   /* radix-sort passes, blocks per SM (default: occupancy)     */
     CH_TUNE_BX_EMIT = 3,        /* chain compaction, blocks per SM (default 4)              */

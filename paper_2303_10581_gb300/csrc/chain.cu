@@ -193,7 +193,7 @@ __device__ void merge_walk(Acc &A, int side, int fa, int la, int fb, int lb)
 }
 
 // ---------------------------------------------------------------------------
-// in-block state; one side (lower or upper) is processed at a time
+// in-block state
 // ---------------------------------------------------------------------------
 template <int LT>
 __device__ __forceinline__ void side_barrier(int side)   // of the warps that work on one side
@@ -517,8 +517,9 @@ __device__ __forceinline__ void block_extreme_y(ChainSmem<LT> &s, float ylo, uns
 
 // Stages the m <= SC unsorted survivors at `base` in the order of x (equal x
 // in any order): pts and perm.  Each warp sorts 32 keys at a time in registers
-// (a bitonic network), then runs are merged in pairs: every key finds its
-// place from its rank in its own run and a binary search in the other.
+// (a bitonic network), then runs are merged in pairs by merge path (Odeh, Green
+// et al. 2012): a thread finds by binary search where its stretch of the
+// output begins in both runs and merges that stretch.
 // Bound by latency.  A set that fits one block need not be written back
 // between digits: the histogram and four passes over global memory take 57 us
 // on 4200 survivors, this 27 on 4096.  (Every key by a binary search in the
@@ -973,7 +974,7 @@ __device__ __forceinline__ void superchunk(ChainSmem<LT> &sm, const ChainPtrs &P
             sm.hi[t] = (int16_t)(h - 1);
             sm.first[t] = sm.last[t] = (int16_t)(h > 0 ? t : -1);
             __syncwarp();
-            // ---- merge tree: five levels inside the warp, then three across warps
+            // ---- merge tree: five levels inside the warp, then three (256 threads) or four (512) across warps
             const SmemAcc<LT> A{sm, flat};
             for (int w = 1; w < 32; w *= 2) {
                 if (lane < 32 / (2 * w)) {

@@ -66,9 +66,9 @@ struct Octagon {
     uint32_t valid;         // bit k: edge k has non-zero length
     uint32_t has_edges;     // at least one valid edge
     uint32_t abort;         // non-finite input: later stages do nothing
-    uint32_t spec;          // 1: the speculative sweep's candidates hold every survivor (spec.cu)
+    uint32_t spec;          // 1: the speculative sweep's candidates hold every survivor
     float xl, xh, yl, yh;   // closed quick-discard rectangle (xl > xh: none)
-    float cx, cy;           // bounding-box centre, for the edge order
+    float cx, cy;           // bounding-box centre: origin of the affine forms, centre of the fan
     float bxl, bxh, byl, byh;   // closed bounding box of the eight vertices
     uint32_t box_check;     // 1: points may lie outside that box (caller-supplied vertices)
     float scale;            // power of two: the fan works on points times this (1 for boxes of ordinary sizes)
@@ -744,8 +744,8 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
 // end first.  Every thread passes here, before any return, so a kernel's
 // completion implies that of all kernels before it.  A call's pipeline holds
 // up to a dozen kernels that find nothing to do for a given set, each 2.8 us
-// when launched the ordinary way: ch_hull of 1000 points 62 -> 40 us, of 2^20
-// normal points 105 -> 68, of 10^8 circle points 970 -> 919.  No kernel lets the
+// when launched the ordinary way: ch_hull of 1000 points 62 -> 42 us, of 2^20
+// normal points 105 -> 68, of 10^8 circle points 970 -> 928.  No kernel lets the
 // next one in earlier (launch_dependents): its blocks would then fill the
 // first SMs to become free, and grids of fewer blocks than the chip holds
 // would run on half of it (circle 1057, 2^20 normal points 75).

@@ -395,7 +395,7 @@ __device__ __forceinline__ T edge_bound(float cx, float cy, float2 v, float2 w, 
     return lo * lo / (len2 * ((T)1 + (T)16 * U)) * ((T)1 - (T)16 * U);
 }
 
-// In binary32 first (27648 binary64 quotients on 28 SMs would take 15 us),
+// In binary32 first (27648 binary64 quotients on 27 SMs would take 15 us),
 // in binary64 where that proves nothing: a value in binary32, rounded down.
 __device__ __forceinline__ float disk_bound(float cx, float cy, float2 v, float2 w)
 {
