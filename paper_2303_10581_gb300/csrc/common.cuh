@@ -238,7 +238,7 @@ struct Layout {
     size_t utmp;          // u32[n]
     size_t spec, p0;        // SpecCtrl, the speculative sweep's test region (SpecBox, extremes.cu)
     size_t learn;           // the learned proposal's scratch (LearnScratch)
-    size_t fan2_v;          // float2[fan2_bins + 3]: the second fan level's vertices, the ends repeated
+    size_t fan2_v;          // float2[fan2_bins + 4]: the second fan level's vertices, the ends repeated
     size_t total;
     int64_t n, filt_tiles, sort_tiles, n_chunks, n_nodes, emit_tiles;
     int64_t fan2_bins;      // kFan2Bins for sets of at least kFan2MinN points, else 0 (no second level)
@@ -398,7 +398,7 @@ __host__ __device__ inline Layout make_layout(int64_t n, int64_t sets = 0)
     L.spec = take(sizeof(SpecCtrl));
     L.p0 = take(256);
     L.learn = take(sizeof(LearnScratch));
-    L.fan2_v = take((size_t)(L.fan2_bins + 3) * 8);
+    L.fan2_v = take((size_t)(L.fan2_bins + 4) * 8);
     L.total = o;
     return L;
 }

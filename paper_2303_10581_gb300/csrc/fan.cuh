@@ -49,8 +49,11 @@ __device__ __forceinline__ float fan_phi(Bins nb, float dx, float dy)
     return __fmaf_rn(fan_turn(dx, dy), nb.quarter(), left ? 3.0f * nb.quarter() : nb.quarter());
 }
 
-// kBinBias + its bin, the bin in [0, NB] (a NaN: kBinBias + NB): the same FMA
+// kBinBias + its bin, the bin in [-1, NB] (a NaN: kBinBias + NB): the same FMA
 // shifted by 2^23 and rounded down leaves the bin in the low mantissa bits.
+// (-1: straight below, a reciprocal one ulp too large makes t less than -1.  A
+// table that is read at such an index has an entry, and one beside it, on
+// either side; inner_bin tells where one is not wanted.)
 constexpr uint32_t kBinBias = 0x4b000000u;
 template <class Bins>
 __device__ __forceinline__ uint32_t fan_bin_biased(Bins nb, float dx, float dy)
@@ -60,6 +63,10 @@ __device__ __forceinline__ uint32_t fan_bin_biased(Bins nb, float dx, float dy)
                               left ? 0x1p23f + 3.0f * nb.quarter() : 0x1p23f + nb.quarter());
     return min(__float_as_uint(f), kBinBias + nb.count());
 }
+
+// Whether bin b (less kBinBias, modulo 2^32) has neighbours on both sides: in
+// [1, nb - 2].
+__host__ __device__ inline bool inner_bin(uint32_t b, uint32_t nb) { return b - 1u < nb - 2u; }
 
 // The direction of pseudo-angle a (|x| + |y| = 1).
 template <class Bins>

@@ -77,7 +77,7 @@ namespace {
 
 constexpr int CT = 768;                  // threads per block of the filter pass: groups
 constexpr int CG = CT / kFiltThreads;    // groups of kFiltThreads, each with its own tiles
-constexpr int kFanTable = (kFanBins + 4) * 8;  // vertices, the last again before them and the first two after them (and padding)
+constexpr int kFanTable = (kFanBins + 4) * 8;  // vertices, the last two again before them and the first two after them
 constexpr int kQueue = 64;                     // points a warp of the filter pass queues (under 32, and 32 more)
 constexpr uint32_t kMany = 128;                // a warp's survivors of a tile that go straight to the list
 constexpr int kQueueSmem = CT / 32 * kQueue * 4;
@@ -119,12 +119,12 @@ struct SharedFan {
 // The same in global memory.
 struct GlobalFan {
     const float2 *V;
-    __device__ __forceinline__ const float2 *at(uint32_t biased) const { return V + (biased - kBinBias); }
+    __device__ __forceinline__ const float2 *at(uint32_t biased) const { return V + (int)(biased - kBinBias); }   // (may be -1)
     __device__ __forceinline__ float2 get(const float2 *a, int d) const { return __ldg(a + d); }
 };
 
 // Strictly inside the fan, proven (see the top of the file).  F: the
-// vertices; before the first comes the last, after the last the first two
+// vertices; before the first come the last two, after the last the first two
 // again; d = fl(p - c).  Two vertices are read: in shared memory the reads of
 // 32 random bins conflict (six wavefronts each), and a third would bound the
 // pass.
@@ -893,6 +893,7 @@ __device__ __forceinline__ void load_fan(float2 *sv, const float2 *V, int nb)
 #pragma unroll 4
     for (int i = threadIdx.x; i < nb / 2; i += blockDim.x) dst[i] = __ldg(src + i);
     if (threadIdx.x == 0) {
+        sv[-2] = __ldg(V + nb - 2);
         sv[-1] = __ldg(V + nb - 1);
         sv[nb] = __ldg(V);
         sv[nb + 1] = __ldg(V + 1);
@@ -1012,7 +1013,7 @@ __global__ void __launch_bounds__(F2T) fan2_max_kernel(void *ws, Layout L, uint3
 }
 
 // One thread per sub-bin, as fan_build_kernel; the table's ends are repeated
-// at V[-1] and V[kFan2Bins], V[kFan2Bins + 1].
+// at V[-2], V[-1] and V[kFan2Bins], V[kFan2Bins + 1].
 __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
 {
     kernel_entry();
@@ -1024,7 +1025,7 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
     const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
     const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
     const Kgon *g = at<Kgon>(ws, L.kgon);
-    float2 *V = at<float2>(ws, L.fan2_v) + 1;
+    float2 *V = at<float2>(ws, L.fan2_v) + 2;
     const int b = (int)(blockIdx.x * BT + threadIdx.x);
     const int src = vertex_source([&](int j) { return slot[j] != 0ull; }, s_w, s_scan);
     if (src < 0) {   // no survivor reached a slot: keep everything
@@ -1041,7 +1042,7 @@ __global__ void __launch_bounds__(BT) fan2_build_kernel(void *ws, Layout L)
     if (gap) v.x = __int_as_float(0x7fc00000);
     V[b] = v;
     if (b < 2) V[kFan2Bins + b] = v;
-    if (b == kFan2Bins - 1) V[-1] = v;
+    if (b >= kFan2Bins - 2) V[b - kFan2Bins] = v;
     const uint32_t edges = __popc(__ballot_sync(0xffffffffu, edge && !gap));
     if (lane_id() == 0 && edges) atomicAdd(&f2->edges, edges);
 }
@@ -1061,7 +1062,7 @@ __global__ void __launch_bounds__(F2T) fan2_test_kernel(void *ws, Layout L)
     const Kgon *g = at<Kgon>(ws, L.kgon);
     const float2 c = make_float2(g->cx, g->cy);
     const float scale = at<Octagon>(ws, L.oct)->scale;
-    const GlobalFan F{at<float2>(ws, L.fan2_v) + 1};
+    const GlobalFan F{at<float2>(ws, L.fan2_v) + 2};
     const uint32_t *keys = at<uint32_t>(ws, L.keys[0]);
     const unsigned long long *pay = at<unsigned long long>(ws, L.pay[0]);
     uint32_t *okeys = at<uint32_t>(ws, L.keys[1]);
@@ -1540,7 +1541,7 @@ __global__ void __launch_bounds__(BT, 2) bx_fan_build_kernel(const float *__rest
             const float2 d = sub2(p, c);
             const uint32_t b = fan_bin_biased(nb, d.x, d.y) - kBinBias;
             bool in = false;
-            const bool seen = b >= 1u && b + 1u < nb.n;
+            const bool seen = inner_bin(b, nb.n);
             if (seen) {
                 const float2 Q = __ldcg(V + b);
                 float e1, e2;
